@@ -356,7 +356,10 @@ int ridfa_last_status(const ridfa_program *prog, void *stream);
 int ridfa_last_timings(const ridfa_program *prog, float *reach_ms, float *join_ms);
 
 /* The reach plan of the last ridfa_recognize / ridfa_recognize_dfa / ridfa_recognize_host call of
- * `prog` on the current device (diagnostics; the automatic choices the tuning fields override). */
+ * `prog` on the current device (diagnostics; the automatic choices the tuning fields override).
+ * A call with the automatic tuning on an automaton whose runs merge runs in the stream kernels,
+ * which have tables and a launch shape of their own; the report then describes the general reach
+ * kernel's plan for the same call, the one that explicit tuning fields start from. */
 typedef struct {
     uint32_t table_mode;    /* table layout, numbered as ridfa_tuning::table_mode (1..11) */
     uint32_t text_path;     /* 1 global loads, 3 staged, 4 staged two chunks a lane, 5 set path */

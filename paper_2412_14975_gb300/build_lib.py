@@ -25,7 +25,7 @@ def _cuda_home():
 
 def sources():
     return [os.path.join(CSRC, f) for f in sorted(os.listdir(CSRC))
-            if f.endswith((".cu", ".cpp", ".h"))] + [os.path.join(INC, "ridfa.h")]
+            if f.endswith((".cu", ".cpp", ".h", ".cuh"))] + [os.path.join(INC, "ridfa.h")]
 
 
 def up_to_date():

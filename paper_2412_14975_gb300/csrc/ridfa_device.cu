@@ -31,10 +31,13 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "ridfa_internal.h"
+#include "ridfa_join.cuh"
 #include "ridfa_reach.cuh"
+#include "ridfa_stream.h"
 
 namespace ridfa {
 // --------------------------------------------------------------------------- host side
@@ -43,37 +46,68 @@ int cuda_fail(cudaError_t e) {
     return e == cudaErrorMemoryAllocation ? RIDFA_E_NOMEM : RIDFA_E_CUDA;
 }
 
-int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) {
+int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
     D.device = dev;
-    const size_t bt = H.trans.size() * 2, bf = H.final_bits.size() * 4, bi = H.ifmask.size() * 4,
-                 bs = H.slot_state.size() * 2, ba = static_cast<size_t>(H.n_states) * 2;
-    auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
-    const size_t total = al(bt) + al(256) + al(bf) + al(bi) + al(bs) + al(ba);
-    uint8_t *base = nullptr;
-    cudaError_t e = cudaMalloc(&base, total);
-    if (e != cudaSuccess) return cuda_fail(e);
-    size_t off = 0;
-    D.trans = reinterpret_cast<uint16_t *>(base + off); off += al(bt);
-    D.classmap = base + off; off += al(256);
-    D.final_bits = reinterpret_cast<uint32_t *>(base + off); off += al(bf);
-    D.ifmask = reinterpret_cast<uint32_t *>(base + off); off += al(bi);
-    D.slot_state = reinterpret_cast<uint16_t *>(base + off); off += al(bs);
-    D.all_states = reinterpret_cast<uint16_t *>(base + off); off += al(ba);
-    D.bytes = total;
     std::vector<uint16_t> iota(H.n_states);
     for (uint32_t i = 0; i < H.n_states; ++i) iota[i] = static_cast<uint16_t>(i);
-    e = cudaMemcpy(D.trans, H.trans.data(), bt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(D.classmap, H.classmap.data(), 256, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && bf) e = cudaMemcpy(D.final_bits, H.final_bits.data(), bf, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && bi) e = cudaMemcpy(D.ifmask, H.ifmask.data(), bi, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && bs) e = cudaMemcpy(D.slot_state, H.slot_state.data(), bs, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && ba) e = cudaMemcpy(D.all_states, iota.data(), ba, cudaMemcpyHostToDevice);
+    // all tables in one host image, one allocation and one copy
+    std::vector<uint8_t> img;
+    auto put = [&](const void *src, size_t n) {
+        const size_t off = img.size();
+        img.resize(off + ((n + 255) & ~static_cast<size_t>(255)));
+        if (n) std::memcpy(img.data() + off, src, n);
+        return off;
+    };
+    auto put_v = [&](const auto &v) { return put(v.data(), v.size() * sizeof(v[0])); };
+    const HostMerge &G = H.merge;
+    const HostStream &T = H.stream;
+    const size_t o_trans = put_v(H.trans), o_cls = put_v(H.classmap), o_fin = put_v(H.final_bits), o_ifm = put_v(H.ifmask),
+                 o_slot = put_v(H.slot_state), o_all = put_v(iota);
+    const bool stream = T.kind != kStreamNone;
+    size_t o_next = 0, o_leaf = 0, o_np = 0, o_ni = 0, o_img = 0, o_part = 0, o_alive = 0, o_code = 0, o_words = 0;
+    if (stream) {
+        o_next = put_v(G.next);
+        o_leaf = put_v(G.leaf);
+        o_np = put_v(G.node_part);
+        o_ni = put_v(G.node_img);
+        o_img = put_v(G.images);
+        o_part = put_v(G.part);
+        o_alive = put_v(G.slot_alive);
+        o_code = put_v(T.byte_code);
+        o_words = put_v(T.words);
+    }
+    uint8_t *base = nullptr;
+    cudaError_t e = cudaMalloc(&base, img.size());
+    if (e != cudaSuccess) return cuda_fail(e);
+    e = cudaMemcpy(base, img.data(), img.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(base);
         D = DeviceAutomaton{};
         return cuda_fail(e);
     }
+    auto u16 = [&](size_t off) { return reinterpret_cast<uint16_t *>(base + off); };
+    auto u32 = [&](size_t off) { return reinterpret_cast<uint32_t *>(base + off); };
+    D.trans = u16(o_trans);
+    D.classmap = base + o_cls;
+    D.final_bits = u32(o_fin);
+    D.ifmask = u32(o_ifm);
+    D.slot_state = u16(o_slot);
+    D.all_states = u16(o_all);
+    if (stream) {
+        D.mg_next = u16(o_next);
+        D.mg_leaf = u32(o_leaf);
+        D.mg_node_part = u16(o_np);
+        D.mg_node_img = u32(o_ni);
+        D.mg_images = u16(o_img);
+        D.mg_part = u16(o_part);
+        D.mg_slot_alive = u32(o_alive);
+        D.st_code = u32(o_code);
+        D.st_words = u32(o_words);
+    }
+    D.bytes = img.size();
     return RIDFA_OK;
+} catch (const std::bad_alloc &) {
+    return RIDFA_E_NOMEM;
 }
 
 const DeviceAutomaton *device_copy(const ridfa_program *P, bool dfa, int dev, int *err) {
@@ -111,208 +145,6 @@ int smem_optin_limit() {
 
 namespace {
 
-// ------------------------------------------------------------------------------- join
-struct JoinArgs {
-    Automaton A;
-    uint32_t c;
-    const uint16_t *maps;
-    const uint32_t *dinfo;
-    uint32_t *status;
-    uint32_t *partials;       // [gridDim.x][2 + kMaxD]
-    uint32_t *ticket;
-    uint8_t *accept;
-    uint32_t per_thread;      // boundaries per thread
-    ridfa_shard_summary *summary;   // non-null: write the shard's relation instead of accept
-};
-
-// Distinct defined values of lambda_i, ascending (at most kMaxD; caller checked m <= kMaxD).
-__device__ uint32_t distinct_of(const JoinArgs &p, uint32_t i, uint16_t *D) {
-    const uint32_t info = p.dinfo[i];
-    const uint32_t m = info >> 16;
-    if (m <= 1) {
-        D[0] = static_cast<uint16_t>(info & 0xFFFF);
-        return m;
-    }
-    const uint16_t *row = p.maps + static_cast<uint64_t>(i) * p.A.k;
-    uint32_t cnt = 0;
-    for (uint32_t a = 0; a < p.A.k; ++a) {
-        const uint16_t v = row[a];
-        if (v == kUndef) continue;
-        uint32_t j = 0;
-        while (j < cnt && D[j] < v) ++j;
-        if (j < cnt && D[j] == v) continue;
-        if (cnt == kMaxD) return 0xFFFFFFFFu;
-        for (uint32_t t = cnt; t > j; --t) D[t] = D[t - 1];
-        D[j] = v;
-        ++cnt;
-    }
-    return cnt;
-}
-
-__device__ __forceinline__ uint32_t index_of(const uint16_t *D, uint32_t m, uint16_t v) {
-    for (uint32_t j = 0; j < m; ++j)
-        if (D[j] == v) return j;
-    return 0xFFFFFFFFu;
-}
-
-// Row x of M_i: bits y with lambda_i(a) = D_i[y] for some slot a in if_min({D_{i-1}[x]}).
-__device__ uint32_t transfer_row(const JoinArgs &p, uint32_t i, uint16_t d_prev, const uint16_t *D,
-                                 uint32_t m, bool *bad) {
-    const uint32_t *mask = p.A.ifmask + static_cast<uint64_t>(d_prev) * p.A.kw;
-    const uint16_t *row = p.maps + static_cast<uint64_t>(i) * p.A.k;
-    uint32_t out = 0;
-    for (uint32_t w = 0; w < p.A.kw; ++w) {
-        uint32_t bits = mask[w];
-        while (bits) {
-            const uint32_t a = w * 32 + __ffs(bits) - 1;
-            bits &= bits - 1;
-            const uint16_t v = row[a];
-            if (v == kUndef) continue;
-            const uint32_t y = index_of(D, m, v);
-            if (y == 0xFFFFFFFFu) *bad = true;
-            else out |= 1u << y;
-        }
-    }
-    return out;
-}
-
-// Product of a thread's run of boundaries: rows over D_{s-1}, columns over D_{e-1}.
-struct Prod {
-    uint32_t nrows;           // 0xFFFFFFFF = identity (no boundary)
-    uint32_t rows[kMaxD];
-};
-
-__device__ void compose(Prod &a, const Prod &b) {   // a <- a x b
-    if (b.nrows == 0xFFFFFFFFu) return;
-    if (a.nrows == 0xFFFFFFFFu) {
-        a = b;
-        return;
-    }
-    for (uint32_t x = 0; x < a.nrows; ++x) {
-        uint32_t bits = a.rows[x], out = 0;
-        while (bits) {
-            const uint32_t z = __ffs(bits) - 1;
-            bits &= bits - 1;
-            out |= b.rows[z];
-        }
-        a.rows[x] = out;
-    }
-}
-
-__device__ bool is_final(const Automaton &A, uint32_t s) {
-    return s < A.n && ((A.final_bits[s >> 5] >> (s & 31)) & 1);
-}
-
-// Shard summary when some chunk has more than kMaxD distinct end states (block 0 alone):
-// for every distinct state x the shard's first chunk ends in, propagate if_min({x}) chunk by
-// chunk and record the end states reached, as bits over the last chunk's distinct end states.
-__device__ void summary_wide(const JoinArgs &p, uint32_t *s_vec, uint32_t *s_nvec) {
-    const Automaton &A = p.A;
-    const uint32_t tid = threadIdx.x;
-    ridfa_shard_summary *S = p.summary;
-    __shared__ uint16_t s_out[RIDFA_MAX_SLOTS];
-    __shared__ uint32_t s_nout, s_bits[RIDFA_MAX_SLOTS / 32];
-    const uint16_t *row0 = p.maps;
-    const uint16_t *last = p.maps + static_cast<uint64_t>(p.c - 1) * A.k;
-    if (tid == 0) {
-        // distinct defined end states of the last chunk, ascending
-        uint32_t n = 0;
-        for (uint32_t a = 0; a < A.k; ++a) {
-            const uint16_t v = last[a];
-            if (v == kUndef) continue;
-            uint32_t j = 0;
-            while (j < n && s_out[j] < v) ++j;
-            if (j < n && s_out[j] == v) continue;
-            for (uint32_t t = n; t > j; --t) s_out[t] = s_out[t - 1];
-            s_out[j] = v;
-            ++n;
-        }
-        s_nout = n;
-        S->k = A.k;
-        S->n_out = n;
-    }
-    __syncthreads();
-    for (uint32_t a = tid; a < RIDFA_MAX_SLOTS; a += blockDim.x) {
-        S->out_state[a] = a < s_nout ? s_out[a] : kUndef;
-        S->entry[a] = a < A.k ? row0[a] : kUndef;
-        for (uint32_t w = 0; w < RIDFA_MAX_SLOTS / 32; ++w) S->reach[a][w] = 0;
-    }
-    __syncthreads();
-    for (uint32_t a0 = 0; a0 < A.k; ++a0) {
-        const uint16_t x = row0[a0];
-        if (x == kUndef) continue;
-        bool seen = false;                    // handled with an earlier slot of the same state
-        for (uint32_t b = 0; b < a0 && !seen; ++b) seen = row0[b] == x;
-        if (seen) continue;
-        if (tid < RIDFA_MAX_SLOTS / 32) s_bits[tid] = 0;
-        __syncthreads();
-        if (p.c == 1) {
-            if (tid == 0)
-                for (uint32_t y = 0; y < s_nout; ++y)
-                    if (s_out[y] == x) s_bits[y >> 5] |= 1u << (y & 31);
-        } else {
-            for (uint32_t w = tid; w < A.kw; w += blockDim.x) s_vec[w] = A.ifmask[static_cast<uint64_t>(x) * A.kw + w];
-            __syncthreads();
-            for (uint32_t i = 1; i + 1 < p.c; ++i) {
-                for (uint32_t w = tid; w < A.kw; w += blockDim.x) s_nvec[w] = 0;
-                __syncthreads();
-                const uint16_t *row = p.maps + static_cast<uint64_t>(i) * A.k;
-                for (uint32_t a = tid; a < A.k; a += blockDim.x) {
-                    if (!((s_vec[a >> 5] >> (a & 31)) & 1)) continue;
-                    const uint16_t v = row[a];
-                    if (v == kUndef) continue;
-                    for (uint32_t w = 0; w < A.kw; ++w) {
-                        const uint32_t m = A.ifmask[static_cast<uint64_t>(v) * A.kw + w];
-                        if (m) atomicOr(&s_nvec[w], m);
-                    }
-                }
-                __syncthreads();
-                for (uint32_t w = tid; w < A.kw; w += blockDim.x) s_vec[w] = s_nvec[w];
-                __syncthreads();
-            }
-            for (uint32_t a = tid; a < A.k; a += blockDim.x) {
-                if (!((s_vec[a >> 5] >> (a & 31)) & 1) || last[a] == kUndef) continue;
-                for (uint32_t y = 0; y < s_nout; ++y)
-                    if (s_out[y] == last[a]) atomicOr(&s_bits[y >> 5], 1u << (y & 31));
-            }
-        }
-        __syncthreads();
-        for (uint32_t a = tid; a < A.k; a += blockDim.x)
-            if (row0[a] == x)
-                for (uint32_t w = 0; w < RIDFA_MAX_SLOTS / 32; ++w) S->reach[a][w] = s_bits[w];
-        __syncthreads();
-    }
-}
-
-// Shard summary from the chain product (thread 0 of the last block): tot maps the first chunk's
-// distinct end states D_1 to the last chunk's D_c.
-__device__ void summary_matrix(const JoinArgs &p, const Prod &tot) {
-    const Automaton &A = p.A;
-    ridfa_shard_summary *S = p.summary;
-    uint16_t D0[kMaxD], Dl[kMaxD];
-    const uint32_t m0 = distinct_of(p, 0, D0);
-    const uint32_t ml = distinct_of(p, p.c - 1, Dl);
-    if (m0 == 0xFFFFFFFFu || ml == 0xFFFFFFFFu || (p.c > 1 && tot.nrows == 0xFFFFFFFFu)) {
-        atomicOr(p.status, kStatusBad);
-        return;
-    }
-    S->k = A.k;
-    S->n_out = ml;
-    for (uint32_t y = 0; y < RIDFA_MAX_SLOTS; ++y) S->out_state[y] = y < ml ? Dl[y] : kUndef;
-    for (uint32_t a = 0; a < RIDFA_MAX_SLOTS; ++a) {
-        const uint16_t x = a < A.k ? p.maps[a] : kUndef;
-        S->entry[a] = x;
-        uint32_t bits = 0;
-        if (x != kUndef) {
-            const uint32_t xi = index_of(D0, m0, x);
-            if (xi == 0xFFFFFFFFu) atomicOr(p.status, kStatusBad);
-            else bits = p.c == 1 ? (1u << xi) : tot.rows[xi];
-        }
-        S->reach[a][0] = bits;
-        for (uint32_t w = 1; w < RIDFA_MAX_SLOTS / 32; ++w) S->reach[a][w] = 0;
-    }
-}
-
 __global__ void __launch_bounds__(kJoinThreads) rid_join_kernel(JoinArgs p) {
     __shared__ Prod s_prod[kJoinThreads];
     __shared__ bool s_last;
@@ -324,45 +156,8 @@ __global__ void __launch_bounds__(kJoinThreads) rid_join_kernel(JoinArgs p) {
     if (status0 & kStatusWide) {
         // some chunk has more than kMaxD distinct end states: block 0 propagates if(PLAS_i)
         if (blockIdx.x != 0) return;
-        if (p.summary) {
-            summary_wide(p, s_vec, s_nvec);
-            return;
-        }
-        const uint16_t *row0 = p.maps;
-        const uint16_t v0 = row0[A.q0_slot];
-        if (p.c == 1 || v0 == kUndef) {
-            if (tid == 0) *p.accept = (v0 != kUndef && is_final(A, v0)) ? 1 : 0;
-            return;
-        }
-        for (uint32_t w = tid; w < A.kw; w += blockDim.x)
-            s_vec[w] = A.ifmask[static_cast<uint64_t>(v0) * A.kw + w];
-        __syncthreads();
-        for (uint32_t i = 1; i + 1 < p.c; ++i) {
-            for (uint32_t w = tid; w < A.kw; w += blockDim.x) s_nvec[w] = 0;
-            __syncthreads();
-            const uint16_t *row = p.maps + static_cast<uint64_t>(i) * A.k;
-            for (uint32_t a = tid; a < A.k; a += blockDim.x) {
-                if (!((s_vec[a >> 5] >> (a & 31)) & 1)) continue;
-                const uint16_t v = row[a];
-                if (v == kUndef) continue;
-                for (uint32_t w = 0; w < A.kw; ++w) {
-                    const uint32_t m = A.ifmask[static_cast<uint64_t>(v) * A.kw + w];
-                    if (m) atomicOr(&s_nvec[w], m);
-                }
-            }
-            __syncthreads();
-            for (uint32_t w = tid; w < A.kw; w += blockDim.x) s_vec[w] = s_nvec[w];
-            __syncthreads();
-        }
-        __shared__ uint32_t s_acc;
-        if (tid == 0) s_acc = 0;
-        __syncthreads();
-        const uint16_t *last = p.maps + static_cast<uint64_t>(p.c - 1) * A.k;
-        for (uint32_t a = tid; a < A.k; a += blockDim.x)
-            if (((s_vec[a >> 5] >> (a & 31)) & 1) && last[a] != kUndef && is_final(A, last[a]))
-                s_acc = 1;
-        __syncthreads();
-        if (tid == 0) *p.accept = s_acc ? 1 : 0;
+        if (p.summary) summary_wide(p, s_vec, s_nvec);
+        else accept_wide(p, s_vec, s_nvec);
         return;
     }
 
@@ -795,7 +590,8 @@ DeviceScratch *scratch_for(const ridfa_program *P, int dev, size_t bytes, int *e
         size_t want = std::max(bytes, static_cast<size_t>(1) << 20);
         cudaError_t e = cudaMalloc(&S->base, want);
         if (e != cudaSuccess) { *err = cuda_fail(e); return nullptr; }
-        e = cudaMemset(S->base, 0, 1024);   // ticket and status start at zero
+        e = cudaMemset(S->base, 0, 1024);   // ticket, status and work words start at zero
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
         if (e != cudaSuccess) { *err = cuda_fail(e); return nullptr; }
         S->bytes = want;
     }
@@ -1067,51 +863,25 @@ int plan_reach(const Automaton &A, const ridfa_tuning *tuning, const uint8_t *te
     return RIDFA_OK;
 }
 
-int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, size_t len,
-                   uint32_t n_chunks, const ridfa_tuning *tuning, uint8_t *d_accept_user,
-                   uint8_t *h_accept, uint16_t *d_maps_user, cudaStream_t st,
-                   ridfa_shard_summary *h_summary = nullptr) {
-    if (!P) return RIDFA_E_ARG;
-    if (use_dfa && !P->has_dfa) return RIDFA_E_NO_DFA;
-    const HostAutomaton &H = use_dfa ? P->dfa : P->rid;
-    if (len == 0) {
-        if (n_chunks != 0) return RIDFA_E_CHUNKS;
-        // empty text: accept iff the start state is final (no device work needed for the answer)
-        const uint8_t acc = H.final_flag.empty() ? 0 : H.final_flag[H.slot_state[H.q0_slot]];
-        if (h_accept) *h_accept = acc;
-        if (d_accept_user) {
-            cudaError_t e = cudaMemcpyAsync(d_accept_user, &acc, 1, cudaMemcpyHostToDevice, st);
-            if (e != cudaSuccess) return cuda_fail(e);
-            e = cudaStreamSynchronize(st);
-            if (e != cudaSuccess) return cuda_fail(e);
-        }
-        return RIDFA_OK;
+// How a call runs on the general path: pieces per chunk and the reach launches.
+struct GeneralPlan {
+    uint64_t spc = 1, pieces = 0, grid_warps = 0;
+    uint32_t n_launch = 1, lb_cap = 32;
+    bool lockstep = false, lookback = false;
+    ReachArgs ras[kMaxPieceGroups];
+    ReachPlan plans[kMaxPieceGroups];
+    ridfa_plan_report report() const {
+        const ReachPlan &p0 = plans[0];
+        const bool copies = p0.mode == kModePairF || p0.mode == kModePairH;
+        return ridfa_plan_report{p0.mode,
+                                 p0.path == kPathCoop ? 3u : p0.path == kPathCoop2 ? 4u : p0.path == kPathCoopSet ? 5u : 1u,
+                                 copies ? static_cast<uint32_t>(p0.tis) : 0u, static_cast<uint32_t>(p0.block),
+                                 static_cast<uint32_t>(p0.grid), (spc > 1 || lockstep) ? 1u : 0u};
     }
-    if (!d_text) return RIDFA_E_ARG;
-    if (n_chunks == 0 || n_chunks > len) return RIDFA_E_CHUNKS;
-    if (H.k > RIDFA_MAX_SLOTS) return RIDFA_E_UNSUPPORTED;
+};
 
-    std::lock_guard<std::mutex> lock(P->mu);
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return cuda_fail(e);
-    int err = RIDFA_OK;
-    const DeviceAutomaton *D = device_copy(P, use_dfa, dev, &err);
-    if (!D) return err;
-
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const uint64_t c = n_chunks;
-    const uint64_t nbound = c - 1;
-    const uint64_t per_block_max = 1024;
-    uint32_t per_thread = static_cast<uint32_t>(std::max<uint64_t>(
-        1, (nbound + static_cast<uint64_t>(kJoinThreads) * per_block_max - 1) /
-               (static_cast<uint64_t>(kJoinThreads) * per_block_max)));
-    uint32_t join_blocks = static_cast<uint32_t>(std::max<uint64_t>(
-        1, (nbound + static_cast<uint64_t>(kJoinThreads) * per_thread - 1) /
-               (static_cast<uint64_t>(kJoinThreads) * per_thread)));
-    Automaton A{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state,
-                H.n_states, H.n_classes, H.k, H.kw, H.q0_slot, H.merges};
+int plan_general(const HostAutomaton &H, const DeviceAutomaton *D, const Automaton &A, const uint8_t *d_text, uint64_t len,
+                 uint64_t c, const ridfa_tuning *tuning, int sms, GeneralPlan *out) {
     // intra-chunk speculation: too few chunks to fill the GPU, each long enough to cut into pieces.
     // Pieces run from every state; automata of more than 256 states run theirs in groups of at
     // most 256 states (one reach launch per group into one row of all states).
@@ -1159,8 +929,8 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
     const bool lookback = spc > 1 && lb_able;
     const uint32_t n_launch = spc > 1 ? groups : 1;
     // plan the reach launches first: the run-list scratch is sized by their grids
-    ReachArgs ras[kMaxPieceGroups];
-    ReachPlan plans[kMaxPieceGroups];
+    ReachArgs *ras = out->ras;
+    ReachPlan *plans = out->plans;
     uint64_t grid_warps = 0;
     for (uint32_t g = 0; g < n_launch; ++g) {
         // look-back pieces: 32 start slots per piece, rows of 32 scattered afterwards
@@ -1172,7 +942,7 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
         ras[g] = ReachArgs{Ag, d_text, len, static_cast<uint32_t>(pieces), nullptr, nullptr, nullptr, 8,
                            nullptr, nullptr, lookback ? 32u : spc > 1 ? NS : H.k, nullptr};
         if (tuning && tuning->probe_interval) ras[g].probe = tuning->probe_interval;
-        err = plan_reach(ras[g].A, tuning, d_text, ras[g], sms, &plans[g], !lockstep);
+        const int err = plan_reach(ras[g].A, tuning, d_text, ras[g], sms, &plans[g], !lockstep);
         if (err != RIDFA_OK) return err;
         plans[g].pslot = lookback;
         // warps past the last 32-chunk task never write their run list (the lockstep kernel has none)
@@ -1181,20 +951,161 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
                                                                                (plans[g].block / 32),
                                                                            (pieces + 31) / 32));
     }
+    out->spc = spc;
+    out->pieces = pieces;
+    out->grid_warps = grid_warps;
+    out->n_launch = n_launch;
+    out->lb_cap = lb_cap;
+    out->lockstep = lockstep;
+    out->lookback = lookback;
+    return RIDFA_OK;
+}
+
+// A call that leaves every choice to the library (profiling aside).
+bool automatic(const ridfa_tuning *t) {
+    return !t || !(t->piece_len || t->block_threads || t->probe_interval || t->grid_blocks || t->table_mode || t->text_path ||
+                   t->lookback_cap);
+}
+
+// One call through the stream kernels (ridfa_stream.cu): two launches, results written to the
+// page-locked words by the join itself.  Caller holds P->mu.
+int recognize_stream(const ridfa_program *P, const HostAutomaton &H, const DeviceAutomaton *D, int dev, int sms,
+                     const uint8_t *d_text, uint64_t len, uint32_t n_chunks, bool prof, uint8_t *d_accept_user, uint8_t *h_accept,
+                     uint16_t *d_maps_user, cudaStream_t st, ridfa_shard_summary *h_summary) {
+    const StreamShape sh = stream_shape(H, len, n_chunks, sms);
+    auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
+    // the first 1024 bytes as in Layout: ticket, status (and the stream calls' work word), accept
+    size_t off = 1024;
+    const size_t o_res = off;      off += al(sh.pieces * 4);
+    const size_t o_dinfo = off;    off += al(static_cast<size_t>(n_chunks) * 4);
+    const size_t o_part = off;     off += al(static_cast<size_t>(sh.join_blocks) * kPartialWords * 4);
+    const size_t o_sum = off;      off += al(sizeof(ridfa_shard_summary));
+    const size_t o_maps = off;     off += d_maps_user ? 0 : al(static_cast<size_t>(n_chunks) * H.k * 2);
+    int err = RIDFA_OK;
+    DeviceScratch *S = scratch_for(P, dev, off, &err);
+    if (!S) return err;
+    uint8_t *base = static_cast<uint8_t *>(S->base);
+    StreamCall C;
+    C.H = &H;
+    C.D = D;
+    C.text = d_text;
+    C.len = len;
+    C.c = n_chunks;
+    C.res = reinterpret_cast<uint32_t *>(base + o_res);
+    C.maps = d_maps_user ? d_maps_user : reinterpret_cast<uint16_t *>(base + o_maps);
+    C.dinfo = reinterpret_cast<uint32_t *>(base + o_dinfo);
+    C.partials = reinterpret_cast<uint32_t *>(base + o_part);
+    C.ticket = reinterpret_cast<uint32_t *>(base);
+    C.status = reinterpret_cast<uint32_t *>(base + 256);
+    C.work = C.status + 2;
+    C.accept = d_accept_user ? d_accept_user : base + 512;
+    if (h_accept || h_summary) {
+        C.h_accept = S->h_accept_pinned;
+        C.h_status = S->h_status_pinned;
+    }
+    C.summary = h_summary ? reinterpret_cast<ridfa_shard_summary *>(base + o_sum) : nullptr;
+    cudaError_t e = cudaSuccess;
+    if (prof) {
+        for (auto &ev : S->ev)
+            if (!ev) {
+                cudaEvent_t x;
+                e = cudaEventCreate(&x);
+                if (e != cudaSuccess) return cuda_fail(e);
+                ev = x;
+            }
+        cudaEventRecord(static_cast<cudaEvent_t>(S->ev[0]), st);
+        C.between = static_cast<cudaEvent_t>(S->ev[1]);
+    }
+    NvtxRange range("ridfa reach");
+    e = stream_launch(C, sh, st);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (prof) {
+        cudaEventRecord(static_cast<cudaEvent_t>(S->ev[2]), st);
+        S->profiled = true;
+    }
+    if (!h_accept && !h_summary) return RIDFA_OK;
+    if (h_summary) e = cudaMemcpyAsync(h_summary, C.summary, sizeof(ridfa_shard_summary), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (h_accept) *h_accept = *const_cast<volatile uint8_t *>(S->h_accept_pinned);
+    return *const_cast<volatile uint32_t *>(S->h_status_pinned) & kStatusBad ? RIDFA_E_STATE : RIDFA_OK;
+}
+
+int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, size_t len,
+                   uint32_t n_chunks, const ridfa_tuning *tuning, uint8_t *d_accept_user,
+                   uint8_t *h_accept, uint16_t *d_maps_user, cudaStream_t st,
+                   ridfa_shard_summary *h_summary = nullptr) {
+    if (!P) return RIDFA_E_ARG;
+    if (use_dfa && !P->has_dfa) return RIDFA_E_NO_DFA;
+    const HostAutomaton &H = use_dfa ? P->dfa : P->rid;
+    if (len == 0) {
+        if (n_chunks != 0) return RIDFA_E_CHUNKS;
+        // empty text: accept iff the start state is final (no device work needed for the answer)
+        const uint8_t acc = H.final_flag.empty() ? 0 : H.final_flag[H.slot_state[H.q0_slot]];
+        if (h_accept) *h_accept = acc;
+        if (d_accept_user) {
+            cudaError_t e = cudaMemcpyAsync(d_accept_user, &acc, 1, cudaMemcpyHostToDevice, st);
+            if (e != cudaSuccess) return cuda_fail(e);
+            e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess) return cuda_fail(e);
+        }
+        return RIDFA_OK;
+    }
+    if (!d_text) return RIDFA_E_ARG;
+    if (n_chunks == 0 || n_chunks > len) return RIDFA_E_CHUNKS;
+    if (H.k > RIDFA_MAX_SLOTS) return RIDFA_E_UNSUPPORTED;
+
+    std::lock_guard<std::mutex> lock(P->mu);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e);
+    int err = RIDFA_OK;
+    const DeviceAutomaton *D = device_copy(P, use_dfa, dev, &err);
+    if (!D) return err;
+
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const uint64_t c = n_chunks;
+    const uint64_t nbound = c - 1;
+    const uint64_t per_block_max = 1024;
+    uint32_t per_thread = static_cast<uint32_t>(std::max<uint64_t>(
+        1, (nbound + static_cast<uint64_t>(kJoinThreads) * per_block_max - 1) /
+               (static_cast<uint64_t>(kJoinThreads) * per_block_max)));
+    uint32_t join_blocks = static_cast<uint32_t>(std::max<uint64_t>(
+        1, (nbound + static_cast<uint64_t>(kJoinThreads) * per_thread - 1) /
+               (static_cast<uint64_t>(kJoinThreads) * per_thread)));
+    Automaton A{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state,
+                H.n_states, H.n_classes, H.k, H.kw, H.q0_slot, H.merges};
+    if (automatic(tuning) && stream_takes(H, len, n_chunks)) {
+        err = recognize_stream(P, H, D, dev, sms, d_text, len, n_chunks, tuning && tuning->profile, d_accept_user, h_accept,
+                               d_maps_user, st, h_summary);
+        if (err == RIDFA_OK)
+            for (auto &x : P->scratch)
+                if (x.device == dev) {
+                    x.planned = x.stream_call = true;
+                    x.stream_dfa = use_dfa;
+                    x.stream_text = d_text;
+                    x.stream_len = len;
+                    x.stream_chunks = n_chunks;
+                }
+        return err;
+    }
+    GeneralPlan G;
+    err = plan_general(H, D, A, d_text, len, c, tuning, sms, &G);
+    if (err != RIDFA_OK) return err;
+    const uint64_t spc = G.spc, pieces = G.pieces, grid_warps = G.grid_warps;
+    const uint32_t n_launch = G.n_launch, NS = H.n_states;
+    const bool lockstep = G.lockstep, lookback = G.lookback;
+    ReachArgs *ras = G.ras;
+    ReachPlan *plans = G.plans;
     const uint64_t comp_funcs = spc > 1 ? c * ((spc + kComposeGroup - 1) / kComposeGroup) : 0;
     const Layout L = layout_for(c, H.k, d_maps_user == nullptr, join_blocks, grid_warps, spc > 1 ? pieces : 0,
                                 spc > 1 ? NS : 0, comp_funcs, lookback);
     DeviceScratch *S = scratch_for(P, dev, L.total, &err);
     if (!S) return err;
-    {
-        const ReachPlan &p0 = plans[0];
-        const bool copies = p0.mode == kModePairF || p0.mode == kModePairH;
-        S->last_plan = ridfa_plan_report{p0.mode,
-                                         p0.path == kPathCoop ? 3u : p0.path == kPathCoop2 ? 4u : p0.path == kPathCoopSet ? 5u : 1u,
-                                         copies ? static_cast<uint32_t>(p0.tis) : 0u, static_cast<uint32_t>(p0.block),
-                                         static_cast<uint32_t>(p0.grid), (spc > 1 || lockstep) ? 1u : 0u};
-        S->planned = true;
-    }
+    S->last_plan = G.report();
+    S->planned = true;
+    S->stream_call = false;
     uint8_t *base = static_cast<uint8_t *>(S->base);
     uint32_t *ticket = reinterpret_cast<uint32_t *>(base + L.ticket_off);
     uint32_t *status = reinterpret_cast<uint32_t *>(base + L.status_off);
@@ -1234,7 +1145,7 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
         e = cudaMemsetAsync(pmaps, 0xFF, pieces * NS * 2, st);
         if (e != cudaSuccess) return cuda_fail(e);
         LookbackArgs la{ras[0].A, d_text, len, pieces, static_cast<uint32_t>(spc),
-                        reinterpret_cast<uint16_t *>(base + L.lbslots_off), pmaps, lb_cap};
+                        reinterpret_cast<uint16_t *>(base + L.lbslots_off), pmaps, G.lb_cap};
         la.A.k = H.k;
         e = lookback_dispatch(la, sms, st);
         if (e != cudaSuccess) return cuda_fail(e);
@@ -1482,6 +1393,21 @@ extern "C" int ridfa_last_plan(const ridfa_program *prog, ridfa_plan_report *out
     if (cudaGetDevice(&dev) != cudaSuccess) return ridfa::cuda_fail(cudaGetLastError());
     for (auto &s : prog->scratch)
         if (s.device == dev && s.planned) {
+            if (s.stream_call) {
+                // the general path's plan of the same call
+                const ridfa::HostAutomaton &H = s.stream_dfa ? prog->dfa : prog->rid;
+                int err = RIDFA_OK, sms = 0;
+                const ridfa::DeviceAutomaton *D = ridfa::device_copy(prog, s.stream_dfa, dev, &err);
+                if (!D) return err;
+                cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+                const ridfa::Automaton A{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state,
+                                         H.n_states, H.n_classes, H.k, H.kw, H.q0_slot, H.merges};
+                ridfa::GeneralPlan G;
+                err = ridfa::plan_general(H, D, A, s.stream_text, s.stream_len, s.stream_chunks, nullptr, sms, &G);
+                if (err != RIDFA_OK) return err;
+                s.last_plan = G.report();
+                s.stream_call = false;
+            }
             *out = s.last_plan;
             return RIDFA_OK;
         }

@@ -23,6 +23,49 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
+// The merge graph of an automaton: what becomes of the runs from all of its states at once.
+// A node is a function f from the states to the states (or undefined) that some byte sequence
+// performs; the root is the identity.  Functions with two or more distinct defined values are
+// inner nodes; a function with one value v is a leaf, and the run goes on alone from v.  A function
+// is kept as (partition, images): part[pid][x] = the block of state x (kNoBlock: its run died),
+// images[b] = the state of block b's runs.  A chunk (or any piece of one) is then read by one lane:
+// down the graph until a leaf, on with the leaf's single run to the end.  What is left of the
+// piece's function is one word: (pid, state) -- x goes to state if part[pid][x] is a block -- or an
+// inner node.  Only built where the graph is small (most automata of practical REs: all runs merge
+// within tens of bytes); ok = false otherwise.
+struct HostMerge {
+    bool ok = false;
+    uint32_t inner = 0, parts = 0;
+    std::vector<uint16_t> next;       // [inner][C]: an inner node, or kLeafBit | leaf
+    std::vector<uint32_t> leaf;       // [leaves]: pid << 16 | state; leaf 0: every run dead
+    std::vector<uint16_t> node_part;  // [inner]
+    std::vector<uint32_t> node_img;   // [inner]: offset into images
+    std::vector<uint16_t> images;
+    std::vector<uint16_t> part;       // [parts][n_states]; partition 0: all dead
+    std::vector<uint32_t> slot_alive; // [parts][kw]: slots whose start state has a block
+};
+constexpr uint16_t kLeafBit = 0x8000;
+constexpr uint16_t kNoBlock = 0xFFFF;
+
+// Main-loop table of the stream kernels (ridfa_stream.cu), chosen per automaton on the host.
+//   kStreamField: the live bytes (those some position reads) differ in a field of `width` <= 2 bits
+//     at bit `shift`; codes come from the field by arithmetic, `canon` holds the byte of each code
+//     (a byte that is not its code's is not in the alphabet and kills the run), one lookup takes
+//     `group` bytes: column = the codes, first byte lowest.
+//   kStreamPair / kStreamSingle: two / one bytes a lookup; byte_code[b] = the column offset of b as
+//     first byte (low half) and second byte (high half) of a pair, whose sum is the column.
+// Entries are next states of `entry` bytes (1 when all ids and the dead state fit 8 bits, else 2);
+// row s, column col: word s * row_words + col / (4 / entry), each word in `copies` lane copies.
+enum StreamKind : uint32_t { kStreamNone = 0, kStreamField = 1, kStreamPair = 2, kStreamSingle = 3 };
+struct HostStream {
+    uint32_t kind = kStreamNone;
+    uint32_t entry = 1, copies = 32, row_words = 0, group = 1, shift = 0, width = 0;
+    uint32_t canon = 0;
+    uint32_t warps = 0;               // warps a block holds beside the table (and its staging)
+    std::vector<uint32_t> byte_code;  // [256] (kStreamPair, kStreamSingle)
+    std::vector<uint32_t> words;      // [(n_states + 1) * row_words]
+};
+
 // One speculative automaton as the device sees it: the RI-DFA B with its interface
 // (Sec. 3.1-3.4) or the minimal DFA with every state initial (Sec. 2).
 struct HostAutomaton {
@@ -38,7 +81,19 @@ struct HostAutomaton {
     std::vector<uint32_t> ifmask;     // [(n_states + 1) * kw]: slots of if_min({p}); dead row = 0
     std::vector<uint16_t> slot_state; // [k]: start state of each slot
     uint32_t merges = 0;              // 1: runs from every slot merge on random text (merge_hint)
+    HostMerge merge;
+    HostStream stream;
 };
+
+// Build H.merge and, where it is small enough, H.stream (ridfa_merge.cpp).
+void build_stream(HostAutomaton &H);
+// Shared memory of a stream kernel's block besides the staging buffers: tables and the compact
+// copies for the ragged ends.
+size_t stream_table_bytes(const HostAutomaton &H);
+constexpr size_t kStreamSmem = 226 * 1024;        // shared memory a stream block may take
+constexpr size_t kStreamTransSmem = 24 * 1024;    // ragged-end tables up to these sizes sit in shared
+constexpr size_t kStreamNextSmem = 12 * 1024;     // memory, larger ones are read through L1
+constexpr size_t kStreamStaging = 4096;           // per-warp staging (kStreamPair, kStreamSingle)
 
 // Device copy of one automaton (one per device it was uploaded to).
 struct DeviceAutomaton {
@@ -49,6 +104,10 @@ struct DeviceAutomaton {
     uint32_t *ifmask = nullptr;
     uint16_t *slot_state = nullptr;
     uint16_t *all_states = nullptr;   // [n_states]: state s (every state as a start, for pieces)
+    // merge graph and stream table (HostMerge, HostStream); null when not built
+    uint16_t *mg_next = nullptr, *mg_node_part = nullptr, *mg_images = nullptr, *mg_part = nullptr;
+    uint32_t *mg_leaf = nullptr, *mg_node_img = nullptr, *mg_slot_alive = nullptr;
+    uint32_t *st_code = nullptr, *st_words = nullptr;
     size_t bytes = 0;
 };
 
@@ -87,6 +146,11 @@ struct DeviceScratch {
     bool profiled = false;
     ridfa_plan_report last_plan{};               // the reach plan of the last call on this device
     bool planned = false;
+    bool stream_call = false;                    // the last call took the stream kernels: its plan on the
+    bool stream_dfa = false;                     // general path is worked out when asked for
+    const uint8_t *stream_text = nullptr;        // (only its alignment is looked at)
+    uint64_t stream_len = 0;
+    uint32_t stream_chunks = 0;
 };
 
 }  // namespace ridfa

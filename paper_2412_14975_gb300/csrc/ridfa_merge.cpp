@@ -1,0 +1,386 @@
+// Host construction of the merge graph and of the stream kernels' main-loop table
+// (HostMerge, HostStream in ridfa_internal.h), from a compiled automaton.
+//
+// The graph holds the functions that byte-class sequences perform on the set of all states
+// (Sec. 5's state convergence, precomputed: runs that meet in one state go on as one).  It is the
+// part of the simultaneous automaton over the runs up to the point where one run is left, which
+// stays small where the whole would not.
+#include <algorithm>
+#include <cstring>
+#include <map>
+#include <string>
+#include <unordered_map>
+
+#include "ridfa_internal.h"
+
+namespace ridfa {
+namespace {
+
+// Limits of the graph: inner nodes (codon-like automata, whose runs stay apart, run into it),
+// entries of the partition table, and the images stepped while building (compile time: a step is
+// about 10 ns, so 1.5 M keep the construction under some 15 ms).
+constexpr uint32_t kMaxInner = 6144;
+constexpr uint32_t kMaxInnerApart = 1536;      // without the merge hint
+constexpr uint64_t kMaxPartEntries = 1u << 20;
+constexpr uint64_t kMaxSteps = 500000;
+
+std::string key_of(uint32_t pid, const uint16_t *v, size_t n) {
+    std::string k(4 + n * 2, '\0');
+    std::memcpy(&k[0], &pid, 4);
+    std::memcpy(&k[4], v, n * 2);
+    return k;
+}
+
+bool build_graph(const HostAutomaton &H, HostMerge &G) {
+    const uint32_t n = H.n_states, C = H.n_classes;
+    if (n == 0 || n > 8192) return false;
+    const uint32_t max_inner = H.merges ? kMaxInner : kMaxInnerApart;
+    std::unordered_map<std::string, uint32_t> node_id, part_id, step_id;
+    // partition 0: every run dead; partition 1: the identity
+    G.part.assign(n, kNoBlock);
+    for (uint32_t x = 0; x < n; ++x) G.part.push_back(static_cast<uint16_t>(x));
+    part_id[key_of(0, &G.part[0], n)] = 0;
+    part_id[key_of(0, &G.part[n], n)] = 1;
+    uint32_t parts = 2;
+    G.leaf.push_back(n);                                   // leaf 0: partition 0, the dead state
+    std::unordered_map<uint32_t, uint32_t> leaf_id;
+    std::vector<uint32_t> node_d;                          // blocks of each inner node
+    auto add_node = [&](uint32_t pid, const std::vector<uint16_t> &img) -> uint32_t {
+        const auto r = node_id.emplace(key_of(pid, img.data(), img.size()), static_cast<uint32_t>(node_d.size()));
+        if (r.second) {
+            G.node_part.push_back(static_cast<uint16_t>(pid));
+            G.node_img.push_back(static_cast<uint32_t>(G.images.size()));
+            G.images.insert(G.images.end(), img.begin(), img.end());
+            node_d.push_back(static_cast<uint32_t>(img.size()));
+        }
+        return r.first->second;
+    };
+    auto add_leaf = [&](uint32_t pid, uint32_t state) -> uint32_t {
+        const auto r = leaf_id.emplace(pid << 16 | state, static_cast<uint32_t>(G.leaf.size()));
+        if (r.second) G.leaf.push_back(pid << 16 | state);
+        return r.first->second;
+    };
+    std::vector<uint16_t> img(n), next_img, block(n), pv(n);
+    for (uint32_t x = 0; x < n; ++x) img[x] = static_cast<uint16_t>(x);
+    add_node(1, img);
+    std::vector<uint32_t> where(n + 1, 0), stamp(n + 1, 0);
+    uint32_t gen = 0;
+    uint64_t steps = 0;
+    for (uint32_t u = 0; u < node_d.size(); ++u) {
+        const uint32_t d = node_d[u], pid = G.node_part[u], off = G.node_img[u];
+        for (uint32_t c = 0; c < C; ++c) {
+            // step the distinct images; block[b]: the new block of old block b.  Blocks are numbered
+            // by their smallest state, an order that first appearance keeps.
+            steps += d;
+            ++gen;
+            next_img.clear();
+            for (uint32_t b = 0; b < d; ++b) {
+                const uint32_t t = H.trans[static_cast<size_t>(G.images[off + b]) * C + c];
+                if (t == n) {
+                    block[b] = kNoBlock;
+                } else {
+                    if (stamp[t] != gen) {
+                        stamp[t] = gen;
+                        where[t] = static_cast<uint32_t>(next_img.size());
+                        next_img.push_back(static_cast<uint16_t>(t));
+                    }
+                    block[b] = static_cast<uint16_t>(where[t]);
+                }
+            }
+            uint32_t code;
+            if (next_img.empty()) {
+                code = kLeafBit;                           // leaf 0
+            } else {
+                uint32_t npid = pid;
+                bool same = next_img.size() == d;
+                for (uint32_t b = 0; b < d && same; ++b) same = block[b] == b;
+                if (!same) {
+                    const auto r = step_id.emplace(key_of(pid, block.data(), d), 0u);
+                    if (r.second) {
+                        for (uint32_t x = 0; x < n; ++x) {
+                            const uint16_t o = G.part[static_cast<size_t>(pid) * n + x];
+                            pv[x] = o == kNoBlock ? kNoBlock : block[o];
+                        }
+                        steps += n / 4;
+                        const auto q = part_id.emplace(key_of(0, pv.data(), n), parts);
+                        if (q.second) {
+                            if (static_cast<uint64_t>(parts + 1) * n > kMaxPartEntries || parts >= 0x7FFF) return false;
+                            G.part.insert(G.part.end(), pv.begin(), pv.end());
+                            ++parts;
+                        }
+                        r.first->second = q.first->second;
+                    }
+                    npid = r.first->second;
+                }
+                code = next_img.size() == 1 ? kLeafBit | add_leaf(npid, next_img[0]) : add_node(npid, next_img);
+            }
+            if (!H.merges && node_d.size() > 256 && G.leaf.size() == 1) return false;    // nothing merges
+            if (node_d.size() > max_inner || G.leaf.size() >= 0x8000 || steps > kMaxSteps) return false;
+            G.next.push_back(static_cast<uint16_t>(code));
+        }
+    }
+    G.inner = static_cast<uint32_t>(node_d.size());
+    G.parts = parts;
+    G.slot_alive.assign(static_cast<size_t>(parts) * H.kw, 0);
+    for (uint32_t p = 0; p < parts; ++p)
+        for (uint32_t a = 0; a < H.k; ++a)
+            if (G.part[static_cast<size_t>(p) * n + H.slot_state[a]] != kNoBlock)
+                G.slot_alive[static_cast<size_t>(p) * H.kw + (a >> 5)] |= 1u << (a & 31);
+    return true;
+}
+
+// Every index the kernels take from the graph unchecked.
+bool graph_in_bounds(const HostAutomaton &H, const HostMerge &G) {
+    const uint32_t n = H.n_states;
+    if (G.next.size() != static_cast<size_t>(G.inner) * H.n_classes || G.part.size() != static_cast<size_t>(G.parts) * n ||
+        G.node_part.size() != G.inner || G.node_img.size() != G.inner || G.leaf.empty())
+        return false;
+    for (uint16_t c : G.next)
+        if ((c & kLeafBit) ? (c & 0x7FFFu) >= G.leaf.size() : c >= G.inner) return false;
+    for (uint32_t l : G.leaf)
+        if ((l >> 16) >= G.parts || (l & 0xFFFF) > n) return false;
+    for (uint16_t s : G.images)
+        if (s >= n) return false;
+    for (uint32_t u = 0; u < G.inner; ++u) {
+        if (G.node_part[u] >= G.parts) return false;
+        for (uint32_t x = 0; x < n; ++x) {
+            const uint16_t b = G.part[static_cast<size_t>(G.node_part[u]) * n + x];
+            if (b != kNoBlock && static_cast<size_t>(G.node_img[u]) + b >= G.images.size()) return false;
+        }
+    }
+    return true;
+}
+
+// Shared-memory wavefronts of one 32-lane gather into `copies` lane copies (rows at random): by
+// counting for 32, at most 2 for 16, by simulation below that.
+double wavefronts(uint32_t copies) {
+    switch (copies) {
+        case 32: return 1.0;
+        case 16: return 1.9;
+        case 8: return 2.7;
+        case 4: return 3.2;
+        default: return 3.4;
+    }
+}
+
+size_t rest_bytes(const HostAutomaton &H, uint32_t kind) {
+    // class codes, one-byte table and byte classes for the ragged ends, graph edges
+    const size_t trans = H.trans.size() * 2, next = H.merge.next.size() * 2;
+    return (kind == kStreamField ? 0 : 256 * 128) + (trans <= kStreamTransSmem ? (trans + 15) / 16 * 16 : 0) + 256 +
+           (next <= kStreamNextSmem ? (next + 15) / 16 * 16 : 0) + 256;
+}
+
+// Column offsets of a pair table: offset(c1, c2) = first[c1] + second[c2], where equal sums mean
+// equal columns.  Every first class takes a place (word, part) so that its whole row of columns,
+// the undefined ones included, meets only equal columns; second classes shift by whole words.
+// Tries a few layouts of the second classes and returns the words of a row (0: none found).
+uint32_t place_pairs(const std::vector<uint32_t> &col, uint32_t C, uint32_t per_word, uint32_t limit,
+                     std::vector<uint32_t> &first, std::vector<uint32_t> &second, std::vector<int64_t> &slots) {
+    uint32_t best = 0;
+    std::vector<uint32_t> rows_live(C, 0), cols_live(C, 0), ord(C), rord(C);
+    for (uint32_t a = 0; a < C; ++a)
+        for (uint32_t b = 0; b < C; ++b)
+            if (col[a * C + b]) {
+                ++rows_live[a];
+                ++cols_live[b];
+            }
+    for (uint32_t i = 0; i < C; ++i) ord[i] = rord[i] = i;
+    std::stable_sort(rord.begin(), rord.end(), [&](uint32_t x, uint32_t y) { return rows_live[x] > rows_live[y]; });
+    for (uint32_t gap = 1; gap <= 6; ++gap)
+        for (uint32_t asc = 0; asc < 2; ++asc) {
+            // the class most rows have a move on comes first, `gap` words before the others
+            std::stable_sort(ord.begin(), ord.end(), [&](uint32_t x, uint32_t y) { return cols_live[x] > cols_live[y]; });
+            if (asc) std::reverse(ord.begin() + 1, ord.end());
+            std::vector<uint32_t> sec(C), fst(C);
+            for (uint32_t i = 0; i < C; ++i) sec[ord[i]] = i == 0 ? 0 : gap + i - 1;
+            std::vector<int64_t> occ(static_cast<size_t>(limit + 2 * C + 16) * per_word, -1);
+            uint32_t words = 0;
+            bool ok = true;
+            for (uint32_t ri = 0; ri < C && ok; ++ri) {
+                const uint32_t a = rord[ri];
+                bool placed = false;
+                for (uint32_t w = 0; w < limit && !placed; ++w)
+                    for (uint32_t q = 0; q < per_word && !placed; ++q) {
+                        bool fit = true;
+                        for (uint32_t b = 0; b < C && fit; ++b) {
+                            const int64_t o = occ[static_cast<size_t>(w + sec[b]) * per_word + q];
+                            fit = o < 0 || o == static_cast<int64_t>(col[a * C + b]);
+                        }
+                        if (!fit) continue;
+                        for (uint32_t b = 0; b < C; ++b) {
+                            occ[static_cast<size_t>(w + sec[b]) * per_word + q] = col[a * C + b];
+                            words = std::max(words, w + sec[b] + 1);
+                        }
+                        fst[a] = w * per_word + q;
+                        placed = true;
+                    }
+                ok = placed && words <= limit;
+            }
+            if (ok && (best == 0 || words < best)) {
+                best = words;
+                first = fst;
+                second.assign(C, 0);
+                for (uint32_t b = 0; b < C; ++b) second[b] = sec[b] * per_word;
+                occ.resize(static_cast<size_t>(words) * per_word);
+                slots = occ;
+            }
+        }
+    return best;
+}
+
+void build_table(HostAutomaton &H) {
+    const uint32_t n = H.n_states, C = H.n_classes;
+    HostStream best;
+    double best_cost = 1e9;
+    const uint32_t entry = n + 1 <= 256 ? 1 : 2, per_word = 4 / entry;
+    std::vector<uint8_t> class_live(C, 0);
+    for (uint32_t c = 0; c < C; ++c)
+        for (uint32_t s = 0; s < n && !class_live[c]; ++s) class_live[c] = H.trans[static_cast<size_t>(s) * C + c] != n;
+    // the most copies that fit, with their cost in shared-memory cycles per 32 text bytes
+    auto consider = [&](HostStream t, double fixed, double per_lookup) {
+        const size_t rest = rest_bytes(H, t.kind);
+        for (uint32_t f = 32; f >= 1; f /= 2) {
+            const size_t table = static_cast<size_t>(n + 1) * t.row_words * 4 * f;
+            uint32_t warps = 32;
+            if (t.kind != kStreamField) {
+                if (rest + table + 8 * kStreamStaging > kStreamSmem) continue;
+                warps = static_cast<uint32_t>(std::min<size_t>(32, (kStreamSmem - rest - table) / kStreamStaging));
+            } else if (rest + table > kStreamSmem) {
+                continue;
+            }
+            // fewer warps hide less of the lookups' latency
+            const double thin = warps >= 24 ? 1.0 : warps >= 16 ? 1.08 : warps >= 12 ? 1.2 : 1.45;
+            const double cost = std::max(1.75, fixed + wavefronts(f) * per_lookup) * thin;
+            if (cost < best_cost) {
+                best_cost = cost;
+                t.copies = f;
+                t.warps = warps;
+                best = t;
+            }
+        }
+    };
+    HostStream t;
+    t.entry = entry;
+    // codes by a bit field of the byte
+    std::vector<uint32_t> live;
+    for (uint32_t b = 0; b < 256; ++b)
+        if (class_live[H.classmap[b]]) live.push_back(b);
+    bool field = false;
+    for (uint32_t w = 1; w <= 2 && !field && live.size() <= 4; ++w)
+        for (uint32_t sh = 0; sh + w <= 8 && !field; ++sh) {
+            uint32_t seen = 0, canon = 0, m = (1u << w) - 1;
+            bool inj = live.size() <= m + 1;
+            for (uint32_t b : live) {
+                const uint32_t code = (b >> sh) & m;
+                if (seen >> code & 1) inj = false;
+                seen |= 1u << code;
+                canon |= b << (8 * code);
+            }
+            // a code no live byte has: its canonical byte has another code, so no byte passes
+            for (uint32_t code = 0; code <= 3; ++code)
+                if (!(seen >> code & 1)) canon |= ((code ^ 1) & m) << sh << (8 * code);
+            if (inj) {
+                field = true;
+                t.shift = sh;
+                t.width = w;
+                t.canon = canon;
+            }
+        }
+    if (field) {
+        t.kind = kStreamField;
+        for (uint32_t g : {4u, 2u}) {
+            t.group = g;
+            const uint32_t cols = 1u << (t.width * g);
+            t.row_words = (cols + per_word - 1) / per_word;
+            consider(t, 1.2, 1.0 / g);
+        }
+    }
+    // two bytes a lookup through class codes
+    std::vector<uint32_t> col(static_cast<size_t>(C) * C, 0), first, second, firsts, seconds;
+    std::vector<uint32_t> reps(1, 0);                   // a class pair of each distinct column
+    std::vector<int64_t> slots, best_slots;
+    if (!field && C <= 24) {
+        std::map<std::vector<uint16_t>, uint32_t> ids;
+        std::vector<uint16_t> v(n);
+        for (uint32_t a = 0; a < C; ++a)
+            for (uint32_t b = 0; b < C; ++b) {
+                bool any = false;
+                for (uint32_t s = 0; s < n; ++s) {
+                    v[s] = H.trans[static_cast<size_t>(H.trans[static_cast<size_t>(s) * C + a]) * C + b];
+                    any |= v[s] != n;
+                }
+                if (!any) continue;
+                const auto r = ids.emplace(v, static_cast<uint32_t>(ids.size() + 1));
+                if (r.second) reps.push_back(a * C + b);
+                col[a * C + b] = r.first->second;
+            }
+        const uint32_t limit = static_cast<uint32_t>(std::min<size_t>(256, kStreamSmem / 4 / (n + 1)));
+        const uint32_t words = place_pairs(col, C, per_word, limit, first, second, slots);
+        if (words) {
+            t.kind = kStreamPair;
+            t.group = 2;
+            t.row_words = words;
+            consider(t, 1.64, 0.5);
+        }
+    }
+    if (!field) {
+        t.kind = kStreamSingle;
+        t.group = 1;
+        t.row_words = (C + per_word - 1) / per_word;
+        consider(t, 1.64, 1.0);
+    }
+    if (best_cost >= 1e9) return;
+    // entries, then the codes in byte offsets of the chosen number of copies
+    const uint32_t W = best.row_words;
+    best.words.assign(static_cast<size_t>(n + 1) * W, 0);
+    auto put = [&](uint32_t s, uint32_t c, uint32_t v) {
+        const uint32_t bits = 8 * entry;
+        best.words[static_cast<size_t>(s) * W + c / per_word] |= v << (bits * (c % per_word));
+    };
+    auto step = [&](uint32_t s, uint32_t c) -> uint32_t { return H.trans[static_cast<size_t>(s) * C + c]; };
+    auto offset = [&](uint32_t c) { return c / per_word * 4 * best.copies + c % per_word * entry; };
+    if (best.kind == kStreamField) {
+        const uint32_t m = (1u << best.width) - 1;
+        for (uint32_t s = 0; s <= n; ++s)
+            for (uint32_t c = 0; c < W * per_word; ++c) {
+                uint32_t x = c >> (best.width * best.group) ? n : s;
+                for (uint32_t i = 0; i < best.group; ++i)
+                    x = step(x, H.classmap[(best.canon >> (8 * ((c >> (best.width * i)) & m))) & 0xFF]);
+                put(s, c, x);
+            }
+    } else {
+        best.byte_code.assign(256, 0);
+        if (best.kind == kStreamPair) {
+            for (uint32_t s = 0; s <= n; ++s)
+                for (uint32_t c = 0; c < W * per_word; ++c) {
+                    const int64_t id = c < slots.size() ? slots[c] : -1;
+                    put(s, c, id > 0 ? step(step(s, reps[id] / C), reps[id] % C) : n);
+                }
+            for (uint32_t b = 0; b < 256; ++b)
+                best.byte_code[b] = offset(first[H.classmap[b]]) | offset(second[H.classmap[b]]) << 16;
+        } else {
+            for (uint32_t s = 0; s <= n; ++s)
+                for (uint32_t c = 0; c < W * per_word; ++c) put(s, c, c < C ? step(s, c) : n);
+            for (uint32_t b = 0; b < 256; ++b) best.byte_code[b] = offset(H.classmap[b]);
+        }
+        for (uint32_t v : best.byte_code)
+            if ((v & 0xFFFF) + (v >> 16) > 0xFFFF) return;
+    }
+    H.stream = best;
+}
+
+}  // namespace
+
+size_t stream_table_bytes(const HostAutomaton &H) {
+    return rest_bytes(H, H.stream.kind) + static_cast<size_t>(H.n_states + 1) * H.stream.row_words * 4 * H.stream.copies;
+}
+
+void build_stream(HostAutomaton &H) {
+    HostMerge G;
+    if (H.k > RIDFA_MAX_SLOTS || !build_graph(H, G) || !graph_in_bounds(H, G)) return;
+    G.ok = true;
+    H.merge = std::move(G);
+    build_table(H);
+}
+
+}  // namespace ridfa
