@@ -64,10 +64,10 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
     const size_t o_trans = put_v(H.trans), o_cls = put_v(H.classmap), o_fin = put_v(H.final_bits), o_ifm = put_v(H.ifmask),
                  o_slot = put_v(H.slot_state), o_all = put_v(iota);
     const bool stream = T.kind != kStreamNone;
-    size_t o_next = 0, o_leaf = 0, o_np = 0, o_ni = 0, o_img = 0, o_part = 0, o_alive = 0, o_code = 0, o_words = 0;
+    size_t o_walk = 0, o_edge = 0, o_np = 0, o_ni = 0, o_img = 0, o_part = 0, o_alive = 0, o_code = 0, o_words = 0;
     if (stream) {
-        o_next = put_v(G.next);
-        o_leaf = put_v(G.leaf);
+        o_walk = put_v(G.walk);
+        o_edge = put_v(G.edge_pid);
         o_np = put_v(G.node_part);
         o_ni = put_v(G.node_img);
         o_img = put_v(G.images);
@@ -94,8 +94,8 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
     D.slot_state = u16(o_slot);
     D.all_states = u16(o_all);
     if (stream) {
-        D.mg_next = u16(o_next);
-        D.mg_leaf = u32(o_leaf);
+        D.mg_walk = u16(o_walk);
+        D.mg_edge_pid = u16(o_edge);
         D.mg_node_part = u16(o_np);
         D.mg_node_img = u32(o_ni);
         D.mg_images = u16(o_img);

@@ -37,6 +37,10 @@ struct HostMerge {
     bool ok = false;
     uint32_t inner = 0, parts = 0;
     std::vector<uint16_t> next;       // [inner][C]: an inner node, or kLeafBit | leaf
+    std::vector<uint16_t> walk;       // [n_states + 1 + inner][C]: one-byte steps of the states (as
+                                      // trans), then of the nodes (node u as n_states + 1 + u; an
+                                      // edge to a leaf goes to the leaf's state)
+    std::vector<uint16_t> edge_pid;   // [inner][C]: the leaf's partition, for edges to leaves
     std::vector<uint32_t> leaf;       // [leaves]: pid << 16 | state; leaf 0: every run dead
     std::vector<uint16_t> node_part;  // [inner]
     std::vector<uint32_t> node_img;   // [inner]: offset into images
@@ -90,9 +94,10 @@ void build_stream(HostAutomaton &H);
 // Shared memory of a stream kernel's block besides the staging buffers: tables and the compact
 // copies for the ragged ends.
 size_t stream_table_bytes(const HostAutomaton &H);
+size_t stream_walk_bytes(const HostAutomaton &H);      // the one-byte tables alone
 constexpr size_t kStreamSmem = 226 * 1024;        // shared memory a stream block may take
-constexpr size_t kStreamTransSmem = 24 * 1024;    // ragged-end tables up to these sizes sit in shared
-constexpr size_t kStreamNextSmem = 12 * 1024;     // memory, larger ones are read through L1
+constexpr size_t kStreamWalkSmem = 24 * 1024;     // a walk table up to this size sits in shared memory,
+                                                  // a larger one is read through L1
 constexpr size_t kStreamStaging = 4096;           // per-warp staging (kStreamPair, kStreamSingle)
 
 // Device copy of one automaton (one per device it was uploaded to).
@@ -105,8 +110,8 @@ struct DeviceAutomaton {
     uint16_t *slot_state = nullptr;
     uint16_t *all_states = nullptr;   // [n_states]: state s (every state as a start, for pieces)
     // merge graph and stream table (HostMerge, HostStream); null when not built
-    uint16_t *mg_next = nullptr, *mg_node_part = nullptr, *mg_images = nullptr, *mg_part = nullptr;
-    uint32_t *mg_leaf = nullptr, *mg_node_img = nullptr, *mg_slot_alive = nullptr;
+    uint16_t *mg_walk = nullptr, *mg_edge_pid = nullptr, *mg_node_part = nullptr, *mg_images = nullptr, *mg_part = nullptr;
+    uint32_t *mg_node_img = nullptr, *mg_slot_alive = nullptr;
     uint32_t *st_code = nullptr, *st_words = nullptr;
     size_t bytes = 0;
 };

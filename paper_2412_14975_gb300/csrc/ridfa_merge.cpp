@@ -121,6 +121,15 @@ bool build_graph(const HostAutomaton &H, HostMerge &G) {
     }
     G.inner = static_cast<uint32_t>(node_d.size());
     G.parts = parts;
+    if (n + 1 + G.inner > 0xFFFF) return false;
+    // one-byte steps of states and nodes in one table: states first, then the nodes
+    G.walk = H.trans;
+    for (uint16_t e : G.next) {
+        const uint32_t l = e & kLeafBit ? G.leaf[e & 0x7FFF] : 0;
+        G.walk.push_back(static_cast<uint16_t>(e & kLeafBit ? l & 0xFFFF : e + n + 1));
+        G.edge_pid.push_back(static_cast<uint16_t>(l >> 16));
+    }
+    G.walk.resize(G.walk.size() + (G.walk.size() & 1), static_cast<uint16_t>(n));    // whole words
     G.slot_alive.assign(static_cast<size_t>(parts) * H.kw, 0);
     for (uint32_t p = 0; p < parts; ++p)
         for (uint32_t a = 0; a < H.k; ++a)
@@ -135,8 +144,11 @@ bool graph_in_bounds(const HostAutomaton &H, const HostMerge &G) {
     if (G.next.size() != static_cast<size_t>(G.inner) * H.n_classes || G.part.size() != static_cast<size_t>(G.parts) * n ||
         G.node_part.size() != G.inner || G.node_img.size() != G.inner || G.leaf.empty())
         return false;
-    for (uint16_t c : G.next)
-        if ((c & kLeafBit) ? (c & 0x7FFFu) >= G.leaf.size() : c >= G.inner) return false;
+    if (G.walk.size() < static_cast<size_t>(n + 1 + G.inner) * H.n_classes || G.edge_pid.size() != G.next.size()) return false;
+    for (uint16_t c : G.walk)
+        if (c >= n + 1 + G.inner) return false;
+    for (uint16_t q : G.edge_pid)
+        if (q >= G.parts) return false;
     for (uint32_t l : G.leaf)
         if ((l >> 16) >= G.parts || (l & 0xFFFF) > n) return false;
     for (uint16_t s : G.images)
@@ -164,10 +176,9 @@ double wavefronts(uint32_t copies) {
 }
 
 size_t rest_bytes(const HostAutomaton &H, uint32_t kind) {
-    // class codes, one-byte table and byte classes for the ragged ends, graph edges
-    const size_t trans = H.trans.size() * 2, next = H.merge.next.size() * 2;
-    return (kind == kStreamField ? 0 : 256 * 128) + (trans <= kStreamTransSmem ? (trans + 15) / 16 * 16 : 0) + 256 +
-           (next <= kStreamNextSmem ? (next + 15) / 16 * 16 : 0) + 256;
+    // class codes; byte classes and the one-byte table of the ragged ends
+    const size_t walk = H.merge.walk.size() * 2;
+    return (kind == kStreamField ? 0 : 256 * 128) + 256 + (walk <= kStreamWalkSmem ? (walk + 15) / 16 * 16 : 0) + 256;
 }
 
 // Column offsets of a pair table: offset(c1, c2) = first[c1] + second[c2], where equal sums mean
@@ -374,6 +385,8 @@ void build_table(HostAutomaton &H) {
 size_t stream_table_bytes(const HostAutomaton &H) {
     return rest_bytes(H, H.stream.kind) + static_cast<size_t>(H.n_states + 1) * H.stream.row_words * 4 * H.stream.copies;
 }
+
+size_t stream_walk_bytes(const HostAutomaton &H) { return rest_bytes(H, kStreamField); }
 
 void build_stream(HostAutomaton &H) {
     HostMerge G;

@@ -22,60 +22,83 @@
 namespace ridfa {
 namespace {
 
-constexpr uint32_t kNoNode = 0xFFFFFFFFu;
 constexpr uint32_t kNodeResult = 0x80000000u;   // a piece that ended in an inner node
 constexpr uint32_t kGlobal = 0xFFFFFFFFu;       // a ragged-end table left in global memory
 constexpr int kStreamBlock = 1024;
 
 struct StreamArgs {
     const uint8_t *text;
-    uint64_t len, np, q, r;       // np pieces; q = len / np, r = len % np
+    uint64_t len, q, frac;        // chunk i begins at i * q + (i * frac >> 64): floor(i * len / c)
+    uint64_t step;                // bytes per piece of a chunk, 16 fraction bits
+    uint32_t np, per_chunk;       // pieces in all, and per chunk
+    uint32_t warps;               // warps of a block that take pieces (all of them load the tables)
     uint32_t *res;                // [np]: kNodeResult | node, or pid << 16 | state
-    const uint16_t *trans;
+    const uint16_t *walk, *edge_pid;
     const uint8_t *classmap;
-    const uint16_t *next;
-    const uint32_t *leaf, *code, *words;
-    uint32_t n, C, inner;
+    const uint32_t *code, *words;
+    uint32_t n, C, n_walk;        // n_walk: entries of the walk table
     uint32_t n_words, copies, row;                       // row: bytes per state
-    uint32_t shift, mask, mul, sh_w, m_w, sh_q, m_q, canon;   // field codes
-    uint32_t off_table, off_trans, off_cls, off_next, off_stage;
+    // field codes: byte of code 0 (four times) and what each field bit and both add to it; where the
+    // codes of bytes 0.. (and 2.. for two-byte lookups) gather; column -> byte offset
+    uint32_t shift, canon0, d1, d2, d12, mul, mul_h, take_bits, part_mask, col_mul, part_mul;
+    uint32_t off_table, off_walk, off_cls, off_stage;
 };
 
-__device__ __forceinline__ uint64_t piece_begin(const StreamArgs &p, uint64_t i) {
-    return i * p.q + (p.r ? i * p.r / p.np : 0);         // floor(i * len / np)
+__device__ __forceinline__ uint64_t chunk_at(const StreamArgs &p, uint32_t i) {
+    return i * p.q + __umul64hi(i, p.frac);
 }
 
-// The state of one lane between bytes, and one-byte steps for everything that is not a whole
-// granule of a merged run: the graph walk, ragged starts and ends.
-struct Walk {
-    const uint16_t *trans, *next;
-    const uint32_t *leaf;
-    const uint8_t *cls;
-    uint32_t C;
-    uint32_t node, pid, s;
-    __device__ __forceinline__ void start() {
-        node = 0;
-        pid = 0;
-        s = 0;
+// Piece x as addresses [pos, end).  Inside a chunk the pieces meet at 32-byte boundaries.
+__device__ __forceinline__ void piece_range(const StreamArgs &p, uint32_t x, uint64_t t0, uint64_t &pos, uint64_t &end) {
+    if (p.per_chunk == 1) {
+        pos = t0 + chunk_at(p, x);
+        end = t0 + chunk_at(p, x + 1);
+        return;
     }
-    __device__ __forceinline__ void step(uint32_t b) {
-        const uint32_t c = cls[b];
-        if (node == kNoNode) {
-            s = trans[s * C + c];
-            return;
-        }
-        const uint32_t e = next[node * C + c];
-        if (e & kLeafBit) {
-            const uint32_t l = __ldg(leaf + (e & 0x7FFF));
-            pid = l >> 16;
-            s = l & 0xFFFF;
-            node = kNoNode;
+    const uint32_t i = x / p.per_chunk, t = x - i * p.per_chunk;
+    const uint64_t b = t0 + chunk_at(p, i);
+    pos = t ? (b + (t * p.step >> 16)) & ~static_cast<uint64_t>(31) : b;
+    end = t + 1 < p.per_chunk ? (b + ((t + 1) * p.step >> 16)) & ~static_cast<uint64_t>(31) : t0 + chunk_at(p, i + 1);
+}
+
+// A lane between bytes, and the one-byte steps that everything outside whole granules of a merged
+// run takes: the graph walk, ragged starts and ends.  id: a state (id <= n, one run left), or a
+// node of the graph (id - n - 1); edge: the last step taken from a node, which names the leaf.
+struct Walk {
+    const StreamArgs &p;
+    uint32_t cls, tab;           // shared addresses of the byte classes and of the walk table
+    uint32_t id, edge;
+    __device__ __forceinline__ Walk(const StreamArgs &args, uint32_t base) : p(args), cls(base + args.off_cls), tab(base + args.off_walk) {}
+    __device__ __forceinline__ void start() {
+        id = p.n + 1;
+        edge = 0;
+    }
+    __device__ __forceinline__ bool merged() const { return id <= p.n; }
+    __device__ __forceinline__ bool dead() const { return id == p.n; }
+    __device__ __forceinline__ uint32_t class_of(uint32_t b) const { return lds_u8(cls + b); }
+    __device__ __forceinline__ void step_class(uint32_t c) {
+        const uint32_t at = id * p.C + c;
+        edge = id > p.n ? at : edge;
+        id = p.off_walk != kGlobal ? lds_u16(tab + 2 * at) : __ldg(p.walk + at);
+    }
+    // bytes [lo, hi) of 4 * N bytes: the classes are looked up ahead of the dependent steps
+    template <int N>
+    __device__ __forceinline__ void take(const uint32_t (&w)[N], int lo, int hi) {
+        uint32_t c[4 * N];
+#pragma unroll
+        for (int i = 0; i < 4 * N; ++i) c[i] = class_of((w[i >> 2] >> (8 * (i & 3))) & 0xFF);
+        if (lo <= 0 && hi >= 4 * N) {
+#pragma unroll
+            for (int i = 0; i < 4 * N; ++i) step_class(c[i]);
         } else {
-            node = e;
+#pragma unroll
+            for (int i = 0; i < 4 * N; ++i)
+                if (i >= lo && i < hi) step_class(c[i]);
         }
     }
     __device__ __forceinline__ uint32_t result() const {
-        return node == kNoNode ? pid << 16 | s : kNodeResult | node;
+        if (!merged()) return kNodeResult | (id - p.n - 1);
+        return static_cast<uint32_t>(__ldg(p.edge_pid + (edge - (p.n + 1) * p.C))) << 16 | id;
     }
 };
 
@@ -84,70 +107,89 @@ __device__ __forceinline__ uint32_t lds_entry(uint32_t a) {
     return E == 1 ? lds_u8(a) : lds_u16(a);
 }
 
-// Table steps of a merged run.  KIND and G (bytes a lookup) as in HostStream, E: bytes per entry.
-template <int KIND, int G, int E>
+// Table steps of a merged run.  KIND, G (bytes a lookup) and W (field bits) as in HostStream, E: bytes
+// per entry.
+template <int KIND, int G, int E, int W = 0>
 struct Steps {
     static constexpr bool kStaged = KIND != kStreamField;
-    uint32_t lc, lt, row;        // this lane's class codes; its copy of the table; bytes per state
-    uint32_t shift, mask, mul, sh_w, m_w, sh_q, m_q, canon, dead;
-    __device__ __forceinline__ void init(const StreamArgs &p, uint32_t base) {
+    const StreamArgs &p;         // (kernel parameters: constant operands, not registers)
+    uint32_t lc, lt;             // this lane's class codes; its copy of the table
+    __device__ __forceinline__ Steps(const StreamArgs &args, uint32_t base) : p(args) {
         const uint32_t lane = threadIdx.x & 31;
         lc = base + lane * 4;
         lt = base + p.off_table + (lane & (p.copies - 1)) * 4;
-        row = p.row;
-        dead = p.n;
-        if (KIND == kStreamField) {
-            shift = p.shift; mask = p.mask; mul = p.mul; canon = p.canon;
-            sh_w = p.sh_w; m_w = p.m_w; sh_q = p.sh_q; m_q = p.m_q;
-        }
     }
-    __device__ __forceinline__ uint32_t byte_at(const uint32_t *w, int q) const { return (w[q >> 2] >> (8 * (q & 3))) & 0xFF; }
+    // one lookup of G bytes whose codes a multiplication gathered in the top bits of g
+    __device__ __forceinline__ uint32_t column_step(uint32_t s, uint32_t g) const {
+        const uint32_t col = __umulhi(g, p.take_bits);           // (a shift on the multiplier's pipe)
+        return lds_entry<E>(s * p.row + (col * p.col_mul + ((col & p.part_mask) * p.part_mul + lt)));
+    }
+    // address of the class codes of byte q: mask the byte where it is, then one multiply-add for the
+    // shift and the base (the logic pipe is the busier one)
+    __device__ __forceinline__ uint32_t code_at(const uint32_t *w, int q) const {
+        const uint32_t x = w[q >> 2] & (0xFFu << (8 * (q & 3)));
+        if ((q & 3) == 0) return x * 128 + lc;
+        uint32_t a;
+        asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(a) : "r"(x), "r"(1u << (39 - 8 * (q & 3))), "r"(lc));
+        return a;
+    }
     // N 32-bit words of text
     template <int N>
     __device__ __forceinline__ uint32_t take(uint32_t s, const uint32_t (&w)[N]) const {
         if constexpr (KIND == kStreamField) {
-            // codes: mask the field of all four bytes, gather them with one multiplication (byte 0's
-            // code lowest at bit 24), split into word and part of the entry.  A byte that differs
-            // from its code's canonical byte is outside the alphabet: the run is dead after it.
+            // The field of all four bytes is masked out (m) and the codes of a lookup's bytes are
+            // gathered by one multiplication (no two partial products share a bit).  Each byte is
+            // rebuilt from its field bits by multiplications, which share the work with the logic
+            // pipe; a byte that differs is outside the alphabet, and its run is dead after it.
             uint32_t bad = 0;
 #pragma unroll
             for (int i = 0; i < N; ++i) {
-                const uint32_t m = (w[i] >> shift) & mask;
-                const uint32_t y = m | (m >> 4);
-                bad |= __byte_perm(canon, 0, __byte_perm(y, 0, 0x4420)) ^ w[i];
-                if (G == 4) {
-                    const uint32_t g = m * mul;
-                    s = lds_entry<E>(s * row + (((g >> sh_w) & m_w) + ((g >> sh_q) & m_q) + lt));
-                } else {
-                    const uint32_t g = m * mul, h = (m >> 16) * mul;
-                    s = lds_entry<E>(s * row + (((g >> sh_w) & m_w) + ((g >> sh_q) & m_q) + lt));
-                    s = lds_entry<E>(s * row + (((h >> sh_w) & m_w) + ((h >> sh_q) & m_q) + lt));
+                const uint32_t f = w[i] >> p.shift;
+                const uint32_t m1 = f & 0x01010101u;
+                uint32_t m = m1, whole = m1 * p.d1 + p.canon0;
+                if (W == 2) {
+                    const uint32_t m2 = (w[i] >> (p.shift + 1)) & 0x01010101u;
+                    m = f & 0x03030303u;
+                    whole += m2 * p.d2 + (m1 & m2) * p.d12;
                 }
+                bad |= whole ^ w[i];
+                s = column_step(s, m * p.mul);
+                if (G == 2) s = column_step(s, m * p.mul_h);
             }
-            return bad ? dead : s;
+            return bad ? p.n : s;
         } else if constexpr (KIND == kStreamPair) {
             uint32_t x[2 * N];
 #pragma unroll
             for (int i = 0; i < 2 * N; ++i)
-                x[i] = lds_u16(lc + (byte_at(w, 2 * i) << 7)) + lds_u16(lc + 2 + (byte_at(w, 2 * i + 1) << 7)) + lt;
+                x[i] = lds_u16(code_at(w, 2 * i)) + lds_u16(code_at(w, 2 * i + 1) + 2) + lt;
 #pragma unroll
-            for (int i = 0; i < 2 * N; ++i) s = lds_entry<E>(s * row + x[i]);
+            for (int i = 0; i < 2 * N; ++i) s = lds_entry<E>(s * p.row + x[i]);
             return s;
         } else {
             uint32_t x[4 * N];
 #pragma unroll
-            for (int i = 0; i < 4 * N; ++i) x[i] = lds_u32(lc + (byte_at(w, i) << 7)) + lt;
+            for (int i = 0; i < 4 * N; ++i) x[i] = lds_u32(code_at(w, i)) + lt;
 #pragma unroll
-            for (int i = 0; i < 4 * N; ++i) s = lds_entry<E>(s * row + x[i]);
+            for (int i = 0; i < 4 * N; ++i) s = lds_entry<E>(s * p.row + x[i]);
             return s;
         }
     }
 };
 
+// The one-byte tables in shared memory (a large walk table stays in global memory).
+__device__ __forceinline__ void load_walk(const StreamArgs &p, uint8_t *smem) {
+    const uint32_t base = smem_addr(smem);
+    for (uint32_t i = threadIdx.x; i < 64; i += blockDim.x)
+        sts_u32(base + p.off_cls + 4 * i, __ldg(reinterpret_cast<const uint32_t *>(p.classmap) + i));
+    if (p.off_walk != kGlobal)
+        for (uint32_t i = threadIdx.x; i < p.n_walk / 2; i += blockDim.x)
+            sts_u32(base + p.off_walk + 4 * i, __ldg(reinterpret_cast<const uint32_t *>(p.walk) + i));
+}
+
 // Shared-memory tables of a block: class codes (32 lane copies), the main table in its lane copies,
 // and the one-byte tables of the ragged ends.
 template <class S>
-__device__ __forceinline__ void load_tables(const StreamArgs &p, uint8_t *smem, Walk &w) {
+__device__ __forceinline__ void load_tables(const StreamArgs &p, uint8_t *smem) {
     const uint32_t base = smem_addr(smem);
     const uint32_t nt = blockDim.x;
     auto put4 = [&](uint32_t a, uint32_t v) {
@@ -162,68 +204,100 @@ __device__ __forceinline__ void load_tables(const StreamArgs &p, uint8_t *smem, 
         for (uint32_t i = threadIdx.x; i < p.n_words * p.copies; i += nt)
             sts_u32(base + p.off_table + i * 4, __ldg(p.words + i / p.copies));
     }
-    w.cls = smem + p.off_cls;
-    for (uint32_t i = threadIdx.x; i < 64; i += nt)
-        reinterpret_cast<uint32_t *>(smem + p.off_cls)[i] = __ldg(reinterpret_cast<const uint32_t *>(p.classmap) + i);
-    w.trans = p.trans;
-    if (p.off_trans != kGlobal) {
-        uint16_t *t = reinterpret_cast<uint16_t *>(smem + p.off_trans);
-        for (uint32_t i = threadIdx.x; i < (p.n + 1) * p.C; i += nt) t[i] = __ldg(p.trans + i);
-        w.trans = t;
-    }
-    w.next = p.next;
-    if (p.off_next != kGlobal) {
-        uint16_t *t = reinterpret_cast<uint16_t *>(smem + p.off_next);
-        for (uint32_t i = threadIdx.x; i < p.inner * p.C; i += nt) t[i] = __ldg(p.next + i);
-        w.next = t;
-    }
-    w.leaf = p.leaf;
-    w.C = p.C;
+    load_walk(p, smem);
 }
 
-// Text through 32-byte loads of each lane's own piece, one block ahead: an L1 line per lane and
-// load, so 1.2 LSU cycles per 32 text bytes; worth it where the lookups take less than one.
+// Text through 32-byte loads of each lane's own piece: an L1 line per lane and load, so 1.2 LSU
+// cycles per 32 text bytes; worth it where the lookups take less than one.
 __device__ __forceinline__ void load32(const uint8_t *a, uint32_t (&w)[8]) {
     asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
                  : "l"(a));
 }
 
-// One-byte steps over [pos, end) while the run is not merged or `pos` is not 32-byte aligned (or,
-// with `all`, to the end), the text taken in aligned 8-byte loads where they lie inside it.
-__device__ __forceinline__ void walk_ragged(Walk &w, uint64_t &pos, uint64_t end, uint64_t t0, uint64_t t1, bool all) {
-    while (pos < end && (all || w.node != kNoNode || (pos & 31))) {
-        const uint64_t a = pos & ~static_cast<uint64_t>(7);
-        uint64_t v;
-        uint32_t m = 1;
-        if (a >= t0 && a + 8 <= t1) {
-            const uint32_t o = static_cast<uint32_t>(pos & 7);
-            v = __ldg(reinterpret_cast<const unsigned long long *>(a)) >> (8 * o);
-            m = static_cast<uint32_t>(min(static_cast<uint64_t>(8 - o), end - pos));
+// One-byte steps over [pos, end) by 32-byte blocks of the text, one block ahead.
+__device__ __forceinline__ void walk_blocks(Walk &w, uint64_t pos, uint64_t end) {
+    uint32_t cur[8], nxt[8];
+    uint64_t a = pos & ~static_cast<uint64_t>(31);
+    const uint8_t *const text = w.p.text;
+    auto inside = [&](uint64_t x) { return x >= reinterpret_cast<uint64_t>(text) && x + 32 <= reinterpret_cast<uint64_t>(text) + w.p.len; };
+    if (pos < end && inside(a)) load32(reinterpret_cast<const uint8_t *>(a), cur);
+    while (pos < end && !w.dead()) {
+        const uint64_t b = min(end, a + 32);
+        if (b < end && inside(a + 32)) load32(reinterpret_cast<const uint8_t *>(a + 32), nxt);
+        if (inside(a)) {
+            int lo = static_cast<int>(pos - a), hi = static_cast<int>(b - a);
+#pragma unroll 1
+            for (int h = 0; h < 4; ++h, lo -= 8, hi -= 8) {       // (the block moves down 8 bytes a turn)
+                const uint32_t v[2] = {cur[0], cur[1]};
+                if (lo < 8 && hi > 0) w.take(v, lo, hi);
+#pragma unroll
+                for (int i = 0; i < 6; ++i) cur[i] = cur[i + 2];
+            }
+            pos = b;
         } else {
-            v = __ldg(reinterpret_cast<const uint8_t *>(pos));
+            while (pos < b) w.step_class(w.class_of(__ldg(reinterpret_cast<const uint8_t *>(pos++))));
         }
-        pos += m;
-        for (uint32_t i = 0; i < m; ++i, v >>= 8) w.step(static_cast<uint32_t>(v) & 0xFF);
+        a += 32;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
+    }
+}
+
+// One-byte steps over [pos, end), until the end or -- with `to_block` -- until one run is left at a
+// 32-byte boundary: the few ragged bytes at the ends of a long piece, by 8-byte words, with little held in registers beside the main loop's blocks.
+__device__ __forceinline__ void walk_ends(Walk &w, uint64_t &pos, uint64_t end, bool to_block) {
+    const uint64_t t0 = reinterpret_cast<uint64_t>(w.p.text);
+#pragma unroll 1
+    while (pos < end && !w.dead() && !(to_block && w.merged() && !(pos & 31))) {
+        const uint64_t a = pos & ~static_cast<uint64_t>(7);
+        if (a >= t0 && a + 8 <= t0 + w.p.len) {
+            const uint2 x = __ldg(reinterpret_cast<const uint2 *>(a));
+            const uint32_t v[2] = {x.x, x.y};
+            const int lo = static_cast<int>(pos & 7), hi = static_cast<int>(min(static_cast<uint64_t>(8), end - a));
+            w.take(v, lo, hi);
+            pos += hi - lo;
+        } else {
+            w.step_class(w.class_of(__ldg(reinterpret_cast<const uint8_t *>(pos++))));
+        }
     }
 }
 
 template <class S>
-__device__ __forceinline__ void stream_direct(const S &T, Walk &w, uint64_t pos, uint64_t end, uint64_t t0, uint64_t t1) {
-    walk_ragged(w, pos, end, t0, t1, false);
-    uint32_t blocks = pos < end ? static_cast<uint32_t>((end - pos) >> 5) : 0;
-    if (blocks && w.node == kNoNode) {
-        uint32_t cur[8], nxt[8];
-        load32(reinterpret_cast<const uint8_t *>(pos), cur);
-        for (; blocks; --blocks, pos += 32) {
-            if (blocks > 1) load32(reinterpret_cast<const uint8_t *>(pos + 32), nxt);
-            w.s = T.template take<8>(w.s, cur);
-            if (w.s == T.dead) return;
+__device__ __forceinline__ void stream_direct(const S &T, Walk &w, uint64_t pos, uint64_t end) {
+    walk_ends(w, pos, end, true);
+    uint32_t blocks = pos < end && !w.dead() ? static_cast<uint32_t>((end - pos) >> 5) : 0;
+    if (blocks) {
+        auto take_block = [&](const uint32_t (&x)[8]) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
+            for (int h = 0; h < 8; h += 4) {
+                const uint32_t v[4] = {x[h], x[h + 1], x[h + 2], x[h + 3]};
+                w.id = T.template take<4>(w.id, v);
+            }
+        };
+        // three blocks in flight or in hand, each loaded again as soon as it is done with
+        uint32_t b[3][8];
+        const uint8_t *t = reinterpret_cast<const uint8_t *>(pos);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            if (blocks > static_cast<uint32_t>(i)) load32(t + 32 * i, b[i]);
+        pos += static_cast<uint64_t>(blocks) * 32;
+        for (;;) {
+            take_block(b[0]);
+            if (blocks > 3) load32(t + 96, b[0]);
+            if (blocks == 1) break;
+            take_block(b[1]);
+            if (blocks > 4) load32(t + 128, b[1]);
+            if (blocks == 2) break;
+            take_block(b[2]);
+            if (blocks > 5) load32(t + 160, b[2]);
+            if (blocks == 3 || w.dead()) break;
+            blocks -= 3;
+            t += 96;
         }
+        if (w.dead()) return;
     }
-    walk_ragged(w, pos, end, t0, t1, true);
+    walk_ends(w, pos, end, false);
 }
 
 // Text staged by the warp: rounds of one 64-byte window per lane, copied with cp.async (L2 to
@@ -236,7 +310,7 @@ __device__ __forceinline__ void stream_staged(const S &T, Walk &w, uint32_t stag
     const uint64_t lo = (t0 + 15) & ~static_cast<uint64_t>(15), hi = t1 & ~static_cast<uint64_t>(15);
     // offsets are from the start of the warp's first piece (pieces ascend)
     const uint64_t base = __shfl_sync(kFull, pos, 0) & ~static_cast<uint64_t>(15);
-    while (pos < min(end, lo)) w.step(__ldg(reinterpret_cast<const uint8_t *>(pos++)));
+    while (pos < min(end, lo)) w.step_class(w.class_of(__ldg(reinterpret_cast<const uint8_t *>(pos++))));
     const uint64_t stop64 = min(end, hi);
     const bool have = pos < stop64;
     const uint32_t wrel = have ? static_cast<uint32_t>((pos & ~static_cast<uint64_t>(15)) - base) : 0;
@@ -268,30 +342,26 @@ __device__ __forceinline__ void stream_staged(const S &T, Walk &w, uint32_t stag
         else cp_async_commit();
         cp_async_wait1();
         __syncwarp();
-        if (r < nwin && (w.node != kNoNode || w.s != T.dead)) {
+        if (r < nwin && !w.dead()) {
             const uint32_t ws = wrel + kCoopWin * r;
             const uint32_t sb = stage + (r & 1) * kCoopBufBytes + 64 * lane;
             const uint32_t stop = min(srel, ws + kCoopWin);
-            if (w.node == kNoNode && prel == ws && stop == ws + kCoopWin) {
+            if (w.merged() && prel == ws && stop == ws + kCoopWin) {
 #pragma unroll
                 for (uint32_t q = 0; q < 4; ++q) {
                     const uint4 x = lds_v4(sb + 16 * (q ^ sw));
                     const uint32_t v[4] = {x.x, x.y, x.z, x.w};
-                    w.s = T.template take<4>(w.s, v);
+                    w.id = T.template take<4>(w.id, v);
                 }
             } else {
 #pragma unroll 1
                 for (uint32_t q = 0; q < 4; ++q) {
-                    const uint32_t a = max(prel, ws + 16 * q), b = min(stop, ws + 16 * q + 16);
+                    const uint32_t g0 = ws + 16 * q, a = max(prel, g0), b = min(stop, g0 + 16);
                     if (a >= b) continue;
-                    const uint32_t sa = sb + 16 * (q ^ sw);
-                    if (w.node == kNoNode && b - a == 16) {
-                        const uint4 x = lds_v4(sa);
-                        const uint32_t v[4] = {x.x, x.y, x.z, x.w};
-                        w.s = T.template take<4>(w.s, v);
-                    } else {
-                        for (uint32_t o = a; o < b; ++o) w.step(lds_u8(sa + ((o - ws) & 15)));
-                    }
+                    const uint4 x = lds_v4(sb + 16 * (q ^ sw));
+                    const uint32_t v[4] = {x.x, x.y, x.z, x.w};
+                    if (w.merged() && b - a == 16) w.id = T.template take<4>(w.id, v);
+                    else w.take(v, static_cast<int>(a - g0), static_cast<int>(b - g0));
                 }
             }
             prel = stop;
@@ -300,34 +370,33 @@ __device__ __forceinline__ void stream_staged(const S &T, Walk &w, uint32_t stag
     }
     cp_async_wait0();
     __syncwarp();
-    if (w.node == kNoNode && w.s == T.dead) return;
+    if (w.dead()) return;
     if (have) pos = base + prel;
-    while (pos < end) w.step(__ldg(reinterpret_cast<const uint8_t *>(pos++)));
+    while (pos < end) w.step_class(w.class_of(__ldg(reinterpret_cast<const uint8_t *>(pos++))));
 }
 
-template <int KIND, int G, int E>
-__global__ void __launch_bounds__(kStreamBlock, 1) rid_stream_kernel(StreamArgs p) {
+template <int KIND, int G, int E, int W>
+__global__ void __launch_bounds__(kStreamBlock, 1) rid_stream_kernel(const __grid_constant__ StreamArgs p) {
     extern __shared__ __align__(128) uint8_t smem[];
-    using S = Steps<KIND, G, E>;
-    Walk w;
-    load_tables<S>(p, smem, w);
-    S T;
-    T.init(p, smem_addr(smem));
+    using S = Steps<KIND, G, E, W>;
+    load_tables<S>(p, smem);
+    Walk w(p, smem_addr(smem));
+    const S T(p, smem_addr(smem));
     __syncthreads();
-    const uint32_t lane = threadIdx.x & 31;
-    const uint64_t warp0 = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t warps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp >= p.warps) return;                 // (only loaded tables)
     const uint64_t t0 = reinterpret_cast<uint64_t>(p.text), t1 = t0 + p.len;
-    for (uint64_t task = warp0; task * 32 < p.np; task += warps) {
-        const uint64_t i = task * 32 + lane;
-        const bool have = i < p.np;
-        const uint64_t pos = t0 + (have ? piece_begin(p, i) : p.len), end = have ? t0 + piece_begin(p, i + 1) : t1;
+    for (uint32_t task = blockIdx.x * p.warps + warp; task * 32 < p.np; task += gridDim.x * p.warps) {
+        const uint32_t x = task * 32 + lane;
+        const bool have = x < p.np;
+        uint64_t pos = t1, end = t1;
+        if (have) piece_range(p, x, t0, pos, end);
         w.start();
         if constexpr (S::kStaged)
-            stream_staged(T, w, smem_addr(smem) + p.off_stage + (threadIdx.x >> 5) * kWarpCoopBytes, pos, end, t0, t1);
+            stream_staged(T, w, smem_addr(smem) + p.off_stage + warp * kWarpCoopBytes, pos, end, t0, t1);
         else
-            stream_direct(T, w, pos, end, t0, t1);
-        if (have) p.res[i] = w.result();
+            stream_direct(T, w, pos, end);
+        if (have) p.res[x] = w.result();
     }
 }
 
@@ -364,30 +433,63 @@ __device__ __forceinline__ uint32_t apply_piece(const StreamJoinArgs &p, uint32_
 
 // Chunk i's function as one word where all of its pieces merged: pid of the first piece and the last
 // one's state, or partition 0 and the dead state when some piece's state finds no block in the next
-// piece.  By one lane (stride 1), or by a warp, each lane taking every 32nd piece.
-__device__ __forceinline__ void chunk_word(const StreamJoinArgs &p, uint64_t i, uint32_t first, uint32_t stride, bool &general,
-                                           bool &ok) {
-    const uint32_t n = p.j.A.n, s = p.per_chunk;
-    const uint32_t *r = p.res + i * s;
-    for (uint32_t t = first; t < s; t += stride) {
-        const uint32_t f = __ldg(r + t);
-        if (f & kNodeResult) {
-            general = true;
-        } else if (t) {
-            const uint32_t y = __ldg(r + t - 1);
-            if (!(y & kNodeResult)) {
-                const uint32_t x = y & 0xFFFF;
-                if (x >= n || __ldg(p.part + static_cast<uint64_t>(f >> 16) * n + x) == kNoBlock) ok = false;
-            }
-        }
-    }
+// piece; kGeneral when some piece never merged.
+__device__ __forceinline__ bool goes_on(const StreamJoinArgs &p, uint32_t y, uint32_t f) {
+    const uint32_t x = y & 0xFFFF;
+    return x < p.j.A.n && __ldg(p.part + static_cast<uint64_t>(f >> 16) * p.j.A.n + x) != kNoBlock;
 }
 
-__device__ __forceinline__ uint32_t chunk_result(const StreamJoinArgs &p, uint64_t i, bool general, bool ok) {
-    const uint32_t n = p.j.A.n;
-    if (general) return kGeneral;
-    const uint32_t f0 = __ldg(p.res + i * p.per_chunk), fl = __ldg(p.res + (i + 1) * p.per_chunk - 1);
-    return ok && (fl & 0xFFFF) != n ? (f0 & 0xFFFF0000u) | (fl & 0xFFFF) : n;
+// One lane, at most 4 pieces (results are read from L2: the fused join reads other blocks' ones).
+__device__ __forceinline__ uint32_t chunk_word(const StreamJoinArgs &p, uint64_t i) {
+    const uint32_t s = p.per_chunk, *r = p.res + i * s;
+    uint32_t f[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) f[t] = t < s ? __ldcg(r + t) : 0;
+    uint32_t node = f[0], last = f[0];
+    bool ok = true;
+#pragma unroll
+    for (int t = 1; t < 4; ++t)
+        if (t < s) {
+            node |= f[t];
+            last = f[t];
+        }
+    if (node & kNodeResult) return kGeneral;
+#pragma unroll
+    for (int t = 1; t < 4; ++t)
+        if (t < s) ok = goes_on(p, f[t - 1], f[t]) && ok;
+    return ok && (last & 0xFFFF) != p.j.A.n ? (f[0] & 0xFFFF0000u) | (last & 0xFFFF) : p.j.A.n;
+}
+
+// A warp: a piece per lane, up to eight at a time so that their loads overlap.
+__device__ __forceinline__ uint32_t chunk_word_warp(const StreamJoinArgs &p, uint64_t i, uint32_t lane) {
+    const uint32_t s = p.per_chunk, *r = p.res + i * s;
+    uint32_t first = 0, carry = 0;
+    bool node = false, ok = true;
+    for (uint32_t b = 0; b < s; b += 256) {
+        uint32_t f[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = b + 32 * u + lane < s ? __ldcg(r + b + 32 * u + lane) : 0;
+        if (b == 0) first = __shfl_sync(kFull, f[0], 0);
+        bool go[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            uint32_t y = __shfl_up_sync(kFull, f[u], 1);
+            const uint32_t end = __shfl_sync(kFull, f[u], 31);
+            if (lane == 0) y = carry;
+            carry = end;
+            const uint32_t t = b + 32 * u + lane;
+            node = node || (f[u] & kNodeResult);
+            go[u] = true;
+            if (t < s && t && !((f[u] | y) & kNodeResult)) go[u] = goes_on(p, y, f[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) ok = ok && go[u];
+    }
+    const uint32_t last = __ldcg(r + s - 1);
+    node = __any_sync(kFull, node);
+    ok = __all_sync(kFull, ok);
+    if (node) return kGeneral;
+    return ok && (last & 0xFFFF) != p.j.A.n ? (first & 0xFFFF0000u) | (last & 0xFFFF) : p.j.A.n;
 }
 
 // Map row and summary of a chunk some piece of which never merged, by a warp.
@@ -401,7 +503,7 @@ __device__ void general_row(const StreamJoinArgs &p, uint64_t i, uint32_t lane) 
         v[r] = kUndef;
         if (a < A.k) {
             uint32_t x = A.slot_state[a];
-            for (uint32_t t = 0; t < p.per_chunk && x < A.n; ++t) x = apply_piece(p, __ldg(p.res + i * p.per_chunk + t), x);
+            for (uint32_t t = 0; t < p.per_chunk && x < A.n; ++t) x = apply_piece(p, __ldcg(p.res + i * p.per_chunk + t), x);
             if (x < A.n) v[r] = x;
             p.maps[i * A.k + a] = static_cast<uint16_t>(v[r]);
         }
@@ -424,114 +526,170 @@ __device__ void general_row(const StreamJoinArgs &p, uint64_t i, uint32_t lane) 
     }
 }
 
-// Thread 0 of the last block: accept bit (when `acc` is one) and status to their places, counters
-// back to zero for the next call.
-__device__ void publish(const StreamJoinArgs &p) {
+// Thread 0 of the last block: accept bit and status to their places, counters back to zero for the
+// next call.
+__device__ void publish(const StreamJoinArgs &p, uint8_t acc) {
     const uint32_t st = *reinterpret_cast<volatile uint32_t *>(p.work);
     *p.j.status = st;
-    *p.work = 0;
+    if (st) *p.work = 0;
     *p.j.ticket = 0;
+    *p.j.accept = acc;
     if (p.h_accept) {
-        *p.h_accept = *reinterpret_cast<volatile uint8_t *>(p.j.accept);
-        *p.h_status = st;
-        __threadfence_system();
+        *p.h_accept = acc;
+        *p.h_status = st;                // (visible to the host once the kernel has ended)
     }
 }
 
-__global__ void __launch_bounds__(kJoinThreads) rid_stream_join_kernel(StreamJoinArgs p) {
-    __shared__ Prod s_prod[kJoinThreads];
-    __shared__ uint32_t s_info[kBatch + 1];
-    __shared__ uint32_t s_vec[RIDFA_MAX_SLOTS / 32], s_nvec[RIDFA_MAX_SLOTS / 32];
-    __shared__ uint32_t s_general, s_bits, s_last;
+struct JoinShared {
+    Prod prod[kJoinThreads];
+    uint32_t info[kBatch + 1];
+    uint32_t vec[RIDFA_MAX_SLOTS / 32], nvec[RIDFA_MAX_SLOTS / 32];
+    uint32_t general, bits, last;
+};
+
+// Words 31 and 32 of a block's partial product hold the words of its first and last chunk while the
+// product has at most one row.
+constexpr uint32_t kFirstInfo = kPartialWords - 2, kLastInfo = kPartialWords - 1;
+
+// The accept bit when some chunk has more than kMaxD distinct end states, by one block: if_min(PLAS_i)
+// as a k-bit set, chunk by chunk, every slot's end state worked out from the pieces.
+__device__ uint32_t accept_unmerged(const StreamJoinArgs &p, uint32_t *s_vec, uint32_t *s_nvec) {
+    const Automaton &A = p.j.A;
+    __shared__ uint32_t s_acc;
+    for (uint32_t w = threadIdx.x; w < A.kw; w += blockDim.x) s_vec[w] = (A.q0_slot >> 5) == w ? 1u << (A.q0_slot & 31) : 0u;
+    if (threadIdx.x == 0) s_acc = 0;
+    for (uint64_t i = 0; i < p.j.c; ++i) {
+        for (uint32_t w = threadIdx.x; w < A.kw; w += blockDim.x) s_nvec[w] = 0;
+        __syncthreads();
+        for (uint32_t a = threadIdx.x; a < A.k; a += blockDim.x) {
+            if (!((s_vec[a >> 5] >> (a & 31)) & 1)) continue;
+            uint32_t x = A.slot_state[a];
+            for (uint32_t t = 0; t < p.per_chunk && x < A.n; ++t) x = apply_piece(p, __ldcg(p.res + i * p.per_chunk + t), x);
+            if (x >= A.n) continue;
+            if (i + 1 == p.j.c) {
+                if (is_final(A, x)) s_acc = 1;
+            } else {
+                for (uint32_t w = 0; w < A.kw; ++w) {
+                    const uint32_t m = A.ifmask[static_cast<uint64_t>(x) * A.kw + w];
+                    if (m) atomicOr(&s_nvec[w], m);
+                }
+            }
+        }
+        __syncthreads();
+        for (uint32_t w = threadIdx.x; w < A.kw; w += blockDim.x) s_vec[w] = s_nvec[w];
+        __syncthreads();
+    }
+    return s_acc;
+}
+
+// The join of chunks [blk * chunks, ...) by one block of kJoinThreads threads, and by the last of
+// nblk blocks the whole.
+__device__ void stream_join(const StreamJoinArgs &p, uint32_t blk, uint32_t nblk, JoinShared &sh) {
     const Automaton &A = p.j.A;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint64_t c = p.j.c;
-    const uint64_t i0 = static_cast<uint64_t>(blockIdx.x) * p.chunks, i1 = min(c, i0 + p.chunks);
+    const uint64_t i0 = static_cast<uint64_t>(blk) * p.chunks, i1 = min(c, i0 + p.chunks);
     const uint32_t cnt = static_cast<uint32_t>(i1 - i0);
     const uint32_t before = i0 ? 1 : 0;          // the previous chunk is looked at too
     if (tid == 0) {
-        s_general = 0;
-        s_bits = 1;
+        sh.general = 0;
+        sh.bits = 1;
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     __syncthreads();
-    // ---- each chunk's function in one word: s_info[j] = chunk i0 - before + j
-    if (p.per_chunk <= 8) {
+    // ---- each chunk's function in one word: info[j] = chunk i0 - before + j
+    if (p.per_chunk <= 4) {
         for (uint32_t j = tid; j < cnt + before; j += blockDim.x) {
-            bool general = false, ok = true;
-            chunk_word(p, i0 - before + j, 0, 1, general, ok);
-            s_info[j] = chunk_result(p, i0 - before + j, general, ok);
-            if (general) s_general = 1;
+            const uint32_t v = chunk_word(p, i0 - before + j);
+            sh.info[j] = v;
+            if (v == kGeneral) sh.general = 1;
         }
     } else {
         for (uint32_t j = warp; j < cnt + before; j += blockDim.x / 32) {
-            bool general = false, ok = true;
-            chunk_word(p, i0 - before + j, lane, 32, general, ok);
-            general = __any_sync(kFull, general);
-            ok = __all_sync(kFull, ok);
+            const uint32_t v = chunk_word_warp(p, i0 - before + j, lane);
             if (lane == 0) {
-                s_info[j] = chunk_result(p, i0 - before + j, general, ok);
-                if (general) s_general = 1;
+                sh.info[j] = v;
+                if (v == kGeneral) sh.general = 1;
             }
         }
     }
     __syncthreads();
     // ---- map rows and summaries.  A block with an unmerged chunk also writes the row before its
-    // first (the same values as the block that owns it), which its transfer matrices read.
-    const uint32_t skip = s_general ? 0 : before;
+    // first (the same values as the block that owns it), which its transfer matrices read.  Rows that
+    // only the caller reads are written last, beside the other blocks' way to the result.
+    const bool unmerged = sh.general, rows_first = unmerged || p.j.summary;
+    const uint32_t skip = sh.general ? 0 : before;
     const uint32_t nrow = cnt + before - skip;
     const uint64_t r0 = i0 - before + skip;
     uint16_t *rows = p.maps + r0 * A.k;
-    auto cell = [&](uint32_t info, uint32_t a) -> uint32_t {
-        const uint32_t m = __ldg(p.slot_alive + (info >> 16) * A.kw + (a >> 5));
-        return (m >> (a & 31)) & 1 ? info & 0xFFFF : kUndef;
+    auto write_rows = [&]() {
+        if (!unmerged && A.k >= 8 && !(A.k & 1) && !(nrow * A.k & 7) && !(reinterpret_cast<uint64_t>(rows) & 15)) {
+            // 8 entries a thread and store, over at most two rows (k >= 8)
+            for (uint32_t e = tid * 8; e < nrow * A.k; e += blockDim.x * 8) {
+                uint32_t j = __umulhi(e, p.k_magic), a = e - j * A.k, v[4];
+                uint32_t info = sh.info[j + skip];
+                const uint32_t *alive = p.slot_alive + (info >> 16) * A.kw;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (a >= A.k) {
+                        a = 0;
+                        info = sh.info[++j + skip];
+                        alive = p.slot_alive + (info >> 16) * A.kw;
+                    }
+                    const uint32_t m = __ldg(alive + (a >> 5)) >> (a & 31), y = info & 0xFFFF;
+                    v[q] = (m & 1 ? y : kUndef) | (m & 2 ? y : kUndef) << 16;
+                    a += 2;
+                }
+                *reinterpret_cast<uint4 *>(rows + e) = make_uint4(v[0], v[1], v[2], v[3]);
+            }
+        } else if (!unmerged && !(A.k & 1) && !(reinterpret_cast<uint64_t>(rows) & 3)) {
+            uint32_t *rows32 = reinterpret_cast<uint32_t *>(rows);
+            for (uint32_t e = tid; e < nrow * A.k / 2; e += blockDim.x) {
+                const uint32_t j = __umulhi(2 * e, p.k_magic), a = 2 * e - j * A.k;
+                const uint32_t info = sh.info[j + skip];
+                const uint32_t m = __ldg(p.slot_alive + (info >> 16) * A.kw + (a >> 5)) >> (a & 31);
+                const uint32_t y = info & 0xFFFF;
+                rows32[e] = (m & 1 ? y : kUndef) | (m & 2 ? y : kUndef) << 16;
+            }
+        } else {
+            for (uint32_t e = tid; e < nrow * A.k; e += blockDim.x) {
+                const uint32_t j = A.k == 1 ? e : __umulhi(e, p.k_magic), a = e - j * A.k;
+                const uint32_t info = sh.info[j + skip];
+                if (info == kGeneral) continue;
+                const uint32_t m = __ldg(p.slot_alive + (info >> 16) * A.kw + (a >> 5));
+                rows[e] = static_cast<uint16_t>((m >> (a & 31)) & 1 ? info & 0xFFFF : kUndef);
+            }
+        }
     };
-    if (!s_general && !(A.k & 1) && !(reinterpret_cast<uint64_t>(rows) & 3)) {
-        uint32_t *rows32 = reinterpret_cast<uint32_t *>(rows);
-        for (uint32_t e = tid; e < nrow * A.k / 2; e += blockDim.x) {
-            const uint32_t j = A.k == 1 ? e : __umulhi(2 * e, p.k_magic), a = 2 * e - j * A.k;
-            const uint32_t info = s_info[j + skip];
-            const uint32_t m = __ldg(p.slot_alive + (info >> 16) * A.kw + (a >> 5)) >> (a & 31);
-            const uint32_t y = info & 0xFFFF;
-            rows32[e] = (m & 1 ? y : kUndef) | (m & 2 ? y : kUndef) << 16;
-        }
-    } else {
-        for (uint32_t e = tid; e < nrow * A.k; e += blockDim.x) {
-            const uint32_t j = A.k == 1 ? e : __umulhi(e, p.k_magic), a = e - j * A.k;
-            const uint32_t info = s_info[j + skip];
-            if (info != kGeneral) rows[e] = static_cast<uint16_t>(cell(info, a));
-        }
-    }
+    if (rows_first) write_rows();
     for (uint32_t j = tid; j < nrow; j += blockDim.x) {
-        const uint32_t info = s_info[j + skip];
+        const uint32_t info = sh.info[j + skip];
         if (info == kGeneral) continue;
         uint32_t any = 0;
         for (uint32_t w = 0; w < A.kw; ++w) any |= __ldg(p.slot_alive + (info >> 16) * A.kw + w);
         p.dinfo[r0 + j] = any && (info & 0xFFFF) != A.n ? (1u << 16) | (info & 0xFFFF) : static_cast<uint32_t>(kUndef);
     }
-    if (s_general) {
+    if (sh.general) {
         for (uint32_t j = warp; j < nrow; j += blockDim.x / 32)
-            if (s_info[j + skip] == kGeneral) general_row(p, r0 + j, lane);
+            if (sh.info[j + skip] == kGeneral) general_row(p, r0 + j, lane);
     }
     // ---- this block's boundaries (chunk i - 1 to i, i0 <= i < i1, i >= 1): their product
     Prod P;
     P.nrows = 0xFFFFFFFFu;
-    if (!s_general) {
-        const uint32_t j = tid + 1 - before;     // boundary into s_info[j + before]
+    if (!sh.general) {
         bool bit = true;
-        for (uint32_t b = j; b < cnt; b += blockDim.x) {
-            const uint32_t prev = s_info[b + before - 1], cur = s_info[b + before];
+        for (uint32_t b = tid + 1 - before; b < cnt; b += blockDim.x) {      // into info[b + before]
+            const uint32_t prev = sh.info[b + before - 1], cur = sh.info[b + before];
             uint32_t hit = 0;
             if ((prev & 0xFFFF) != A.n && (cur & 0xFFFF) != A.n)
                 for (uint32_t w = 0; w < A.kw; ++w)
                     hit |= __ldg(A.ifmask + static_cast<uint64_t>(prev & 0xFFFF) * A.kw + w) & __ldg(p.slot_alive + (cur >> 16) * A.kw + w);
             bit = bit && hit;
         }
-        if (!bit) s_bits = 0;
+        if (!bit) sh.bits = 0;
         __syncthreads();
         if (cnt + before > 1) {
-            P.nrows = (s_info[0] & 0xFFFF) != A.n ? 1 : 0;
-            P.rows[0] = s_bits;
+            P.nrows = (sh.info[0] & 0xFFFF) != A.n ? 1 : 0;
+            P.rows[0] = sh.bits;
         }
     } else {
         __syncthreads();                         // the rows above are in place
@@ -546,89 +704,117 @@ __global__ void __launch_bounds__(kJoinThreads) rid_stream_join_kernel(StreamJoi
             }
         }
         if (bad) atomicOr(p.work, kStatusBad);
-        s_prod[tid] = P;
+        sh.prod[tid] = P;
         __syncthreads();
         for (uint32_t stride = 1; stride < blockDim.x; stride *= 2) {
-            if ((tid % (2 * stride)) == 0 && tid + stride < blockDim.x) compose(s_prod[tid], s_prod[tid + stride]);
+            if ((tid % (2 * stride)) == 0 && tid + stride < blockDim.x) compose(sh.prod[tid], sh.prod[tid + stride]);
             __syncthreads();
         }
-        if (tid == 0) P = s_prod[0];
+        if (tid == 0) P = sh.prod[0];
     }
-    if (tid == 0) {
-        uint32_t *mine = p.j.partials + static_cast<uint64_t>(blockIdx.x) * kPartialWords;
-        mine[0] = P.nrows;
-        if (P.nrows != 0xFFFFFFFFu)
-            for (uint32_t x = 0; x < P.nrows; ++x) mine[1 + x] = P.rows[x];
-        __threadfence();
-        s_last = atomicAdd(p.j.ticket, 1) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // ---- last block: the product of all blocks, then lambda_1(q0) and the acceptance test
-    if (*reinterpret_cast<volatile uint32_t *>(p.work) & kStatusWide) {
-        if (p.j.summary) summary_wide(p.j, s_vec, s_nvec);
-        else accept_wide(p.j, s_vec, s_nvec);
+    uint32_t first = sh.info[before ? 1 : 0], last = sh.info[cnt + before - 1];
+    bool general = unmerged, bits = sh.bits;
+    if (nblk == 1 && !general && !rows_first) write_rows();
+    if (nblk > 1 || general) {
+        if (tid == 0) {
+            uint32_t *mine = p.j.partials + static_cast<uint64_t>(blk) * kPartialWords;
+            mine[0] = P.nrows;
+            if (P.nrows != 0xFFFFFFFFu)
+                for (uint32_t x = 0; x < P.nrows; ++x) mine[1 + x] = P.rows[x];
+            if (P.nrows == 0xFFFFFFFFu || P.nrows <= 1) {
+                mine[kFirstInfo] = first;
+                mine[kLastInfo] = last;
+            }
+            __threadfence();
+            sh.last = atomicAdd(p.j.ticket, 1) == nblk - 1;
+        }
         __syncthreads();
-        if (tid == 0) publish(p);
+        if (!rows_first) write_rows();
+        if (!sh.last) return;
+        __threadfence();
+        // ---- last block: the product of all blocks
+        if (*reinterpret_cast<volatile uint32_t *>(p.work) & kStatusWide) {
+            uint32_t acc = 0;
+            if (p.j.summary) summary_wide(p.j, sh.vec, sh.nvec);
+            else acc = accept_unmerged(p, sh.vec, sh.nvec);
+            __syncthreads();
+            if (tid == 0) publish(p, static_cast<uint8_t>(acc));
+            return;
+        }
+        // while every product has at most one row and column, it is the AND of their bits
+        if (tid == 0) {
+            sh.general = 0;
+            sh.bits = 1;
+        }
+        __syncthreads();
+        {
+            bool gen = false, bit = true;
+            const uint32_t *qf = p.j.partials + kFirstInfo;
+            const uint32_t *ql = p.j.partials + static_cast<uint64_t>(nblk - 1) * kPartialWords + kLastInfo;
+            first = __ldcg(qf);
+            last = __ldcg(ql);
+#pragma unroll 4
+            for (uint32_t b = tid; b < nblk; b += blockDim.x) {
+                const uint32_t *q = p.j.partials + static_cast<uint64_t>(b) * kPartialWords;
+                const uint32_t nr = __ldcg(q), row = __ldcg(q + 1);
+                if (nr != 0xFFFFFFFFu) {
+                    if (nr > 1 || (nr == 1 && row > 1)) gen = true;
+                    else bit = bit && nr == 1 && row == 1;
+                }
+            }
+            if (gen || first == kGeneral || last == kGeneral) sh.general = 1;
+            if (!bit) sh.bits = 0;
+        }
+        __syncthreads();
+        general = sh.general;
+        bits = sh.bits;
+    }
+    if (!general && !p.j.summary) {
+        if (tid == 0) {
+            const uint32_t q0 = A.q0_slot;
+            const bool enter = (__ldg(p.slot_alive + (first >> 16) * A.kw + (q0 >> 5)) >> (q0 & 31)) & 1;
+            publish(p, enter && bits && (first & 0xFFFF) != A.n && is_final(A, last & 0xFFFF) ? 1 : 0);
+        }
         return;
     }
-    // while every block's product has at most one row and column, it is the AND of their bits
-    if (tid == 0) {
-        s_general = 0;
-        s_bits = 1;
-    }
-    __syncthreads();
-    {
-        bool general = false, bit = true;
-        for (uint32_t b = tid; b < gridDim.x; b += blockDim.x) {
-            const volatile uint32_t *q = p.j.partials + static_cast<uint64_t>(b) * kPartialWords;
-            const uint32_t nr = q[0];
-            if (nr == 0xFFFFFFFFu) continue;
-            if (nr > 1) general = true;
-            else bit = bit && nr == 1 && q[1] == 1;
-            if (nr == 1 && q[1] > 1) general = true;
-        }
-        if (general) s_general = 1;
-        if (!bit) s_bits = 0;
-    }
-    __syncthreads();
     Prod tot;
     tot.nrows = 0xFFFFFFFFu;
-    if (!s_general) {
+    if (!general) {
         if (c > 1) {
             tot.nrows = 1;
-            tot.rows[0] = s_bits;
+            tot.rows[0] = bits;
         }
     } else {
-        for (uint32_t base = 0; base < gridDim.x; base += blockDim.x) {
+        for (uint32_t base = 0; base < nblk; base += blockDim.x) {
             Prod x;
             x.nrows = 0xFFFFFFFFu;
-            if (base + tid < gridDim.x) {
+            if (base + tid < nblk) {
                 const volatile uint32_t *q = p.j.partials + static_cast<uint64_t>(base + tid) * kPartialWords;
                 x.nrows = q[0];
                 if (x.nrows != 0xFFFFFFFFu)
                     for (uint32_t r = 0; r < x.nrows; ++r) x.rows[r] = q[1 + r];
             }
             __syncthreads();
-            s_prod[tid] = x;
+            sh.prod[tid] = x;
             __syncthreads();
             for (uint32_t stride = 1; stride < blockDim.x; stride *= 2) {
-                if ((tid % (2 * stride)) == 0 && tid + stride < blockDim.x) compose(s_prod[tid], s_prod[tid + stride]);
+                if ((tid % (2 * stride)) == 0 && tid + stride < blockDim.x) compose(sh.prod[tid], sh.prod[tid + stride]);
                 __syncthreads();
             }
-            if (tid == 0) compose(tot, s_prod[0]);
+            if (tid == 0) compose(tot, sh.prod[0]);
             __syncthreads();
         }
     }
     if (tid != 0) return;
     if (p.j.summary) {
         summary_matrix(p.j, tot);
-        publish(p);
+        publish(p, 0);
         return;
     }
-    // (chunk 0's row and summary come from another block: read past the caches of this one)
-    const uint16_t v0 = *reinterpret_cast<const volatile uint16_t *>(p.maps + A.q0_slot);
+    // (chunk 0's row may still be on its way: its entry for q0's slot from the pieces instead)
+    uint32_t x = A.slot_state[A.q0_slot];
+    for (uint32_t t = 0; t < p.per_chunk; ++t) x = apply_piece(p, __ldcg(p.res + t), x);
+    const uint16_t v0 = x < A.n ? static_cast<uint16_t>(x) : kUndef;
     uint8_t acc = 0;
     if (v0 != kUndef) {
         if (c == 1) {
@@ -640,37 +826,84 @@ __global__ void __launch_bounds__(kJoinThreads) rid_stream_join_kernel(StreamJoi
             if (x0 == 0xFFFFFFFFu || tot.nrows == 0xFFFFFFFFu || ml == 0xFFFFFFFFu) {
                 atomicOr(p.work, kStatusBad);
             } else if (x0 < tot.nrows) {
-                const uint32_t bits = tot.rows[x0];
+                const uint32_t row = tot.rows[x0];
                 for (uint32_t y = 0; y < ml; ++y)
-                    if (((bits >> y) & 1) && is_final(A, Dl[y])) acc = 1;
+                    if (((row >> y) & 1) && is_final(A, Dl[y])) acc = 1;
             }
         }
     }
-    *p.j.accept = acc;
-    publish(p);
+    publish(p, acc);
+}
+
+__global__ void __launch_bounds__(kJoinThreads) rid_stream_join_kernel(const __grid_constant__ StreamJoinArgs p) {
+    __shared__ JoinShared sh;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    stream_join(p, blockIdx.x, gridDim.x, sh);
+}
+
+// Short pieces: one-byte steps throughout, so a block has only the walk table to set up.  With
+// `fused` the last block to finish runs the join of the whole text (one launch in all).
+__global__ void __launch_bounds__(kJoinThreads) rid_stream_walk_kernel(const __grid_constant__ StreamArgs p, const __grid_constant__ StreamJoinArgs j, int fused) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ JoinShared sh;
+    load_walk(p, smem);
+    Walk w(p, smem_addr(smem));
+    __syncthreads();
+    const uint64_t t0 = reinterpret_cast<uint64_t>(p.text);
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < p.warps) {
+        for (uint32_t task = blockIdx.x * p.warps + warp; task * 32 < p.np; task += gridDim.x * p.warps) {
+            const uint32_t x = task * 32 + lane;
+            if (x >= p.np) break;
+            uint64_t pos, end;
+            piece_range(p, x, t0, pos, end);
+            w.start();
+            walk_blocks(w, pos, end);
+            p.res[x] = w.result();
+        }
+    }
+    if (!fused) return;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        sh.last = atomicAdd(j.j.ticket + 1, 1) == gridDim.x - 1;
+        if (sh.last) j.j.ticket[1] = 0;
+    }
+    __syncthreads();
+    if (!sh.last) return;
+    __threadfence();
+    __syncthreads();
+    stream_join(j, 0, 1, sh);
 }
 
 // --------------------------------------------------------------------------- host side
 using StreamKernel = void (*)(StreamArgs);
 
+template <int G, int E>
+StreamKernel field_kernel(const HostStream &T) {
+    return T.width == 1 ? rid_stream_kernel<kStreamField, G, E, 1> : rid_stream_kernel<kStreamField, G, E, 2>;
+}
+
 StreamKernel stream_kernel(const HostStream &T) {
     const bool b = T.entry == 1;
     switch (T.kind) {
         case kStreamField:
-            return T.group == 4 ? (b ? rid_stream_kernel<kStreamField, 4, 1> : rid_stream_kernel<kStreamField, 4, 2>)
-                                : (b ? rid_stream_kernel<kStreamField, 2, 1> : rid_stream_kernel<kStreamField, 2, 2>);
-        case kStreamPair: return b ? rid_stream_kernel<kStreamPair, 2, 1> : rid_stream_kernel<kStreamPair, 2, 2>;
-        default: return b ? rid_stream_kernel<kStreamSingle, 1, 1> : rid_stream_kernel<kStreamSingle, 1, 2>;
+            return T.group == 4 ? (b ? field_kernel<4, 1>(T) : field_kernel<4, 2>(T))
+                                : (b ? field_kernel<2, 1>(T) : field_kernel<2, 2>(T));
+        case kStreamPair: return b ? rid_stream_kernel<kStreamPair, 2, 1, 0> : rid_stream_kernel<kStreamPair, 2, 2, 0>;
+        default: return b ? rid_stream_kernel<kStreamSingle, 1, 1, 0> : rid_stream_kernel<kStreamSingle, 1, 2, 0>;
     }
 }
 
 constexpr uint64_t kMinPiece = 64;             // bytes a piece has at least, where chunks are cut
+// pieces up to this length (and texts up to kWalkText) take one-byte steps throughout
+constexpr uint64_t kWalkPiece = 192, kWalkText = 8u << 20;
 
 }  // namespace
 
 bool stream_takes(const HostAutomaton &H, uint64_t len, uint32_t c) {
-    // (the kernels keep a warp's 32 pieces within 32-bit offsets; stream_shape cuts any text of up
-    // to 2^40 bytes into pieces far below that)
+    // (the kernels keep a warp's 32 pieces within 32-bit offsets and number pieces in 32 bits;
+    // stream_shape cuts any text of up to 2^40 bytes into pieces far below that)
     return H.stream.kind != kStreamNone && c <= (1u << 26) && len <= (1ull << 40);
 }
 
@@ -679,13 +912,13 @@ StreamShape stream_shape(const HostAutomaton &H, uint64_t len, uint32_t c, int s
     const uint64_t W = H.stream.warps;
     const double L = static_cast<double>(len) / c;
     // Pieces per chunk: the SM with the most warps of pieces decides.  A full round of W warps and a
-    // rest of fewer than 16 take about as long as 16 warps do; a piece costs some 80 bytes beside
+    // rest of fewer than 14 take about as long as 14 warps do; a piece costs some 60 bytes beside
     // its own (ragged ends, graph walk).
     auto time = [&](uint64_t s) {
         const uint64_t warps = (static_cast<uint64_t>(c) * s + 31) / 32, m = (warps + sms - 1) / sms;
         const uint64_t rest = m % W;
-        return static_cast<double>(m / W * W + (rest ? std::max<uint64_t>(rest, std::min<uint64_t>(16, W)) : 0)) *
-               (L / static_cast<double>(s) + 80.0);
+        return static_cast<double>(m / W * W + (rest ? std::max<uint64_t>(rest, std::min<uint64_t>(14, W)) : 0)) *
+               (L / static_cast<double>(s) + 60.0);
     };
     uint64_t best = 1;
     double best_t = time(1);
@@ -700,15 +933,31 @@ StreamShape stream_shape(const HostAutomaton &H, uint64_t len, uint32_t c, int s
     const uint64_t lanes = static_cast<uint64_t>(sms) * 32;
     for (uint64_t s = 2; s <= 16; ++s) consider(s);
     for (uint64_t m = 1; m <= 2 * W; ++m) consider(m * lanes / c);
+    if (len <= kWalkText && len / c / best > kWalkPiece / 2) {
+        // a short text in pieces of some 64 to 128 bytes instead, where that is below kWalkPiece
+        const uint64_t s = std::max<uint64_t>(1, len / c / kMinPiece);
+        if (len / c / s <= kWalkPiece) best = s;
+    }
     S.per_chunk = static_cast<uint32_t>(best);
     S.pieces = static_cast<uint64_t>(c) * best;
+    S.walk_only = len <= kWalkText && len / S.pieces <= kWalkPiece;
     const uint64_t tasks = (S.pieces + 31) / 32;
-    const uint64_t warps = std::min<uint64_t>(W, (tasks + sms - 1) / sms);
-    S.block = static_cast<uint32_t>(warps * 32);
-    S.grid = static_cast<uint32_t>(std::min<uint64_t>(sms, (tasks + warps - 1) / warps));
-    S.smem = stream_table_bytes(H) + (H.stream.kind == kStreamField ? 0 : warps * kStreamStaging);
     // a join block takes 256 chunks, one thread each; where chunks have many pieces, a warp each
-    S.join_chunks = S.per_chunk <= 8 ? kBatch : std::min<uint32_t>(kBatch, std::max<uint32_t>(kJoinThreads / 32, (c + 1023) / 1024));
+    S.join_chunks = S.per_chunk <= 4 ? kBatch : std::min<uint32_t>(kBatch, std::max<uint32_t>(kJoinThreads / 32, (c + 1023) / 1024));
+    if (S.walk_only) {
+        // spread over the SMs first, then up to 8 warps a block, 4 blocks an SM
+        S.block = kJoinThreads;
+        S.warps = static_cast<uint32_t>(std::min<uint64_t>(kJoinThreads / 32, (tasks + sms - 1) / sms));
+        S.grid = static_cast<uint32_t>(std::min<uint64_t>(static_cast<uint64_t>(sms) * 4, (tasks + S.warps - 1) / S.warps));
+        S.smem = stream_walk_bytes(H);
+        S.fused = static_cast<uint64_t>(c) * std::max<uint64_t>(1, S.per_chunk / 32) <= 64;
+        if (S.fused) S.join_chunks = kBatch;
+    } else {
+        S.warps = static_cast<uint32_t>(std::min<uint64_t>(W, (tasks + sms - 1) / sms));
+        S.block = std::max<uint32_t>(S.warps * 32, 512);       // the idle ones help to load the tables
+        S.grid = static_cast<uint32_t>(std::min<uint64_t>(sms, (tasks + S.warps - 1) / S.warps));
+        S.smem = stream_table_bytes(H) + (H.stream.kind == kStreamField ? 0 : S.warps * kStreamStaging);
+    }
     S.join_blocks = static_cast<uint32_t>((static_cast<uint64_t>(c) + S.join_chunks - 1) / S.join_chunks);
     return S;
 }
@@ -720,63 +969,58 @@ cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_
     StreamArgs a{};
     a.text = C.text;
     a.len = C.len;
-    a.np = S.pieces;
-    a.q = C.len / S.pieces;
-    a.r = C.len % S.pieces;
+    a.q = C.len / C.c;
+    // ceil(2^64 * (len mod c) / c): exact floors, as i * frac is off by less than i / 2^64 < 1 / c
+    const uint64_t rem = C.len % C.c;
+    a.frac = rem ? static_cast<uint64_t>((static_cast<unsigned __int128>(rem) << 64) / C.c) + 1 : 0;
+    a.step = static_cast<uint64_t>((static_cast<unsigned __int128>(C.len) << 16) / C.c / S.per_chunk);
+    a.np = static_cast<uint32_t>(S.pieces);
+    a.per_chunk = S.per_chunk;
+    a.warps = S.warps;
     a.res = C.res;
-    a.trans = D.trans;
+    a.walk = D.mg_walk;
     a.classmap = D.classmap;
-    a.next = D.mg_next;
-    a.leaf = D.mg_leaf;
+    a.edge_pid = D.mg_edge_pid;
     a.code = D.st_code;
     a.words = D.st_words;
     a.n = H.n_states;
     a.C = H.n_classes;
-    a.inner = H.merge.inner;
+    a.n_walk = static_cast<uint32_t>(H.merge.walk.size());
     a.n_words = static_cast<uint32_t>(T.words.size());
     a.copies = T.copies;
     a.row = T.row_words * 4 * T.copies;
     if (T.kind == kStreamField) {
-        const uint32_t w = T.width, lgf = static_cast<uint32_t>(__builtin_ctz(T.copies)) + 2;   // log2 of bytes per word
+        const uint32_t w = T.width, bits = w * T.group, part = 4 / T.entry;
+        auto byte = [&](uint32_t code) { return T.canon >> (8 * code) & 0xFF; };
         a.shift = T.shift;
-        a.mask = ((1u << w) - 1) * 0x01010101u;
-        a.canon = T.canon;
-        // byte i's code to bit 24 + w * i
-        a.mul = 1u << 24 | 1u << (16 + w);
-        if (T.group == 4) a.mul |= 1u << (8 + 2 * w) | 1u << (3 * w);
-        // column = the code at bit 24: its low bits are the part of a word, the others the word
-        const uint32_t part = T.entry == 1 ? 2 : 1, cols = w * T.group;      // bits
-        a.m_q = (1u << std::min(part, cols)) - 1;
-        a.sh_q = 24;
-        if (T.entry == 2) {
-            a.m_q <<= 1;
-            a.sh_q = 23;
+        a.canon0 = byte(0) * 0x01010101u;
+        a.d1 = byte(1) - byte(0);
+        a.d2 = byte(2) - byte(0);
+        a.d12 = byte(3) - byte(2) - byte(1) + byte(0);
+        // byte i's code to bit 32 - bits + w * i
+        for (uint32_t i = 0; i < T.group; ++i) {
+            a.mul |= 1u << (32 - bits + w * i - 8 * i);
+            if (T.group == 2) a.mul_h |= 1u << (32 - bits + w * i - 8 * (i + 2));
         }
-        a.m_w = cols > part ? ((1u << (cols - part)) - 1) << lgf : 0;
-        a.sh_w = 24 + part - lgf;
+        a.take_bits = 1u << bits;
+        // column c sits at word c / part, entry c % part
+        a.part_mask = part - 1;
+        a.col_mul = 4 * T.copies / part;
+        a.part_mul = T.entry - a.col_mul;
     }
-    uint32_t off = T.kind == kStreamField ? 0 : 256 * 128;
-    a.off_table = off;
-    off += a.n_words * 4 * T.copies;
-    const uint32_t tb = static_cast<uint32_t>(H.trans.size() * 2), nb = static_cast<uint32_t>(H.merge.next.size() * 2);
-    off = (off + 15) & ~15u;
+    uint32_t off = 0;
+    if (!S.walk_only) {
+        off = T.kind == kStreamField ? 0 : 256 * 128;
+        a.off_table = off;
+        off += a.n_words * 4 * T.copies;
+        off = (off + 15) & ~15u;
+    }
+    const uint32_t wb = a.n_walk * 2;
     a.off_cls = off;
     off += 256;
-    a.off_trans = tb <= kStreamTransSmem ? off : kGlobal;
-    off += tb <= kStreamTransSmem ? (tb + 15) & ~15u : 0;
-    a.off_next = nb <= kStreamNextSmem ? off : kGlobal;
-    off += nb <= kStreamNextSmem ? (nb + 15) & ~15u : 0;
+    a.off_walk = wb <= kStreamWalkSmem ? off : kGlobal;
+    off += wb <= kStreamWalkSmem ? (wb + 15) & ~15u : 0;
     a.off_stage = (off + 127) & ~127u;
-    const StreamKernel kern = stream_kernel(T);
-    cudaError_t e = ensure_smem_cap(reinterpret_cast<const void *>(kern), S.smem);
-    if (e != cudaSuccess) return e;
-    kern<<<S.grid, S.block, S.smem, st>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (C.between) {
-        e = cudaEventRecord(C.between, st);
-        if (e != cudaSuccess) return e;
-    }
     const Automaton A{D.trans, D.classmap, D.final_bits, D.ifmask, D.slot_state,
                       H.n_states, H.n_classes, H.k, H.kw, H.q0_slot, H.merges};
     StreamJoinArgs j{};
@@ -795,6 +1039,25 @@ cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_
     j.work = C.work;
     j.h_accept = C.h_accept;
     j.h_status = C.h_status;
+    cudaError_t e;
+    if (S.walk_only) {
+        // (its static and dynamic shared memory together may pass 48 KB)
+        e = ensure_smem_cap(reinterpret_cast<const void *>(rid_stream_walk_kernel), 64 * 1024);
+        if (e != cudaSuccess) return e;
+        rid_stream_walk_kernel<<<S.grid, S.block, S.smem, st>>>(a, j, S.fused ? 1 : 0);
+    } else {
+        const StreamKernel kern = stream_kernel(T);
+        e = ensure_smem_cap(reinterpret_cast<const void *>(kern), S.smem);
+        if (e != cudaSuccess) return e;
+        kern<<<S.grid, S.block, S.smem, st>>>(a);
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (C.between) {
+        e = cudaEventRecord(C.between, st);
+        if (e != cudaSuccess) return e;
+    }
+    if (S.fused) return cudaSuccess;
     // the join's blocks may be set up while the last stream blocks run (they wait at their start)
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(S.join_blocks);

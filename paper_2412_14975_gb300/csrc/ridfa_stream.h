@@ -11,13 +11,15 @@ namespace ridfa {
 struct StreamShape {
     uint32_t per_chunk = 1;      // pieces a chunk is cut into
     uint64_t pieces = 0;
-    uint32_t block = 32, grid = 1;
+    bool walk_only = false;      // short pieces: one-byte steps only, no main table to set up
+    uint32_t block = 32, grid = 1, warps = 1;   // warps of a block that take pieces
     uint32_t join_chunks = 256;  // chunks per join block
     uint32_t join_blocks = 1;
+    bool fused = false;          // the join runs in the last block of the reach launch
     size_t smem = 0;
 };
 
-// Buffers of one call.  ticket and work are zero before and after every call.
+// Buffers of one call.  ticket (two words) and work are zero before and after every call.
 struct StreamCall {
     const HostAutomaton *H = nullptr;
     const DeviceAutomaton *D = nullptr;
