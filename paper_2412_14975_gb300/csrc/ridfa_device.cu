@@ -1223,6 +1223,16 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
 
 }  // namespace
 
+int scan_words(const ridfa_program *prog, int dev, size_t bytes, uint64_t **d_words, uint64_t **h_words, uint32_t **work) {
+    int err = RIDFA_OK;
+    DeviceScratch *S = scratch_for(prog, dev, 1024 + bytes, &err);
+    if (!S) return err;
+    *d_words = reinterpret_cast<uint64_t *>(static_cast<uint8_t *>(S->base) + 768);    // (past Layout's words)
+    *h_words = reinterpret_cast<uint64_t *>(S->h_accept_pinned + 32);
+    if (work) *work = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(S->base) + 1024);
+    return RIDFA_OK;
+}
+
 void release_device(const ridfa_program *P) {
     int cur = 0;
     if (cudaGetDevice(&cur) != cudaSuccess) {

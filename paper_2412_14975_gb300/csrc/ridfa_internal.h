@@ -201,6 +201,9 @@ int cuda_fail(cudaError_t e);
 int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev);
 const DeviceAutomaton *device_copy(const ridfa_program *P, bool dfa, int dev, int *err);
 int smem_optin_limit();
+// For the join scan: two device words and two page-locked host words of the program's scratch on
+// `dev`, and `bytes` of working space in it.  Caller holds prog->mu.
+int scan_words(const ridfa_program *prog, int dev, size_t bytes, uint64_t **d_words, uint64_t **h_words, uint32_t **work);
 // Raise a kernel's dynamic shared-memory cap on the current device to at least `bytes`.  The cap
 // is never lowered, so a launch sized by another thread (or an earlier plan) stays valid.
 cudaError_t ensure_smem_cap(const void *kern, size_t bytes);

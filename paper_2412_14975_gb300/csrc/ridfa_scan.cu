@@ -2,15 +2,24 @@
 //
 // For every chunk i the entry set E_i = if_min(PLAS_{i-1}) ∩ PIS_i (E_1 = {q0's slot} ∩ PIS_1),
 // i.e. the interface slots through which chunk i is entered on the way to PLAS_i = λ_i(E_i), and
-// the first chunk whose PLAS_i is empty (the text is rejected there).  The recurrence
-// PLAS_i = PLAS_{i-1} · M_i runs over the distinct end states D_i of each chunk (M_i as in the
-// join kernel), in three launches:
-//   1. one thread per segment of kScanSeg boundaries: the product of the segment's M_i;
-//   2. one block: the product of each thread's run of segments, then the incoming PLAS vector of
-//      every segment (vector × matrix, sequential over 256 thread totals, then per segment);
-//   3. one thread per segment: walk its boundaries from the incoming vector, writing E_i.
+// the first chunk whose PLAS_i is empty (the text is rejected there).
+//
+// While every chunk has at most one end state (runs that merge), E_i does not depend on how the
+// chunks before i - 1 went, only on whether PLAS_{i-1} is empty: one warp per row works out every
+// E_i as if it were not, the first empty one is where the text is rejected, and the sets after it
+// are cleared.  Otherwise PLAS_i = PLAS_{i-1} · M_i over the distinct end states D_i of each chunk
+// (M_i as in the join kernel):
+//   1. a warp per boundary forms M_i;
+//   2. a warp per segment of kScanSeg boundaries multiplies them, a row of the product per lane;
+//   3. one block: the incoming PLAS vector of every segment;
+//   4. a warp per segment walks its boundaries from that vector;
+//   5. a warp per chunk forms E_i from PLAS_{i-1}.
 // When some chunk has more than 32 distinct end states, one block propagates the k-bit sets
 // chunk by chunk instead (exact, sequential in c).
+//
+// Record lines, 65,537 chunks of 68 slots: a whole call 1,750 us with one thread walking 64 rows at a
+// time (every row sorted entry by entry, twice), 39 us by the first form; the codon RE, 65,536
+// chunks with several end states, 197 us by the second.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -21,183 +30,282 @@
 namespace ridfa {
 namespace {
 
-constexpr uint32_t kScanSeg = 64;          // boundaries per thread of launches 1 and 3
+constexpr uint32_t kScanSeg = 32;          // boundaries per warp of launches 2 and 4
 constexpr uint32_t kScanThreads = 256;
-constexpr uint32_t kScanWords = 1 + kMaxD; // a product: nrows (0xFFFFFFFF = identity) + rows
+constexpr uint32_t kScanWarps = kScanThreads / 32;
+constexpr uint32_t kScanRows = 8;          // consecutive rows per warp of rid_scan_rows
+constexpr uint32_t kStatusSeveral = 8u;    // some chunk has two or more end states
+constexpr int kScanRegs = RIDFA_MAX_SLOTS / 32;
 
 struct ScanArgs {
     Automaton A;
     const uint16_t *maps;      // [c][k]
     uint32_t c, nseg;
-    uint32_t *prods;           // [nseg][kScanWords]
+    uint32_t *mats;            // [c][32]: row z of M_i, bits over D_i
+    uint32_t *prods;           // [nseg][32]
     uint32_t *vin;             // [nseg]: PLAS before the segment's first boundary, over its D
+    uint32_t *plas;            // [c]: PLAS_i as bits over D_i
     uint32_t *entry;           // [c][kw], or null
     unsigned long long *reject;
     uint32_t *status;
 };
 
-// Distinct defined values of a row, ascending (0xFFFFFFFF when more than kMaxD).
-__device__ uint32_t row_distinct(const uint16_t *row, uint32_t k, uint16_t *D) {
-    uint32_t cnt = 0;
-    for (uint32_t a = 0; a < k; ++a) {
-        const uint16_t v = row[a];
-        if (v == kUndef) continue;
-        uint32_t j = 0;
-        while (j < cnt && D[j] < v) ++j;
-        if (j < cnt && D[j] == v) continue;
-        if (cnt == kMaxD) return 0xFFFFFFFFu;
-        for (uint32_t t = cnt; t > j; --t) D[t] = D[t - 1];
-        D[j] = v;
+// Row i across the warp: lane l holds entries l, 32 + l, ...
+__device__ __forceinline__ void load_row(const ScanArgs &p, uint64_t i, uint32_t lane, uint32_t (&v)[kScanRegs]) {
+    const uint16_t *row = p.maps + i * p.A.k;
+#pragma unroll
+    for (int r = 0; r < kScanRegs; ++r) {
+        const uint32_t a = r * 32 + lane;
+        v[r] = a < p.A.k ? __ldg(row + a) : kUndef;
+    }
+}
+
+// The distinct defined values of a row, ascending: lane g gets the g-th; returns their number
+// (kMaxD + 1: more than kMaxD).
+__device__ __forceinline__ uint32_t warp_distinct(const uint32_t (&v)[kScanRegs], uint32_t lane, uint32_t &mine) {
+    uint32_t cnt = 0, cur = 0;
+    mine = kUndef;
+    for (;;) {
+        uint32_t m = 0xFFFFFFFFu;
+#pragma unroll
+        for (int r = 0; r < kScanRegs; ++r)
+            if (v[r] != kUndef && (cnt == 0 || v[r] > cur)) m = min(m, v[r]);
+        m = __reduce_min_sync(kFull, m);
+        if (m == 0xFFFFFFFFu) return cnt;
+        if (cnt == static_cast<uint32_t>(kMaxD)) return kMaxD + 1;
+        if (lane == cnt) mine = m;
+        cur = m;
         ++cnt;
     }
-    return cnt;
 }
 
-__device__ __forceinline__ uint32_t row_index(const uint16_t *D, uint32_t m, uint16_t v) {
-    for (uint32_t j = 0; j < m; ++j)
-        if (D[j] == v) return j;
-    return 0xFFFFFFFFu;
-}
-
-// Entry slots of a chunk from the previous chunk's PLAS (bits v over Dp): if_min(PLAS) ∩ PIS.
-// Writes them to out (kw words) when non-null and returns the next PLAS as bits over Dc.
-__device__ uint32_t step_plas(const Automaton &A, const uint16_t *row, const uint16_t *Dp, uint32_t v,
-                              const uint16_t *Dc, uint32_t mc, uint32_t *out, bool *bad) {
-    uint32_t next = 0;
-    for (uint32_t w = 0; w < A.kw; ++w) {
-        uint32_t e = 0;
-        for (uint32_t bits = v; bits; bits &= bits - 1)
-            e |= A.ifmask[static_cast<uint64_t>(Dp[__ffs(bits) - 1]) * A.kw + w];
-        uint32_t live = 0;
-        for (uint32_t bits = e; bits; bits &= bits - 1) {
-            const uint32_t a = w * 32 + __ffs(bits) - 1;
-            const uint16_t s = row[a];
-            if (s == kUndef) continue;
-            live |= 1u << (a & 31);
-            const uint32_t y = row_index(Dc, mc, s);
-            if (y == 0xFFFFFFFFu) *bad = true;
-            else next |= 1u << y;
-        }
-        if (out) out[w] = live;
+// Word `lane` of the row's set of defined slots (lanes below kw).
+__device__ __forceinline__ uint32_t alive_word(const uint32_t (&v)[kScanRegs], uint32_t lane) {
+    uint32_t alive = 0;
+#pragma unroll
+    for (int r = 0; r < kScanRegs; ++r) {
+        const uint32_t b = __ballot_sync(kFull, v[r] != kUndef);
+        if (lane == static_cast<uint32_t>(r)) alive = b;
     }
-    return next;
+    return alive;
 }
 
-__device__ uint32_t vec_times(uint32_t v, const uint32_t *prod) {   // v · P (P may be identity)
-    if (prod[0] == 0xFFFFFFFFu) return v;
+// The case of at most one end state per chunk, a warp per kScanRows rows: E_i as if PLAS_{i-1} were
+// not empty, and the first empty one.  Bound by the maps' bytes (L2 or HBM).
+__global__ void __launch_bounds__(kScanThreads) rid_scan_rows(ScanArgs p) {
+    const Automaton &A = p.A;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t i0 = (static_cast<uint64_t>(blockIdx.x) * kScanWarps + (threadIdx.x >> 5)) * kScanRows;
+    if (i0 >= p.c) return;
+    const uint64_t i1 = min(static_cast<uint64_t>(p.c), i0 + kScanRows);
+    uint32_t v[kScanRegs], y = kUndef;       // y: the previous chunk's end state
+    uint32_t bad = 0;
+    auto only = [&]() -> uint32_t {          // the row's one defined value
+        uint32_t lo = 0xFFFFFFFFu, hi = 0;
+#pragma unroll
+        for (int r = 0; r < kScanRegs; ++r)
+            if (v[r] != kUndef) {
+                lo = min(lo, v[r]);
+                hi = max(hi, v[r]);
+            }
+        lo = __reduce_min_sync(kFull, lo);
+        hi = __reduce_max_sync(kFull, hi);
+        if (lo == 0xFFFFFFFFu) return kUndef;
+        if (lo != hi) bad |= kStatusSeveral;
+        if (hi >= A.n) bad |= kStatusBad;
+        return min(lo, A.n);
+    };
+    if (i0) {
+        load_row(p, i0 - 1, lane, v);
+        y = only();
+    }
+    for (uint64_t i = i0; i < i1; ++i) {
+        load_row(p, i, lane, v);
+        uint32_t in = 0;                     // word `lane` of if_min of the previous end state
+        if (lane < A.kw) {
+            if (i == 0) in = (A.q0_slot >> 5) == lane ? 1u << (A.q0_slot & 31) : 0u;
+            else if (y != kUndef) in = __ldg(A.ifmask + static_cast<uint64_t>(y) * A.kw + lane);
+        }
+        const uint32_t e = in & alive_word(v, lane);
+        if (p.entry && lane < A.kw) p.entry[i * A.kw + lane] = e;
+        if (!__any_sync(kFull, e != 0) && lane == 0) atomicMin(p.reject, static_cast<unsigned long long>(i));
+        y = only();
+    }
+    if (bad && lane == 0) atomicOr(p.status, bad);
+}
+
+// ... and the sets after the first empty one.
+__global__ void __launch_bounds__(kScanThreads) rid_scan_clear(ScanArgs p) {
+    const unsigned long long f = *p.reject;
+    if (f >= p.c) return;
+    const uint64_t lo = (f + 1) * p.A.kw, hi = static_cast<uint64_t>(p.c) * p.A.kw;
+    for (uint64_t e = lo + static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < hi; e += static_cast<uint64_t>(gridDim.x) * blockDim.x)
+        p.entry[e] = 0;
+}
+
+// Launch 1: M_i, a warp per boundary.
+__global__ void __launch_bounds__(kScanThreads) rid_scan_matrices(ScanArgs p) {
+    __shared__ uint8_t s_idx[kScanWarps][RIDFA_MAX_SLOTS];
+    const Automaton &A = p.A;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t i = 1 + static_cast<uint64_t>(blockIdx.x) * kScanWarps + warp;
+    if (i >= p.c) return;
+    uint32_t v[kScanRegs], prev, mine;
+    load_row(p, i - 1, lane, v);
+    const uint32_t mp = warp_distinct(v, lane, prev);
+    load_row(p, i, lane, v);
+    const uint32_t mc = warp_distinct(v, lane, mine);
+    if (mp > static_cast<uint32_t>(kMaxD) || mc > static_cast<uint32_t>(kMaxD)) {
+        if (lane == 0) atomicOr(p.status, kStatusWide);
+        return;
+    }
+    // each slot's place in D_i
+    uint32_t idx[kScanRegs];
+#pragma unroll
+    for (int r = 0; r < kScanRegs; ++r) idx[r] = 0xFF;
+    for (uint32_t g = 0; g < mc; ++g) {
+        const uint32_t d = __shfl_sync(kFull, mine, g);
+#pragma unroll
+        for (int r = 0; r < kScanRegs; ++r)
+            if (v[r] == d) idx[r] = g;
+    }
+#pragma unroll
+    for (int r = 0; r < kScanRegs; ++r) s_idx[warp][r * 32 + lane] = static_cast<uint8_t>(idx[r]);
+    __syncwarp();
+    uint32_t row = 0;
+    if (lane < mp) {
+        if (prev >= A.n) atomicOr(p.status, kStatusBad);
+        else
+            for (uint32_t w = 0; w < A.kw; ++w)
+                for (uint32_t bits = __ldg(A.ifmask + static_cast<uint64_t>(prev) * A.kw + w); bits; bits &= bits - 1) {
+                    const uint32_t g = s_idx[warp][w * 32 + __ffs(bits) - 1];
+                    if (g != 0xFF) row |= 1u << g;
+                }
+    }
+    p.mats[i * 32 + lane] = row;
+}
+
+// rows <- rows · M, a row per lane; m: the lane's row of M.
+__device__ __forceinline__ uint32_t times(uint32_t row, uint32_t m) {
     uint32_t out = 0;
-    for (uint32_t bits = v; bits; bits &= bits - 1) out |= prod[1 + __ffs(bits) - 1];
+    for (uint32_t nz = __ballot_sync(kFull, m != 0); nz; nz &= nz - 1) {
+        const uint32_t z = __ffs(nz) - 1, mz = __shfl_sync(kFull, m, z);
+        if ((row >> z) & 1) out |= mz;
+    }
     return out;
 }
 
-__device__ void prod_compose(uint32_t *a, const uint32_t *b) {       // a <- a · b
-    if (b[0] == 0xFFFFFFFFu) return;
-    if (a[0] == 0xFFFFFFFFu) {
-        for (uint32_t r = 0; r < kScanWords; ++r) a[r] = b[r];
-        return;
-    }
-    for (uint32_t x = 0; x < a[0]; ++x) a[1 + x] = vec_times(a[1 + x], b);
+// v · M for a vector that every lane holds.
+__device__ __forceinline__ uint32_t vec_times(uint32_t v, uint32_t m, uint32_t lane) {
+    return __reduce_or_sync(kFull, (v >> lane) & 1 ? m : 0u);
 }
 
-// Launch 1: the product of each segment's transfer matrices.
+// Launch 2: the product of each segment's matrices.
 __global__ void __launch_bounds__(kScanThreads) rid_scan_products(ScanArgs p) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= p.nseg) return;
-    const Automaton &A = p.A;
-    const uint64_t b0 = 1 + static_cast<uint64_t>(t) * kScanSeg;
-    const uint64_t b1 = b0 + kScanSeg < p.c ? b0 + kScanSeg : p.c;
-    uint16_t Dp[kMaxD], Dc[kMaxD];
-    uint32_t *P = p.prods + static_cast<uint64_t>(t) * kScanWords;
-    uint32_t mp = row_distinct(p.maps + (b0 - 1) * A.k, A.k, Dp);
-    if (mp == 0xFFFFFFFFu) {
-        atomicOr(p.status, kStatusWide);
-        return;
-    }
-    // rows stay over the segment's first D; the columns move on to each next D
-    uint32_t rows[kMaxD];
-    for (uint32_t x = 0; x < mp; ++x) rows[x] = 1u << x;
-    uint32_t mcur = mp;
-    bool bad = false;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t sg = blockIdx.x * kScanWarps + (threadIdx.x >> 5);
+    if (sg >= p.nseg) return;
+    const uint64_t b0 = 1 + static_cast<uint64_t>(sg) * kScanSeg, b1 = min(static_cast<uint64_t>(p.c), b0 + kScanSeg);
+    uint32_t row = 1u << lane, m = p.mats[b0 * 32 + lane];
     for (uint64_t i = b0; i < b1; ++i) {
-        const uint16_t *row = p.maps + i * A.k;
-        const uint32_t mc = row_distinct(row, A.k, Dc);
-        if (mc == 0xFFFFFFFFu) {
-            atomicOr(p.status, kStatusWide);
-            return;
-        }
-        uint32_t M[kMaxD];                       // row z of M_i: D_{i-1}[z] -> bits over D_i
-        for (uint32_t z = 0; z < mcur; ++z) M[z] = step_plas(A, row, Dp, 1u << z, Dc, mc, nullptr, &bad);
-        for (uint32_t x = 0; x < mp; ++x) {
-            uint32_t out = 0;
-            for (uint32_t bits = rows[x]; bits; bits &= bits - 1) out |= M[__ffs(bits) - 1];
-            rows[x] = out;
-        }
-        for (uint32_t j = 0; j < mc; ++j) Dp[j] = Dc[j];
-        mcur = mc;
+        const uint32_t next = i + 1 < b1 ? p.mats[(i + 1) * 32 + lane] : 0;
+        row = times(row, m);
+        m = next;
     }
-    if (bad) atomicOr(p.status, kStatusBad);
-    P[0] = mp;
-    for (uint32_t x = 0; x < kMaxD; ++x) P[1 + x] = x < mp ? rows[x] : 0;
+    p.prods[static_cast<uint64_t>(sg) * 32 + lane] = row;
 }
 
-// Launch 2 (one block): incoming PLAS vector of every segment, and chunk 0's entry set.
-__global__ void __launch_bounds__(kScanThreads) rid_scan_prefix(ScanArgs p) {
-    __shared__ uint32_t s_tot[kScanThreads][kScanWords];
-    __shared__ uint32_t s_in[kScanThreads];
+// Launch 3 (one block of 32 warps): the incoming PLAS vector of every segment, PLAS and entry set of
+// chunk 0.
+__global__ void __launch_bounds__(1024) rid_scan_prefix(ScanArgs p) {
+    __shared__ uint32_t s_tot[32][32], s_in[32];
     const Automaton &A = p.A;
-    const uint32_t tid = threadIdx.x;
-    const uint32_t per = (p.nseg + kScanThreads - 1) / kScanThreads;
-    const uint32_t s0 = tid * per, s1 = min(p.nseg, s0 + per);
-    s_tot[tid][0] = 0xFFFFFFFFu;
-    for (uint32_t sg = s0; sg < s1; ++sg) prod_compose(s_tot[tid], p.prods + static_cast<uint64_t>(sg) * kScanWords);
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t per = (p.nseg + 31) / 32, s0 = min(p.nseg, warp * per), s1 = min(p.nseg, s0 + per);
+    // (four products are loaded together: one after the other, the loads' latency was the time)
+    auto load4 = [&](uint32_t sg, uint32_t (&m)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) m[u] = sg + u < s1 ? p.prods[static_cast<uint64_t>(sg + u) * 32 + lane] : 0;
+    };
+    uint32_t row = 1u << lane;
+    for (uint32_t sg = s0; sg < s1; sg += 4) {
+        uint32_t m[4];
+        load4(sg, m);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (sg + u < s1) row = times(row, m[u]);
+    }
+    s_tot[warp][lane] = row;
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0) {
         // PLAS_1 = {λ_1(q0)} over D_1 (chunk 0 here); E_1 = {q0's slot} if that move is defined
-        uint16_t D0[kMaxD];
-        const uint32_t m0 = row_distinct(p.maps, A.k, D0);
-        const uint16_t v0 = p.maps[A.q0_slot];
-        uint32_t v = 0;
-        if (v0 != kUndef && m0 != 0xFFFFFFFFu) {
-            const uint32_t x = row_index(D0, m0, v0);
-            if (x != 0xFFFFFFFFu) v = 1u << x;
+        uint32_t v[kScanRegs], mine;
+        load_row(p, 0, lane, v);
+        const uint32_t m0 = warp_distinct(v, lane, mine);
+        const uint32_t v0 = p.maps[A.q0_slot];
+        uint32_t x = m0 <= static_cast<uint32_t>(kMaxD) ? __ballot_sync(kFull, v0 != kUndef && lane < m0 && mine == v0) : 0;
+        if (p.entry && lane < A.kw) p.entry[lane] = (v0 != kUndef && (A.q0_slot >> 5) == lane) ? 1u << (A.q0_slot & 31) : 0u;
+        if (lane == 0) {
+            p.plas[0] = x;
+            if (v0 == kUndef) atomicMin(p.reject, 0ull);
         }
-        if (p.entry)
-            for (uint32_t w = 0; w < A.kw; ++w)
-                p.entry[w] = (v0 != kUndef && (A.q0_slot >> 5) == w) ? (1u << (A.q0_slot & 31)) : 0u;
-        if (v0 == kUndef) atomicMin(p.reject, 0ull);
-        for (uint32_t t = 0; t < kScanThreads; ++t) {
-            s_in[t] = v;
-            v = vec_times(v, s_tot[t]);
+        for (uint32_t t = 0; t < 32; ++t) {
+            if (lane == 0) s_in[t] = x;
+            x = vec_times(x, s_tot[t][lane], lane);
         }
     }
     __syncthreads();
-    uint32_t v = s_in[tid];
-    for (uint32_t sg = s0; sg < s1; ++sg) {
-        p.vin[sg] = v;
-        v = vec_times(v, p.prods + static_cast<uint64_t>(sg) * kScanWords);
+    uint32_t v = s_in[warp];
+    for (uint32_t sg = s0; sg < s1; sg += 4) {
+        uint32_t m[4];
+        load4(sg, m);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (sg + u < s1) {
+                if (lane == 0) p.vin[sg + u] = v;
+                v = vec_times(v, m[u], lane);
+            }
     }
 }
 
-// Launch 3: walk each segment's boundaries from its incoming vector.
+// Launch 4: PLAS after every boundary of a segment.
 __global__ void __launch_bounds__(kScanThreads) rid_scan_walk(ScanArgs p) {
-    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= p.nseg) return;
-    const Automaton &A = p.A;
-    const uint64_t b0 = 1 + static_cast<uint64_t>(t) * kScanSeg;
-    const uint64_t b1 = b0 + kScanSeg < p.c ? b0 + kScanSeg : p.c;
-    uint16_t Dp[kMaxD], Dc[kMaxD];
-    row_distinct(p.maps + (b0 - 1) * A.k, A.k, Dp);
-    uint32_t v = p.vin[t];
-    bool bad = false;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t sg = blockIdx.x * kScanWarps + (threadIdx.x >> 5);
+    if (sg >= p.nseg) return;
+    const uint64_t b0 = 1 + static_cast<uint64_t>(sg) * kScanSeg, b1 = min(static_cast<uint64_t>(p.c), b0 + kScanSeg);
+    uint32_t v = p.vin[sg], keep = 0, m = p.mats[b0 * 32 + lane];
     for (uint64_t i = b0; i < b1; ++i) {
-        const uint16_t *row = p.maps + i * A.k;
-        const uint32_t mc = row_distinct(row, A.k, Dc);
-        const uint32_t nv = step_plas(A, row, Dp, v, Dc, mc, p.entry ? p.entry + i * A.kw : nullptr, &bad);
-        if (nv == 0 && v != 0) atomicMin(p.reject, static_cast<unsigned long long>(i));
+        const uint32_t next = i + 1 < b1 ? p.mats[(i + 1) * 32 + lane] : 0;
+        const uint32_t nv = vec_times(v, m, lane);
+        if (nv == 0 && v != 0 && lane == 0) atomicMin(p.reject, static_cast<unsigned long long>(i));
+        if (lane == i - b0) keep = nv;
         v = nv;
-        for (uint32_t j = 0; j < mc; ++j) Dp[j] = Dc[j];
+        m = next;
     }
-    if (bad) atomicOr(p.status, kStatusBad);
+    if (b0 + lane < b1) p.plas[b0 + lane] = keep;
+}
+
+// Launch 5: E_i from PLAS_{i-1}, a warp per chunk.
+__global__ void __launch_bounds__(kScanThreads) rid_scan_entries(ScanArgs p) {
+    const Automaton &A = p.A;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t i = 1 + static_cast<uint64_t>(blockIdx.x) * kScanWarps + (threadIdx.x >> 5);
+    if (i >= p.c) return;
+    const uint32_t plas = p.plas[i - 1];
+    uint32_t e = 0;
+    if (plas) {
+        uint32_t v[kScanRegs], prev;
+        load_row(p, i - 1, lane, v);
+        warp_distinct(v, lane, prev);
+        load_row(p, i, lane, v);
+        const uint32_t alive = alive_word(v, lane);
+        for (uint32_t w = 0; w < A.kw; ++w) {
+            const uint32_t in = __reduce_or_sync(kFull, ((plas >> lane) & 1) && prev < A.n ? __ldg(A.ifmask + static_cast<uint64_t>(prev) * A.kw + w) : 0u);
+            if (lane == w) e = in & alive;
+        }
+    }
+    if (lane < A.kw) p.entry[i * A.kw + lane] = e;
 }
 
 // Some chunk has more than kMaxD end states: one block propagates the k-bit slot sets.
@@ -217,6 +325,10 @@ __global__ void __launch_bounds__(kScanThreads) rid_scan_wide(ScanArgs p) {
         for (uint32_t a = tid; a < A.k; a += blockDim.x) {
             const bool in = (s_vec[a >> 5] >> (a & 31)) & 1;
             if (!in || row[a] == kUndef) continue;
+            if (row[a] >= A.n) {
+                atomicOr(p.status, kStatusBad);
+                continue;
+            }
             s_any = 1;
             for (uint32_t w = 0; w < A.kw; ++w) {
                 const uint32_t m = A.ifmask[static_cast<uint64_t>(row[a]) * A.kw + w];
@@ -253,53 +365,77 @@ extern "C" int ridfa_join_scan(const ridfa_program *prog, const uint16_t *d_maps
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
-    const DeviceAutomaton *D = nullptr;
-    {
-        std::lock_guard<std::mutex> lock(prog->mu);
-        int err = RIDFA_OK;
-        D = device_copy(prog, false, dev, &err);
-        if (!D) return err;
-    }
-    const uint32_t c = n_chunks;
-    const uint32_t nseg = c > 1 ? (c - 1 + kScanSeg - 1) / kScanSeg : 0;
-    const size_t bytes = 256 + static_cast<size_t>(nseg) * (kScanWords + 1) * 4;
-    uint8_t *scratch = nullptr;
-    e = cudaMallocAsync(reinterpret_cast<void **>(&scratch), bytes, st);
-    if (e != cudaSuccess) return cuda_fail(e);
-    unsigned long long *reject = reinterpret_cast<unsigned long long *>(scratch);
-    uint32_t *status = reinterpret_cast<uint32_t *>(scratch + 8);
-    uint32_t *prods = reinterpret_cast<uint32_t *>(scratch + 256);
-    uint32_t *vin = prods + static_cast<size_t>(nseg) * kScanWords;
-    ScanArgs a{Automaton{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state, H.n_states, H.n_classes,
-                         H.k, H.kw, H.q0_slot},
-               d_maps, c, nseg, prods, vin, d_entry, reject, status};
-    uint64_t h[2] = {~0ull, 0};
-    e = cudaMemsetAsync(scratch, 0xFF, 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(status, 0, 4, st);
-    if (e == cudaSuccess && nseg) {
-        rid_scan_products<<<(nseg + kScanThreads - 1) / kScanThreads, kScanThreads, 0, st>>>(a);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h[1], status, 4, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    std::lock_guard<std::mutex> lock(prog->mu);
     int err = RIDFA_OK;
-    if (e == cudaSuccess && (h[1] & kStatusBad)) err = RIDFA_E_STATE;
-    if (e == cudaSuccess && err == RIDFA_OK) {
-        if (h[1] & kStatusWide) {
-            rid_scan_wide<<<1, kScanThreads, 0, st>>>(a);
-        } else {
-            rid_scan_prefix<<<1, kScanThreads, 0, st>>>(a);
-            if (nseg) rid_scan_walk<<<(nseg + kScanThreads - 1) / kScanThreads, kScanThreads, 0, st>>>(a);
+    const DeviceAutomaton *D = device_copy(prog, false, dev, &err);
+    if (!D) return err;
+    // the result words: {first rejecting chunk, status}, on the device and page-locked on the host
+    uint64_t *words = nullptr, *h = nullptr;
+    err = scan_words(prog, dev, 0, &words, &h, nullptr);
+    if (err != RIDFA_OK) return err;
+    const uint32_t c = n_chunks;
+    ScanArgs a{};
+    a.A = Automaton{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state, H.n_states, H.n_classes,
+                    H.k, H.kw, H.q0_slot};
+    a.maps = d_maps;
+    a.c = c;
+    a.nseg = c > 1 ? (c - 1 + kScanSeg - 1) / kScanSeg : 0;
+    a.entry = d_entry;
+    a.reject = reinterpret_cast<unsigned long long *>(words);
+    a.status = reinterpret_cast<uint32_t *>(words + 1);
+    auto blocks = [](uint64_t items, uint64_t per) { return static_cast<unsigned>((items + per - 1) / per); };
+    auto fetch = [&]() {
+        e = cudaMemcpyAsync(h, words, 16, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        return e;
+    };
+    auto clear = [&]() {
+        e = cudaMemsetAsync(words, 0xFF, 8, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(words + 1, 0, 8, st);
+        return e;
+    };
+    if (clear() != cudaSuccess) return cuda_fail(e);
+    rid_scan_rows<<<blocks(c, kScanWarps * kScanRows), kScanThreads, 0, st>>>(a);
+    if (d_entry) rid_scan_clear<<<blocks(static_cast<uint64_t>(c) * H.kw, 4096) < 608 ? blocks(static_cast<uint64_t>(c) * H.kw, 4096) : 608, kScanThreads, 0, st>>>(a);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) fetch();
+    if (e != cudaSuccess) return cuda_fail(e);
+    uint32_t status = static_cast<uint32_t>(h[1]);
+    if (status & kStatusSeveral) {
+        const size_t bytes = (static_cast<size_t>(c) * 33 + static_cast<size_t>(a.nseg) * 33) * 4;
+        uint32_t *scratch = nullptr;
+        err = scan_words(prog, dev, bytes, &words, &h, &scratch);
+        if (err != RIDFA_OK) return err;
+        a.reject = reinterpret_cast<unsigned long long *>(words);
+        a.status = reinterpret_cast<uint32_t *>(words + 1);
+        if (clear() != cudaSuccess) return cuda_fail(e);
+        a.mats = scratch;
+        a.prods = a.mats + static_cast<size_t>(c) * 32;
+        a.vin = a.prods + static_cast<size_t>(a.nseg) * 32;
+        a.plas = a.vin + a.nseg;
+        if (c > 1) {
+            rid_scan_matrices<<<blocks(c - 1, kScanWarps), kScanThreads, 0, st>>>(a);
+            rid_scan_products<<<blocks(a.nseg, kScanWarps), kScanThreads, 0, st>>>(a);
+        }
+        rid_scan_prefix<<<1, 1024, 0, st>>>(a);
+        if (c > 1) {
+            rid_scan_walk<<<blocks(a.nseg, kScanWarps), kScanThreads, 0, st>>>(a);
+            if (d_entry) rid_scan_entries<<<blocks(c - 1, kScanWarps), kScanThreads, 0, st>>>(a);
         }
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h[0], reject, 8, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&h[1], status, 4, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e == cudaSuccess && (h[1] & kStatusBad)) err = RIDFA_E_STATE;
+        if (e == cudaSuccess) fetch();
+        if (e != cudaSuccess) return cuda_fail(e);
+        status = static_cast<uint32_t>(h[1]);
+        if (status & kStatusWide) {
+            if (clear() != cudaSuccess) return cuda_fail(e);
+            rid_scan_wide<<<1, kScanThreads, 0, st>>>(a);
+            e = cudaGetLastError();
+            if (e == cudaSuccess) fetch();
+            if (e != cudaSuccess) return cuda_fail(e);
+            status = static_cast<uint32_t>(h[1]);
+        }
     }
-    cudaFreeAsync(scratch, st);
-    if (e != cudaSuccess) return cuda_fail(e);
-    if (err != RIDFA_OK) return err;
+    if (status & kStatusBad) return RIDFA_E_STATE;
     *h_reject = h[0] == ~0ull ? -1 : static_cast<int64_t>(h[0]);
     return RIDFA_OK;
 }
