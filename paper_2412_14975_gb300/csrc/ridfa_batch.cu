@@ -4,6 +4,8 @@
 // exactly, for every (text, program) item, with all items' chunks in one persistent reach launch
 // per table layout and one join launch, captured once into a CUDA graph and replayed by
 // ridfa_batch_run:
+// Texts of programs with a merge graph take the stream kernels (ridfa_stream_batch.cu), side by side
+// with the launches here, which take the others:
 //   * reach: CTAs take tasks (up to 32 chunks per warp of one program) from an atomic ticket;
 //     tasks are ordered by program, so a CTA reloads its shared-memory tables only when the
 //     program changes.  Each warp runs the speculative phase of its chunks (lanes = runs) and
@@ -28,6 +30,7 @@
 #include "ridfa_batch_plan.h"
 #include "ridfa_internal.h"
 #include "ridfa_kernels.cuh"
+#include "ridfa_stream_batch.h"
 
 namespace ridfa {
 namespace {
@@ -564,6 +567,9 @@ struct BatchPlan {
     std::vector<TaskDesc> tasks;
     std::vector<SegDesc> segs;
     std::vector<LaunchGroup> groups;
+    // the texts of programs with a merge graph, at most kStreamBatchProgs programs a plan
+    std::vector<StreamBatchPlan> stream;
+    std::vector<size_t> o_stream, o_sres;        // image and result offsets of each
     uint32_t n_items = 0;
     uint64_t total_bytes = 0, total_chunks = 0;
     // block layout; everything before o_part is the host image
@@ -585,6 +591,11 @@ PlanStats plan_stats(const BatchPlan *pl) {
     s.n_launches = static_cast<uint32_t>(pl->groups.size()) + (pl->segs.empty() ? 0 : 1);
     s.n_tasks = static_cast<uint32_t>(pl->tasks.size());
     s.n_segments = static_cast<uint32_t>(pl->segs.size());
+    for (const StreamBatchPlan &b : pl->stream) {
+        s.n_launches += 2 * static_cast<uint32_t>(b.launches.size());
+        for (const StreamBatchPart &p : b.parts) s.n_tasks += p.task1 - p.task0;
+        s.n_segments += static_cast<uint32_t>(b.texts.size());
+    }
     return s;
 }
 
@@ -616,6 +627,7 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
         P.dev[p] = device_copy(R, false, device, &err);
         if (!P.dev[p]) return err;
         const HostAutomaton &H = R->rid;
+        if (H.stream.kind != kStreamNone) continue;          // (planned below)
         Automaton A{nullptr, nullptr, nullptr, nullptr, nullptr, H.n_states, H.n_classes, H.k, H.kw, H.q0_slot};
         const size_t r16 = LutRep<true>::smem_bytes(A), r32 = LutRep<false>::smem_bytes(A),
                      pln = LutPlain::smem_bytes(A), flt = LutFlat::smem_bytes(A);
@@ -640,22 +652,36 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
     P.n_texts_of.assign(np, 0);
     bool aligned_all = true;
     P.total_bytes = 0;
+    P.total_chunks = 0;
+    std::vector<StreamBatchSource> sources;
+    uint64_t stream_bytes = 0;
     for (uint32_t p = 0; p < np; ++p) {
         P.text0[p] = static_cast<uint32_t>(P.texts.size());
-        P.n_texts_of[p] = static_cast<uint32_t>(by_prog[p].size());
+        const bool stream = progs[p]->rid.stream.kind != kStreamNone;
+        if (stream && !by_prog[p].empty()) {
+            sources.push_back(StreamBatchSource{&progs[p]->rid, P.dev[p], {}});
+        }
+        P.n_texts_of[p] = stream ? 0 : static_cast<uint32_t>(by_prog[p].size());
         for (uint32_t i : by_prog[p]) {
             const ridfa_batch_item &it = items[i];
             TextDesc td{it.d_text, it.len, prog_chunks[p], 0, i};
             if (it.len == 0) td.c = 0;
             else if (it.n_chunks) td.c = it.n_chunks;
             else td.c = static_cast<uint32_t>(std::max<uint64_t>(1, std::min<uint64_t>(it.len, (it.len + L - 1) / L)));
+            if (stream) {
+                // (its chunks only count: the accept bit does not depend on where a text is cut)
+                sources.back().items.push_back(StreamBatchItem{it.d_text, it.len, i});
+                P.total_chunks += td.c;
+                P.total_bytes += it.len;
+                stream_bytes += it.len;
+                continue;
+            }
             if (it.len && (reinterpret_cast<uintptr_t>(it.d_text) & 15)) aligned_all = false;
             prog_chunks[p] += td.c;
             P.total_bytes += it.len;
             P.texts.push_back(td);
         }
     }
-    P.total_chunks = 0;
     for (uint32_t p = 0; p < np; ++p) P.total_chunks += prog_chunks[p];
     // launch groups by layout; tasks ordered by group then program
     P.groups.clear();
@@ -688,15 +714,38 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
             for (uint64_t c0 = 0; c0 < prog_chunks[p]; c0 += per_task)
                 P.tasks.push_back(TaskDesc{c0, p, static_cast<uint32_t>(std::min<uint64_t>(per_task, prog_chunks[p] - c0))});
         g.n_tasks = static_cast<uint32_t>(P.tasks.size()) - g.task0;
+        P.groups.push_back(g);
+    }
+    // The stream launches and the general groups run side by side, a block of either filling an SM: each
+    // side gets SMs by its share of the work (the general kernels take some four times the time per
+    // byte), the general groups no more than they have tasks.
+    uint32_t stream_sms = static_cast<uint32_t>(sms);
+    const uint64_t other_bytes = P.total_bytes - stream_bytes;
+    if (other_bytes && stream_bytes) {
+        uint64_t tasks = 0;
+        for (const LaunchGroup &g : P.groups) tasks += g.n_tasks;
+        const double share = static_cast<double>(stream_bytes) / (static_cast<double>(stream_bytes) + 4.0 * static_cast<double>(other_bytes));
+        stream_sms = std::max<uint32_t>(1, std::min<uint32_t>(static_cast<uint32_t>(sms) - 1, static_cast<uint32_t>(share * sms + 0.5)));
+        stream_sms = std::max<uint32_t>(stream_sms, static_cast<uint32_t>(sms - std::min<uint64_t>(tasks, static_cast<uint64_t>(sms) - 1)));
+    }
+    P.stream.clear();
+    for (size_t p0 = 0; p0 < sources.size(); p0 += kStreamBatchProgs) {
+        std::vector<StreamBatchSource> part(sources.begin() + p0, sources.begin() + std::min<size_t>(sources.size(), p0 + kStreamBatchProgs));
+        P.stream.emplace_back();
+        plan_stream_batch(P.stream.back(), part, stream_sms);
+    }
+    const bool apart = stream_bytes && !P.stream.front().walk_only;
+    const int group_sms = stream_bytes ? std::max(1, sms - static_cast<int>(stream_sms)) : sms;
+    for (LaunchGroup &g : P.groups) {
+        if (apart) g.smem = std::max(g.smem, kStreamBatchSmem);
         // persistent: as many blocks as fit on every SM, no more than there are tasks
         int per_sm = 0;
         const int err = blocks_per_sm(device, g, &per_sm);
         if (err != RIDFA_OK) return err;
         if (per_sm < 1) return RIDFA_E_UNSUPPORTED;
-        g.grid = static_cast<int>(std::min<uint64_t>(g.n_tasks, static_cast<uint64_t>(sms) * per_sm));
+        g.grid = static_cast<int>(std::min<uint64_t>(g.n_tasks, static_cast<uint64_t>(group_sms) * per_sm));
         g.run0 = run_warps;
-        run_warps += static_cast<uint64_t>(g.grid) * warps;
-        P.groups.push_back(g);
+        run_warps += static_cast<uint64_t>(g.grid) * (g.block / 32);
     }
     // join segments
     P.segs.clear();
@@ -730,11 +779,21 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
     P.o_segs = off;     off += al256(P.segs.size() * sizeof(SegDesc));
     P.o_tick = off;     off += al256(P.texts.size() * 4);
     P.o_flags = off;    off += al256(P.texts.size() * 4);
+    P.o_stream.clear();
+    for (const StreamBatchPlan &b : P.stream) {
+        P.o_stream.push_back(off);
+        off += al256(b.image_bytes);
+    }
     P.o_part = off;     off += al256(P.segs.size() * kPartialWords * 4);
     P.o_runs = off;     off += al256(run_warps * kRunsPerWarp * sizeof(RunEntry));
     P.o_finals = off;   off += al256(run_warps * kFinalsPerWarp * 4);
     P.o_maps = off;     off += maps_bytes;
     P.o_dinfo = off;    off += dinfo_bytes;
+    P.o_sres.clear();
+    for (const StreamBatchPlan &b : P.stream) {
+        P.o_sres.push_back(off);
+        off += al256(b.result_words * 4);
+    }
     P.total = off;
     return RIDFA_OK;
 }
@@ -760,6 +819,8 @@ void plan_image(const BatchPlan *pl, uint8_t *base, uint8_t *img) {
     if (!P.texts.empty()) std::memcpy(img + P.o_texts, P.texts.data(), P.texts.size() * sizeof(TextDesc));
     if (!P.tasks.empty()) std::memcpy(img + P.o_tasks, P.tasks.data(), P.tasks.size() * sizeof(TaskDesc));
     if (!P.segs.empty()) std::memcpy(img + P.o_segs, P.segs.data(), P.segs.size() * sizeof(SegDesc));
+    for (size_t i = 0; i < P.stream.size(); ++i)
+        stream_batch_image(P.stream[i], base + P.o_stream[i], reinterpret_cast<uint32_t *>(base + P.o_sres[i]), img + P.o_stream[i]);
 }
 
 int make_fork(LaunchFork *f) {
@@ -768,7 +829,7 @@ int make_fork(LaunchFork *f) {
         cudaError_t e = cudaStreamCreateWithFlags(&f->aux[i], cudaStreamNonBlocking);
         if (e != cudaSuccess) return cuda_fail(e);
     }
-    for (int i = 0; i < kMaxLaunchGroups; ++i) {
+    for (int i = 0; i < kForkEvents; ++i) {
         cudaError_t e = cudaEventCreateWithFlags(&f->ev[i], cudaEventDisableTiming);
         if (e != cudaSuccess) return cuda_fail(e);
     }
@@ -797,34 +858,59 @@ int plan_enqueue(const BatchPlan *pl, uint8_t *base, uint8_t *d_accept, cudaStre
     const TaskDesc *tasks = reinterpret_cast<const TaskDesc *>(base + P.o_tasks);
     RunEntry *runs = reinterpret_cast<RunEntry *>(base + P.o_runs);
     uint32_t *finals = reinterpret_cast<uint32_t *>(base + P.o_finals);
-    const bool concurrent = fork && fork->ok && P.groups.size() > 1 && P.groups.size() <= kMaxLaunchGroups;
+    // launches side by side: the first on `st`, every further one on a stream of its own (in turn,
+    // should there be more of them than streams)
+    size_t n_side = P.groups.size();
+    for (const StreamBatchPlan &b : P.stream) n_side += b.launches.size();
+    const bool concurrent = fork && fork->ok && n_side > 1;
+    const size_t n_aux = concurrent ? std::min<size_t>(n_side - 1, kMaxLaunchGroups - 1) : 0;
+    size_t side = 0;
+    auto side_stream = [&]() {
+        const size_t i = side++;
+        return n_aux && i ? fork->aux[(i - 1) % n_aux] : st;
+    };
     if (concurrent) {
         cudaError_t e = cudaEventRecord(fork->ev[0], st);
-        for (size_t gi = 1; gi < P.groups.size() && e == cudaSuccess; ++gi) e = cudaStreamWaitEvent(fork->aux[gi - 1], fork->ev[0], 0);
+        for (size_t a = 0; a < n_aux && e == cudaSuccess; ++a) e = cudaStreamWaitEvent(fork->aux[a], fork->ev[0], 0);
         if (e != cudaSuccess) return cuda_fail(e);
     }
+    for (size_t i = 0; i < P.stream.size(); ++i)
+        for (const StreamBatchLaunch &L : P.stream[i].launches) {
+            const cudaStream_t on = side_stream();
+            cudaError_t e = stream_batch_reach(P.stream[i], L, base + P.o_stream[i], on);
+            if (e == cudaSuccess) e = stream_batch_join(P.stream[i], L, base + P.o_stream[i], d_accept, on);
+            if (e != cudaSuccess) return cuda_fail(e);
+        }
+    // the general groups, then their join on the first one's stream once the others are done
+    cudaStream_t join_on = st;
+    size_t waits = 0;
     for (size_t gi = 0; gi < P.groups.size(); ++gi) {
         const LaunchGroup &g = P.groups[gi];
         if (g.n_tasks == 0) continue;
         BatchReachArgs a{progs, tasks + g.task0, g.n_tasks, 8, counters + gi, status, runs + g.run0 * kRunsPerWarp,
                          finals + g.run0 * kFinalsPerWarp};
-        cudaError_t e = batch_reach(g, a, (concurrent && gi > 0) ? fork->aux[gi - 1] : st, nullptr);
-        if (e != cudaSuccess) return cuda_fail(e);
-    }
-    if (concurrent) {
-        for (size_t gi = 1; gi < P.groups.size(); ++gi) {
-            cudaError_t e = cudaEventRecord(fork->ev[gi], fork->aux[gi - 1]);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, fork->ev[gi], 0);
-            if (e != cudaSuccess) return cuda_fail(e);
+        const cudaStream_t on = side_stream();
+        if (gi == 0) join_on = on;
+        cudaError_t e = batch_reach(g, a, on, nullptr);
+        if (e == cudaSuccess && on != join_on) {
+            e = cudaEventRecord(fork->ev[kMaxLaunchGroups + waits], on);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(join_on, fork->ev[kMaxLaunchGroups + waits], 0);
+            ++waits;
         }
+        if (e != cudaSuccess) return cuda_fail(e);
     }
     if (!P.segs.empty()) {
         BatchJoinArgs J{progs, reinterpret_cast<const TextDesc *>(base + P.o_texts),
                         reinterpret_cast<const SegDesc *>(base + P.o_segs),
                         reinterpret_cast<uint32_t *>(base + P.o_part), reinterpret_cast<uint32_t *>(base + P.o_tick),
                         reinterpret_cast<uint32_t *>(base + P.o_flags), d_accept, status};
-        rid_join_batch_kernel<<<static_cast<unsigned>(P.segs.size()), kBatchJoinThreads, 0, st>>>(J);
+        rid_join_batch_kernel<<<static_cast<unsigned>(P.segs.size()), kBatchJoinThreads, 0, join_on>>>(J);
         cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e);
+    }
+    for (size_t a = 0; a < n_aux; ++a) {
+        cudaError_t e = cudaEventRecord(fork->ev[1 + a], fork->aux[a]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, fork->ev[1 + a], 0);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     return RIDFA_OK;
@@ -920,11 +1006,18 @@ int batch_run(ridfa_batch *B, cudaStream_t st) {
 int batch_autotune(ridfa_batch *B, bool fixed_warps, bool fixed_set, BatchTune *out) {
     std::vector<std::tuple<int, int, int>> keys;
     bool large_table = false;
+    // (programs with a merge graph are cut by plan_stream_batch: nothing to tune for them)
     for (const ridfa_program *P : B->progs) {
+        if (P->rid.stream.kind != kStreamNone) continue;
         keys.emplace_back(log2i(P->rid.n_states), log2i(P->rid.k), log2i(P->rid.n_classes));
         const HostAutomaton &H = P->rid;
         Automaton A{nullptr, nullptr, nullptr, nullptr, nullptr, H.n_states, H.n_classes, H.k, H.kw, H.q0_slot};
         if (!LutRep<true>::fits16(A) && !LutRep16x4::fits(A)) large_table = true;
+    }
+    if (keys.empty()) {
+        out->chunk_len = 8192;
+        out->shape = B->shape;
+        return RIDFA_OK;
     }
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);

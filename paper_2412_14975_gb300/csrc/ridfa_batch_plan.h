@@ -44,13 +44,14 @@ size_t plan_status_offset(const BatchPlan *pl);  // byte offset of the status wo
 // descriptors depend on it); `img` holds plan_image_bytes bytes.
 void plan_image(const BatchPlan *pl, uint8_t *base, uint8_t *img);
 
-// Streams and events that let the reach groups of one batch (one per table layout) run
-// concurrently: group 0 on the caller's stream, group g > 0 on aux[g - 1], joined back before the
-// join launch.  Owned by the caller; created once with make_fork, released with free_fork.
-constexpr int kMaxLaunchGroups = 5;
+// Streams and events that let the reach launches of one batch (one per table layout or form) run
+// concurrently: the first launch on the caller's stream, the further ones on the streams of aux,
+// joined back before the join launches.  Owned by the caller; created once with make_fork, released with free_fork.
+constexpr int kMaxLaunchGroups = 9;
+constexpr int kForkEvents = kMaxLaunchGroups + 4;    // (and one per further general group)
 struct LaunchFork {
     cudaStream_t aux[kMaxLaunchGroups - 1] = {};
-    cudaEvent_t ev[kMaxLaunchGroups] = {};
+    cudaEvent_t ev[kForkEvents] = {};
     bool ok = false;
 };
 int make_fork(LaunchFork *f);

@@ -66,6 +66,7 @@ struct HostStream {
     uint32_t entry = 1, copies = 32, row_words = 0, group = 1, shift = 0, width = 0;
     uint32_t canon = 0;
     uint32_t warps = 0;               // warps a block holds beside the table (and its staging)
+    float cost = 0;                   // estimated shared-memory cycles per 32 text bytes
     std::vector<uint32_t> byte_code;  // [256] (kStreamPair, kStreamSingle)
     std::vector<uint32_t> words;      // [(n_states + 1) * row_words]
 };

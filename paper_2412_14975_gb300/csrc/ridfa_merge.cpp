@@ -264,6 +264,7 @@ void build_table(HostAutomaton &H) {
             const double cost = std::max(1.75, fixed + wavefronts(f) * per_lookup) * thin;
             if (cost < best_cost) {
                 best_cost = cost;
+                t.cost = static_cast<float>(cost);
                 t.copies = f;
                 t.warps = warps;
                 best = t;
