@@ -37,6 +37,7 @@
 #include "ridfa_internal.h"
 #include "ridfa_join.cuh"
 #include "ridfa_reach.cuh"
+#include "ridfa_set.h"
 #include "ridfa_stream.h"
 
 namespace ridfa {
@@ -76,6 +77,16 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
         o_code = put_v(T.byte_code);
         o_words = put_v(T.words);
     }
+    const HostSet &Z = H.set;
+    size_t z_next = 0, z_leaf = 0, z_img = 0, z_part = 0, z_mask = 0, z_words = 0;
+    if (Z.ok) {
+        z_next = put_v(Z.next);
+        z_leaf = put_v(Z.leaf);
+        z_img = put_v(Z.images);
+        z_part = put_v(Z.part);
+        z_mask = put_v(Z.block_mask);
+        z_words = put_v(Z.table.words);
+    }
     uint8_t *base = nullptr;
     cudaError_t e = cudaMalloc(&base, img.size());
     if (e != cudaSuccess) return cuda_fail(e);
@@ -103,6 +114,14 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
         D.mg_slot_alive = u32(o_alive);
         D.st_code = u32(o_code);
         D.st_words = u32(o_words);
+    }
+    if (Z.ok) {
+        D.set_next = u16(z_next);
+        D.set_leaf = u32(z_leaf);
+        D.set_images = u16(z_img);
+        D.set_part = base + z_part;
+        D.set_block_mask = u32(z_mask);
+        D.set_words = u32(z_words);
     }
     D.bytes = img.size();
     return RIDFA_OK;
@@ -967,6 +986,17 @@ bool automatic(const ridfa_tuning *t) {
                    t->lookback_cap);
 }
 
+cudaError_t profile_events(DeviceScratch *S) {
+    for (auto &ev : S->ev)
+        if (!ev) {
+            cudaEvent_t x;
+            const cudaError_t e = cudaEventCreate(&x);
+            if (e != cudaSuccess) return e;
+            ev = x;
+        }
+    return cudaSuccess;
+}
+
 // One call through the stream kernels (ridfa_stream.cu): two launches, results written to the
 // page-locked words by the join itself.  Caller holds P->mu.
 int recognize_stream(const ridfa_program *P, const HostAutomaton &H, const DeviceAutomaton *D, int dev, int sms,
@@ -1006,13 +1036,8 @@ int recognize_stream(const ridfa_program *P, const HostAutomaton &H, const Devic
     C.summary = h_summary ? reinterpret_cast<ridfa_shard_summary *>(base + o_sum) : nullptr;
     cudaError_t e = cudaSuccess;
     if (prof) {
-        for (auto &ev : S->ev)
-            if (!ev) {
-                cudaEvent_t x;
-                e = cudaEventCreate(&x);
-                if (e != cudaSuccess) return cuda_fail(e);
-                ev = x;
-            }
+        e = profile_events(S);
+        if (e != cudaSuccess) return cuda_fail(e);
         cudaEventRecord(static_cast<cudaEvent_t>(S->ev[0]), st);
         C.between = static_cast<cudaEvent_t>(S->ev[1]);
     }
@@ -1029,6 +1054,59 @@ int recognize_stream(const ridfa_program *P, const HostAutomaton &H, const Devic
     if (e != cudaSuccess) return cuda_fail(e);
     if (h_accept) *h_accept = *const_cast<volatile uint8_t *>(S->h_accept_pinned);
     return *const_cast<volatile uint32_t *>(S->h_status_pinned) & kStatusBad ? RIDFA_E_STATE : RIDFA_OK;
+}
+
+// One call through the set kernels (ridfa_set.cu), as recognize_stream.
+int recognize_set(const ridfa_program *P, const HostAutomaton &H, const DeviceAutomaton *D, int dev, int sms,
+                  const uint8_t *d_text, uint64_t len, uint32_t n_chunks, bool prof, uint8_t *d_accept_user, uint8_t *h_accept,
+                  uint16_t *d_maps_user, cudaStream_t st) {
+    auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
+    size_t off = 1024;
+    const size_t o_ends = off;     off += al(static_cast<size_t>(n_chunks) * kSetRuns * 2);
+    const size_t o_reps = off;     off += al(static_cast<size_t>(n_chunks) * 8);
+    const size_t o_pids = off;     off += al(static_cast<size_t>(n_chunks) * 4);
+    const size_t o_part = off;     off += al(static_cast<size_t>(set_join_blocks(n_chunks)) * kSetRuns * 4);
+    int err = RIDFA_OK;
+    DeviceScratch *S = scratch_for(P, dev, off, &err);
+    if (!S) return err;
+    uint8_t *base = static_cast<uint8_t *>(S->base);
+    SetCall C;
+    C.H = &H;
+    C.D = D;
+    C.text = d_text;
+    C.len = len;
+    C.c = n_chunks;
+    C.ends = reinterpret_cast<uint16_t *>(base + o_ends);
+    C.reps = reinterpret_cast<uint64_t *>(base + o_reps);
+    C.pids = reinterpret_cast<uint32_t *>(base + o_pids);
+    C.maps = d_maps_user;
+    C.partials = reinterpret_cast<uint32_t *>(base + o_part);
+    C.ticket = reinterpret_cast<uint32_t *>(base);
+    C.status = reinterpret_cast<uint32_t *>(base + 256);
+    C.accept = d_accept_user ? d_accept_user : base + 512;
+    if (h_accept) {
+        C.h_accept = S->h_accept_pinned;
+        C.h_status = S->h_status_pinned;
+    }
+    cudaError_t e = cudaSuccess;
+    if (prof) {
+        e = profile_events(S);
+        if (e != cudaSuccess) return cuda_fail(e);
+        cudaEventRecord(static_cast<cudaEvent_t>(S->ev[0]), st);
+        C.between = static_cast<cudaEvent_t>(S->ev[1]);
+    }
+    NvtxRange range("ridfa reach");
+    e = set_launch(C, sms, st);
+    if (e != cudaSuccess) return cuda_fail(e);
+    if (prof) {
+        cudaEventRecord(static_cast<cudaEvent_t>(S->ev[2]), st);
+        S->profiled = true;
+    }
+    if (!h_accept) return RIDFA_OK;
+    e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e);
+    *h_accept = *const_cast<volatile uint8_t *>(S->h_accept_pinned);
+    return RIDFA_OK;
 }
 
 int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, size_t len,
@@ -1076,9 +1154,12 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
                (static_cast<uint64_t>(kJoinThreads) * per_thread)));
     Automaton A{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state,
                 H.n_states, H.n_classes, H.k, H.kw, H.q0_slot, H.merges};
-    if (automatic(tuning) && stream_takes(H, len, n_chunks)) {
-        err = recognize_stream(P, H, D, dev, sms, d_text, len, n_chunks, tuning && tuning->profile, d_accept_user, h_accept,
-                               d_maps_user, st, h_summary);
+    const bool to_stream = automatic(tuning) && stream_takes(H, len, n_chunks);
+    const bool to_set = automatic(tuning) && !h_summary && set_takes(H, len, n_chunks, sms);
+    if (to_stream || to_set) {
+        const bool prof = tuning && tuning->profile;
+        err = to_stream ? recognize_stream(P, H, D, dev, sms, d_text, len, n_chunks, prof, d_accept_user, h_accept, d_maps_user, st, h_summary)
+                        : recognize_set(P, H, D, dev, sms, d_text, len, n_chunks, prof, d_accept_user, h_accept, d_maps_user, st);
         if (err == RIDFA_OK)
             for (auto &x : P->scratch)
                 if (x.device == dev) {
@@ -1130,13 +1211,8 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
 
     const bool prof = tuning && tuning->profile;
     if (prof) {
-        for (auto &ev : S->ev)
-            if (!ev) {
-                cudaEvent_t x;
-                e = cudaEventCreate(&x);
-                if (e != cudaSuccess) return cuda_fail(e);
-                ev = x;
-            }
+        e = profile_events(S);
+        if (e != cudaSuccess) return cuda_fail(e);
         cudaEventRecord(static_cast<cudaEvent_t>(S->ev[0]), st);
     }
     if (lookback) {

@@ -71,6 +71,21 @@ struct HostStream {
     std::vector<uint32_t> words;      // [(n_states + 1) * row_words]
 };
 
+// Automata whose runs stay apart, over an alphabet of at most four bytes (set kernels, ridfa_set.cu): the
+// functions that the first `depth` bytes perform on the interface slots, all of which have at most
+// kSetRuns distinct values, so that a lane takes up a chunk's runs after walking `depth` edges.
+struct HostSet {
+    bool ok = false;
+    uint32_t depth = 0, inner = 0, parts = 0;
+    std::vector<uint16_t> next;       // [inner][C]: an inner node, or kLeafBit | leaf (leaf 0: all dead)
+    std::vector<uint32_t> leaf;       // [leaves][2]: partition, offset into images
+    std::vector<uint16_t> images;     // states of a leaf's blocks, kSetRuns each (unused ones: n_states)
+    std::vector<uint8_t> part;        // [parts][k]: block of each slot, 0xFF: dead
+    std::vector<uint32_t> block_mask; // [parts][kw][kSetRuns]: slots of each block
+    HostStream table;                 // kStreamField, entries of 2 bytes
+};
+constexpr uint32_t kSetRuns = 16;     // places; at most 15 are taken (15 marks a dead run in 4 bits)
+
 // One speculative automaton as the device sees it: the RI-DFA B with its interface
 // (Sec. 3.1-3.4) or the minimal DFA with every state initial (Sec. 2).
 struct HostAutomaton {
@@ -88,14 +103,16 @@ struct HostAutomaton {
     uint32_t merges = 0;              // 1: runs from every slot merge on random text (merge_hint)
     HostMerge merge;
     HostStream stream;
+    HostSet set;                      // only where merge is not built
 };
 
-// Build H.merge and, where it is small enough, H.stream (ridfa_merge.cpp).
+// Build H.merge with H.stream, or H.set, where they are small enough (ridfa_merge.cpp).
 void build_stream(HostAutomaton &H);
 // Shared memory of a stream kernel's block besides the staging buffers: tables and the compact
 // copies for the ragged ends.
 size_t stream_table_bytes(const HostAutomaton &H);
 size_t stream_walk_bytes(const HostAutomaton &H);      // the one-byte tables alone
+size_t set_rest_bytes(const HostAutomaton &H);         // of a set kernel's block besides the table
 constexpr size_t kStreamSmem = 226 * 1024;        // shared memory a stream block may take
 constexpr size_t kStreamWalkSmem = 24 * 1024;     // a walk table up to this size sits in shared memory,
                                                   // a larger one is read through L1
@@ -114,6 +131,10 @@ struct DeviceAutomaton {
     uint16_t *mg_walk = nullptr, *mg_edge_pid = nullptr, *mg_node_part = nullptr, *mg_images = nullptr, *mg_part = nullptr;
     uint32_t *mg_node_img = nullptr, *mg_slot_alive = nullptr;
     uint32_t *st_code = nullptr, *st_words = nullptr;
+    // set tables (HostSet)
+    uint16_t *set_next = nullptr, *set_images = nullptr;
+    uint32_t *set_leaf = nullptr, *set_block_mask = nullptr, *set_words = nullptr;
+    uint8_t *set_part = nullptr;
     size_t bytes = 0;
 };
 

@@ -239,14 +239,58 @@ uint32_t place_pairs(const std::vector<uint32_t> &col, uint32_t C, uint32_t per_
     return best;
 }
 
+// Codes by a bit field of the byte: the field's place and the byte of each code, when the live bytes
+// differ in at most two adjacent bits.
+bool find_field(const HostAutomaton &H, HostStream &t) {
+    const uint32_t n = H.n_states, C = H.n_classes;
+    std::vector<uint8_t> class_live(C, 0);
+    for (uint32_t c = 0; c < C; ++c)
+        for (uint32_t s = 0; s < n && !class_live[c]; ++s) class_live[c] = H.trans[static_cast<size_t>(s) * C + c] != n;
+    std::vector<uint32_t> live;
+    for (uint32_t b = 0; b < 256; ++b)
+        if (class_live[H.classmap[b]]) live.push_back(b);
+    bool field = false;
+    for (uint32_t w = 1; w <= 2 && !field && live.size() <= 4; ++w)
+        for (uint32_t sh = 0; sh + w <= 8 && !field; ++sh) {
+            uint32_t seen = 0, canon = 0, m = (1u << w) - 1;
+            bool inj = live.size() <= m + 1;
+            for (uint32_t b : live) {
+                const uint32_t code = (b >> sh) & m;
+                if (seen >> code & 1) inj = false;
+                seen |= 1u << code;
+                canon |= b << (8 * code);
+            }
+            // a code no live byte has: its canonical byte has another code, so no byte passes
+            for (uint32_t code = 0; code <= 3; ++code)
+                if (!(seen >> code & 1)) canon |= ((code ^ 1) & m) << sh << (8 * code);
+            if (inj) {
+                field = true;
+                t.shift = sh;
+                t.width = w;
+                t.canon = canon;
+            }
+        }
+    return field;
+}
+
+// Entries of a field table: column = the codes of `group` bytes, the first one lowest.
+void fill_field(const HostAutomaton &H, HostStream &t) {
+    const uint32_t n = H.n_states, per_word = 4 / t.entry, W = t.row_words, m = (1u << t.width) - 1;
+    t.words.assign(static_cast<size_t>(n + 1) * W, 0);
+    for (uint32_t s = 0; s <= n; ++s)
+        for (uint32_t c = 0; c < W * per_word; ++c) {
+            uint32_t x = c >> (t.width * t.group) ? n : s;
+            for (uint32_t i = 0; i < t.group; ++i)
+                x = H.trans[static_cast<size_t>(x) * H.n_classes + H.classmap[(t.canon >> (8 * ((c >> (t.width * i)) & m))) & 0xFF]];
+            t.words[static_cast<size_t>(s) * W + c / per_word] |= x << (8 * t.entry * (c % per_word));
+        }
+}
+
 void build_table(HostAutomaton &H) {
     const uint32_t n = H.n_states, C = H.n_classes;
     HostStream best;
     double best_cost = 1e9;
     const uint32_t entry = n + 1 <= 256 ? 1 : 2, per_word = 4 / entry;
-    std::vector<uint8_t> class_live(C, 0);
-    for (uint32_t c = 0; c < C; ++c)
-        for (uint32_t s = 0; s < n && !class_live[c]; ++s) class_live[c] = H.trans[static_cast<size_t>(s) * C + c] != n;
     // the most copies that fit, with their cost in shared-memory cycles per 32 text bytes
     auto consider = [&](HostStream t, double fixed, double per_lookup) {
         const size_t rest = rest_bytes(H, t.kind);
@@ -273,31 +317,7 @@ void build_table(HostAutomaton &H) {
     };
     HostStream t;
     t.entry = entry;
-    // codes by a bit field of the byte
-    std::vector<uint32_t> live;
-    for (uint32_t b = 0; b < 256; ++b)
-        if (class_live[H.classmap[b]]) live.push_back(b);
-    bool field = false;
-    for (uint32_t w = 1; w <= 2 && !field && live.size() <= 4; ++w)
-        for (uint32_t sh = 0; sh + w <= 8 && !field; ++sh) {
-            uint32_t seen = 0, canon = 0, m = (1u << w) - 1;
-            bool inj = live.size() <= m + 1;
-            for (uint32_t b : live) {
-                const uint32_t code = (b >> sh) & m;
-                if (seen >> code & 1) inj = false;
-                seen |= 1u << code;
-                canon |= b << (8 * code);
-            }
-            // a code no live byte has: its canonical byte has another code, so no byte passes
-            for (uint32_t code = 0; code <= 3; ++code)
-                if (!(seen >> code & 1)) canon |= ((code ^ 1) & m) << sh << (8 * code);
-            if (inj) {
-                field = true;
-                t.shift = sh;
-                t.width = w;
-                t.canon = canon;
-            }
-        }
+    const bool field = find_field(H, t);
     if (field) {
         t.kind = kStreamField;
         for (uint32_t g : {4u, 2u}) {
@@ -352,14 +372,7 @@ void build_table(HostAutomaton &H) {
     auto step = [&](uint32_t s, uint32_t c) -> uint32_t { return H.trans[static_cast<size_t>(s) * C + c]; };
     auto offset = [&](uint32_t c) { return c / per_word * 4 * best.copies + c % per_word * entry; };
     if (best.kind == kStreamField) {
-        const uint32_t m = (1u << best.width) - 1;
-        for (uint32_t s = 0; s <= n; ++s)
-            for (uint32_t c = 0; c < W * per_word; ++c) {
-                uint32_t x = c >> (best.width * best.group) ? n : s;
-                for (uint32_t i = 0; i < best.group; ++i)
-                    x = step(x, H.classmap[(best.canon >> (8 * ((c >> (best.width * i)) & m))) & 0xFF]);
-                put(s, c, x);
-            }
+        fill_field(H, best);
     } else {
         best.byte_code.assign(256, 0);
         if (best.kind == kStreamPair) {
@@ -381,7 +394,122 @@ void build_table(HostAutomaton &H) {
     H.stream = best;
 }
 
+// The functions of the first bytes on the slots, level by level, down to the first level on which all
+// have fewer than kSetRuns distinct values.
+bool build_set(const HostAutomaton &H, HostSet &Z) {
+    constexpr uint32_t kMaxNodes = 4096;
+    const uint32_t n = H.n_states, C = H.n_classes, k = H.k;
+    if (n == 0 || n > 8192 || k > RIDFA_MAX_SLOTS) return false;
+    HostStream t;
+    t.entry = 2;
+    if (!find_field(H, t)) return false;
+    t.kind = kStreamField;
+    // four bytes a lookup in one copy, else two bytes in the most copies that fit
+    const size_t rest = set_rest_bytes(H);
+    for (uint32_t g : {4u, 2u}) {
+        t.group = g;
+        t.row_words = ((1u << (t.width * g)) + 1) / 2;
+        t.copies = 0;
+        for (uint32_t f = 32; f >= 1 && !t.copies; f /= 2)
+            if (rest + static_cast<size_t>(n + 1) * t.row_words * 4 * f <= kStreamSmem) t.copies = f;
+        if (t.copies) break;
+    }
+    if (!t.copies) return false;
+    fill_field(H, t);
+    Z.table = t;
+    using Fn = std::vector<uint16_t>;                     // state of each slot, n: dead
+    std::map<Fn, uint32_t> ids, part_ids;
+    std::vector<Fn> level, next_level;
+    Z.leaf = {0, 0};
+    Z.images.assign(kSetRuns, static_cast<uint16_t>(n));
+    auto add_leaf = [&](const Fn &f) -> uint32_t {
+        Fn img;
+        Fn block(k, 0xFF);
+        for (uint32_t a = 0; a < k; ++a) {
+            if (f[a] == n) continue;
+            const uint32_t b = static_cast<uint32_t>(std::find(img.begin(), img.end(), f[a]) - img.begin());
+            if (b == img.size()) img.push_back(f[a]);
+            block[a] = static_cast<uint16_t>(b);
+        }
+        img.resize(kSetRuns, static_cast<uint16_t>(n));
+        const auto r = part_ids.emplace(block, Z.parts);
+        if (r.second) {
+            ++Z.parts;
+            for (uint16_t b : block) Z.part.push_back(static_cast<uint8_t>(b));
+        }
+        Z.leaf.push_back(r.first->second);
+        Z.leaf.push_back(static_cast<uint32_t>(Z.images.size()));
+        Z.images.insert(Z.images.end(), img.begin(), img.end());
+        return static_cast<uint32_t>(Z.leaf.size() / 2 - 1);
+    };
+    part_ids.emplace(Fn(k, 0xFF), 0u);                     // partition 0: all dead
+    Z.parts = 1;
+    Z.part.assign(k, 0xFF);
+    level.push_back(Fn(H.slot_state.begin(), H.slot_state.end()));
+    for (uint32_t d = 1; d <= 32; ++d) {
+        ids.clear();
+        next_level.clear();
+        std::vector<uint16_t> edges;
+        size_t most = 0;
+        for (const Fn &f : level)
+            for (uint32_t c = 0; c < C; ++c) {
+                Fn g(k);
+                bool any = false;
+                for (uint32_t a = 0; a < k; ++a) {
+                    g[a] = f[a] == n ? static_cast<uint16_t>(n) : H.trans[static_cast<size_t>(f[a]) * C + c];
+                    any |= g[a] != n;
+                }
+                if (!any) {
+                    edges.push_back(kLeafBit);
+                    continue;
+                }
+                const auto r = ids.emplace(g, static_cast<uint32_t>(next_level.size()));
+                if (r.second) {
+                    next_level.push_back(g);
+                    std::sort(g.begin(), g.end());
+                    size_t v = std::unique(g.begin(), g.end()) - g.begin();
+                    if (std::binary_search(g.begin(), g.begin() + v, static_cast<uint16_t>(n))) --v;
+                    most = std::max(most, v);
+                }
+                edges.push_back(static_cast<uint16_t>(r.first->second));
+            }
+        if (Z.inner + level.size() + next_level.size() > kMaxNodes) return false;
+        const bool last = most < kSetRuns;
+        std::vector<uint32_t> leaf_of;
+        if (last)
+            for (const Fn &f : next_level) leaf_of.push_back(add_leaf(f));
+        const uint32_t base = Z.inner + static_cast<uint32_t>(level.size());       // first node of the next level
+        for (uint16_t e : edges)
+            Z.next.push_back(e & kLeafBit ? kLeafBit : static_cast<uint16_t>(last ? kLeafBit | leaf_of[e] : base + e));
+        Z.inner = base;
+        if (last) {
+            Z.depth = d;
+            break;
+        }
+        level.swap(next_level);
+        if (level.empty()) return false;
+    }
+    if (!Z.depth) return false;
+    Z.block_mask.assign(static_cast<size_t>(Z.parts) * kSetRuns * H.kw, 0);
+    for (uint32_t p = 0; p < Z.parts; ++p)
+        for (uint32_t a = 0; a < k; ++a) {
+            const uint8_t b = Z.part[static_cast<size_t>(p) * k + a];
+            if (b != 0xFF) Z.block_mask[(static_cast<size_t>(p) * H.kw + (a >> 5)) * kSetRuns + b] |= 1u << (a & 31);
+        }
+    // every index the kernels take unchecked
+    if (Z.next.size() != static_cast<size_t>(Z.inner) * C || Z.parts > 0xFFFF) return false;
+    for (uint16_t e : Z.next)
+        if ((e & kLeafBit) ? 2u * (e & 0x7FFFu) + 1 >= Z.leaf.size() : e >= Z.inner) return false;
+    for (size_t l = 0; l < Z.leaf.size(); l += 2)
+        if (Z.leaf[l] >= Z.parts || Z.leaf[l + 1] + kSetRuns > Z.images.size()) return false;
+    for (uint16_t s : Z.images)
+        if (s > n) return false;
+    return true;
+}
+
 }  // namespace
+
+size_t set_rest_bytes(const HostAutomaton &H) { return 256 + (H.trans.size() * 2 + 15) / 16 * 16 + 256; }
 
 size_t stream_table_bytes(const HostAutomaton &H) {
     return rest_bytes(H, H.stream.kind) + static_cast<size_t>(H.n_states + 1) * H.stream.row_words * 4 * H.stream.copies;
@@ -391,7 +519,15 @@ size_t stream_walk_bytes(const HostAutomaton &H) { return rest_bytes(H, kStreamF
 
 void build_stream(HostAutomaton &H) {
     HostMerge G;
-    if (H.k > RIDFA_MAX_SLOTS || !build_graph(H, G) || !graph_in_bounds(H, G)) return;
+    if (H.k > RIDFA_MAX_SLOTS) return;
+    if (!build_graph(H, G) || !graph_in_bounds(H, G)) {
+        HostSet Z;
+        if (build_set(H, Z)) {
+            Z.ok = true;
+            H.set = std::move(Z);
+        }
+        return;
+    }
     G.ok = true;
     H.merge = std::move(G);
     build_table(H);

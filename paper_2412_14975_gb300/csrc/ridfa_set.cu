@@ -1,0 +1,519 @@
+// Set kernels: automata whose runs stay apart (the codon RE's three reading frames), over an alphabet
+// of at most four bytes, a chunk per lane from its first byte to its last.
+//
+// The lane walks the first bytes of its chunk through the graph of functions on the interface slots
+// (HostSet) and takes up the distinct runs it finds there, fewer than 16; from then on every byte is
+// stepped once for all of them: the column of four bytes comes from arithmetic on their bit fields, and
+// each run pays one lookup per four bytes into a table of one copy that fills the SM's shared memory
+// (no staging: text comes by 32-byte loads of each lane's own chunk, the next 64 bytes under way; one
+// 32-byte load ahead hid too little, 558 -> 586 us at 65,536 chunks of 1 GiB and 566 -> 768 us at
+// 77,824, whose chunks begin between blocks).  Every 256 bytes the lane's runs are compacted and the
+// warp's loop respecialised to its largest count.
+// Bound by the table's bank conflicts, about 3.1 wavefronts a gather (the shared memory pipe is 78 %
+// busy).  The general kernel spends 1 + M/2 lookups per byte on M runs, and a warp's time on its chunks'
+// first 16 bytes one after another: 1 GiB of codon text in 65,536 chunks 797 -> 559 us, in 1,048,576
+// chunks 2863 -> 1334 us with the join, 128 MiB in 65,536 chunks 226 -> 127 us.
+//
+// The join works on the lane's places: chunk i's function is block of the slot -> place of the block's
+// run -> the place's end state, and the transfer from a place of chunk i - 1 that ended in y to the
+// places of chunk i comes from the blocks that if_min({y}) meets.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "ridfa_set.h"
+#include "ridfa_stream.cuh"
+
+namespace ridfa {
+namespace {
+
+constexpr int kSetBlock = 512;
+constexpr int kHalf = kSetRuns / 2;
+
+struct SetArgs {
+    const uint8_t *text;
+    uint64_t len, q, frac;        // chunk i begins at i * q + (i * frac >> 64)
+    uint32_t c, depth, k;
+    const uint16_t *next, *images, *trans;
+    const uint32_t *leaf;
+    uint16_t *ends;               // [c][kSetRuns]: distinct end states, dead beyond them
+    uint64_t *reps;               // [c]: place of each run of the graph's leaf (4 bits; 15: dead)
+    uint32_t *pids;               // [c]: the leaf's partition
+    StreamTables t;
+};
+
+__device__ __forceinline__ uint64_t set_chunk_at(const SetArgs &p, uint32_t i) { return i * p.q + __umul64hi(i, p.frac); }
+
+// Drop dead runs and runs in the same state as an earlier one of the places [0, N), pack the others
+// to the front, and follow them in `rep` (4 bits per original run: its place, 15 once dead).  As
+// compact_runs, by select networks only.
+template <int N>
+__device__ __forceinline__ uint32_t compact_set(uint32_t (&s)[kSetRuns], uint64_t &rep, uint32_t dead) {
+    uint64_t place = 0;
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        uint32_t at = 15;
+        if (s[j] != dead) {
+#pragma unroll
+            for (int i = 0; i < j; ++i)
+                if (at == 15 && s[i] == s[j]) at = static_cast<uint32_t>(place >> (4 * i)) & 15;
+            if (at == 15) at = cnt++;
+        }
+        place |= static_cast<uint64_t>(at) << (4 * j);
+    }
+    uint32_t t[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) t[j] = dead;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const uint32_t at = static_cast<uint32_t>(place >> (4 * j)) & 15;
+#pragma unroll
+        for (int i = 0; i <= j; ++i)
+            if (at == static_cast<uint32_t>(i)) t[i] = s[j];
+    }
+#pragma unroll
+    for (int j = 0; j < N; ++j) s[j] = t[j];
+    uint64_t nrep = 0;
+#pragma unroll
+    for (int g = 0; g < static_cast<int>(kSetRuns); ++g) {
+        const uint32_t r = static_cast<uint32_t>(rep >> (4 * g)) & 15;
+        nrep |= (r == 15 ? 15ull : (place >> (4 * r)) & 15) << (4 * g);
+    }
+    rep = nrep;
+    return cnt;
+}
+
+// One word of text for the first m places (m is the same in the whole warp).
+template <int G>
+__device__ __forceinline__ void set_word(const StreamTables &p, uint32_t lt, uint32_t w, uint32_t (&s)[kSetRuns], uint32_t m_runs) {
+    const uint32_t f = w >> p.shift;
+    const uint32_t m1 = f & 0x01010101u, m2 = (w >> (p.shift + 1)) & p.second;
+    const uint32_t m = m1 + 2 * m2;
+    const bool bad = (m1 * p.d1 + m2 * p.d2 + (m1 & m2) * p.d12 + p.canon0) != w;
+#pragma unroll
+    for (int h = 0; h < 4 / G; ++h) {
+        const uint32_t col = __umulhi(m * (h ? p.mul_h : p.mul), p.take_bits);
+        const uint32_t x = col * p.col_mul + (col & p.part_mask) * p.part_mul + lt;
+#pragma unroll
+        for (int g = 0; g < static_cast<int>(kSetRuns); ++g)
+            if (static_cast<uint32_t>(g) < m_runs) s[g] = lds_u16(s[g] * p.row + x);
+    }
+    if (bad) {
+#pragma unroll
+        for (int g = 0; g < static_cast<int>(kSetRuns); ++g) s[g] = p.n;
+    }
+}
+
+// Eight words of text for the first M runs of places [B, B + 8).  Returns whether all bytes were in the
+// alphabet.
+template <int G, int M, int B>
+__device__ __forceinline__ bool set_block(const StreamTables &p, uint32_t lt, const uint32_t (&w)[8], uint32_t (&s)[kSetRuns]) {
+    uint32_t bad = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t f = w[i] >> p.shift;
+        const uint32_t m1 = f & 0x01010101u, m2 = (w[i] >> (p.shift + 1)) & p.second;
+        const uint32_t m = m1 + 2 * m2;
+        bad |= (m1 * p.d1 + m2 * p.d2 + (m1 & m2) * p.d12 + p.canon0) ^ w[i];
+#pragma unroll
+        for (int h = 0; h < 4 / G; ++h) {
+            const uint32_t col = __umulhi(m * (h ? p.mul_h : p.mul), p.take_bits);
+            const uint32_t x = col * p.col_mul + (col & p.part_mask) * p.part_mul + lt;
+#pragma unroll
+            for (int g = 0; g < M; ++g) s[B + g] = lds_u16(s[B + g] * p.row + x);
+        }
+    }
+    return bad == 0;
+}
+
+template <int G, int B>
+__device__ __forceinline__ bool set_block_m(const StreamTables &p, uint32_t lt, const uint32_t (&w)[8], uint32_t (&s)[kSetRuns], uint32_t M) {
+    switch (M) {
+        case 1: return set_block<G, 1, B>(p, lt, w, s);
+        case 2: return set_block<G, 2, B>(p, lt, w, s);
+        case 3: return set_block<G, 3, B>(p, lt, w, s);
+        case 4: return set_block<G, 4, B>(p, lt, w, s);
+        case 5: return set_block<G, 5, B>(p, lt, w, s);
+        case 6: return set_block<G, 6, B>(p, lt, w, s);
+        case 7: return set_block<G, 7, B>(p, lt, w, s);
+        default: return set_block<G, 8, B>(p, lt, w, s);
+    }
+}
+
+template <int G>
+__global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_constant__ SetArgs p) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const uint32_t base = smem_addr(smem);
+    load_tables<Steps<kStreamField, G, 2, 2>>(p.t, smem);        // (the walk table is the one-byte table)
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31, dead = p.t.n;
+    const uint32_t lt = base + p.t.off_table + (lane & (p.t.copies - 1)) * 4;
+    const uint32_t cls = base + p.t.off_cls, one = base + p.t.off_walk;
+    const uint64_t t0 = reinterpret_cast<uint64_t>(p.text);
+    const uint32_t warps = blockDim.x / 32;
+    for (uint32_t task = blockIdx.x * warps + (threadIdx.x >> 5); task * 32 < p.c; task += gridDim.x * warps) {
+        const uint32_t ch = task * 32 + lane;
+        const bool have = ch < p.c;
+        uint64_t pos = t0, end = t0;
+        if (have) {
+            pos = t0 + set_chunk_at(p, ch);
+            end = t0 + set_chunk_at(p, ch + 1);
+        }
+        // ---- the first bytes through the graph (chunks are longer than its depth)
+        uint32_t leaf = 0;
+        if (have) {
+            uint32_t node = 0;
+            for (uint32_t d = 0; d < p.depth; ++d) {
+                const uint32_t e = __ldg(p.next + node * p.t.C + lds_u8(cls + __ldg(reinterpret_cast<const uint8_t *>(pos++))));
+                node = e;
+                if (e & kLeafBit) break;
+            }
+            leaf = node & 0x7FFF;
+        }
+        const uint32_t pid = __ldg(p.leaf + 2 * leaf), img = __ldg(p.leaf + 2 * leaf + 1);
+        uint32_t s[kSetRuns];
+        uint64_t rep = ~0ull;
+        uint32_t cnt = 0;
+#pragma unroll
+        for (int g = 0; g < static_cast<int>(kSetRuns); ++g) {
+            s[g] = __ldg(p.images + img + g);
+            if (s[g] != dead) {
+                rep = (rep & ~(15ull << (4 * g))) | static_cast<uint64_t>(g) << (4 * g);
+                ++cnt;
+            }
+        }
+        // ---- one-byte steps for all runs up to a 64-byte boundary
+        const uint32_t most = __reduce_max_sync(kFull, cnt);
+        auto step_all = [&](uint32_t m) {
+            const uint32_t c = lds_u8(cls + __ldg(reinterpret_cast<const uint8_t *>(pos++)));
+#pragma unroll
+            for (int g = 0; g < static_cast<int>(kSetRuns); ++g)
+                if (static_cast<uint32_t>(g) < m) s[g] = lds_u16(one + 2 * (s[g] * p.t.C + c));
+        };
+        // (by words once those are aligned: a lookup a run for four bytes)
+        while (cnt && pos < end && (pos & 3)) step_all(most);
+        while (cnt && pos + 4 <= end && (pos & 63)) {
+            set_word<G>(p.t, lt, __ldg(reinterpret_cast<const uint32_t *>(pos)), s, most);
+            pos += 4;
+        }
+        cnt = compact_set<kSetRuns>(s, rep, dead);
+        // ---- blocks of 64 bytes, the next one under way
+        uint32_t blocks = cnt && pos < end ? static_cast<uint32_t>((end - pos) >> 6) : 0;
+        const uint32_t rounds = __reduce_max_sync(kFull, blocks);
+        uint32_t M = __reduce_max_sync(kFull, cnt);
+        uint32_t a[8], b[8], na[8], nb[8];
+        if (blocks) {
+            load32(reinterpret_cast<const uint8_t *>(pos), a);
+            load32(reinterpret_cast<const uint8_t *>(pos + 32), b);
+        }
+        for (uint32_t r = 0; r < rounds; ++r) {
+            if (r + 1 < blocks) {
+                load32(reinterpret_cast<const uint8_t *>(pos + 64), na);
+                load32(reinterpret_cast<const uint8_t *>(pos + 96), nb);
+            }
+            if (r < blocks) {
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    bool ok = set_block_m<G, 0>(p.t, lt, a, s, min(M, 8u));
+                    if (M > kHalf) ok = set_block_m<G, kHalf>(p.t, lt, a, s, M - kHalf);
+                    if (!ok) {
+#pragma unroll
+                        for (int g = 0; g < static_cast<int>(kSetRuns); ++g) s[g] = dead;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) a[i] = b[i];
+                }
+                pos += 64;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    a[i] = na[i];
+                    b[i] = nb[i];
+                }
+            }
+            if ((r & 3) == 3) {
+                if (M > kHalf) cnt = compact_set<kSetRuns>(s, rep, dead);
+                else cnt = compact_set<kHalf>(s, rep, dead);
+                M = __reduce_max_sync(kFull, r + 1 < blocks ? cnt : 0u);
+                if (M == 0) break;
+            }
+        }
+        // ---- ragged end
+        uint32_t used = 0;                       // places up to the last live run
+#pragma unroll
+        for (int g = 0; g < static_cast<int>(kSetRuns); ++g)
+            if (s[g] != dead) used = g + 1;
+        M = __reduce_max_sync(kFull, used);
+        while (used && !(pos & 3) && pos + 4 <= end) {
+            set_word<G>(p.t, lt, __ldg(reinterpret_cast<const uint32_t *>(pos)), s, M);
+            pos += 4;
+        }
+        while (used && pos < end) step_all(M);
+        compact_set<kSetRuns>(s, rep, dead);
+        if (!have) continue;
+        uint32_t w[kHalf];
+#pragma unroll
+        for (int g = 0; g < kHalf; ++g) w[g] = s[2 * g] | s[2 * g + 1] << 16;
+        uint4 *out = reinterpret_cast<uint4 *>(p.ends + static_cast<uint64_t>(ch) * kSetRuns);
+        out[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        out[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        p.reps[ch] = rep;
+        p.pids[ch] = pid;
+    }
+}
+
+// ------------------------------------------------------------------------------- join
+struct SetJoinArgs {
+    uint32_t c, k, kw, n, q0_slot, per_warp;
+    const uint16_t *ends;
+    const uint64_t *reps;
+    const uint32_t *pids, *block_mask, *ifmask, *final_bits;
+    const uint8_t *part;
+    uint16_t *maps;               // null: not asked for
+    uint32_t *partials, *ticket, *status;
+    uint8_t *accept, *h_accept;
+    uint32_t *h_status;
+};
+
+constexpr uint32_t kSetJoinWarps = 16;
+constexpr uint32_t kSetTile = 16;                // chunks a warp stages at a time
+
+// rows <- rows · M in each half-warp: lane h * 16 + x has row x of both (at most 15 places).  `from`
+// is added to the lane M's row z is read from (z + from): the own half's, or a fixed half's.
+__device__ __forceinline__ uint32_t set_times(uint32_t row, uint32_t m, uint32_t from) {
+    const uint32_t any = __ballot_sync(kFull, m != 0);
+    uint32_t out = 0;
+    for (uint32_t nz = (any | any >> 16) & 0xFFFFu; nz; nz &= nz - 1) {
+        const uint32_t z = __ffs(nz) - 1, mz = __shfl_sync(kFull, m, z + from);
+        if ((row >> z) & 1) out |= mz;
+    }
+    return out;
+}
+
+// Chunk maps, and the product over all boundaries.  A warp takes per_warp consecutive chunks by tiles
+// of 16 that it stages in shared memory, a tile ahead in registers; each half-warp forms the product of
+// eight boundaries, a place of the chunk before per lane, so that a boundary costs a quarter of the
+// loads and half of the serial steps that a warp per boundary takes (46 -> 26 us at 65,536 chunks, 409
+// -> 232 us at 1,048,576; the general join took 65 and about 500 us).  Bound by latency: tables through
+// L1 and the products' shuffles.  A block takes the product of its warps', the last block that of all.
+__global__ void __launch_bounds__(32 * kSetJoinWarps) rid_set_join_kernel(const __grid_constant__ SetJoinArgs p) {
+    __shared__ __align__(16) uint16_t s_end[kSetJoinWarps][kSetTile + 1][kSetRuns];  // row 0: the chunk before
+    __shared__ uint64_t s_rep[kSetJoinWarps][kSetTile];
+    __shared__ uint32_t s_pid[kSetJoinWarps][kSetTile];
+    __shared__ uint32_t s_prod[2 * kSetJoinWarps][kSetRuns];
+    __shared__ uint32_t s_last;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, x = lane & 15, half = lane & 16;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint64_t i0 = (static_cast<uint64_t>(blockIdx.x) * kSetJoinWarps + warp) * p.per_warp;
+    const uint64_t i1 = min(static_cast<uint64_t>(p.c), i0 + p.per_warp);
+    uint32_t row = 1u << x;
+    uint4 e{};
+    uint64_t rep = 0;
+    uint32_t pid = 0;
+    // lane l: half a row of ends; the first 16 lanes: a chunk's places and partition
+    auto fetch = [&](uint64_t i) {
+        if (i + (lane >> 1) < i1) e = __ldg(reinterpret_cast<const uint4 *>(p.ends + i * kSetRuns) + lane);
+        if (lane < kSetTile && i + lane < i1) {
+            rep = __ldg(reinterpret_cast<const unsigned long long *>(p.reps) + i + lane);
+            pid = __ldg(p.pids + i + lane);
+        }
+    };
+    if (i0 < i1) {
+        if (lane < kSetRuns) s_end[warp][kSetTile][lane] = i0 ? __ldg(p.ends + (i0 - 1) * kSetRuns + lane) : static_cast<uint16_t>(p.n);
+        fetch(i0);
+    }
+    for (uint64_t i = i0; i < i1; i += kSetTile) {
+        const uint32_t cnt = static_cast<uint32_t>(min(static_cast<uint64_t>(kSetTile), i1 - i));
+        if (lane < kSetRuns) s_end[warp][0][lane] = s_end[warp][kSetTile][lane];
+        __syncwarp();
+        reinterpret_cast<uint4 *>(s_end[warp][1])[lane] = e;
+        if (lane < kSetTile) {
+            s_rep[warp][lane] = rep;
+            s_pid[warp][lane] = pid;
+        }
+        __syncwarp();
+        if (i + kSetTile < i1) fetch(i + kSetTile);
+        // boundaries before chunks i + u, i + 8 + u
+        uint32_t prod = 1u << x;
+#pragma unroll 2
+        for (uint32_t u = 0; u < 8; ++u) {
+            const uint32_t at = (half >> 1) + u;
+            uint32_t m = 1u << x;                            // (no boundary before chunk 0 or beyond the end)
+            if (at < cnt && i + at != 0) {
+                m = 0;
+                const uint32_t y = s_end[warp][at][x], id = s_pid[warp][at];
+                const uint64_t rp = s_rep[warp][at];
+                for (uint32_t w = 0; w < p.kw; ++w) {
+                    const uint32_t in = y < p.n ? __ldg(p.ifmask + static_cast<uint64_t>(y) * p.kw + w) : 0u;
+                    const uint4 *bm = reinterpret_cast<const uint4 *>(p.block_mask + (static_cast<uint64_t>(id) * p.kw + w) * kSetRuns);
+#pragma unroll
+                    for (int q = 0; q < static_cast<int>(kSetRuns) / 4; ++q) {
+                        const uint4 v = __ldg(bm + q);
+                        const uint32_t b[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int t = 0; t < 4; ++t)
+                            if (in & b[t]) m |= 1u << (static_cast<uint32_t>(rp >> (4 * (4 * q + t))) & 15);
+                    }
+                }
+                m &= 0x7FFFu;                                // (place 15: the run died)
+            }
+            prod = set_times(prod, m, half);
+        }
+        row = set_times(row, prod, 0);
+        row = set_times(row, prod, 16);
+        if (p.maps) {
+            for (uint32_t j = lane; j < cnt * p.k; j += 32) {
+                const uint32_t u = j / p.k, a = j - u * p.k;
+                const uint32_t b = __ldg(p.part + static_cast<uint64_t>(s_pid[warp][u]) * p.k + a);
+                const uint32_t at = b == 0xFF ? 15u : static_cast<uint32_t>(s_rep[warp][u] >> (4 * (b & 15))) & 15;
+                const uint32_t v = s_end[warp][u + 1][at];   // (place 15 stays dead)
+                p.maps[i * p.k + j] = static_cast<uint16_t>(v >= p.n ? kUndef : v);
+            }
+        }
+        __syncwarp();
+    }
+    if (lane < kSetRuns) s_prod[warp][lane] = row;
+    __syncthreads();
+    if (warp == 0) {
+        // the upper half its eight warps, then both
+        row = 1u << x;
+        for (uint32_t w = 0; w < kSetJoinWarps / 2; ++w) row = set_times(row, s_prod[(half ? kSetJoinWarps / 2 : 0) + w][x], half);
+        const uint32_t all = set_times(row, row, 16);        // (lower half: first · second)
+        if (lane < kSetRuns) p.partials[static_cast<uint64_t>(blockIdx.x) * kSetRuns + lane] = all;
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            s_last = atomicAdd(p.ticket, 1) == gridDim.x - 1;
+        }
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // ---- last block: each half-warp its share of the blocks' products
+    const uint32_t per = (gridDim.x + 2 * kSetJoinWarps - 1) / (2 * kSetJoinWarps), hw = 2 * warp + (half >> 4);
+    const uint32_t b0 = min(gridDim.x, hw * per), b1 = min(gridDim.x, b0 + per);
+    row = 1u << x;
+    for (uint32_t b = 0; b < per; b += 4) {
+        uint32_t m[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) m[u] = b0 + b + u < b1 ? __ldcg(p.partials + static_cast<uint64_t>(b0 + b + u) * kSetRuns + x) : 1u << x;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) row = set_times(row, m[u], half);
+    }
+    s_prod[hw][x] = row;
+    __syncthreads();
+    if (warp) return;
+    // the place of q0's slot in chunk 0, through all boundaries, to a final state
+    const uint32_t q0 = __ldg(p.part + static_cast<uint64_t>(__ldg(p.pids)) * p.k + p.q0_slot);
+    const uint32_t at = q0 == 0xFF ? 15u : static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned long long *>(p.reps)) >> (4 * q0)) & 15;
+    uint32_t v = at == 15 ? 0u : 1u << at;
+    for (uint32_t w = 0; w < 2 * kSetJoinWarps; ++w) v = __reduce_or_sync(kFull, (v >> x) & 1 ? s_prod[w][x] : 0u);
+    const uint32_t z = lane < kSetRuns ? __ldg(p.ends + static_cast<uint64_t>(p.c - 1) * kSetRuns + lane) : p.n;
+    const bool fin = ((v >> x) & 1) && z < p.n && ((__ldg(p.final_bits + (z >> 5)) >> (z & 31)) & 1);
+    const uint32_t acc = __any_sync(kFull, fin) ? 1 : 0;
+    if (lane == 0) {
+        *p.accept = static_cast<uint8_t>(acc);
+        *p.status = 0;
+        *p.ticket = 0;
+        if (p.h_accept) {
+            *p.h_accept = static_cast<uint8_t>(acc);
+            *p.h_status = 0;
+        }
+    }
+}
+
+// Whole tiles, for a few blocks on each of about 150 SMs: 256 blocks' products are short work for the
+// last block, and a warp's chain is short up to 65,536 chunks.
+uint32_t join_per_warp(uint32_t c) { return std::max<uint32_t>(kSetTile, (c / 8192 + kSetTile - 1) / kSetTile * kSetTile); }
+
+}  // namespace
+
+bool set_takes(const HostAutomaton &H, uint64_t len, uint32_t c, int sms) {
+    // chunks for at least a quarter of the lanes (fewer are cut into pieces by the general path), each
+    // with some whole blocks
+    return H.set.ok && c <= (1u << 26) && len / c >= 128 && len <= (1ull << 40) && static_cast<uint64_t>(c) * 4 > static_cast<uint64_t>(sms) * 1024;
+}
+
+uint32_t set_join_blocks(uint32_t c) {
+    const uint64_t per = static_cast<uint64_t>(join_per_warp(c)) * kSetJoinWarps;
+    return static_cast<uint32_t>((c + per - 1) / per);
+}
+
+cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
+    const HostAutomaton &H = *C.H;
+    const DeviceAutomaton &D = *C.D;
+    const HostStream &T = H.set.table;
+    SetArgs a{};
+    a.text = C.text;
+    a.len = C.len;
+    a.q = C.len / C.c;
+    const uint64_t rem = C.len % C.c;
+    a.frac = rem ? static_cast<uint64_t>((static_cast<unsigned __int128>(rem) << 64) / C.c) + 1 : 0;   // (as the stream kernels)
+    a.c = C.c;
+    a.depth = H.set.depth;
+    a.k = H.k;
+    a.next = D.set_next;
+    a.images = D.set_images;
+    a.leaf = D.set_leaf;
+    a.ends = C.ends;
+    a.reps = C.reps;
+    a.pids = C.pids;
+    a.t = stream_field_tables(T);
+    a.t.walk = D.trans;
+    a.t.classmap = D.classmap;
+    a.t.words = D.set_words;
+    a.t.n = H.n_states;
+    a.t.C = H.n_classes;
+    a.t.n_walk = static_cast<uint32_t>(H.trans.size() + 1) & ~1u;      // (whole words; the upload is padded)
+    uint32_t off = a.t.n_words * 4 * T.copies;
+    a.t.off_table = 0;
+    a.t.off_cls = (off + 15) & ~15u;
+    a.t.off_walk = a.t.off_cls + 256;
+    const size_t smem = set_rest_bytes(H) + static_cast<size_t>(off);
+    const uint32_t tasks = (C.c + 31) / 32;
+    const uint32_t warps = std::max<uint32_t>(4, std::min<uint32_t>(kSetBlock / 32, (tasks + sms - 1) / sms));
+    const uint32_t grid = std::min<uint32_t>(sms, (tasks + warps - 1) / warps);
+    auto kern = T.group == 4 ? rid_set_kernel<4> : rid_set_kernel<2>;
+    cudaError_t e = ensure_smem_cap(reinterpret_cast<const void *>(kern), smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, warps * 32, smem, st>>>(a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (C.between) {
+        e = cudaEventRecord(C.between, st);
+        if (e != cudaSuccess) return e;
+    }
+    SetJoinArgs j{};
+    j.c = C.c;
+    j.k = H.k;
+    j.kw = H.kw;
+    j.n = H.n_states;
+    j.q0_slot = H.q0_slot;
+    j.per_warp = join_per_warp(C.c);
+    j.ends = C.ends;
+    j.reps = C.reps;
+    j.pids = C.pids;
+    j.block_mask = D.set_block_mask;
+    j.ifmask = D.ifmask;
+    j.final_bits = D.final_bits;
+    j.part = D.set_part;
+    j.maps = C.maps;
+    j.partials = C.partials;
+    j.ticket = C.ticket;
+    j.status = C.status;
+    j.accept = C.accept;
+    j.h_accept = C.h_accept;
+    j.h_status = C.h_status;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(set_join_blocks(C.c));
+    cfg.blockDim = dim3(32 * kSetJoinWarps);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = C.between ? 0 : 1;
+    return cudaLaunchKernelEx(&cfg, rid_set_join_kernel, j);
+}
+
+}  // namespace ridfa

@@ -22,7 +22,8 @@ struct StreamTables {
     uint32_t n_words, copies, row;                       // row: bytes per state
     // field codes: byte of code 0 (four times) and what each field bit and both add to it; where the
     // codes of bytes 0.. (and 2.. for two-byte lookups) gather; column -> byte offset
-    uint32_t shift, canon0, d1, d2, d12, mul, mul_h, take_bits, part_mask, col_mul, part_mul;
+    // (second: mask of the field's second bit, 0 in a field of one)
+    uint32_t shift, second, canon0, d1, d2, d12, mul, mul_h, take_bits, part_mask, col_mul, part_mul;
     uint32_t off_table, off_walk, off_cls, off_stage;
 };
 
@@ -166,9 +167,19 @@ __device__ __forceinline__ void load_tables(const StreamTables &p, uint8_t *smem
     if (p.copies >= 4) {
         const uint32_t lg = __ffs(p.copies) - 3;         // 16-byte stores per word: copies / 4
         for (uint32_t i = threadIdx.x; i < p.n_words << lg; i += nt) put4(base + p.off_table + i * 16, __ldg(p.words + (i >> lg)));
+    } else if (p.copies == 2) {
+        for (uint32_t i = threadIdx.x; i < p.n_words; i += nt) {
+            const uint32_t v = __ldg(p.words + i);
+            sts_u32(base + p.off_table + i * 8, v);
+            sts_u32(base + p.off_table + i * 8 + 4, v);
+        }
     } else {
-        for (uint32_t i = threadIdx.x; i < p.n_words * p.copies; i += nt)
-            sts_u32(base + p.off_table + i * 4, __ldg(p.words + i / p.copies));
+        // one copy, as it is: 16 bytes a thread (the upload is padded to whole ones)
+#pragma unroll 4
+        for (uint32_t i = threadIdx.x; i < (p.n_words + 3) / 4; i += nt) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p.words) + i);
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(base + p.off_table + i * 16), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+        }
     }
     load_walk(p, smem);
 }
@@ -339,19 +350,9 @@ __device__ __forceinline__ void stream_staged(const S &T, Walk &w, uint32_t stag
     while (pos < end) w.step_class(w.class_of(__ldg(reinterpret_cast<const uint8_t *>(pos++))));
 }
 
-// Host: the tables' part of a launch's arguments.  walk_only: no main table.
-inline StreamTables stream_tables(const HostAutomaton &H, const DeviceAutomaton &D, bool walk_only, uint32_t warps) {
-    const HostStream &T = H.stream;
+// Host: what a table says of itself, the field codes among it.
+inline StreamTables stream_field_tables(const HostStream &T) {
     StreamTables a{};
-    a.warps = warps;
-    a.walk = D.mg_walk;
-    a.classmap = D.classmap;
-    a.edge_pid = D.mg_edge_pid;
-    a.code = D.st_code;
-    a.words = D.st_words;
-    a.n = H.n_states;
-    a.C = H.n_classes;
-    a.n_walk = static_cast<uint32_t>(H.merge.walk.size());
     a.n_words = static_cast<uint32_t>(T.words.size());
     a.copies = T.copies;
     a.row = T.row_words * 4 * T.copies;
@@ -359,6 +360,7 @@ inline StreamTables stream_tables(const HostAutomaton &H, const DeviceAutomaton 
         const uint32_t w = T.width, bits = w * T.group, part = 4 / T.entry;
         auto byte = [&](uint32_t code) { return T.canon >> (8 * code) & 0xFF; };
         a.shift = T.shift;
+        a.second = w == 2 ? 0x01010101u : 0u;
         a.canon0 = byte(0) * 0x01010101u;
         a.d1 = byte(1) - byte(0);
         a.d2 = byte(2) - byte(0);
@@ -374,6 +376,22 @@ inline StreamTables stream_tables(const HostAutomaton &H, const DeviceAutomaton 
         a.col_mul = 4 * T.copies / part;
         a.part_mul = T.entry - a.col_mul;
     }
+    return a;
+}
+
+// Host: the tables' part of a launch's arguments.  walk_only: no main table.
+inline StreamTables stream_tables(const HostAutomaton &H, const DeviceAutomaton &D, bool walk_only, uint32_t warps) {
+    const HostStream &T = H.stream;
+    StreamTables a = stream_field_tables(T);
+    a.warps = warps;
+    a.walk = D.mg_walk;
+    a.classmap = D.classmap;
+    a.edge_pid = D.mg_edge_pid;
+    a.code = D.st_code;
+    a.words = D.st_words;
+    a.n = H.n_states;
+    a.C = H.n_classes;
+    a.n_walk = static_cast<uint32_t>(H.merge.walk.size());
     uint32_t off = 0;
     if (!walk_only) {
         off = T.kind == kStreamField ? 0 : 256 * 128;
