@@ -78,7 +78,7 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
         o_words = put_v(T.words);
     }
     const HostSet &Z = H.set;
-    size_t z_next = 0, z_leaf = 0, z_img = 0, z_part = 0, z_mask = 0, z_words = 0;
+    size_t z_next = 0, z_leaf = 0, z_img = 0, z_part = 0, z_mask = 0, z_words = 0, z_bn = 0, z_bi = 0;
     if (Z.ok) {
         z_next = put_v(Z.next);
         z_leaf = put_v(Z.leaf);
@@ -86,6 +86,8 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
         z_part = put_v(Z.part);
         z_mask = put_v(Z.block_mask);
         z_words = put_v(Z.table.words);
+        z_bn = put_v(Z.back_next);
+        z_bi = put_v(Z.back_images);
     }
     uint8_t *base = nullptr;
     cudaError_t e = cudaMalloc(&base, img.size());
@@ -122,6 +124,8 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
         D.set_part = base + z_part;
         D.set_block_mask = u32(z_mask);
         D.set_words = u32(z_words);
+        D.set_back_next = u16(z_bn);
+        D.set_back_images = u16(z_bi);
     }
     D.bytes = img.size();
     return RIDFA_OK;
@@ -1058,16 +1062,10 @@ int recognize_stream(const ridfa_program *P, const HostAutomaton &H, const Devic
 
 // One call through the set kernels (ridfa_set.cu), as recognize_stream.
 int recognize_set(const ridfa_program *P, const HostAutomaton &H, const DeviceAutomaton *D, int dev, int sms,
-                  const uint8_t *d_text, uint64_t len, uint32_t n_chunks, bool prof, uint8_t *d_accept_user, uint8_t *h_accept,
+                  const uint8_t *d_text, uint64_t len, uint32_t n_chunks, uint32_t spc, bool prof, uint8_t *d_accept_user, uint8_t *h_accept,
                   uint16_t *d_maps_user, cudaStream_t st) {
-    auto al = [](size_t x) { return (x + 255) & ~static_cast<size_t>(255); };
-    size_t off = 1024;
-    const size_t o_ends = off;     off += al(static_cast<size_t>(n_chunks) * kSetRuns * 2);
-    const size_t o_reps = off;     off += al(static_cast<size_t>(n_chunks) * 8);
-    const size_t o_pids = off;     off += al(static_cast<size_t>(n_chunks) * 4);
-    const size_t o_part = off;     off += al(static_cast<size_t>(set_join_blocks(n_chunks)) * kSetRuns * 4);
     int err = RIDFA_OK;
-    DeviceScratch *S = scratch_for(P, dev, off, &err);
+    DeviceScratch *S = scratch_for(P, dev, 1024 + set_scratch(n_chunks, spc), &err);
     if (!S) return err;
     uint8_t *base = static_cast<uint8_t *>(S->base);
     SetCall C;
@@ -1076,11 +1074,9 @@ int recognize_set(const ridfa_program *P, const HostAutomaton &H, const DeviceAu
     C.text = d_text;
     C.len = len;
     C.c = n_chunks;
-    C.ends = reinterpret_cast<uint16_t *>(base + o_ends);
-    C.reps = reinterpret_cast<uint64_t *>(base + o_reps);
-    C.pids = reinterpret_cast<uint32_t *>(base + o_pids);
+    C.spc = spc;
+    C.scratch = base + 1024;
     C.maps = d_maps_user;
-    C.partials = reinterpret_cast<uint32_t *>(base + o_part);
     C.ticket = reinterpret_cast<uint32_t *>(base);
     C.status = reinterpret_cast<uint32_t *>(base + 256);
     C.accept = d_accept_user ? d_accept_user : base + 512;
@@ -1155,11 +1151,11 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
     Automaton A{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state,
                 H.n_states, H.n_classes, H.k, H.kw, H.q0_slot, H.merges};
     const bool to_stream = automatic(tuning) && stream_takes(H, len, n_chunks);
-    const bool to_set = automatic(tuning) && !h_summary && set_takes(H, len, n_chunks, sms);
-    if (to_stream || to_set) {
+    const uint32_t set_spc = automatic(tuning) && !h_summary ? set_pieces(H, len, n_chunks, sms) : 0;
+    if (to_stream || set_spc) {
         const bool prof = tuning && tuning->profile;
         err = to_stream ? recognize_stream(P, H, D, dev, sms, d_text, len, n_chunks, prof, d_accept_user, h_accept, d_maps_user, st, h_summary)
-                        : recognize_set(P, H, D, dev, sms, d_text, len, n_chunks, prof, d_accept_user, h_accept, d_maps_user, st);
+                        : recognize_set(P, H, D, dev, sms, d_text, len, n_chunks, set_spc, prof, d_accept_user, h_accept, d_maps_user, st);
         if (err == RIDFA_OK)
             for (auto &x : P->scratch)
                 if (x.device == dev) {

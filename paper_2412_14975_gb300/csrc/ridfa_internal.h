@@ -83,6 +83,9 @@ struct HostSet {
     std::vector<uint8_t> part;        // [parts][k]: block of each slot, 0xFF: dead
     std::vector<uint32_t> block_mask; // [parts][kw][kSetRuns]: slots of each block
     HostStream table;                 // kStreamField, entries of 2 bytes
+    uint32_t back_depth = 0;          // 0: not built.  The sets the bytes before a piece leave of all states:
+    std::vector<uint16_t> back_next;  // [inner sets][C]: an inner set, or kLeafBit | leaf (leaf 0: all dead)
+    std::vector<uint16_t> back_images;// [leaves][kSetRuns]: states (unused ones: n_states)
 };
 constexpr uint32_t kSetRuns = 16;     // places; at most 15 are taken (15 marks a dead run in 4 bits)
 
@@ -132,7 +135,7 @@ struct DeviceAutomaton {
     uint32_t *mg_node_img = nullptr, *mg_slot_alive = nullptr;
     uint32_t *st_code = nullptr, *st_words = nullptr;
     // set tables (HostSet)
-    uint16_t *set_next = nullptr, *set_images = nullptr;
+    uint16_t *set_next = nullptr, *set_images = nullptr, *set_back_next = nullptr, *set_back_images = nullptr;
     uint32_t *set_leaf = nullptr, *set_block_mask = nullptr, *set_words = nullptr;
     uint8_t *set_part = nullptr;
     size_t bytes = 0;

@@ -394,6 +394,74 @@ void build_table(HostAutomaton &H) {
     H.stream = best;
 }
 
+// The sets that strings of up to `back_depth` bytes lead the set of all states to, each followed until
+// fewer than kSetRuns states are left: what a piece in the middle of a chunk can be entered with.  Sets
+// are bit rows; left out when they are too many.
+void build_back(const HostAutomaton &H, HostSet &Z) {
+    constexpr uint32_t kMaxNodes = 4096, kMaxDepth = 24, kHash = 4 * kMaxNodes;
+    const uint32_t n = H.n_states, C = H.n_classes, words = (n + 63) / 64;
+    if (n < kSetRuns) return;
+    std::vector<uint64_t> sets(words, 0), row(words);     // bit row of every set met; 0: all states
+    std::vector<uint32_t> depth{0}, code{0}, hash(kHash, UINT32_MAX), order{0};
+    for (uint32_t x = 0; x < n; ++x) sets[x >> 6] |= 1ull << (x & 63);
+    std::vector<uint16_t> images(kSetRuns, static_cast<uint16_t>(n)), next;   // leaf 0: all dead
+    uint64_t steps = 0;
+    uint32_t inner = 1, leaves = 1, most = 0;             // code: the inner node's index, or kLeafBit | leaf
+    for (uint32_t u = 0; u < order.size(); ++u) {
+        const uint32_t from = order[u];
+        most = std::max(most, depth[from] + 1);
+        if (most > kMaxDepth) return;
+        for (uint32_t c = 0; c < C; ++c) {
+            std::fill(row.begin(), row.end(), 0);
+            for (uint32_t w = 0; w < words; ++w)
+                for (uint64_t b = sets[static_cast<size_t>(from) * words + w]; b; b &= b - 1) {
+                    const uint32_t t = H.trans[static_cast<size_t>(w * 64 + __builtin_ctzll(b)) * C + c];
+                    if (t < n) row[t >> 6] |= 1ull << (t & 63);
+                }
+            uint32_t count = 0;
+            uint64_t h = 0;
+            for (uint64_t v : row) {
+                count += static_cast<uint32_t>(__builtin_popcountll(v));
+                h = (h ^ v) * 0x9E3779B97F4A7C15ull;
+                h ^= h >> 29;
+            }
+            if ((steps += count) > kMaxSteps) return;
+            if (!count) {
+                next.push_back(kLeafBit);
+                continue;
+            }
+            uint32_t at = static_cast<uint32_t>(h >> 32) % kHash;
+            while (hash[at] != UINT32_MAX && !std::equal(row.begin(), row.end(), sets.begin() + static_cast<size_t>(hash[at]) * words))
+                at = (at + 1) % kHash;
+            if (hash[at] == UINT32_MAX) {
+                const uint32_t id = static_cast<uint32_t>(depth.size());
+                if (id >= 2 * kMaxNodes) return;
+                hash[at] = id;
+                sets.insert(sets.end(), row.begin(), row.end());
+                depth.push_back(depth[from] + 1);
+                if (count < kSetRuns) {
+                    code.push_back(kLeafBit | leaves++);
+                    for (uint32_t w = 0; w < words; ++w)
+                        for (uint64_t b = row[w]; b; b &= b - 1) images.push_back(static_cast<uint16_t>(w * 64 + __builtin_ctzll(b)));
+                    images.resize(static_cast<size_t>(leaves) * kSetRuns, static_cast<uint16_t>(n));
+                } else {
+                    if (inner >= kMaxNodes) return;
+                    code.push_back(inner++);
+                    order.push_back(id);
+                }
+            }
+            next.push_back(static_cast<uint16_t>(code[hash[at]]));
+        }
+    }
+    // every index the kernels take unchecked
+    if (next.size() != static_cast<size_t>(inner) * C || images.size() != static_cast<size_t>(leaves) * kSetRuns) return;
+    for (uint16_t e : next)
+        if ((e & kLeafBit) ? (e & 0x7FFFu) >= leaves : e >= inner) return;
+    Z.back_next = std::move(next);
+    Z.back_images = std::move(images);
+    Z.back_depth = most;
+}
+
 // The functions of the first bytes on the slots, level by level, down to the first level on which all
 // have fewer than kSetRuns distinct values.
 bool build_set(const HostAutomaton &H, HostSet &Z) {
@@ -496,6 +564,7 @@ bool build_set(const HostAutomaton &H, HostSet &Z) {
             const uint8_t b = Z.part[static_cast<size_t>(p) * k + a];
             if (b != 0xFF) Z.block_mask[(static_cast<size_t>(p) * H.kw + (a >> 5)) * kSetRuns + b] |= 1u << (a & 31);
         }
+    build_back(H, Z);
     // every index the kernels take unchecked
     if (Z.next.size() != static_cast<size_t>(Z.inner) * C || Z.parts > 0xFFFF) return false;
     for (uint16_t e : Z.next)

@@ -33,11 +33,13 @@ constexpr int kHalf = kSetRuns / 2;
 struct SetArgs {
     const uint8_t *text;
     uint64_t len, q, frac;        // chunk i begins at i * q + (i * frac >> 64)
-    uint32_t c, depth, k;
-    const uint16_t *next, *images, *trans;
+    uint32_t c, depth, spc, back_depth;
+    uint64_t pieces;              // c * spc; pieces of a chunk are equal up to 64 bytes
+    const uint16_t *next, *images, *back_next, *back_images;
     const uint32_t *leaf;
-    uint16_t *ends;               // [c][kSetRuns]: distinct end states, dead beyond them
-    uint64_t *reps;               // [c]: place of each run of the graph's leaf (4 bits; 15: dead)
+    uint16_t *ends;               // [pieces][kSetRuns]: distinct end states, dead beyond them
+    uint64_t *reps;               // [pieces]: place of each run of the graph's leaf (4 bits; 15: dead)
+    uint16_t *entry;              // [pieces][kSetRuns]: states a later piece's runs begin in
     uint32_t *pids;               // [c]: the leaf's partition
     StreamTables t;
 };
@@ -141,6 +143,15 @@ __device__ __forceinline__ bool set_block_m(const StreamTables &p, uint32_t lt, 
     }
 }
 
+// Byte i of 32.
+__device__ __forceinline__ uint32_t byte_of(const uint32_t (&w)[8], uint32_t i) {
+    uint32_t v = w[0];
+#pragma unroll
+    for (int k = 1; k < 8; ++k)
+        if (i >> 2 == static_cast<uint32_t>(k)) v = w[k];
+    return v >> (8 * (i & 3)) & 0xFF;
+}
+
 template <int G>
 __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_constant__ SetArgs p) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -151,18 +162,42 @@ __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_cons
     const uint32_t lt = base + p.t.off_table + (lane & (p.t.copies - 1)) * 4;
     const uint32_t cls = base + p.t.off_cls, one = base + p.t.off_walk;
     const uint64_t t0 = reinterpret_cast<uint64_t>(p.text);
-    const uint32_t warps = blockDim.x / 32;
-    for (uint32_t task = blockIdx.x * warps + (threadIdx.x >> 5); task * 32 < p.c; task += gridDim.x * warps) {
-        const uint32_t ch = task * 32 + lane;
-        const bool have = ch < p.c;
+    for (uint64_t task = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; task * 32 < p.pieces; task += gridDim.x * (kSetBlock / 32)) {
+        const uint64_t pc = task * 32 + lane;
+        const bool have = pc < p.pieces;
+        uint32_t ch = static_cast<uint32_t>(pc), j = 0;
         uint64_t pos = t0, end = t0;
         if (have) {
+            if (p.spc > 1) {
+                ch = static_cast<uint32_t>(pc / p.spc);
+                j = static_cast<uint32_t>(pc - static_cast<uint64_t>(ch) * p.spc);
+            }
             pos = t0 + set_chunk_at(p, ch);
             end = t0 + set_chunk_at(p, ch + 1);
+            if (p.spc > 1) {
+                // (cuts on 64-byte boundaries of the text: no ragged ends but the chunk's)
+                const uint64_t s0 = pos, per = (end - s0) / p.spc, rem = (end - s0) - per * p.spc;
+                if (j) pos = (s0 + j * per + min(static_cast<uint64_t>(j), rem)) & ~63ull;
+                if (j + 1 < p.spc) end = (s0 + (j + 1) * per + min(static_cast<uint64_t>(j + 1), rem)) & ~63ull;
+            }
         }
-        // ---- the first bytes through the graph (chunks are longer than its depth)
+        // ---- the first bytes through the graph (chunks are longer than its depth); for a later piece,
+        // the bytes before it, from all states (pieces are longer than back_depth)
         uint32_t leaf = 0;
-        if (have) {
+        uint32_t before[8];                      // the 32 bytes before a later piece
+        uint32_t taken = 32;
+        if (j) {
+            load32(reinterpret_cast<const uint8_t *>(pos - 32), before);
+            uint32_t node = 0;
+            taken = 32 - p.back_depth;
+            for (; taken < 32; ++taken) {
+                const uint32_t e = __ldg(p.back_next + node * p.t.C + lds_u8(cls + byte_of(before, taken)));
+                node = e;
+                if (e & kLeafBit) break;
+            }
+            ++taken;
+            leaf = node & 0x7FFF;
+        } else if (have) {
             uint32_t node = 0;
             for (uint32_t d = 0; d < p.depth; ++d) {
                 const uint32_t e = __ldg(p.next + node * p.t.C + lds_u8(cls + __ldg(reinterpret_cast<const uint8_t *>(pos++))));
@@ -171,13 +206,14 @@ __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_cons
             }
             leaf = node & 0x7FFF;
         }
-        const uint32_t pid = __ldg(p.leaf + 2 * leaf), img = __ldg(p.leaf + 2 * leaf + 1);
+        const uint32_t pid = j ? 0u : __ldg(p.leaf + 2 * leaf);
+        const uint16_t *img = j ? p.back_images + leaf * kSetRuns : p.images + __ldg(p.leaf + 2 * leaf + 1);
         uint32_t s[kSetRuns];
         uint64_t rep = ~0ull;
         uint32_t cnt = 0;
 #pragma unroll
         for (int g = 0; g < static_cast<int>(kSetRuns); ++g) {
-            s[g] = __ldg(p.images + img + g);
+            s[g] = __ldg(img + g);
             if (s[g] != dead) {
                 rep = (rep & ~(15ull << (4 * g))) | static_cast<uint64_t>(g) << (4 * g);
                 ++cnt;
@@ -185,12 +221,25 @@ __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_cons
         }
         // ---- one-byte steps for all runs up to a 64-byte boundary
         const uint32_t most = __reduce_max_sync(kFull, cnt);
-        auto step_all = [&](uint32_t m) {
-            const uint32_t c = lds_u8(cls + __ldg(reinterpret_cast<const uint8_t *>(pos++)));
+        auto step_byte = [&](uint32_t m, uint32_t byte) {
+            const uint32_t c = lds_u8(cls + byte);
 #pragma unroll
             for (int g = 0; g < static_cast<int>(kSetRuns); ++g)
                 if (static_cast<uint32_t>(g) < m) s[g] = lds_u16(one + 2 * (s[g] * p.t.C + c));
         };
+        auto step_all = [&](uint32_t m) { step_byte(m, __ldg(reinterpret_cast<const uint8_t *>(pos++))); };
+        auto store = [&](uint16_t *to) {
+            uint32_t w[kHalf];
+#pragma unroll
+            for (int g = 0; g < kHalf; ++g) w[g] = s[2 * g] | s[2 * g + 1] << 16;
+            uint4 *out = reinterpret_cast<uint4 *>(to + pc * kSetRuns);
+            out[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            out[1] = make_uint4(w[4], w[5], w[6], w[7]);
+        };
+        if (j) {
+            for (; taken < 32; ++taken) step_byte(most, byte_of(before, taken));
+            store(p.entry);                      // (states may repeat: those runs end in one place)
+        }
         // (by words once those are aligned: a lookup a run for four bytes)
         while (cnt && pos < end && (pos & 3)) step_all(most);
         while (cnt && pos + 4 <= end && (pos & 63)) {
@@ -231,7 +280,7 @@ __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_cons
                     b[i] = nb[i];
                 }
             }
-            if ((r & 3) == 3) {
+            if (r < 3 || (r & 3) == 3) {         // (the most runs die in the first bytes)
                 if (M > kHalf) cnt = compact_set<kSetRuns>(s, rep, dead);
                 else cnt = compact_set<kHalf>(s, rep, dead);
                 M = __reduce_max_sync(kFull, r + 1 < blocks ? cnt : 0u);
@@ -251,15 +300,75 @@ __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_cons
         while (used && pos < end) step_all(M);
         compact_set<kSetRuns>(s, rep, dead);
         if (!have) continue;
-        uint32_t w[kHalf];
-#pragma unroll
-        for (int g = 0; g < kHalf; ++g) w[g] = s[2 * g] | s[2 * g + 1] << 16;
-        uint4 *out = reinterpret_cast<uint4 *>(p.ends + static_cast<uint64_t>(ch) * kSetRuns);
-        out[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        out[1] = make_uint4(w[4], w[5], w[6], w[7]);
-        p.reps[ch] = rep;
-        p.pids[ch] = pid;
+        store(p.ends);
+        p.reps[pc] = rep;
+        if (j == 0) p.pids[ch] = pid;
     }
+}
+
+// Up to kComposeSet consecutive pieces of a chunk as one: a half-warp follows the places of the first
+// through the others, whose runs it finds by the states they begin in.  Bound by latency: the words of
+// four pieces are loaded at a time.
+constexpr uint32_t kComposeSet = 32, kComposeOne = 64;       // (up to kComposeOne pieces in one launch)
+struct SetComposeArgs {
+    uint32_t c, in, out, group, n;                           // pieces a chunk, before and after
+    const uint16_t *ends, *entry;
+    const uint64_t *reps;
+    uint16_t *to_ends, *to_entry;
+    uint64_t *to_reps;
+};
+
+__global__ void __launch_bounds__(256) rid_set_compose_kernel(const __grid_constant__ SetComposeArgs p) {
+    const uint32_t lane = threadIdx.x & 31, x = lane & 15, half = lane & 16;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const uint64_t all = static_cast<uint64_t>(p.c) * p.out;
+    const uint64_t id = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 4;
+    const uint64_t mine = min(id, all - 1);
+    const uint64_t ch = mine / p.out;
+    const uint32_t g0 = static_cast<uint32_t>(mine - ch * p.out) * p.group;
+    const uint32_t n_in = min(p.group, p.in - g0);
+    const uint64_t at = ch * p.in + g0;
+    uint32_t y = __ldg(p.ends + at * kSetRuns + x);
+    uint32_t ew[4] = {}, z[4] = {}, ne[4] = {}, nz[4] = {};
+    uint64_t rp[4] = {}, nr[4] = {};
+    auto fetch = [&](uint32_t j0) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (j0 + u >= n_in) continue;
+            const uint64_t o = at + j0 + u;
+            ne[u] = __ldg(reinterpret_cast<const uint32_t *>(p.entry + o * kSetRuns) + (x & 7));
+            nz[u] = __ldg(p.ends + o * kSetRuns + x);
+            nr[u] = __ldg(reinterpret_cast<const unsigned long long *>(p.reps) + o);
+        }
+    };
+    fetch(1);
+    for (uint32_t j0 = 1; j0 < p.group; j0 += 4) {           // (the whole warp takes p.group pieces)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            ew[u] = ne[u];
+            z[u] = nz[u];
+            rp[u] = nr[u];
+        }
+        fetch(j0 + 4);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const bool on = j0 + u < n_in;
+            uint32_t place = 15;
+#pragma unroll
+            for (int g = 0; g < kHalf; ++g) {
+                const uint32_t w = __shfl_sync(kFull, ew[u], half + g);
+                if (y == (w & 0xFFFFu)) place = static_cast<uint32_t>(rp[u] >> (8 * g)) & 15;
+                if (y == w >> 16) place = static_cast<uint32_t>(rp[u] >> (8 * g + 4)) & 15;
+            }
+            if (y >= p.n) place = 15;
+            const uint32_t to = __shfl_sync(kFull, z[u], half + place);     // (place 15 stays dead)
+            if (on) y = to;
+        }
+    }
+    if (id >= all) return;
+    p.to_ends[mine * kSetRuns + x] = static_cast<uint16_t>(y);
+    if (p.out > 1) p.to_entry[mine * kSetRuns + x] = __ldg(p.entry + at * kSetRuns + x);
+    if (x == 0) p.to_reps[mine] = __ldg(reinterpret_cast<const unsigned long long *>(p.reps) + at);
 }
 
 // ------------------------------------------------------------------------------- join
@@ -281,6 +390,7 @@ constexpr uint32_t kSetTile = 16;                // chunks a warp stages at a ti
 // rows <- rows · M in each half-warp: lane h * 16 + x has row x of both (at most 15 places).  `from`
 // is added to the lane M's row z is read from (z + from): the own half's, or a fixed half's.
 __device__ __forceinline__ uint32_t set_times(uint32_t row, uint32_t m, uint32_t from) {
+    if (__all_sync(kFull, m == 1u << (threadIdx.x & 15))) return row;       // (identities would be the longest)
     const uint32_t any = __ballot_sync(kFull, m != 0);
     uint32_t out = 0;
     for (uint32_t nz = (any | any >> 16) & 0xFFFFu; nz; nz &= nz - 1) {
@@ -426,23 +536,46 @@ __global__ void __launch_bounds__(32 * kSetJoinWarps) rid_set_join_kernel(const 
 // last block, and a warp's chain is short up to 65,536 chunks.
 uint32_t join_per_warp(uint32_t c) { return std::max<uint32_t>(kSetTile, (c / 8192 + kSetTile - 1) / kSetTile * kSetTile); }
 
-}  // namespace
-
-bool set_takes(const HostAutomaton &H, uint64_t len, uint32_t c, int sms) {
-    // chunks for at least a quarter of the lanes (fewer are cut into pieces by the general path), each
-    // with some whole blocks
-    return H.set.ok && c <= (1u << 26) && len / c >= 128 && len <= (1ull << 40) && static_cast<uint64_t>(c) * 4 > static_cast<uint64_t>(sms) * 1024;
-}
-
 uint32_t set_join_blocks(uint32_t c) {
     const uint64_t per = static_cast<uint64_t>(join_per_warp(c)) * kSetJoinWarps;
     return static_cast<uint32_t>((c + per - 1) / per);
+}
+
+}  // namespace
+
+uint32_t set_pieces(const HostAutomaton &H, uint64_t len, uint32_t c, int sms) {
+    if (!H.set.ok || c > (1u << 26) || len > (1ull << 40) || len / c < 128) return 0;
+    const uint64_t lanes = static_cast<uint64_t>(sms) * kSetBlock;
+    // Without the sets of what a piece is entered with, a chunk is one lane's work: at least half of the
+    // lanes have to have one (at a quarter the general path was as fast).
+    if (!H.set.back_depth) return static_cast<uint64_t>(c) * 2 > lanes ? 1 : 0;
+    // As many pieces as the lanes take at once, of 256 bytes or more: a second round costs its pieces'
+    // first bytes, with the most runs, again (1 GiB in 20,000 chunks: 721 us in 3 pieces each, 883 in 7;
+    // in 40,000 chunks 782 in one, 978 in 3), and a shorter piece is mostly such bytes.
+    return static_cast<uint32_t>(std::max<uint64_t>(1, std::min<uint64_t>(len / c / 256, lanes / c)));
+}
+
+size_t set_scratch(uint32_t c, uint32_t spc) {
+    size_t n = 0;
+    for (uint64_t s = spc; s > 1; s = (s + kComposeSet - 1) / kComposeSet) n += c * s;       // each level's pieces
+    return (n + c) * (2 * kSetRuns * 2 + 8) + static_cast<size_t>(c) * 4 + static_cast<size_t>(set_join_blocks(c)) * kSetRuns * 4 + 64 * 256;
 }
 
 cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     const HostAutomaton &H = *C.H;
     const DeviceAutomaton &D = *C.D;
     const HostStream &T = H.set.table;
+    const uint64_t pieces = static_cast<uint64_t>(C.c) * C.spc;
+    uint8_t *next = C.scratch;
+    auto take = [&](size_t bytes) {
+        uint8_t *r = next;
+        next += (bytes + 255) & ~static_cast<size_t>(255);
+        return r;
+    };
+    auto u16 = [&](uint64_t n) { return reinterpret_cast<uint16_t *>(take(n * kSetRuns * 2)); };
+    auto u64 = [&](uint64_t n) { return reinterpret_cast<uint64_t *>(take(n * 8)); };
+    uint32_t *pids = reinterpret_cast<uint32_t *>(take(C.c * 4ull));
+    uint32_t *partials = reinterpret_cast<uint32_t *>(take(static_cast<size_t>(set_join_blocks(C.c)) * kSetRuns * 4));
     SetArgs a{};
     a.text = C.text;
     a.len = C.len;
@@ -450,14 +583,19 @@ cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     const uint64_t rem = C.len % C.c;
     a.frac = rem ? static_cast<uint64_t>((static_cast<unsigned __int128>(rem) << 64) / C.c) + 1 : 0;   // (as the stream kernels)
     a.c = C.c;
+    a.spc = C.spc;
+    a.pieces = pieces;
     a.depth = H.set.depth;
-    a.k = H.k;
+    a.back_depth = H.set.back_depth;
     a.next = D.set_next;
     a.images = D.set_images;
+    a.back_next = D.set_back_next;
+    a.back_images = D.set_back_images;
     a.leaf = D.set_leaf;
-    a.ends = C.ends;
-    a.reps = C.reps;
-    a.pids = C.pids;
+    a.ends = u16(pieces);
+    a.reps = u64(pieces);
+    a.entry = C.spc > 1 ? u16(pieces) : nullptr;
+    a.pids = pids;
     a.t = stream_field_tables(T);
     a.t.walk = D.trans;
     a.t.classmap = D.classmap;
@@ -470,15 +608,42 @@ cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     a.t.off_cls = (off + 15) & ~15u;
     a.t.off_walk = a.t.off_cls + 256;
     const size_t smem = set_rest_bytes(H) + static_cast<size_t>(off);
-    const uint32_t tasks = (C.c + 31) / 32;
-    const uint32_t warps = std::max<uint32_t>(4, std::min<uint32_t>(kSetBlock / 32, (tasks + sms - 1) / sms));
-    const uint32_t grid = std::min<uint32_t>(sms, (tasks + warps - 1) / warps);
+    const uint64_t tasks = (pieces + 31) / 32;
+    const uint32_t grid = static_cast<uint32_t>(std::min<uint64_t>(sms, tasks));
     auto kern = T.group == 4 ? rid_set_kernel<4> : rid_set_kernel<2>;
     cudaError_t e = ensure_smem_cap(reinterpret_cast<const void *>(kern), smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, warps * 32, smem, st>>>(a);
+    kern<<<grid, kSetBlock, smem, st>>>(a);       // (all warps load the table)
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    SetComposeArgs m{};
+    m.c = C.c;
+    m.n = H.n_states;
+    m.ends = a.ends;
+    m.entry = a.entry;
+    m.reps = a.reps;
+    for (m.in = C.spc; m.in > 1; m.in = m.out) {
+        m.group = m.in <= kComposeOne ? m.in : kComposeSet;
+        m.out = (m.in + m.group - 1) / m.group;
+        const uint64_t n = static_cast<uint64_t>(C.c) * m.out;
+        m.to_ends = u16(n);
+        m.to_reps = u64(n);
+        m.to_entry = m.out > 1 ? u16(n) : nullptr;
+        cfg.gridDim = dim3(static_cast<unsigned>((n + 15) / 16));
+        cfg.blockDim = dim3(256);
+        e = cudaLaunchKernelEx(&cfg, rid_set_compose_kernel, m);
+        if (e != cudaSuccess) return e;
+        m.ends = m.to_ends;
+        m.entry = m.to_entry;
+        m.reps = m.to_reps;
+    }
     if (C.between) {
         e = cudaEventRecord(C.between, st);
         if (e != cudaSuccess) return e;
@@ -490,28 +655,22 @@ cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     j.n = H.n_states;
     j.q0_slot = H.q0_slot;
     j.per_warp = join_per_warp(C.c);
-    j.ends = C.ends;
-    j.reps = C.reps;
-    j.pids = C.pids;
+    j.ends = m.ends;
+    j.reps = m.reps;
+    j.pids = pids;
     j.block_mask = D.set_block_mask;
     j.ifmask = D.ifmask;
     j.final_bits = D.final_bits;
     j.part = D.set_part;
     j.maps = C.maps;
-    j.partials = C.partials;
+    j.partials = partials;
     j.ticket = C.ticket;
     j.status = C.status;
     j.accept = C.accept;
     j.h_accept = C.h_accept;
     j.h_status = C.h_status;
-    cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(set_join_blocks(C.c));
     cfg.blockDim = dim3(32 * kSetJoinWarps);
-    cfg.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
     cfg.numAttrs = C.between ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, rid_set_join_kernel, j);
 }

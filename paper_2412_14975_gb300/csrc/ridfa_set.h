@@ -13,12 +13,9 @@ struct SetCall {
     const DeviceAutomaton *D = nullptr;
     const uint8_t *text = nullptr;
     uint64_t len = 0;
-    uint32_t c = 0;
-    uint16_t *ends = nullptr;        // [c][kSetRuns]
-    uint64_t *reps = nullptr;        // [c]
-    uint32_t *pids = nullptr;        // [c]
+    uint32_t c = 0, spc = 0;         // chunks, pieces of each (set_pieces)
+    uint8_t *scratch = nullptr;      // set_scratch(c, spc) bytes, aligned to 256
     uint16_t *maps = nullptr;        // [c][k], or null
-    uint32_t *partials = nullptr;    // [set_join_blocks(c)][kSetRuns]
     uint32_t *ticket = nullptr, *status = nullptr;   // ticket: zero before and after every call
     uint8_t *accept = nullptr;
     uint8_t *h_accept = nullptr;     // page-locked host copies of the results, or null
@@ -26,8 +23,9 @@ struct SetCall {
     cudaEvent_t between = nullptr;   // recorded between the two launches when set
 };
 
-bool set_takes(const HostAutomaton &H, uint64_t len, uint32_t c, int sms);
-uint32_t set_join_blocks(uint32_t c);
+// Pieces the set kernels cut each chunk into; 0: the call is not theirs.
+uint32_t set_pieces(const HostAutomaton &H, uint64_t len, uint32_t c, int sms);
+size_t set_scratch(uint32_t c, uint32_t spc);
 cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st);
 
 }  // namespace ridfa

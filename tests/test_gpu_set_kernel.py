@@ -1,8 +1,8 @@
-"""GPU set kernels: automata over at most four bytes whose runs stay apart (the codon RE), a chunk per
-lane.  Every chunk-map entry against stepping the RI-DFA's own table on the host, the accept bit against
-the serial host recognizer, at chunk counts above the few-chunk regime, short and ragged chunks, aligned
-and unaligned texts, bytes outside the alphabet, chunk counts around a warp's, a block's and a join
-block's; and the same answers as the general kernel.  Tolerance 0."""
+"""GPU set kernels: automata over at most four bytes whose runs stay apart (the codon RE), a chunk or a
+piece of one per lane.  Chunk maps against stepping the RI-DFA's own table on the host, the accept bit
+against the serial host recognizer, with many and few chunks, short and ragged ones, aligned and unaligned
+texts, bytes outside the alphabet, chunk counts around a warp's, a block's and a join block's; and the same
+answers as the general kernel.  Tolerance 0."""
 import numpy as np
 import pytest
 
@@ -43,7 +43,8 @@ def check(re_src, x, c, offset=0):
     acc = lib.ridfa_recognize(prog, d[offset:], x.size, c, d_chunk_maps=maps)
     got = maps.cpu().numpy().view(np.uint16)
     rng = np.random.Generator(np.random.PCG64(c))
-    rows = sorted({0, 1, 31, 32, c // 2, c - 33, c - 2, c - 1} | set(rng.integers(0, c, 40).tolist()))
+    rows = sorted({i for i in (0, 1, 31, 32, c // 2, c - 33, c - 2, c - 1) if 0 <= i < c} | set(rng.integers(0, c, 40).tolist()))
+    rows = rows[:400_000 // (x.size // c)]                   # (long chunks: against the general kernel alone)
     for i, want in step_rows(prog, x, c, rows).items():
         assert np.array_equal(got[i], want), (c, i)
     assert acc == lib.ridfa_cpu_recognize(prog, x, 1)
@@ -80,3 +81,19 @@ def test_set_other_res(re_src, alphabet):
     y = x.copy()
     y[y.size // 3] = ord("Z")
     check(re_src, y, 40_000)
+
+
+@pytest.mark.parametrize("c,per", [(1, 20_000_003), (2, 9_000_001), (67, 300_017), (1024, 19_001), (1030, 40_507), (4096, 5_003), (30_000, 701),
+                                   (1, 128), (1, 511), (1, 512), (3, 1_400), (33, 1_000)])
+@pytest.mark.parametrize("re_src,alphabet", [(CODON, None), (BINARY, b"ab")])
+def test_set_pieces(re_src, alphabet, c, per):
+    """Few chunks, cut into pieces: one level of composition and several, ragged groups of pieces."""
+    n = c * per + c // 3
+    if alphabet is None:
+        x = textgen.c2_text(n, seed=c)
+    else:
+        x = np.frombuffer(alphabet, dtype=np.uint8)[np.random.Generator(np.random.PCG64(c)).integers(0, len(alphabet), n)]
+    check(re_src, x, c, offset=c % 32)
+    y = x.copy()
+    y[n // 2] = ord("Z")
+    check(re_src, y, c)
