@@ -30,6 +30,7 @@
 #include "ridfa_batch_plan.h"
 #include "ridfa_internal.h"
 #include "ridfa_kernels.cuh"
+#include "ridfa_set.h"
 #include "ridfa_stream_batch.h"
 
 namespace ridfa {
@@ -570,6 +571,9 @@ struct BatchPlan {
     // the texts of programs with a merge graph, at most kStreamBatchProgs programs a plan
     std::vector<StreamBatchPlan> stream;
     std::vector<size_t> o_stream, o_sres;        // image and result offsets of each
+    // programs whose runs stay apart, over few bytes, with enough text
+    std::vector<SetBatchPlan> set;
+    std::vector<size_t> o_set, o_setres;
     uint32_t n_items = 0;
     uint64_t total_bytes = 0, total_chunks = 0;
     // block layout; everything before o_part is the host image
@@ -594,6 +598,11 @@ PlanStats plan_stats(const BatchPlan *pl) {
     for (const StreamBatchPlan &b : pl->stream) {
         s.n_launches += 2 * static_cast<uint32_t>(b.launches.size());
         for (const StreamBatchPart &p : b.parts) s.n_tasks += p.task1 - p.task0;
+        s.n_segments += static_cast<uint32_t>(b.texts.size());
+    }
+    for (const SetBatchPlan &b : pl->set) {
+        s.n_launches += 2;
+        s.n_tasks += (b.pieces + 31) / 32;
         s.n_segments += static_cast<uint32_t>(b.texts.size());
     }
     return s;
@@ -653,15 +662,25 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
     bool aligned_all = true;
     P.total_bytes = 0;
     P.total_chunks = 0;
-    std::vector<StreamBatchSource> sources;
-    uint64_t stream_bytes = 0;
+    std::vector<StreamBatchSource> sources, set_sources;
+    std::vector<uint64_t> set_bytes;
+    uint64_t stream_bytes = 0, all_set_bytes = 0;
     for (uint32_t p = 0; p < np; ++p) {
         P.text0[p] = static_cast<uint32_t>(P.texts.size());
         const bool stream = progs[p]->rid.stream.kind != kStreamNone;
         if (stream && !by_prog[p].empty()) {
             sources.push_back(StreamBatchSource{&progs[p]->rid, P.dev[p], {}});
         }
-        P.n_texts_of[p] = stream ? 0 : static_cast<uint32_t>(by_prog[p].size());
+        uint64_t long_bytes = 0;                             // in texts that the set kernels take
+        if (progs[p]->rid.set.ok)
+            for (uint32_t i : by_prog[p])
+                if (items[i].len >= kSetBatchText) long_bytes += items[i].len;
+        const bool set = long_bytes >= kSetBatchBytes && set_sources.size() < kSetBatchProgs;
+        if (set) {
+            set_sources.push_back(StreamBatchSource{&progs[p]->rid, P.dev[p], {}});
+            set_bytes.push_back(long_bytes);
+            all_set_bytes += long_bytes;
+        }
         for (uint32_t i : by_prog[p]) {
             const ridfa_batch_item &it = items[i];
             TextDesc td{it.d_text, it.len, prog_chunks[p], 0, i};
@@ -676,11 +695,18 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
                 stream_bytes += it.len;
                 continue;
             }
+            if (set && it.len >= kSetBatchText) {
+                set_sources.back().items.push_back(StreamBatchItem{it.d_text, it.len, i});
+                P.total_chunks += td.c;
+                P.total_bytes += it.len;
+                continue;
+            }
             if (it.len && (reinterpret_cast<uintptr_t>(it.d_text) & 15)) aligned_all = false;
             prog_chunks[p] += td.c;
             P.total_bytes += it.len;
             P.texts.push_back(td);
         }
+        P.n_texts_of[p] = static_cast<uint32_t>(P.texts.size()) - P.text0[p];
     }
     for (uint32_t p = 0; p < np; ++p) P.total_chunks += prog_chunks[p];
     // launch groups by layout; tasks ordered by group then program
@@ -716,17 +742,30 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
         g.n_tasks = static_cast<uint32_t>(P.tasks.size()) - g.task0;
         P.groups.push_back(g);
     }
-    // The stream launches and the general groups run side by side, a block of either filling an SM: each
-    // side gets SMs by its share of the work (the general kernels take some four times the time per
+    // The stream and set launches and the general groups run side by side, a block of any filling an SM:
+    // each gets SMs by its share of the work (the general kernels take some four times the time per
     // byte), the general groups no more than they have tasks.
-    uint32_t stream_sms = static_cast<uint32_t>(sms);
-    const uint64_t other_bytes = P.total_bytes - stream_bytes;
+    const uint64_t other_bytes = P.total_bytes - stream_bytes - all_set_bytes;
+    double work = static_cast<double>(stream_bytes) + 4.0 * static_cast<double>(other_bytes);
+    for (size_t i = 0; i < set_sources.size(); ++i) work += set_batch_weight(*set_sources[i].H) * static_cast<double>(set_bytes[i]);
+    uint32_t left = static_cast<uint32_t>(sms);
+    P.set.clear();
+    for (size_t i = 0; i < set_sources.size(); ++i) {
+        const double share = set_batch_weight(*set_sources[i].H) * static_cast<double>(set_bytes[i]) / work;
+        const uint32_t most = std::max<uint32_t>(1, left - std::min<uint32_t>(left, 2));
+        const uint32_t n = std::max<uint32_t>(1, std::min<uint32_t>(most, static_cast<uint32_t>(share * sms + 0.5)));
+        P.set.emplace_back();
+        plan_set_batch(P.set.back(), set_sources[i], stream_bytes || other_bytes || set_sources.size() > 1 ? n : static_cast<uint32_t>(sms));
+        left -= std::min(left - 1, n);
+    }
+    uint32_t stream_sms = left;
     if (other_bytes && stream_bytes) {
         uint64_t tasks = 0;
         for (const LaunchGroup &g : P.groups) tasks += g.n_tasks;
         const double share = static_cast<double>(stream_bytes) / (static_cast<double>(stream_bytes) + 4.0 * static_cast<double>(other_bytes));
-        stream_sms = std::max<uint32_t>(1, std::min<uint32_t>(static_cast<uint32_t>(sms) - 1, static_cast<uint32_t>(share * sms + 0.5)));
-        stream_sms = std::max<uint32_t>(stream_sms, static_cast<uint32_t>(sms - std::min<uint64_t>(tasks, static_cast<uint64_t>(sms) - 1)));
+        const uint32_t most = std::max<uint32_t>(1, left - 1);
+        stream_sms = std::max<uint32_t>(1, std::min<uint32_t>(most, static_cast<uint32_t>(share * left + 0.5)));
+        stream_sms = std::max<uint32_t>(stream_sms, left - static_cast<uint32_t>(std::min<uint64_t>(tasks, most)));
     }
     P.stream.clear();
     for (size_t p0 = 0; p0 < sources.size(); p0 += kStreamBatchProgs) {
@@ -734,8 +773,8 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
         P.stream.emplace_back();
         plan_stream_batch(P.stream.back(), part, stream_sms);
     }
-    const bool apart = stream_bytes && !P.stream.front().walk_only;
-    const int group_sms = stream_bytes ? std::max(1, sms - static_cast<int>(stream_sms)) : sms;
+    const bool apart = !P.set.empty() || (stream_bytes && !P.stream.front().walk_only);
+    const int group_sms = static_cast<int>(stream_bytes ? std::max(1u, left - std::min(left, stream_sms)) : left);
     for (LaunchGroup &g : P.groups) {
         if (apart) g.smem = std::max(g.smem, kStreamBatchSmem);
         // persistent: as many blocks as fit on every SM, no more than there are tasks
@@ -784,6 +823,11 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
         P.o_stream.push_back(off);
         off += al256(b.image_bytes);
     }
+    P.o_set.clear();
+    for (const SetBatchPlan &b : P.set) {
+        P.o_set.push_back(off);
+        off += al256(b.image_bytes);
+    }
     P.o_part = off;     off += al256(P.segs.size() * kPartialWords * 4);
     P.o_runs = off;     off += al256(run_warps * kRunsPerWarp * sizeof(RunEntry));
     P.o_finals = off;   off += al256(run_warps * kFinalsPerWarp * 4);
@@ -793,6 +837,11 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
     for (const StreamBatchPlan &b : P.stream) {
         P.o_sres.push_back(off);
         off += al256(b.result_words * 4);
+    }
+    P.o_setres.clear();
+    for (const SetBatchPlan &b : P.set) {
+        P.o_setres.push_back(off);
+        off += al256(b.result_bytes);
     }
     P.total = off;
     return RIDFA_OK;
@@ -821,6 +870,7 @@ void plan_image(const BatchPlan *pl, uint8_t *base, uint8_t *img) {
     if (!P.segs.empty()) std::memcpy(img + P.o_segs, P.segs.data(), P.segs.size() * sizeof(SegDesc));
     for (size_t i = 0; i < P.stream.size(); ++i)
         stream_batch_image(P.stream[i], base + P.o_stream[i], reinterpret_cast<uint32_t *>(base + P.o_sres[i]), img + P.o_stream[i]);
+    for (size_t i = 0; i < P.set.size(); ++i) set_batch_image(P.set[i], img + P.o_set[i]);
 }
 
 int make_fork(LaunchFork *f) {
@@ -860,7 +910,7 @@ int plan_enqueue(const BatchPlan *pl, uint8_t *base, uint8_t *d_accept, cudaStre
     uint32_t *finals = reinterpret_cast<uint32_t *>(base + P.o_finals);
     // launches side by side: the first on `st`, every further one on a stream of its own (in turn,
     // should there be more of them than streams)
-    size_t n_side = P.groups.size();
+    size_t n_side = P.groups.size() + P.set.size();
     for (const StreamBatchPlan &b : P.stream) n_side += b.launches.size();
     const bool concurrent = fork && fork->ok && n_side > 1;
     const size_t n_aux = concurrent ? std::min<size_t>(n_side - 1, kMaxLaunchGroups - 1) : 0;
@@ -881,6 +931,10 @@ int plan_enqueue(const BatchPlan *pl, uint8_t *base, uint8_t *d_accept, cudaStre
             if (e == cudaSuccess) e = stream_batch_join(P.stream[i], L, base + P.o_stream[i], d_accept, on);
             if (e != cudaSuccess) return cuda_fail(e);
         }
+    for (size_t i = 0; i < P.set.size(); ++i) {
+        cudaError_t e = set_batch_launch(P.set[i], base + P.o_set[i], base + P.o_setres[i], d_accept, side_stream());
+        if (e != cudaSuccess) return cuda_fail(e);
+    }
     // the general groups, then their join on the first one's stream once the others are done
     cudaStream_t join_on = st;
     size_t waits = 0;

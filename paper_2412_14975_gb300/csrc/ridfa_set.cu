@@ -20,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 
 #include "ridfa_set.h"
 #include "ridfa_stream.cuh"
@@ -41,6 +42,9 @@ struct SetArgs {
     uint64_t *reps;               // [pieces]: place of each run of the graph's leaf (4 bits; 15: dead)
     uint16_t *entry;              // [pieces][kSetRuns]: states a later piece's runs begin in
     uint32_t *pids;               // [c]: the leaf's partition
+    const StreamBatchText *texts; // a batch's texts (null: one text), every piece of them a chunk
+    const uint32_t *bases;        // their first pieces
+    uint32_t n_texts;
     StreamTables t;
 };
 
@@ -167,7 +171,19 @@ __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_cons
         const bool have = pc < p.pieces;
         uint32_t ch = static_cast<uint32_t>(pc), j = 0;
         uint64_t pos = t0, end = t0;
-        if (have) {
+        if (have && p.texts) {
+            uint32_t lo = 0, hi = p.n_texts - 1;             // the last text that begins at pc or before
+            while (lo < hi) {
+                const uint32_t mid = (lo + hi + 1) / 2;
+                if (__ldg(p.bases + mid) <= ch) lo = mid;
+                else hi = mid - 1;
+            }
+            const StreamBatchText td = p.texts[lo];
+            const uint32_t t = ch - td.base;
+            const uint64_t s0 = reinterpret_cast<uint64_t>(td.text);
+            pos = t ? (s0 + (t * td.step >> 16)) & ~63ull : s0;
+            end = t + 1 < td.pieces ? (s0 + ((t + 1) * td.step >> 16)) & ~63ull : s0 + td.len;
+        } else if (have) {
             if (p.spc > 1) {
                 ch = static_cast<uint32_t>(pc / p.spc);
                 j = static_cast<uint32_t>(pc - static_cast<uint64_t>(ch) * p.spc);
@@ -382,6 +398,7 @@ struct SetJoinArgs {
     uint32_t *partials, *ticket, *status;
     uint8_t *accept, *h_accept;
     uint32_t *h_status;
+    const StreamBatchText *texts; // a batch's texts, a block each (null: one text)
 };
 
 constexpr uint32_t kSetJoinWarps = 16;
@@ -405,8 +422,9 @@ __device__ __forceinline__ uint32_t set_times(uint32_t row, uint32_t m, uint32_t
 // eight boundaries, a place of the chunk before per lane, so that a boundary costs a quarter of the
 // loads and half of the serial steps that a warp per boundary takes (46 -> 26 us at 65,536 chunks, 409
 // -> 232 us at 1,048,576; the general join took 65 and about 500 us).  Bound by latency: tables through
-// L1 and the products' shuffles.  A block takes the product of its warps', the last block that of all.
-__global__ void __launch_bounds__(32 * kSetJoinWarps) rid_set_join_kernel(const __grid_constant__ SetJoinArgs p) {
+// L1 and the products' shuffles.  A block takes the product of its warps', the last block that of all;
+// of a batch's texts each has one block.
+__global__ void __launch_bounds__(32 * kSetJoinWarps) rid_set_join_kernel(const __grid_constant__ SetJoinArgs a) {
     __shared__ __align__(16) uint16_t s_end[kSetJoinWarps][kSetTile + 1][kSetRuns];  // row 0: the chunk before
     __shared__ uint64_t s_rep[kSetJoinWarps][kSetTile];
     __shared__ uint32_t s_pid[kSetJoinWarps][kSetTile];
@@ -414,7 +432,19 @@ __global__ void __launch_bounds__(32 * kSetJoinWarps) rid_set_join_kernel(const 
     __shared__ uint32_t s_last;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, x = lane & 15, half = lane & 16;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const uint64_t i0 = (static_cast<uint64_t>(blockIdx.x) * kSetJoinWarps + warp) * p.per_warp;
+    SetJoinArgs p = a;
+    uint32_t first_block = blockIdx.x;
+    if (a.texts) {
+        const StreamBatchText td = a.texts[blockIdx.x];
+        p.c = td.pieces;
+        p.ends += static_cast<uint64_t>(td.base) * kSetRuns;
+        p.reps += td.base;
+        p.pids += td.base;
+        p.accept += td.item;
+        p.per_warp = ((td.pieces + kSetJoinWarps - 1) / kSetJoinWarps + kSetTile - 1) / kSetTile * kSetTile;
+        first_block = 0;
+    }
+    const uint64_t i0 = (static_cast<uint64_t>(first_block) * kSetJoinWarps + warp) * p.per_warp;
     const uint64_t i1 = min(static_cast<uint64_t>(p.c), i0 + p.per_warp);
     uint32_t row = 1u << x;
     uint4 e{};
@@ -484,6 +514,22 @@ __global__ void __launch_bounds__(32 * kSetJoinWarps) rid_set_join_kernel(const 
     }
     if (lane < kSetRuns) s_prod[warp][lane] = row;
     __syncthreads();
+    auto accepts = [&](uint32_t products) {                  // (one warp)
+        // the place of q0's slot in chunk 0, through all boundaries, to a final state
+        const uint32_t q0 = __ldg(p.part + static_cast<uint64_t>(__ldg(p.pids)) * p.k + p.q0_slot);
+        const uint32_t at = q0 == 0xFF ? 15u : static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned long long *>(p.reps)) >> (4 * q0)) & 15;
+        uint32_t v = at == 15 ? 0u : 1u << at;
+        for (uint32_t w = 0; w < products; ++w) v = __reduce_or_sync(kFull, (v >> x) & 1 ? s_prod[w][x] : 0u);
+        const uint32_t z = lane < kSetRuns ? __ldg(p.ends + static_cast<uint64_t>(p.c - 1) * kSetRuns + lane) : p.n;
+        const bool fin = ((v >> x) & 1) && z < p.n && ((__ldg(p.final_bits + (z >> 5)) >> (z & 31)) & 1);
+        return __any_sync(kFull, fin) ? 1u : 0u;
+    };
+    if (p.texts) {
+        if (warp) return;
+        const uint32_t acc = accepts(kSetJoinWarps);
+        if (lane == 0) *p.accept = static_cast<uint8_t>(acc);
+        return;
+    }
     if (warp == 0) {
         // the upper half its eight warps, then both
         row = 1u << x;
@@ -513,14 +559,7 @@ __global__ void __launch_bounds__(32 * kSetJoinWarps) rid_set_join_kernel(const 
     s_prod[hw][x] = row;
     __syncthreads();
     if (warp) return;
-    // the place of q0's slot in chunk 0, through all boundaries, to a final state
-    const uint32_t q0 = __ldg(p.part + static_cast<uint64_t>(__ldg(p.pids)) * p.k + p.q0_slot);
-    const uint32_t at = q0 == 0xFF ? 15u : static_cast<uint32_t>(__ldg(reinterpret_cast<const unsigned long long *>(p.reps)) >> (4 * q0)) & 15;
-    uint32_t v = at == 15 ? 0u : 1u << at;
-    for (uint32_t w = 0; w < 2 * kSetJoinWarps; ++w) v = __reduce_or_sync(kFull, (v >> x) & 1 ? s_prod[w][x] : 0u);
-    const uint32_t z = lane < kSetRuns ? __ldg(p.ends + static_cast<uint64_t>(p.c - 1) * kSetRuns + lane) : p.n;
-    const bool fin = ((v >> x) & 1) && z < p.n && ((__ldg(p.final_bits + (z >> 5)) >> (z & 31)) & 1);
-    const uint32_t acc = __any_sync(kFull, fin) ? 1 : 0;
+    const uint32_t acc = accepts(2 * kSetJoinWarps);
     if (lane == 0) {
         *p.accept = static_cast<uint8_t>(acc);
         *p.status = 0;
@@ -541,6 +580,48 @@ uint32_t set_join_blocks(uint32_t c) {
     return static_cast<uint32_t>((c + per - 1) / per);
 }
 
+}  // namespace
+
+namespace {
+// The parts of the kernels' arguments that depend on the automaton alone; returns the shared memory.
+size_t set_args(const HostAutomaton &H, const DeviceAutomaton &D, SetArgs &a, SetJoinArgs &j) {
+    const HostStream &T = H.set.table;
+    a.depth = H.set.depth;
+    a.back_depth = H.set.back_depth;
+    a.next = D.set_next;
+    a.images = D.set_images;
+    a.back_next = D.set_back_next;
+    a.back_images = D.set_back_images;
+    a.leaf = D.set_leaf;
+    a.t = stream_field_tables(T);
+    a.t.walk = D.trans;
+    a.t.classmap = D.classmap;
+    a.t.words = D.set_words;
+    a.t.n = H.n_states;
+    a.t.C = H.n_classes;
+    a.t.n_walk = static_cast<uint32_t>(H.trans.size() + 1) & ~1u;      // (whole words; the upload is padded)
+    const uint32_t off = a.t.n_words * 4 * T.copies;
+    a.t.off_table = 0;
+    a.t.off_cls = (off + 15) & ~15u;
+    a.t.off_walk = a.t.off_cls + 256;
+    j.k = H.k;
+    j.kw = H.kw;
+    j.n = H.n_states;
+    j.q0_slot = H.q0_slot;
+    j.block_mask = D.set_block_mask;
+    j.ifmask = D.ifmask;
+    j.final_bits = D.final_bits;
+    j.part = D.set_part;
+    return set_rest_bytes(H) + static_cast<size_t>(off);
+}
+
+cudaError_t set_reach(const HostAutomaton &H, const SetArgs &a, uint32_t grid, size_t smem, cudaStream_t st) {
+    auto kern = H.set.table.group == 4 ? rid_set_kernel<4> : rid_set_kernel<2>;
+    cudaError_t e = ensure_smem_cap(reinterpret_cast<const void *>(kern), smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, kSetBlock, smem, st>>>(a);       // (all warps load the table)
+    return cudaGetLastError();
+}
 }  // namespace
 
 uint32_t set_pieces(const HostAutomaton &H, uint64_t len, uint32_t c, int sms) {
@@ -564,7 +645,6 @@ size_t set_scratch(uint32_t c, uint32_t spc) {
 cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     const HostAutomaton &H = *C.H;
     const DeviceAutomaton &D = *C.D;
-    const HostStream &T = H.set.table;
     const uint64_t pieces = static_cast<uint64_t>(C.c) * C.spc;
     uint8_t *next = C.scratch;
     auto take = [&](size_t bytes) {
@@ -585,36 +665,13 @@ cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     a.c = C.c;
     a.spc = C.spc;
     a.pieces = pieces;
-    a.depth = H.set.depth;
-    a.back_depth = H.set.back_depth;
-    a.next = D.set_next;
-    a.images = D.set_images;
-    a.back_next = D.set_back_next;
-    a.back_images = D.set_back_images;
-    a.leaf = D.set_leaf;
     a.ends = u16(pieces);
     a.reps = u64(pieces);
     a.entry = C.spc > 1 ? u16(pieces) : nullptr;
     a.pids = pids;
-    a.t = stream_field_tables(T);
-    a.t.walk = D.trans;
-    a.t.classmap = D.classmap;
-    a.t.words = D.set_words;
-    a.t.n = H.n_states;
-    a.t.C = H.n_classes;
-    a.t.n_walk = static_cast<uint32_t>(H.trans.size() + 1) & ~1u;      // (whole words; the upload is padded)
-    uint32_t off = a.t.n_words * 4 * T.copies;
-    a.t.off_table = 0;
-    a.t.off_cls = (off + 15) & ~15u;
-    a.t.off_walk = a.t.off_cls + 256;
-    const size_t smem = set_rest_bytes(H) + static_cast<size_t>(off);
-    const uint64_t tasks = (pieces + 31) / 32;
-    const uint32_t grid = static_cast<uint32_t>(std::min<uint64_t>(sms, tasks));
-    auto kern = T.group == 4 ? rid_set_kernel<4> : rid_set_kernel<2>;
-    cudaError_t e = ensure_smem_cap(reinterpret_cast<const void *>(kern), smem);
-    if (e != cudaSuccess) return e;
-    kern<<<grid, kSetBlock, smem, st>>>(a);       // (all warps load the table)
-    e = cudaGetLastError();
+    SetJoinArgs j{};
+    const size_t smem = set_args(H, D, a, j);
+    cudaError_t e = set_reach(H, a, static_cast<uint32_t>(std::min<uint64_t>(sms, (pieces + 31) / 32)), smem, st);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -648,20 +705,11 @@ cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
         e = cudaEventRecord(C.between, st);
         if (e != cudaSuccess) return e;
     }
-    SetJoinArgs j{};
     j.c = C.c;
-    j.k = H.k;
-    j.kw = H.kw;
-    j.n = H.n_states;
-    j.q0_slot = H.q0_slot;
     j.per_warp = join_per_warp(C.c);
     j.ends = m.ends;
     j.reps = m.reps;
     j.pids = pids;
-    j.block_mask = D.set_block_mask;
-    j.ifmask = D.ifmask;
-    j.final_bits = D.final_bits;
-    j.part = D.set_part;
     j.maps = C.maps;
     j.partials = partials;
     j.ticket = C.ticket;
@@ -673,6 +721,60 @@ cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     cfg.blockDim = dim3(32 * kSetJoinWarps);
     cfg.numAttrs = C.between ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, rid_set_join_kernel, j);
+}
+
+// (measured on the batch of 2,000 texts against 16 REs: 4 bytes a clock of an SM, a two-byte stream
+// table 10 to 12)
+double set_batch_weight(const HostAutomaton &H) { return H.set.table.group == 4 ? 2.5 : 4.0; }
+
+void plan_set_batch(SetBatchPlan &P, const StreamBatchSource &src, uint32_t sms) {
+    P = SetBatchPlan{};
+    P.H = src.H;
+    P.D = src.D;
+    uint64_t bytes = 0;
+    for (const auto &it : src.items) bytes += it.len;
+    // one round of pieces for the SMs' lanes, none longer than the others
+    const uint64_t piece = std::max<uint64_t>(1024, bytes / (static_cast<uint64_t>(sms) * kSetBlock) + 1);
+    for (const auto &it : src.items) {
+        StreamBatchText t{it.text, it.len, 0, P.pieces, 0, 0, it.item};
+        t.pieces = static_cast<uint32_t>((it.len + piece - 1) / piece);
+        t.step = static_cast<uint64_t>((static_cast<unsigned __int128>(it.len) << 16) / t.pieces);
+        P.pieces += t.pieces;
+        P.texts.push_back(t);
+        P.bases.push_back(t.base);
+    }
+    P.grid = std::min<uint32_t>(sms, (P.pieces + 31) / 32);
+    P.o_bases = (P.texts.size() * sizeof(StreamBatchText) + 255) & ~static_cast<size_t>(255);
+    P.image_bytes = P.o_bases + P.bases.size() * 4;
+    P.result_bytes = static_cast<size_t>(P.pieces) * (kSetRuns * 2 + 8 + 4);
+}
+
+void set_batch_image(const SetBatchPlan &P, uint8_t *img) {
+    std::memcpy(img, P.texts.data(), P.texts.size() * sizeof(StreamBatchText));
+    std::memcpy(img + P.o_bases, P.bases.data(), P.bases.size() * 4);
+}
+
+cudaError_t set_batch_launch(const SetBatchPlan &P, const uint8_t *dev, uint8_t *res, uint8_t *d_accept, cudaStream_t st) {
+    SetArgs a{};
+    SetJoinArgs j{};
+    const size_t smem = set_args(*P.H, *P.D, a, j);
+    a.texts = reinterpret_cast<const StreamBatchText *>(dev);
+    a.bases = reinterpret_cast<const uint32_t *>(dev + P.o_bases);
+    a.n_texts = static_cast<uint32_t>(P.texts.size());
+    a.spc = 1;
+    a.pieces = P.pieces;
+    a.ends = reinterpret_cast<uint16_t *>(res);
+    a.reps = reinterpret_cast<uint64_t *>(res + static_cast<size_t>(P.pieces) * kSetRuns * 2);
+    a.pids = reinterpret_cast<uint32_t *>(a.reps + P.pieces);
+    cudaError_t e = set_reach(*P.H, a, P.grid, smem, st);
+    if (e != cudaSuccess) return e;
+    j.texts = a.texts;
+    j.ends = a.ends;
+    j.reps = a.reps;
+    j.pids = a.pids;
+    j.accept = d_accept;
+    rid_set_join_kernel<<<a.n_texts, 32 * kSetJoinWarps, 0, st>>>(j);
+    return cudaGetLastError();
 }
 
 }  // namespace ridfa

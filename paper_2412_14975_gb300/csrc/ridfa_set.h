@@ -4,7 +4,10 @@
 
 #include <cuda_runtime_api.h>
 
+#include <vector>
+
 #include "ridfa_internal.h"
+#include "ridfa_stream_batch.h"
 
 namespace ridfa {
 
@@ -27,5 +30,25 @@ struct SetCall {
 uint32_t set_pieces(const HostAutomaton &H, uint64_t len, uint32_t c, int sms);
 size_t set_scratch(uint32_t c, uint32_t spc);
 cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st);
+
+// The texts of one program of a batch, each of kSetBatchText bytes or more, on `grid` SMs: only accept
+// bits are asked for, so a piece is entered through the interface slots, as a chunk is.
+constexpr uint64_t kSetBatchText = 128;
+// What a batch's launch has to have: a table takes 10 us to set up, and shorter pieces than 1 KB are
+// mostly first bytes.
+constexpr uint64_t kSetBatchBytes = 1 << 20;
+constexpr uint32_t kSetBatchProgs = 16;
+struct SetBatchPlan {
+    const HostAutomaton *H = nullptr;
+    const DeviceAutomaton *D = nullptr;
+    std::vector<StreamBatchText> texts;
+    std::vector<uint32_t> bases;
+    uint32_t pieces = 0, grid = 0;
+    size_t image_bytes = 0, result_bytes = 0, o_bases = 0;
+};
+double set_batch_weight(const HostAutomaton &H);         // time per byte, a two-byte stream table's being 1
+void plan_set_batch(SetBatchPlan &P, const StreamBatchSource &src, uint32_t sms);
+void set_batch_image(const SetBatchPlan &P, uint8_t *img);
+cudaError_t set_batch_launch(const SetBatchPlan &P, const uint8_t *dev_image, uint8_t *dev_results, uint8_t *d_accept, cudaStream_t st);
 
 }  // namespace ridfa
