@@ -559,6 +559,9 @@ int log2i(uint32_t v) {
 
 }  // namespace
 
+// Time per byte of the general batch kernels, a two-byte stream table's being 1.
+constexpr double kGeneralWeight = 2.3;
+
 struct BatchPlan {
     std::vector<const ridfa_program *> progs;
     std::vector<const DeviceAutomaton *> dev;
@@ -746,7 +749,7 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
     // each gets SMs by its share of the work (the general kernels take some four times the time per
     // byte), the general groups no more than they have tasks.
     const uint64_t other_bytes = P.total_bytes - stream_bytes - all_set_bytes;
-    double work = static_cast<double>(stream_bytes) + 4.0 * static_cast<double>(other_bytes);
+    double work = static_cast<double>(stream_bytes) + kGeneralWeight * static_cast<double>(other_bytes);
     for (size_t i = 0; i < set_sources.size(); ++i) work += set_batch_weight(*set_sources[i].H) * static_cast<double>(set_bytes[i]);
     uint32_t left = static_cast<uint32_t>(sms);
     P.set.clear();
@@ -762,10 +765,20 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
     if (other_bytes && stream_bytes) {
         uint64_t tasks = 0;
         for (const LaunchGroup &g : P.groups) tasks += g.n_tasks;
-        const double share = static_cast<double>(stream_bytes) / (static_cast<double>(stream_bytes) + 4.0 * static_cast<double>(other_bytes));
+        // A task is a block's for long, so the groups' SMs are those of whole rounds of tasks (36 tasks
+        // took 248 us on 36 SMs, 474 us on 25), with the number of rounds that ends both sides earliest.
+        const double task = kGeneralWeight * static_cast<double>(other_bytes) / static_cast<double>(std::max<uint64_t>(1, tasks));
         const uint32_t most = std::max<uint32_t>(1, left - 1);
-        stream_sms = std::max<uint32_t>(1, std::min<uint32_t>(most, static_cast<uint32_t>(share * left + 0.5)));
-        stream_sms = std::max<uint32_t>(stream_sms, left - static_cast<uint32_t>(std::min<uint64_t>(tasks, most)));
+        double best = 0;
+        for (uint32_t r = 1; r <= 64; ++r) {
+            const uint32_t n = static_cast<uint32_t>(std::min<uint64_t>(std::max<uint64_t>(1, (tasks + r - 1) / r), most));
+            const double rounds = std::ceil(static_cast<double>(tasks) / n);
+            const double t = std::max(rounds * task, static_cast<double>(stream_bytes) / std::max(1u, left - n));
+            if (r == 1 || t < best) {
+                best = t;
+                stream_sms = std::max(1u, left - n);
+            }
+        }
     }
     P.stream.clear();
     for (size_t p0 = 0; p0 < sources.size(); p0 += kStreamBatchProgs) {

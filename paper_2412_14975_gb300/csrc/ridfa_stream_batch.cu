@@ -6,7 +6,7 @@
 // program's tables when its share comes to that program.  The launches of the forms run side by side,
 // each on its share of the SMs.  (One kernel for all forms spilled 1.7 KB a thread.)  (The general batch kernel hands out tasks of up to 16 MB by
 // tickets, which left half of the SMs idle on batches of a GB over 16 programs.)  A text is accepted
-// iff the join of its pieces' functions is: a warp per text tests every boundary, as the single-text
+// iff the join of its pieces' functions is: a block per text tests every boundary, as the single-text
 // join does.
 #include <cuda_runtime.h>
 
@@ -137,35 +137,30 @@ __device__ __forceinline__ uint32_t piece_to(const StreamBatchProg &P, uint32_t 
     return __ldg(P.part + static_cast<uint64_t>(f >> 16) * n + x) == kNoBlock ? n : f & 0xFFFF;
 }
 
-// Accept bits, a warp per text.  While every piece merged, piece i is entered iff if_min of piece
-// i - 1's end state meets the slots alive in piece i.  With a piece that did not, the run from q0's
-// start state is followed piece by piece instead (repeats of one function on its fixed point at
-// once).
-__global__ void __launch_bounds__(256) rid_stream_batch_join_kernel(const StreamBatchProg *progs, const StreamBatchText *texts,
-                                                                    uint32_t n_texts, uint8_t *accept) {
+// Accept bits, a block per text, a piece per thread (a warp per text took 25 us on texts of up to 2,000
+// pieces, one after another).  While every piece merged, piece i is entered iff if_min of piece i - 1's
+// end state meets the slots alive in piece i.  With a piece that did not, the run from q0's start state
+// is followed piece by piece instead (repeats of one function on its fixed point at once).
+constexpr int kBatchJoinBlock = 128;
+__global__ void __launch_bounds__(kBatchJoinBlock) rid_stream_batch_join_kernel(const StreamBatchProg *progs, const StreamBatchText *texts,
+                                                                               uint8_t *accept) {
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t ti = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (ti >= n_texts) return;
-    const StreamBatchText td = texts[ti];
+    const StreamBatchText td = texts[blockIdx.x];
     const StreamBatchProg &P = progs[td.prog];
     const uint32_t n = P.n;
     const uint32_t start = __ldg(P.slot_state + P.q0_slot);
     auto final_state = [&](uint32_t s) { return s < n && ((__ldg(P.final_bits + (s >> 5)) >> (s & 31)) & 1); };
     if (td.pieces == 0) {                        // empty text: is the empty word in L?
-        if (lane == 0) accept[td.item] = final_state(start) ? 1 : 0;
+        if (threadIdx.x == 0) accept[td.item] = final_state(start) ? 1 : 0;
         return;
     }
     const uint32_t *r = P.res + td.base;
     bool node = false, ok = true;
-    uint32_t carry = 0;
-    for (uint32_t b = 0; b < td.pieces; b += 32) {
-        const uint32_t t = b + lane;
-        const uint32_t f = t < td.pieces ? __ldg(r + t) : 0;
-        uint32_t y = __shfl_up_sync(kFull, f, 1);
-        if (lane == 0) y = carry;
-        carry = __shfl_sync(kFull, f, 31);
-        node = node || (t < td.pieces && (f & kNodeResult));
-        if (t < td.pieces && !((f | y) & kNodeResult)) {
+#pragma unroll 2
+    for (uint32_t t = threadIdx.x; t < td.pieces; t += kBatchJoinBlock) {
+        const uint32_t f = __ldg(r + t), y = t ? __ldg(r + t - 1) : 0;
+        node = node || (f & kNodeResult);
+        if (!((f | y) & kNodeResult)) {
             const uint32_t *alive = P.slot_alive + (f >> 16) * P.kw;
             uint32_t hit = 0;
             if (t == 0) hit = (__ldg(alive + (P.q0_slot >> 5)) >> (P.q0_slot & 31)) & 1;
@@ -174,11 +169,12 @@ __global__ void __launch_bounds__(256) rid_stream_batch_join_kernel(const Stream
             ok = ok && hit && (f & 0xFFFF) < n;
         }
     }
-    if (!__any_sync(kFull, node)) {
-        ok = __all_sync(kFull, ok);
-        if (lane == 0) accept[td.item] = ok && final_state(__ldg(r + td.pieces - 1) & 0xFFFF) ? 1 : 0;
+    if (!__syncthreads_or(node)) {
+        const int all = __syncthreads_and(ok);
+        if (threadIdx.x == 0) accept[td.item] = all && final_state(__ldg(r + td.pieces - 1) & 0xFFFF) ? 1 : 0;
         return;
     }
+    if (threadIdx.x >= 32) return;
     uint32_t x = start;
     for (uint32_t b = 0; b < td.pieces && x < n; b += 32) {
         const uint32_t f = b + lane < td.pieces ? __ldg(r + b + lane) : 0;
@@ -204,7 +200,7 @@ inline uint32_t batch_warps(const HostStream &T) { return std::min<uint32_t>(T.w
 // clock for the two-byte table, 8.6 for the one-byte one, 10.7 for field codes, whose single-text
 // kernel HBM holds back before an SM does).
 inline double time_of(const HostStream &T) {
-    return T.kind == kStreamPair ? 0.78 * T.cost : T.kind == kStreamField ? std::max(2.0f, T.cost) : T.entry == 2 ? 0.86 * T.cost : T.cost;
+    return T.kind == kStreamPair ? 0.78 * T.cost : T.kind == kStreamField ? std::max(2.0f, T.cost) : T.entry == 2 ? 0.86 * T.cost : 1.2 * T.cost;
 }
 
 using BatchKernel = void (*)(BatchTables, const StreamBatchProg *, const StreamBatchPart *, const uint32_t *);
@@ -396,9 +392,9 @@ cudaError_t stream_batch_reach(const StreamBatchPlan &P, const StreamBatchLaunch
 }
 
 cudaError_t stream_batch_join(const StreamBatchPlan &P, const StreamBatchLaunch &L, const uint8_t *dev, uint8_t *d_accept, cudaStream_t st) {
-    rid_stream_batch_join_kernel<<<(L.n_texts + 7) / 8, 256, 0, st>>>(reinterpret_cast<const StreamBatchProg *>(dev + P.o_progs),
-                                                                     reinterpret_cast<const StreamBatchText *>(dev + P.o_texts) + L.text0,
-                                                                     L.n_texts, d_accept);
+    rid_stream_batch_join_kernel<<<L.n_texts, kBatchJoinBlock, 0, st>>>(reinterpret_cast<const StreamBatchProg *>(dev + P.o_progs),
+                                                                       reinterpret_cast<const StreamBatchText *>(dev + P.o_texts) + L.text0,
+                                                                       d_accept);
     return cudaGetLastError();
 }
 
