@@ -734,7 +734,7 @@ void plan_set_batch(SetBatchPlan &P, const StreamBatchSource &src, uint32_t sms)
     uint64_t bytes = 0;
     for (const auto &it : src.items) bytes += it.len;
     // one round of pieces for the SMs' lanes, none longer than the others
-    const uint64_t piece = std::max<uint64_t>(1024, bytes / (static_cast<uint64_t>(sms) * kSetBlock) + 1);
+    const uint64_t piece = std::max<uint64_t>(512, bytes / (static_cast<uint64_t>(sms) * kSetBlock) + 1);
     for (const auto &it : src.items) {
         StreamBatchText t{it.text, it.len, 0, P.pieces, 0, 0, it.item};
         t.pieces = static_cast<uint32_t>((it.len + piece - 1) / piece);
