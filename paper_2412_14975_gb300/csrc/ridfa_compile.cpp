@@ -800,6 +800,7 @@ extern "C" int ridfa_compile(const char *re, size_t re_len, const ridfa_compile_
         build_rid(N, cap, o.minimize_interface != 0, *P);
         P->has_dfa = o.build_dfa ? build_min_dfa(N, cap, *P) : false;
         if (tables_in_bounds(P->rid)) ridfa::build_stream(P->rid);
+        if (P->has_dfa && tables_in_bounds(P->dfa)) ridfa::build_stream(P->dfa);
     } catch (const SyntaxError &) {
         delete P;
         return RIDFA_E_SYNTAX;

@@ -137,15 +137,6 @@ const DeviceAutomaton *device_copy(const ridfa_program *P, bool dfa, int dev, in
     auto &vec = dfa ? P->dev_dfa : P->dev_rid;
     for (auto &d : vec)
         if (d.device == dev) return &d;
-    if (dfa && !P->dfa_stream) {
-        try {
-            build_stream(P->dfa);
-        } catch (const std::bad_alloc &) {
-            *err = RIDFA_E_NOMEM;
-            return nullptr;
-        }
-        P->dfa_stream = true;
-    }
     DeviceAutomaton D;
     *err = upload(dfa ? P->dfa : P->rid, D, dev);
     if (*err != RIDFA_OK) return nullptr;

@@ -192,8 +192,7 @@ struct ridfa_program {
     std::vector<uint32_t> slots;                      // representative NFA state per slot
     std::vector<uint32_t> delegate_slot;              // NFA state -> slot of its representative
     ridfa::HostAutomaton rid;
-    mutable ridfa::HostAutomaton dfa;                 // (its stream tables are built on its first upload:
-    mutable bool dfa_stream = false;                  // few programs run it on the GPU)
+    ridfa::HostAutomaton dfa;
     bool has_dfa = false;
     ridfa::HostNfa nfa;                               // the NFA variant's tables (n <= 128)
     // device side (filled lazily by the device code)
