@@ -1015,6 +1015,9 @@ int recognize_stream(const ridfa_program *P, const HostAutomaton &H, const Devic
     const size_t o_part = off;     off += al(static_cast<size_t>(sh.join_blocks) * kPartialWords * 4);
     const size_t o_sum = off;      off += al(sizeof(ridfa_shard_summary));
     const size_t o_maps = off;     off += d_maps_user ? 0 : al(static_cast<size_t>(n_chunks) * H.k * 2);
+    const size_t groups = static_cast<size_t>(n_chunks) * sh.groups;
+    const size_t o_groups = off;   off += al(groups * 4);
+    const size_t o_tables = off;   off += al(groups * H.n_states * 2);
     int err = RIDFA_OK;
     DeviceScratch *S = scratch_for(P, dev, off, &err);
     if (!S) return err;
@@ -1026,6 +1029,8 @@ int recognize_stream(const ridfa_program *P, const HostAutomaton &H, const Devic
     C.len = len;
     C.c = n_chunks;
     C.res = reinterpret_cast<uint32_t *>(base + o_res);
+    C.groups = reinterpret_cast<uint32_t *>(base + o_groups);
+    C.tables = reinterpret_cast<uint16_t *>(base + o_tables);
     C.maps = d_maps_user ? d_maps_user : reinterpret_cast<uint16_t *>(base + o_maps);
     C.dinfo = reinterpret_cast<uint32_t *>(base + o_dinfo);
     C.partials = reinterpret_cast<uint32_t *>(base + o_part);

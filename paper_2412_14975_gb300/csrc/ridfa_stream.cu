@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "ridfa_join.cuh"
 #include "ridfa_stream.cuh"
@@ -84,7 +85,8 @@ struct StreamJoinArgs {
     const uint32_t *res;
     const uint16_t *part, *node_part, *images;
     const uint32_t *node_img, *slot_alive;
-    uint32_t per_chunk;      // pieces per chunk
+    const uint16_t *tables;  // of the groups that did not merge (kTableResult)
+    uint32_t per_chunk;      // pieces (or groups of them) per chunk
     uint32_t chunks;         // chunks per block
     uint32_t k_magic;        // ceil(2^32 / k): e / k = umulhi(e, k_magic) for e < 2^16
     uint32_t *work;          // status bits of this call while it runs
@@ -93,6 +95,8 @@ struct StreamJoinArgs {
 };
 
 constexpr uint32_t kGeneral = 0xFFFFFFFFu;   // a chunk with a piece that never merged
+constexpr uint32_t kTableResult = 0xC0000000u;   // | g: group g's function is row g of the tables (a node
+                                                 // id is below 2^15)
 constexpr uint32_t kBatch = 256;             // chunks a join block handles at a time
 
 // The state that a piece's function takes x to (the dead state n: none).
@@ -100,11 +104,44 @@ __device__ __forceinline__ uint32_t apply_piece(const StreamJoinArgs &p, uint32_
     const uint32_t n = p.j.A.n;
     if (x >= n) return n;
     if (f & kNodeResult) {
+        if (f >= kTableResult) return __ldcg(p.tables + static_cast<uint64_t>(f & ~kTableResult) * n + x);
         const uint32_t u = f & ~kNodeResult;
         const uint16_t b = __ldg(p.part + static_cast<uint64_t>(__ldg(p.node_part + u)) * n + x);
         return b == kNoBlock ? n : __ldg(p.images + __ldg(p.node_img + u) + b);
     }
     return __ldg(p.part + static_cast<uint64_t>(f >> 16) * n + x) == kNoBlock ? n : f & 0xFFFF;
+}
+
+// x through the functions r[0, s), eight words and their tables' places ahead of the states (one after
+// another a piece took 0.55 us).
+__device__ __forceinline__ uint32_t apply_pieces(const StreamJoinArgs &p, const uint32_t *r, uint32_t s, uint32_t x) {
+    const uint32_t n = p.j.A.n;
+    if (s < 4) {
+        for (uint32_t t = 0; t < s && x < n; ++t) x = apply_piece(p, __ldcg(r + t), x);
+        return x;
+    }
+    for (uint32_t t0 = 0; t0 < s && x < n; t0 += 8) {
+        uint32_t f[8], row[8], img[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = t0 + u < s ? __ldcg(r + t0 + u) : 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool node = (f[u] & kNodeResult) && f[u] < kTableResult;
+            row[u] = node ? __ldg(p.node_part + (f[u] & ~kNodeResult)) : f[u] >> 16;
+            img[u] = node ? __ldg(p.node_img + (f[u] & ~kNodeResult)) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (t0 + u >= s || x >= n) continue;
+            if (f[u] >= kTableResult) {
+                x = apply_piece(p, f[u], x);
+            } else {
+                const uint16_t b = __ldg(p.part + static_cast<uint64_t>(row[u]) * n + x);
+                x = b == kNoBlock ? n : f[u] & kNodeResult ? __ldg(p.images + img[u] + b) : f[u] & 0xFFFF;
+            }
+        }
+    }
+    return x;
 }
 
 // Chunk i's function as one word where all of its pieces merged: pid of the first piece and the last
@@ -136,9 +173,8 @@ __device__ __forceinline__ uint32_t chunk_word(const StreamJoinArgs &p, uint64_t
     return ok && (last & 0xFFFF) != p.j.A.n ? (f[0] & 0xFFFF0000u) | (last & 0xFFFF) : p.j.A.n;
 }
 
-// A warp: a piece per lane, up to eight at a time so that their loads overlap.
-__device__ __forceinline__ uint32_t chunk_word_warp(const StreamJoinArgs &p, uint64_t i, uint32_t lane) {
-    const uint32_t s = p.per_chunk, *r = p.res + i * s;
+// The s pieces at r by a warp: a piece per lane, up to eight at a time so that their loads overlap.
+__device__ __forceinline__ uint32_t chunk_word_warp(const StreamJoinArgs &p, const uint32_t *r, uint32_t s, uint32_t lane) {
     uint32_t first = 0, carry = 0;
     bool node = false, ok = true;
     for (uint32_t b = 0; b < s; b += 256) {
@@ -178,8 +214,7 @@ __device__ void general_row(const StreamJoinArgs &p, uint64_t i, uint32_t lane) 
         const uint32_t a = r * 32 + lane;
         v[r] = kUndef;
         if (a < A.k) {
-            uint32_t x = A.slot_state[a];
-            for (uint32_t t = 0; t < p.per_chunk && x < A.n; ++t) x = apply_piece(p, __ldcg(p.res + i * p.per_chunk + t), x);
+            const uint32_t x = apply_pieces(p, p.res + i * p.per_chunk, p.per_chunk, A.slot_state[a]);
             if (x < A.n) v[r] = x;
             p.maps[i * A.k + a] = static_cast<uint16_t>(v[r]);
         }
@@ -239,8 +274,7 @@ __device__ uint32_t accept_unmerged(const StreamJoinArgs &p, uint32_t *s_vec, ui
         __syncthreads();
         for (uint32_t a = threadIdx.x; a < A.k; a += blockDim.x) {
             if (!((s_vec[a >> 5] >> (a & 31)) & 1)) continue;
-            uint32_t x = A.slot_state[a];
-            for (uint32_t t = 0; t < p.per_chunk && x < A.n; ++t) x = apply_piece(p, __ldcg(p.res + i * p.per_chunk + t), x);
+            const uint32_t x = apply_pieces(p, p.res + i * p.per_chunk, p.per_chunk, A.slot_state[a]);
             if (x >= A.n) continue;
             if (i + 1 == p.j.c) {
                 if (is_final(A, x)) s_acc = 1;
@@ -281,7 +315,7 @@ __device__ void stream_join(const StreamJoinArgs &p, uint32_t blk, uint32_t nblk
         }
     } else {
         for (uint32_t j = warp; j < cnt + before; j += blockDim.x / 32) {
-            const uint32_t v = chunk_word_warp(p, i0 - before + j, lane);
+            const uint32_t v = chunk_word_warp(p, p.res + (i0 - before + j) * p.per_chunk, p.per_chunk, lane);
             if (lane == 0) {
                 sh.info[j] = v;
                 if (v == kGeneral) sh.general = 1;
@@ -488,8 +522,7 @@ __device__ void stream_join(const StreamJoinArgs &p, uint32_t blk, uint32_t nblk
         return;
     }
     // (chunk 0's row may still be on its way: its entry for q0's slot from the pieces instead)
-    uint32_t x = A.slot_state[A.q0_slot];
-    for (uint32_t t = 0; t < p.per_chunk; ++t) x = apply_piece(p, __ldcg(p.res + t), x);
+    const uint32_t x = apply_pieces(p, p.res, p.per_chunk, A.slot_state[A.q0_slot]);
     const uint16_t v0 = x < A.n ? static_cast<uint16_t>(x) : kUndef;
     uint8_t acc = 0;
     if (v0 != kUndef) {
@@ -515,6 +548,42 @@ __global__ void __launch_bounds__(kJoinThreads) rid_stream_join_kernel(const __g
     __shared__ JoinShared sh;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     stream_join(p, blockIdx.x, gridDim.x, sh);
+}
+
+// Where a chunk has very many pieces: groups of consecutive ones as one word each, a warp per group.  A group with a piece that did not merge becomes a row of tables, on the states that the piece
+// before it (or, for a chunk's first group, the slots) can end in.  Bound by latency.  (64 MiB in one
+// chunk: one warp of the join over its 77,824 pieces 292 us in all, and 42.6 ms where runs stay apart.)
+struct StreamGroupArgs {
+    StreamJoinArgs j;
+    uint64_t groups;
+    uint32_t per_chunk, size;                // groups per chunk, pieces per group
+    uint32_t inner, n_images;                // nodes of the graph and their images
+    uint32_t *out;                           // [groups]
+    uint16_t *tables;                        // [groups][n]
+};
+
+__global__ void __launch_bounds__(kJoinThreads) rid_stream_group_kernel(const __grid_constant__ StreamGroupArgs p) {
+    const Automaton &A = p.j.j.A;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t g = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (g >= p.groups) return;
+    const uint64_t i = g / p.per_chunk;
+    const uint32_t first = static_cast<uint32_t>(g - i * p.per_chunk) * p.size, s = min(p.size, p.j.per_chunk - first);
+    const uint32_t *r = p.j.res + i * p.j.per_chunk + first;
+    uint32_t word = chunk_word_warp(p.j, r, s, lane);
+    if (word == kGeneral) {
+        word = kTableResult | static_cast<uint32_t>(g);
+        const uint32_t f = first ? __ldcg(r - 1) : 0, u = f & ~kNodeResult;
+        const bool slots = first == 0, node = !slots && (f & kNodeResult);
+        const uint32_t at = node ? __ldg(p.j.node_img + u) : 0;
+        const uint32_t d = slots ? A.k : node ? (u + 1 < p.inner ? __ldg(p.j.node_img + u + 1) : p.n_images) - at : 1;
+        for (uint32_t b = lane; b < d; b += 32) {
+            const uint32_t x = slots ? A.slot_state[b] : node ? __ldg(p.j.images + at + b) : f & 0xFFFF;
+            if (x < A.n) p.tables[g * A.n + x] = static_cast<uint16_t>(apply_pieces(p.j, r, s, x));
+        }
+    }
+    if (lane == 0) p.out[g] = word;
 }
 
 // Short pieces: one-byte steps throughout, so a block has only the walk table to set up.  With
@@ -571,9 +640,16 @@ StreamKernel stream_kernel(const HostStream &T) {
     }
 }
 
+// Chunks of more pieces are joined by groups of about the square root of their number (a launch more, 3
+// us).  Merged pieces: a warp tests some 4,096 in 10 us.  Where runs stay apart every slot's run goes
+// through the pieces one by one, 0.35 us each (1 MiB in 64 chunks of 256 pieces: 168 us without groups).
+constexpr uint32_t kGroupFrom = 4096, kGroupApart = 32;
 constexpr uint64_t kMinPiece = 64;             // bytes a piece has at least, where chunks are cut
-// pieces up to this length (and texts up to kWalkText) take one-byte steps throughout
-constexpr uint64_t kWalkPiece = 192, kWalkText = 8u << 20;
+// Pieces up to this length (and texts up to kWalkText) take one-byte steps throughout: a block then
+// has only the walk table to set up, and pieces of 64 bytes are the shortest chains.  Measured with
+// pieces of 64 / 96 to 192 bytes: 1 MiB in 64 chunks 30.4 / 32.6 us.  With the walk kernel / the table
+// kernels: 256 KiB 29.0 / 33.3 us, 1 MiB of record lines 33.2 / 35.4, 8 MiB in 64 chunks 47.8 / 41.0.
+constexpr uint64_t kWalkPiece = 96, kWalkText = 2u << 20;
 
 }  // namespace
 
@@ -618,6 +694,10 @@ StreamShape stream_shape(const HostAutomaton &H, uint64_t len, uint32_t c, int s
     S.pieces = static_cast<uint64_t>(c) * best;
     S.walk_only = len <= kWalkText && len / S.pieces <= kWalkPiece;
     const uint64_t tasks = (S.pieces + 31) / 32;
+    if (S.per_chunk > (H.merges ? kGroupFrom : kGroupApart)) {
+        S.group = std::min<uint32_t>(256, std::max<uint32_t>(8, static_cast<uint32_t>(std::sqrt(static_cast<double>(S.per_chunk)))));
+        S.groups = (S.per_chunk + S.group - 1) / S.group;
+    }
     // a join block takes 256 chunks, one thread each; where chunks have many pieces, a warp each
     S.join_chunks = S.per_chunk <= 4 ? kBatch : std::min<uint32_t>(kBatch, std::max<uint32_t>(kJoinThreads / 32, (c + 1023) / 1024));
     if (S.walk_only) {
@@ -626,7 +706,7 @@ StreamShape stream_shape(const HostAutomaton &H, uint64_t len, uint32_t c, int s
         S.warps = static_cast<uint32_t>(std::min<uint64_t>(kJoinThreads / 32, (tasks + sms - 1) / sms));
         S.grid = static_cast<uint32_t>(std::min<uint64_t>(static_cast<uint64_t>(sms) * 4, (tasks + S.warps - 1) / S.warps));
         S.smem = stream_walk_bytes(H);
-        S.fused = static_cast<uint64_t>(c) * std::max<uint64_t>(1, S.per_chunk / 32) <= 64;
+        S.fused = !S.groups && static_cast<uint64_t>(c) * std::max<uint64_t>(1, S.per_chunk / 32) <= 64;
         if (S.fused) S.join_chunks = kBatch;
     } else {
         S.warps = static_cast<uint32_t>(std::min<uint64_t>(W, (tasks + sms - 1) / sms));
@@ -693,7 +773,6 @@ cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_
     if (S.fused) return cudaSuccess;
     // the join's blocks may be set up while the last stream blocks run (they wait at their start)
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(S.join_blocks);
     cfg.blockDim = dim3(kJoinThreads);
     cfg.stream = st;
     cudaLaunchAttribute at{};
@@ -701,6 +780,25 @@ cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = C.between ? 0 : 1;
+    if (S.groups) {
+        StreamGroupArgs g{};
+        g.j = j;
+        g.per_chunk = S.groups;
+        g.size = S.group;
+        g.groups = static_cast<uint64_t>(C.c) * S.groups;
+        g.inner = H.merge.inner;
+        g.n_images = static_cast<uint32_t>(H.merge.images.size());
+        g.out = C.groups;
+        g.tables = C.tables;
+        cfg.gridDim = dim3(static_cast<unsigned>((g.groups + kJoinThreads / 32 - 1) / (kJoinThreads / 32)));
+        e = cudaLaunchKernelEx(&cfg, rid_stream_group_kernel, g);
+        if (e != cudaSuccess) return e;
+        cfg.numAttrs = 1;
+        j.res = C.groups;
+        j.tables = C.tables;
+        j.per_chunk = S.groups;
+    }
+    cfg.gridDim = dim3(S.join_blocks);
     return cudaLaunchKernelEx(&cfg, rid_stream_join_kernel, j);
 }
 

@@ -16,6 +16,7 @@ struct StreamShape {
     uint32_t join_chunks = 256;  // chunks per join block
     uint32_t join_blocks = 1;
     bool fused = false;          // the join runs in the last block of the reach launch
+    uint32_t group = 0, groups = 0;  // pieces a group, groups a chunk is joined by; 0: its pieces themselves
     size_t smem = 0;
 };
 
@@ -27,6 +28,8 @@ struct StreamCall {
     uint64_t len = 0;
     uint32_t c = 0;
     uint32_t *res = nullptr;         // [pieces]
+    uint32_t *groups = nullptr;      // [c * groups], with groups
+    uint16_t *tables = nullptr;      // [c * groups][n]
     uint16_t *maps = nullptr;        // [c][k]
     uint32_t *dinfo = nullptr;       // [c]
     uint32_t *partials = nullptr;    // [join_blocks][kPartialWords]

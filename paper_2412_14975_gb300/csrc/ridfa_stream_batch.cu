@@ -24,6 +24,7 @@ struct StreamBatchProg {
     uint32_t n;                  // states
     uint32_t form;               // which instantiation of Steps
     uint32_t k, kw, q0_slot, n_texts, np;
+    uint32_t inner, n_images;    // nodes of the graph and their images
     const StreamBatchText *texts;
     const uint32_t *bases;
     uint32_t *res;
@@ -140,9 +141,13 @@ __device__ __forceinline__ uint32_t piece_to(const StreamBatchProg &P, uint32_t 
 // Accept bits, a block per text, a piece per thread (a warp per text took 25 us on texts of up to 2,000
 // pieces, one after another).  While every piece merged, piece i is entered iff if_min of piece i - 1's
 // end state meets the slots alive in piece i.  With a piece that did not, the run from q0's start state
-// is followed piece by piece instead (repeats of one function on its fixed point at once).
-constexpr int kBatchJoinBlock = 128;
-__global__ void __launch_bounds__(kBatchJoinBlock) rid_stream_batch_join_kernel(const StreamBatchProg *progs, const StreamBatchText *texts,
+// is followed piece by piece instead: every warp takes a strip of the pieces from all states that the
+// piece before the strip can end in (up to 32; repeats of one function on fixed points at once), and one
+// warp strings the strips together.
+// Threads a block; 1,024 where a text has very many pieces (two texts of 32 MB whose runs stay apart
+// took 5.9 ms with one warp's chain).
+constexpr uint32_t kBatchJoinBlock = 128, kBatchJoinMany = 4096;
+__global__ void __launch_bounds__(1024) rid_stream_batch_join_kernel(const StreamBatchProg *progs, const StreamBatchText *texts,
                                                                                uint8_t *accept) {
     const uint32_t lane = threadIdx.x & 31;
     const StreamBatchText td = texts[blockIdx.x];
@@ -157,7 +162,7 @@ __global__ void __launch_bounds__(kBatchJoinBlock) rid_stream_batch_join_kernel(
     const uint32_t *r = P.res + td.base;
     bool node = false, ok = true;
 #pragma unroll 2
-    for (uint32_t t = threadIdx.x; t < td.pieces; t += kBatchJoinBlock) {
+    for (uint32_t t = threadIdx.x; t < td.pieces; t += blockDim.x) {
         const uint32_t f = __ldg(r + t), y = t ? __ldg(r + t - 1) : 0;
         node = node || (f & kNodeResult);
         if (!((f | y) & kNodeResult)) {
@@ -174,21 +179,53 @@ __global__ void __launch_bounds__(kBatchJoinBlock) rid_stream_batch_join_kernel(
         if (threadIdx.x == 0) accept[td.item] = all && final_state(__ldg(r + td.pieces - 1) & 0xFFFF) ? 1 : 0;
         return;
     }
-    if (threadIdx.x >= 32) return;
-    uint32_t x = start;
-    for (uint32_t b = 0; b < td.pieces && x < n; b += 32) {
-        const uint32_t f = b + lane < td.pieces ? __ldg(r + b + lane) : 0;
-        const uint32_t cnt = min(32u, td.pieces - b);
-        for (uint32_t j = 0; j < cnt && x < n;) {
-            const uint32_t fj = __shfl_sync(kFull, f, j);
-            const uint32_t nx = piece_to(P, fj, x);
-            ++j;
-            if (nx == x) {                       // the same function again changes nothing
-                const uint32_t other = __ballot_sync(kFull, lane >= j && lane < cnt && f != fj);
-                j = other ? __ffs(other) - 1 : cnt;
+    __shared__ uint32_t s_from[32][32], s_to[32][32];
+    const uint32_t warp = threadIdx.x >> 5, strips = blockDim.x / 32, per = (td.pieces + strips - 1) / strips;
+    // the functions r[b0, b1) on every lane's state x
+    auto follow = [&](uint32_t b0, uint32_t b1, uint32_t x) {
+        for (uint32_t b = b0; b < b1 && __any_sync(kFull, x < n); b += 32) {
+            const uint32_t f = b + lane < b1 ? __ldg(r + b + lane) : 0;
+            const uint32_t cnt = min(32u, b1 - b);
+            for (uint32_t j = 0; j < cnt;) {
+                const uint32_t fj = __shfl_sync(kFull, f, j);
+                const uint32_t nx = piece_to(P, fj, x);
+                ++j;
+                if (__all_sync(kFull, nx == x)) {    // the same function again changes nothing
+                    const uint32_t other = __ballot_sync(kFull, lane >= j && lane < cnt && f != fj);
+                    j = other ? __ffs(other) - 1 : cnt;
+                }
+                x = nx;
             }
-            x = nx;
         }
+        return x;
+    };
+    const uint32_t b0 = min(td.pieces, warp * per), b1 = min(td.pieces, b0 + per);
+    const uint32_t before = warp && b0 < b1 ? __ldg(r + b0 - 1) : 0, u = before & ~kNodeResult;
+    uint32_t x = n, wide = 0;
+    if (warp == 0) {
+        if (lane == 0) x = start;
+    } else if (b0 < b1 && (before & kNodeResult)) {
+        const uint32_t at = __ldg(P.node_img + u), d = (u + 1 < P.inner ? __ldg(P.node_img + u + 1) : P.n_images) - at;
+        wide = d > 32;
+        if (lane < d) x = __ldg(P.images + at + lane);
+    } else if (b0 < b1 && lane == 0) {
+        x = before & 0xFFFF;
+    }
+    wide = __syncthreads_or(wide);
+    if (wide) {
+        if (warp) return;
+        x = follow(0, td.pieces, x);
+        if (lane == 0) accept[td.item] = final_state(x) ? 1 : 0;
+        return;
+    }
+    s_from[warp][lane] = x;
+    s_to[warp][lane] = follow(b0, b1, x);
+    __syncthreads();
+    if (warp) return;
+    x = s_to[0][0];
+    for (uint32_t w = 1; w < strips && w * per < td.pieces && x < n; ++w) {
+        const uint32_t hit = __ballot_sync(kFull, s_from[w][lane] == x);
+        x = hit ? s_to[w][__ffs(hit) - 1] : n;
     }
     if (lane == 0) accept[td.item] = final_state(x) ? 1 : 0;
 }
@@ -298,6 +335,7 @@ void plan_stream_batch(StreamBatchPlan &P, std::vector<StreamBatchSource> &src, 
         for (uint32_t p : forms[fi].second) {
             const HostAutomaton &A = *H[p];
             L.n_texts += static_cast<uint32_t>(src[p].items.size());
+            for (uint32_t t = P.text0[p]; t < P.text0[p] + src[p].items.size(); ++t) L.most = std::max(L.most, P.texts[t].pieces);
             L.smem = std::max(L.smem, P.walk_only ? stream_walk_bytes(A)
                                                   : stream_table_bytes(A) + (A.stream.kind == kStreamField ? 0 : batch_warps(A.stream) * kStreamStaging));
         }
@@ -359,6 +397,8 @@ void stream_batch_image(const StreamBatchPlan &P, uint8_t *dev, uint32_t *res, u
         b.q0_slot = H.q0_slot;
         b.n_texts = (p + 1 < P.H.size() ? P.text0[p + 1] : static_cast<uint32_t>(P.texts.size())) - P.text0[p];
         b.np = P.np[p];
+        b.inner = H.merge.inner;
+        b.n_images = static_cast<uint32_t>(H.merge.images.size());
         b.texts = reinterpret_cast<const StreamBatchText *>(dev + P.o_texts) + P.text0[p];
         b.bases = reinterpret_cast<const uint32_t *>(dev + P.o_bases) + P.text0[p];
         b.res = res + P.res0[p];
@@ -392,7 +432,7 @@ cudaError_t stream_batch_reach(const StreamBatchPlan &P, const StreamBatchLaunch
 }
 
 cudaError_t stream_batch_join(const StreamBatchPlan &P, const StreamBatchLaunch &L, const uint8_t *dev, uint8_t *d_accept, cudaStream_t st) {
-    rid_stream_batch_join_kernel<<<L.n_texts, kBatchJoinBlock, 0, st>>>(reinterpret_cast<const StreamBatchProg *>(dev + P.o_progs),
+    rid_stream_batch_join_kernel<<<L.n_texts, L.most > kBatchJoinMany ? 1024 : kBatchJoinBlock, 0, st>>>(reinterpret_cast<const StreamBatchProg *>(dev + P.o_progs),
                                                                        reinterpret_cast<const StreamBatchText *>(dev + P.o_texts) + L.text0,
                                                                        d_accept);
     return cudaGetLastError();

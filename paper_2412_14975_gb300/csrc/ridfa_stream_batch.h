@@ -32,7 +32,7 @@ struct StreamBatchLaunch {
     uint32_t form = 0, first = 0;                    // first: its entry in first_part
     uint32_t grid = 0, block = 0;
     size_t smem = 0;
-    uint32_t text0 = 0, n_texts = 0;                 // its texts, joined right after it
+    uint32_t text0 = 0, n_texts = 0, most = 0;       // its texts, joined right after it; pieces of the longest
 };
 
 // Plan of a batch's stream part.  The descriptors of plan_stream_image() go to the device as they
