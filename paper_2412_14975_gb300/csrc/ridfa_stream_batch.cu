@@ -1,13 +1,14 @@
-// Batched recognition by automata with a merge graph: the texts of all such programs in one launch,
-// whatever their table forms, and their accept bits in a second one.
+// Batched recognition by automata with a merge graph.
 //
 // A lane takes a piece of a text as in the single-text kernels.  The pieces of all programs of one
 // table form are one list, cut into equal shares of estimated cost, one per block; a block loads a
 // program's tables when its share comes to that program.  The launches of the forms run side by side,
-// each on its share of the SMs.  (One kernel for all forms spilled 1.7 KB a thread.)  (The general batch kernel hands out tasks of up to 16 MB by
-// tickets, which left half of the SMs idle on batches of a GB over 16 programs.)  A text is accepted
-// iff the join of its pieces' functions is: a block per text tests every boundary, as the single-text
-// join does.
+// each on its share of the SMs.  (One kernel for all forms spilled 1.7 KB a thread; the general batch
+// kernel hands out tasks of up to 16 MB by tickets, which left half of the SMs idle on batches of a GB
+// over 16 programs.)  A text is accepted iff the join of its pieces' functions is: a block per text
+// tests every boundary, as the single-text join does.
+// Bound by the shared-memory pipe, the one-byte tables above all (2,000 texts of 0.8 GB against 16 REs:
+// 789 us in the general kernels, 450 us with these and the set kernels).
 #include <cuda_runtime.h>
 
 #include <algorithm>
