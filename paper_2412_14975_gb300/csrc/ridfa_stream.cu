@@ -692,7 +692,7 @@ StreamShape stream_shape(const HostAutomaton &H, uint64_t len, uint32_t c, int s
     for (uint64_t s = 2; s <= 16; ++s) consider(s);
     for (uint64_t m = 1; m <= 2 * W; ++m) consider(m * lanes / c);
     if (len <= kWalkText && len / c / best > kWalkPiece / 2) {
-        // a short text in pieces of some 64 to 128 bytes instead, where that is below kWalkPiece
+        // a short text in pieces of some 64 bytes instead
         const uint64_t s = std::max<uint64_t>(1, len / c / kMinPiece);
         if (len / c / s <= kWalkPiece) best = s;
     }

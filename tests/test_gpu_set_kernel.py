@@ -64,7 +64,7 @@ def test_set_chunk_counts(c):
     check(CODON, x, c, offset=5)
 
 
-@pytest.mark.parametrize("per", [128, 129, 159, 160, 161, 300, 1000])
+@pytest.mark.parametrize("per", [31, 32, 33, 64, 95, 127, 128, 129, 159, 160, 161, 300, 1000])
 def test_set_chunk_lengths(per):
     c = 39000
     x = textgen.c2_text(c * per + 1, seed=per)
@@ -84,7 +84,7 @@ def test_set_other_res(re_src, alphabet):
 
 
 @pytest.mark.parametrize("c,per", [(1, 20_000_003), (2, 9_000_001), (67, 300_017), (1024, 19_001), (1030, 40_507), (4096, 5_003), (30_000, 701),
-                                   (1, 128), (1, 511), (1, 512), (3, 1_400), (33, 1_000)])
+                                   (1, 32), (1, 128), (1, 511), (1, 512), (3, 1_400), (33, 1_000), (80, 64), (5045, 64)])
 @pytest.mark.parametrize("re_src,alphabet", [(CODON, None), (BINARY, b"ab")])
 def test_set_pieces(re_src, alphabet, c, per):
     """Few chunks, cut into pieces: one level of composition and several, ragged groups of pieces."""
