@@ -141,10 +141,10 @@ class ClockSampler:
 
 # DRAM bytes (read + write) per text byte of the reach kernel, from one ncu capture of it
 # (record-line RE, 1 GiB, 155,648 chunks: dram__bytes_read.sum + dram__bytes_write.sum); applied
-# to the record-line workload in the same launch shape (Rep16 tables, cooperative staging), scaled
+# to the record-line workload in the same launch shape (two-byte table, staged text), scaled
 # by the text bytes.  Must be re-measured (or dropped) whenever that kernel changes.
-REACH_TRAFFIC = {"workload": "c3", "kernel": "rid_reach_kernel<4, LutRep<true>, 1024, 2>",
-                 "dram_bytes_per_text_byte": 1.0312}
+REACH_TRAFFIC = {"workload": "c3", "kernel": "rid_stream_kernel<2, 2, 1, 0>",
+                 "dram_bytes_per_text_byte": 1.0222}
 
 
 def measured_peaks():
@@ -827,12 +827,15 @@ def main():
     # measured on this GPU by the library's microbenchmark
     lut_rate = lib.ridfa_bench_smem_gather(1 << 16) / 1e9
     text_rate = n / (reach_ms / 1e3) / 1e9
+    # (the library's own choice; any override takes the general kernel)
+    override = args.table_mode or args.text_path or args.piece_len or args.probe
+    reach_kernel = "rid_reach_kernel" if override else "rid_set_kernel" if name == "c2" else "rid_stream_kernel"
     traffic = None
     if name == REACH_TRAFFIC["workload"] and args.table_mode == 0 and args.text_path == 0 and c == 155648:
         traffic = int(REACH_TRAFFIC["dram_bytes_per_text_byte"] * n)
     roofline = {"bound": "hbm", "achieved": round(achieved, 2), "peak": peaks["hbm_gbs"],
                 "unit": "GB/s", "frac": round(achieved / peaks["hbm_gbs"], 4), "traffic": traffic,
-                "kernel": "rid_reach_kernel", "peak_source": peak_kind,
+                "kernel": reach_kernel, "peak_source": peak_kind,
                 "algorithmic_bytes_per_launch": alg_bytes, "kernel_ms": round(reach_ms, 4),
                 "join_ms": round(join_ms, 4),
                 "smem_gather": {"peak_text_GBps": round(lut_rate, 1), "achieved_text_GBps": round(text_rate, 1),
@@ -905,8 +908,9 @@ def main():
         work["count_s"] = round(time.perf_counter() - t0, 2)
         lpb = 1 + rc["w_conv"] / n
         roofline["smem_gather"]["lookups_per_byte"] = round(lpb, 5)
-        # the binding roof: the slower of the text at HBM bandwidth and the lookups at the
-        # measured gather rate (the microbenchmark does 2 lookups per byte)
+        # the binding roof: the slower of the text at HBM bandwidth and the lookups of one-byte steps
+        # at the measured gather rate (the microbenchmark does 2 lookups per byte); kernels that step
+        # two or four bytes a lookup may pass the latter
         lut_text_rate = lut_rate * 2.0 / lpb
         roofline["smem_gather"]["roof_text_GBps"] = round(lut_text_rate, 1)
         roofline["smem_gather"]["roof_frac"] = round(text_rate / lut_text_rate, 4)
