@@ -277,11 +277,21 @@ bool find_field(const HostAutomaton &H, HostStream &t) {
 void fill_field(const HostAutomaton &H, HostStream &t) {
     const uint32_t n = H.n_states, per_word = 4 / t.entry, W = t.row_words, m = (1u << t.width) - 1;
     t.words.assign(static_cast<size_t>(n + 1) * W, 0);
+    // columns of half a group, then of two halves
+    const uint32_t half = t.width * t.group / 2, cols = 1u << half;
+    std::vector<uint16_t> mid(static_cast<size_t>(n + 1) * cols);
+    std::vector<uint32_t> cls(m + 1);
+    for (uint32_t v = 0; v <= m; ++v) cls[v] = H.classmap[(t.canon >> (8 * v)) & 0xFF];
+    for (uint32_t s = 0; s <= n; ++s)
+        for (uint32_t c = 0; c < cols; ++c) {
+            uint32_t x = s;
+            for (uint32_t i = 0; i < t.group / 2; ++i) x = H.trans[static_cast<size_t>(x) * H.n_classes + cls[(c >> (t.width * i)) & m]];
+            mid[static_cast<size_t>(s) * cols + c] = static_cast<uint16_t>(x);
+        }
     for (uint32_t s = 0; s <= n; ++s)
         for (uint32_t c = 0; c < W * per_word; ++c) {
-            uint32_t x = c >> (t.width * t.group) ? n : s;
-            for (uint32_t i = 0; i < t.group; ++i)
-                x = H.trans[static_cast<size_t>(x) * H.n_classes + H.classmap[(t.canon >> (8 * ((c >> (t.width * i)) & m))) & 0xFF]];
+            const uint32_t y = mid[static_cast<size_t>(s) * cols + (c & (cols - 1))];
+            const uint32_t x = c >> (2 * half) ? n : mid[static_cast<size_t>(y) * cols + (c >> half)];
             t.words[static_cast<size_t>(s) * W + c / per_word] |= x << (8 * t.entry * (c % per_word));
         }
 }
@@ -406,12 +416,20 @@ void build_back(const HostAutomaton &H, HostSet &Z) {
     for (uint32_t x = 0; x < n; ++x) sets[x >> 6] |= 1ull << (x & 63);
     std::vector<uint16_t> images(kSetRuns, static_cast<uint16_t>(n)), next;   // leaf 0: all dead
     uint64_t steps = 0;
+    std::vector<bool> dead_class(C, true);
+    for (uint32_t x = 0; x < n; ++x)
+        for (uint32_t c = 0; c < C; ++c)
+            if (H.trans[static_cast<size_t>(x) * C + c] < n) dead_class[c] = false;
     uint32_t inner = 1, leaves = 1, most = 0;             // code: the inner node's index, or kLeafBit | leaf
     for (uint32_t u = 0; u < order.size(); ++u) {
         const uint32_t from = order[u];
         most = std::max(most, depth[from] + 1);
         if (most > kMaxDepth) return;
         for (uint32_t c = 0; c < C; ++c) {
+            if (dead_class[c]) {
+                next.push_back(kLeafBit);
+                continue;
+            }
             std::fill(row.begin(), row.end(), 0);
             for (uint32_t w = 0; w < words; ++w)
                 for (uint64_t b = sets[static_cast<size_t>(from) * words + w]; b; b &= b - 1) {
