@@ -305,8 +305,12 @@ __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_cons
                 }
             }
             if (r < 3 || (r & 3) == 3) {         // (the most runs die in the first bytes)
-                if (M > kHalf) cnt = compact_set<kSetRuns>(s, rep, dead);
-                else cnt = compact_set<kHalf>(s, rep, dead);
+                // (M is the most runs of the lanes that had a block: a lane that ended its own earlier may
+                // hold more, beyond the places a narrow compaction looks at, and waits for the one at the end)
+                if (r < blocks) {
+                    if (M > kHalf) cnt = compact_set<kSetRuns>(s, rep, dead);
+                    else cnt = compact_set<kHalf>(s, rep, dead);
+                }
                 M = __reduce_max_sync(kFull, r + 1 < blocks ? cnt : 0u);
                 if (M == 0) break;
             }
