@@ -83,7 +83,8 @@ struct HostSet {
     std::vector<uint8_t> part;        // [parts][k]: block of each slot, 0xFF: dead
     std::vector<uint32_t> block_mask; // [parts][kw][kSetRuns]: slots of each block
     HostStream table;                 // kStreamField, entries of 2 bytes
-    uint32_t back_depth = 0;          // 0: not built.  The sets the bytes before a piece leave of all states:
+    uint32_t back_depth = 0;          // 0: not built.  The sets the bytes before a piece leave of all states;
+                                      // every string of back_depth bytes comes to a leaf:
     std::vector<uint16_t> back_next;  // [inner sets][C]: an inner set, or kLeafBit | leaf (leaf 0: all dead)
     std::vector<uint16_t> back_images;// [leaves][kSetRuns]: states (unused ones: n_states)
 };

@@ -406,7 +406,7 @@ void build_table(HostAutomaton &H) {
 
 // The sets that strings of up to `back_depth` bytes lead the set of all states to, each followed until
 // fewer than kSetRuns states are left: what a piece in the middle of a chunk can be entered with.  Sets
-// are bit rows; left out when they are too many.
+// are bit rows; left out when they are too many, or when some string of kMaxDepth bytes leaves more states.
 void build_back(const HostAutomaton &H, HostSet &Z) {
     constexpr uint32_t kMaxNodes = 4096, kMaxDepth = 24, kHash = 4 * kMaxNodes;
     const uint32_t n = H.n_states, C = H.n_classes, words = (n + 63) / 64;
@@ -420,11 +420,10 @@ void build_back(const HostAutomaton &H, HostSet &Z) {
     for (uint32_t x = 0; x < n; ++x)
         for (uint32_t c = 0; c < C; ++c)
             if (H.trans[static_cast<size_t>(x) * C + c] < n) dead_class[c] = false;
-    uint32_t inner = 1, leaves = 1, most = 0;             // code: the inner node's index, or kLeafBit | leaf
+    uint32_t inner = 1, leaves = 1;                       // code: the inner node's index, or kLeafBit | leaf
     for (uint32_t u = 0; u < order.size(); ++u) {
         const uint32_t from = order[u];
-        most = std::max(most, depth[from] + 1);
-        if (most > kMaxDepth) return;
+        if (depth[from] >= kMaxDepth) return;
         for (uint32_t c = 0; c < C; ++c) {
             if (dead_class[c]) {
                 next.push_back(kLeafBit);
@@ -475,9 +474,29 @@ void build_back(const HostAutomaton &H, HostSet &Z) {
     if (next.size() != static_cast<size_t>(inner) * C || images.size() != static_cast<size_t>(leaves) * kSetRuns) return;
     for (uint16_t e : next)
         if ((e & kLeafBit) ? (e & 0x7FFFu) >= leaves : e >= inner) return;
+    // A string's way to a leaf may be longer than the shortest one to it, and a set that leads back to itself
+    // has ways without end: the kernels walk as many bytes as the longest way has, if there is one.
+    std::vector<uint32_t> ways(inner, 0), longest(inner, 0), ready{0};
+    for (uint16_t e : next)
+        if (!(e & kLeafBit)) ++ways[e];
+    uint32_t done = 0, deepest = 0;
+    if (ways[0]) return;
+    while (!ready.empty()) {
+        const uint32_t u = ready.back();
+        ready.pop_back();
+        ++done;
+        deepest = std::max(deepest, longest[u] + 1);
+        for (uint32_t c = 0; c < C; ++c) {
+            const uint16_t e = next[static_cast<size_t>(u) * C + c];
+            if (e & kLeafBit) continue;
+            longest[e] = std::max(longest[e], longest[u] + 1);
+            if (--ways[e] == 0) ready.push_back(e);
+        }
+    }
+    if (done != inner || deepest > kMaxDepth) return;
     Z.back_next = std::move(next);
     Z.back_images = std::move(images);
-    Z.back_depth = most;
+    Z.back_depth = deepest;
 }
 
 // The functions of the first bytes on the slots, level by level, down to the first level on which all

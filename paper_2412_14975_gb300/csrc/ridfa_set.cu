@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kSetBlock, 1) rid_set_kernel(const __grid_cons
                 if (e & kLeafBit) break;
             }
             ++taken;
-            leaf = node & 0x7FFF;
+            leaf = node & kLeafBit ? node & 0x7FFF : 0;      // (always a leaf: back_depth is the longest way to one)
         } else if (have) {
             uint32_t node = 0;
             for (uint32_t d = 0; d < p.depth; ++d) {
