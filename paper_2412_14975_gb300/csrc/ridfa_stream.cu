@@ -95,7 +95,7 @@ struct StreamJoinArgs {
     uint32_t per_chunk;      // pieces (or groups of them) per chunk
     uint32_t chunks;         // chunks per block
     uint32_t k_magic;        // ceil(2^32 / k): e / k = umulhi(e, k_magic) for e < 2^16
-    uint32_t *work;          // status bits of this call while it runs
+    uint32_t *status;        // the call's status, written once by publish(); while it runs its bits are in j.status
     uint8_t *h_accept;
     uint32_t *h_status;
 };
@@ -239,16 +239,16 @@ __device__ void general_row(const StreamJoinArgs &p, uint64_t i, uint32_t lane) 
     }
     if (lane == 0) {
         p.dinfo[i] = cnt > kMaxD ? (0xFFu << 16) | first : cnt ? (cnt << 16) | first : static_cast<uint32_t>(kUndef);
-        if (cnt > kMaxD) atomicOr(p.work, kStatusWide);
+        if (cnt > kMaxD) atomicOr(p.j.status, kStatusWide);
     }
 }
 
 // Thread 0 of the last block: accept bit and status to their places, counters back to zero for the
 // next call.
 __device__ void publish(const StreamJoinArgs &p, uint8_t acc) {
-    const uint32_t st = *reinterpret_cast<volatile uint32_t *>(p.work);
-    *p.j.status = st;
-    if (st) *p.work = 0;
+    const uint32_t st = *reinterpret_cast<volatile uint32_t *>(p.j.status);
+    *p.status = st;
+    if (st) *p.j.status = 0;
     *p.j.ticket = 0;
     *p.j.accept = acc;
     if (p.h_accept) {
@@ -419,7 +419,7 @@ __device__ void stream_join(const StreamJoinArgs &p, uint32_t blk, uint32_t nblk
                 for (uint32_t z = 0; z < mp; ++z) P.rows[z] = transfer_row(p.j, static_cast<uint32_t>(i), Dp[z], Dc, mc, &bad);
             }
         }
-        if (bad) atomicOr(p.work, kStatusBad);
+        if (bad) atomicOr(p.j.status, kStatusBad);
         sh.prod[tid] = P;
         __syncthreads();
         for (uint32_t stride = 1; stride < blockDim.x; stride *= 2) {
@@ -449,7 +449,7 @@ __device__ void stream_join(const StreamJoinArgs &p, uint32_t blk, uint32_t nblk
         if (!sh.last) return;
         __threadfence();
         // ---- last block: the product of all blocks
-        if (*reinterpret_cast<volatile uint32_t *>(p.work) & kStatusWide) {
+        if (*reinterpret_cast<volatile uint32_t *>(p.j.status) & kStatusWide) {
             uint32_t acc = 0;
             if (p.j.summary) summary_wide(p.j, sh.vec, sh.nvec);
             else acc = accept_unmerged(p, sh.vec, sh.nvec);
@@ -539,7 +539,7 @@ __device__ void stream_join(const StreamJoinArgs &p, uint32_t blk, uint32_t nblk
             const uint32_t m0 = distinct_of(p.j, 0, D0), x0 = index_of(D0, m0, v0);
             const uint32_t ml = distinct_of(p.j, static_cast<uint32_t>(c - 1), Dl);
             if (x0 == 0xFFFFFFFFu || tot.nrows == 0xFFFFFFFFu || ml == 0xFFFFFFFFu) {
-                atomicOr(p.work, kStatusBad);
+                atomicOr(p.j.status, kStatusBad);
             } else if (x0 < tot.nrows) {
                 const uint32_t row = tot.rows[x0];
                 for (uint32_t y = 0; y < ml; ++y)
@@ -743,7 +743,7 @@ cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_
     const Automaton A{D.trans, D.classmap, D.final_bits, D.ifmask, D.slot_state,
                       H.n_states, H.n_classes, H.k, H.kw, H.q0_slot, H.merges};
     StreamJoinArgs j{};
-    j.j = JoinArgs{A, C.c, C.maps, C.dinfo, C.status, C.partials, C.ticket, C.accept, 1, C.summary};
+    j.j = JoinArgs{A, C.c, C.maps, C.dinfo, C.work, C.partials, C.ticket, C.accept, 1, C.summary};
     j.maps = C.maps;
     j.dinfo = C.dinfo;
     j.res = C.res;
@@ -755,7 +755,7 @@ cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_
     j.per_chunk = S.per_chunk;
     j.chunks = S.join_chunks;
     j.k_magic = static_cast<uint32_t>((0xFFFFFFFFull + H.k) / H.k);
-    j.work = C.work;
+    j.status = C.status;
     j.h_accept = C.h_accept;
     j.h_status = C.h_status;
     cudaError_t e;
