@@ -14,6 +14,8 @@
 //   3. one block: the incoming PLAS vector of every segment;
 //   4. a warp per segment walks its boundaries from that vector;
 //   5. a warp per chunk forms E_i from PLAS_{i-1}.
+// Boundaries go through these launches kScanTile at a time, so that the matrices take 35 MB at most, however many
+// chunks there are.
 // When some chunk has more than 32 distinct end states, one block propagates the k-bit sets
 // chunk by chunk instead (exact, sequential in c).
 //
@@ -22,6 +24,7 @@
 // chunks with several end states, 197 us by the second.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "ridfa_internal.h"
@@ -35,16 +38,19 @@ constexpr uint32_t kScanThreads = 256;
 constexpr uint32_t kScanWarps = kScanThreads / 32;
 constexpr uint32_t kScanRows = 8;          // consecutive rows per warp of rid_scan_rows
 constexpr uint32_t kStatusSeveral = 8u;    // some chunk has two or more end states
+constexpr uint32_t kScanTile = 1u << 18;   // boundaries that launches 1 to 5 take at a time (2^20 chunks of the
+                                           // codon RE: 2,530 us in one, 2,546 in 4 tiles, 2,910 in 16)
 constexpr int kScanRegs = RIDFA_MAX_SLOTS / 32;
 
 struct ScanArgs {
     Automaton A;
     const uint16_t *maps;      // [c][k]
-    uint32_t c, nseg;
-    uint32_t *mats;            // [c][32]: row z of M_i, bits over D_i
+    uint32_t c;
+    uint32_t first, end, nseg; // boundaries [first, end) of this tile, in nseg segments
+    uint32_t *mats;            // [boundary - first][32]: row z of M_i, bits over D_i
     uint32_t *prods;           // [nseg][32]
     uint32_t *vin;             // [nseg]: PLAS before the segment's first boundary, over its D
-    uint32_t *plas;            // [c]: PLAS_i as bits over D_i
+    uint32_t *plas;            // [1 + kScanTile]: PLAS_i as bits over D_i, i from first - 1
     uint32_t *entry;           // [c][kw], or null
     unsigned long long *reject;
     uint32_t *status;
@@ -148,8 +154,8 @@ __global__ void __launch_bounds__(kScanThreads) rid_scan_matrices(ScanArgs p) {
     __shared__ uint8_t s_idx[kScanWarps][RIDFA_MAX_SLOTS];
     const Automaton &A = p.A;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t i = 1 + static_cast<uint64_t>(blockIdx.x) * kScanWarps + warp;
-    if (i >= p.c) return;
+    const uint64_t i = p.first + static_cast<uint64_t>(blockIdx.x) * kScanWarps + warp;
+    if (i >= p.end) return;
     uint32_t v[kScanRegs], prev, mine;
     load_row(p, i - 1, lane, v);
     const uint32_t mp = warp_distinct(v, lane, prev);
@@ -182,7 +188,7 @@ __global__ void __launch_bounds__(kScanThreads) rid_scan_matrices(ScanArgs p) {
                     if (g != 0xFF) row |= 1u << g;
                 }
     }
-    p.mats[i * 32 + lane] = row;
+    p.mats[(i - p.first) * 32 + lane] = row;
 }
 
 // rows <- rows · M, a row per lane; m: the lane's row of M.
@@ -205,9 +211,9 @@ __global__ void __launch_bounds__(kScanThreads) rid_scan_products(ScanArgs p) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t sg = blockIdx.x * kScanWarps + (threadIdx.x >> 5);
     if (sg >= p.nseg) return;
-    const uint64_t b0 = 1 + static_cast<uint64_t>(sg) * kScanSeg, b1 = min(static_cast<uint64_t>(p.c), b0 + kScanSeg);
+    const uint32_t b0 = sg * kScanSeg, b1 = min(p.end - p.first, b0 + kScanSeg);
     uint32_t row = 1u << lane, m = p.mats[b0 * 32 + lane];
-    for (uint64_t i = b0; i < b1; ++i) {
+    for (uint32_t i = b0; i < b1; ++i) {
         const uint32_t next = i + 1 < b1 ? p.mats[(i + 1) * 32 + lane] : 0;
         row = times(row, m);
         m = next;
@@ -215,8 +221,8 @@ __global__ void __launch_bounds__(kScanThreads) rid_scan_products(ScanArgs p) {
     p.prods[static_cast<uint64_t>(sg) * 32 + lane] = row;
 }
 
-// Launch 3 (one block of 32 warps): the incoming PLAS vector of every segment, PLAS and entry set of
-// chunk 0.
+// Launch 3 (one block of 32 warps): the incoming PLAS vector of every segment; in the first tile, PLAS and
+// entry set of chunk 0.
 __global__ void __launch_bounds__(1024) rid_scan_prefix(ScanArgs p) {
     __shared__ uint32_t s_tot[32][32], s_in[32];
     const Automaton &A = p.A;
@@ -238,17 +244,20 @@ __global__ void __launch_bounds__(1024) rid_scan_prefix(ScanArgs p) {
     s_tot[warp][lane] = row;
     __syncthreads();
     if (warp == 0) {
-        // PLAS_1 = {λ_1(q0)} over D_1 (chunk 0 here); E_1 = {q0's slot} if that move is defined
-        uint32_t v[kScanRegs], mine;
-        load_row(p, 0, lane, v);
-        const uint32_t m0 = warp_distinct(v, lane, mine);
-        const uint32_t v0 = p.maps[A.q0_slot];
-        uint32_t x = m0 <= static_cast<uint32_t>(kMaxD) ? __ballot_sync(kFull, v0 != kUndef && lane < m0 && mine == v0) : 0;
-        if (p.entry && lane < A.kw) p.entry[lane] = (v0 != kUndef && (A.q0_slot >> 5) == lane) ? 1u << (A.q0_slot & 31) : 0u;
-        if (lane == 0) {
-            p.plas[0] = x;
-            if (v0 == kUndef) atomicMin(p.reject, 0ull);
+        uint32_t x;
+        if (p.first > 1) {
+            x = p.plas[kScanTile];               // (the tile before was a whole one)
+        } else {
+            // PLAS_1 = {λ_1(q0)} over D_1 (chunk 0 here); E_1 = {q0's slot} if that move is defined
+            uint32_t v[kScanRegs], mine;
+            load_row(p, 0, lane, v);
+            const uint32_t m0 = warp_distinct(v, lane, mine);
+            const uint32_t v0 = p.maps[A.q0_slot];
+            x = m0 <= static_cast<uint32_t>(kMaxD) ? __ballot_sync(kFull, v0 != kUndef && lane < m0 && mine == v0) : 0;
+            if (p.entry && lane < A.kw) p.entry[lane] = (v0 != kUndef && (A.q0_slot >> 5) == lane) ? 1u << (A.q0_slot & 31) : 0u;
+            if (lane == 0 && v0 == kUndef) atomicMin(p.reject, 0ull);
         }
+        if (lane == 0) p.plas[0] = x;
         for (uint32_t t = 0; t < 32; ++t) {
             if (lane == 0) s_in[t] = x;
             x = vec_times(x, s_tot[t][lane], lane);
@@ -273,26 +282,26 @@ __global__ void __launch_bounds__(kScanThreads) rid_scan_walk(ScanArgs p) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t sg = blockIdx.x * kScanWarps + (threadIdx.x >> 5);
     if (sg >= p.nseg) return;
-    const uint64_t b0 = 1 + static_cast<uint64_t>(sg) * kScanSeg, b1 = min(static_cast<uint64_t>(p.c), b0 + kScanSeg);
+    const uint32_t b0 = sg * kScanSeg, b1 = min(p.end - p.first, b0 + kScanSeg);
     uint32_t v = p.vin[sg], keep = 0, m = p.mats[b0 * 32 + lane];
-    for (uint64_t i = b0; i < b1; ++i) {
+    for (uint32_t i = b0; i < b1; ++i) {
         const uint32_t next = i + 1 < b1 ? p.mats[(i + 1) * 32 + lane] : 0;
         const uint32_t nv = vec_times(v, m, lane);
-        if (nv == 0 && v != 0 && lane == 0) atomicMin(p.reject, static_cast<unsigned long long>(i));
+        if (nv == 0 && v != 0 && lane == 0) atomicMin(p.reject, static_cast<unsigned long long>(p.first) + i);
         if (lane == i - b0) keep = nv;
         v = nv;
         m = next;
     }
-    if (b0 + lane < b1) p.plas[b0 + lane] = keep;
+    if (b0 + lane < b1) p.plas[b0 + lane + 1] = keep;
 }
 
 // Launch 5: E_i from PLAS_{i-1}, a warp per chunk.
 __global__ void __launch_bounds__(kScanThreads) rid_scan_entries(ScanArgs p) {
     const Automaton &A = p.A;
     const uint32_t lane = threadIdx.x & 31;
-    const uint64_t i = 1 + static_cast<uint64_t>(blockIdx.x) * kScanWarps + (threadIdx.x >> 5);
-    if (i >= p.c) return;
-    const uint32_t plas = p.plas[i - 1];
+    const uint64_t i = p.first + static_cast<uint64_t>(blockIdx.x) * kScanWarps + (threadIdx.x >> 5);
+    if (i >= p.end) return;
+    const uint32_t plas = p.plas[i - p.first];
     uint32_t e = 0;
     if (plas) {
         uint32_t v[kScanRegs], prev;
@@ -379,7 +388,6 @@ extern "C" int ridfa_join_scan(const ridfa_program *prog, const uint16_t *d_maps
                     H.k, H.kw, H.q0_slot};
     a.maps = d_maps;
     a.c = c;
-    a.nseg = c > 1 ? (c - 1 + kScanSeg - 1) / kScanSeg : 0;
     a.entry = d_entry;
     a.reject = reinterpret_cast<unsigned long long *>(words);
     a.status = reinterpret_cast<uint32_t *>(words + 1);
@@ -402,7 +410,8 @@ extern "C" int ridfa_join_scan(const ridfa_program *prog, const uint16_t *d_maps
     if (e != cudaSuccess) return cuda_fail(e);
     uint32_t status = static_cast<uint32_t>(h[1]);
     if (status & kStatusSeveral) {
-        const size_t bytes = (static_cast<size_t>(c) * 33 + static_cast<size_t>(a.nseg) * 33) * 4;
+        const size_t tile = std::min<size_t>(kScanTile, c - 1), segs = (tile + kScanSeg - 1) / kScanSeg;
+        const size_t bytes = (tile * 32 + segs * 33 + kScanTile + 1) * 4;
         uint32_t *scratch = nullptr;
         err = scan_words(prog, dev, bytes, &words, &h, &scratch);
         if (err != RIDFA_OK) return err;
@@ -410,19 +419,27 @@ extern "C" int ridfa_join_scan(const ridfa_program *prog, const uint16_t *d_maps
         a.status = reinterpret_cast<uint32_t *>(words + 1);
         if (clear() != cudaSuccess) return cuda_fail(e);
         a.mats = scratch;
-        a.prods = a.mats + static_cast<size_t>(c) * 32;
-        a.vin = a.prods + static_cast<size_t>(a.nseg) * 32;
-        a.plas = a.vin + a.nseg;
-        if (c > 1) {
-            rid_scan_matrices<<<blocks(c - 1, kScanWarps), kScanThreads, 0, st>>>(a);
-            rid_scan_products<<<blocks(a.nseg, kScanWarps), kScanThreads, 0, st>>>(a);
-        }
-        rid_scan_prefix<<<1, 1024, 0, st>>>(a);
-        if (c > 1) {
-            rid_scan_walk<<<blocks(a.nseg, kScanWarps), kScanThreads, 0, st>>>(a);
-            if (d_entry) rid_scan_entries<<<blocks(c - 1, kScanWarps), kScanThreads, 0, st>>>(a);
-        }
-        e = cudaGetLastError();
+        a.prods = a.mats + tile * 32;
+        a.vin = a.prods + segs * 32;
+        a.plas = a.vin + segs;
+        uint64_t at = 1;
+        do {                                     // (one tile without boundaries where there is one chunk)
+            a.first = static_cast<uint32_t>(at);
+            a.end = static_cast<uint32_t>(std::min<uint64_t>(c, at + kScanTile));
+            const uint32_t n = a.end - a.first;
+            a.nseg = (n + kScanSeg - 1) / kScanSeg;
+            if (n) {
+                rid_scan_matrices<<<blocks(n, kScanWarps), kScanThreads, 0, st>>>(a);
+                rid_scan_products<<<blocks(a.nseg, kScanWarps), kScanThreads, 0, st>>>(a);
+            }
+            rid_scan_prefix<<<1, 1024, 0, st>>>(a);
+            if (n) {
+                rid_scan_walk<<<blocks(a.nseg, kScanWarps), kScanThreads, 0, st>>>(a);
+                if (d_entry) rid_scan_entries<<<blocks(n, kScanWarps), kScanThreads, 0, st>>>(a);
+            }
+            e = cudaGetLastError();
+            at = a.end;
+        } while (e == cudaSuccess && at < c);
         if (e == cudaSuccess) fetch();
         if (e != cudaSuccess) return cuda_fail(e);
         status = static_cast<uint32_t>(h[1]);
