@@ -1300,14 +1300,36 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
 
 }  // namespace
 
-int scan_words(const ridfa_program *prog, int dev, size_t bytes, uint64_t **d_words, uint64_t **h_words, uint32_t **work) {
+int scan_take(const ridfa_program *prog, int dev, ScanSpace *out) {
     int err = RIDFA_OK;
-    DeviceScratch *S = scratch_for(prog, dev, 1024 + bytes, &err);
+    DeviceScratch *S = scratch_for(prog, dev, 0, &err);
     if (!S) return err;
-    *d_words = reinterpret_cast<uint64_t *>(static_cast<uint8_t *>(S->base) + 768);    // (past Layout's words)
-    *h_words = reinterpret_cast<uint64_t *>(S->h_accept_pinned + 32);
-    if (work) *work = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(S->base) + 1024);
-    return RIDFA_OK;
+    *out = S->scan;
+    S->scan = ScanSpace{};
+    if (out->host) return RIDFA_OK;
+    const cudaError_t e = cudaMallocHost(&out->host, 64);
+    if (e != cudaSuccess) out->host = nullptr;
+    return e == cudaSuccess ? RIDFA_OK : cuda_fail(e);
+}
+
+int scan_grow(ScanSpace *sp, size_t bytes) {
+    if (sp->base && sp->bytes >= bytes) return RIDFA_OK;
+    if (sp->base) cudaFree(sp->base);
+    sp->base = nullptr;
+    const cudaError_t e = cudaMalloc(&sp->base, 256 + bytes);
+    if (e != cudaSuccess) sp->base = nullptr;
+    sp->bytes = sp->base ? bytes : 0;
+    return e == cudaSuccess ? RIDFA_OK : cuda_fail(e);
+}
+
+void scan_give(const ridfa_program *prog, int dev, const ScanSpace &sp) {
+    for (auto &s : prog->scratch)
+        if (s.device == dev && !s.scan.host) {
+            s.scan = sp;
+            return;
+        }
+    if (sp.base) cudaFree(sp.base);
+    if (sp.host) cudaFreeHost(sp.host);
 }
 
 void release_device(const ridfa_program *P) {
@@ -1327,6 +1349,8 @@ void release_device(const ridfa_program *P) {
     for (auto &s : P->scratch) {
         free_on(s.device, s.base);
         if (s.h_accept_pinned) cudaFreeHost(s.h_accept_pinned);
+        free_on(s.device, s.scan.base);
+        if (s.scan.host) cudaFreeHost(s.scan.host);
         for (void *ev : s.ev)
             if (ev) cudaEventDestroy(static_cast<cudaEvent_t>(ev));
     }

@@ -165,6 +165,13 @@ struct DeviceNfa {
     uint8_t *h_accept_pinned = nullptr;
 };
 
+// What one join scan works in: two result words and working space on the device, two page-locked words.
+struct ScanSpace {
+    void *base = nullptr;             // the words, then (256 bytes on) the working space
+    size_t bytes = 0;
+    uint64_t *host = nullptr;
+};
+
 // Per-device scratch of a program: chunk maps when the caller passes none, per-chunk summaries,
 // the join's partial products, a block ticket, the status word and the accept byte.
 struct DeviceScratch {
@@ -182,6 +189,7 @@ struct DeviceScratch {
     const uint8_t *stream_text = nullptr;        // (only its alignment is looked at)
     uint64_t stream_len = 0;
     uint32_t stream_chunks = 0;
+    ScanSpace scan;                              // of the last join scan, while none runs
 };
 
 }  // namespace ridfa
@@ -227,9 +235,12 @@ int cuda_fail(cudaError_t e);
 int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev);
 const DeviceAutomaton *device_copy(const ridfa_program *P, bool dfa, int dev, int *err);
 int smem_optin_limit();
-// For the join scan: two device words and two page-locked host words of the program's scratch on
-// `dev`, and `bytes` of working space in it.  Caller holds prog->mu.
-int scan_words(const ridfa_program *prog, int dev, size_t bytes, uint64_t **d_words, uint64_t **h_words, uint32_t **work);
+// The space of one join scan, taken from the program (or made) and given back, so that prog->mu need not be
+// held while the scan runs: scans that overlap have one each, of which the program keeps one a device.
+// Callers of take and give hold prog->mu; grow makes room for `bytes` of working space.
+int scan_take(const ridfa_program *prog, int dev, ScanSpace *out);
+int scan_grow(ScanSpace *sp, size_t bytes);
+void scan_give(const ridfa_program *prog, int dev, const ScanSpace &sp);
 // Raise a kernel's dynamic shared-memory cap on the current device to at least `bytes`.  The cap
 // is never lowered, so a launch sized by another thread (or an earlier plan) stays valid.
 cudaError_t ensure_smem_cap(const void *kern, size_t bytes);

@@ -374,30 +374,52 @@ extern "C" int ridfa_join_scan(const ridfa_program *prog, const uint16_t *d_maps
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_fail(e);
-    std::lock_guard<std::mutex> lock(prog->mu);
+    ScanArgs a{};
+    struct Space {                               // given back once nothing of the call is in flight
+        const ridfa_program *prog;
+        int dev;
+        cudaStream_t st;
+        ScanSpace sp;
+        bool idle = true;
+        ~Space() {
+            if (!idle) cudaStreamSynchronize(st);
+            std::lock_guard<std::mutex> lock(prog->mu);
+            scan_give(prog, dev, sp);
+        }
+    } space{prog, dev, st, {}};
     int err = RIDFA_OK;
-    const DeviceAutomaton *D = device_copy(prog, false, dev, &err);
-    if (!D) return err;
+    {
+        std::lock_guard<std::mutex> lock(prog->mu);
+        const DeviceAutomaton *D = device_copy(prog, false, dev, &err);
+        if (!D) return err;
+        a.A = Automaton{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state, H.n_states, H.n_classes,
+                        H.k, H.kw, H.q0_slot};
+        err = scan_take(prog, dev, &space.sp);
+    }
     // the result words: {first rejecting chunk, status}, on the device and page-locked on the host
-    uint64_t *words = nullptr, *h = nullptr;
-    err = scan_words(prog, dev, 0, &words, &h, nullptr);
+    if (err == RIDFA_OK) err = scan_grow(&space.sp, 0);
     if (err != RIDFA_OK) return err;
     const uint32_t c = n_chunks;
-    ScanArgs a{};
-    a.A = Automaton{D->trans, D->classmap, D->final_bits, D->ifmask, D->slot_state, H.n_states, H.n_classes,
-                    H.k, H.kw, H.q0_slot};
+    uint64_t *words = nullptr;
+    const uint64_t *h = space.sp.host;
+    auto place = [&]() {
+        words = static_cast<uint64_t *>(space.sp.base);
+        a.reject = reinterpret_cast<unsigned long long *>(words);
+        a.status = reinterpret_cast<uint32_t *>(words + 1);
+    };
+    place();
     a.maps = d_maps;
     a.c = c;
     a.entry = d_entry;
-    a.reject = reinterpret_cast<unsigned long long *>(words);
-    a.status = reinterpret_cast<uint32_t *>(words + 1);
     auto blocks = [](uint64_t items, uint64_t per) { return static_cast<unsigned>((items + per - 1) / per); };
     auto fetch = [&]() {
-        e = cudaMemcpyAsync(h, words, 16, cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(space.sp.host, words, 16, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        space.idle = e == cudaSuccess;
         return e;
     };
     auto clear = [&]() {
+        space.idle = false;
         e = cudaMemsetAsync(words, 0xFF, 8, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(words + 1, 0, 8, st);
         return e;
@@ -412,13 +434,11 @@ extern "C" int ridfa_join_scan(const ridfa_program *prog, const uint16_t *d_maps
     if (status & kStatusSeveral) {
         const size_t tile = std::min<size_t>(kScanTile, c - 1), segs = (tile + kScanSeg - 1) / kScanSeg;
         const size_t bytes = (tile * 32 + segs * 33 + kScanTile + 1) * 4;
-        uint32_t *scratch = nullptr;
-        err = scan_words(prog, dev, bytes, &words, &h, &scratch);
+        err = scan_grow(&space.sp, bytes);
         if (err != RIDFA_OK) return err;
-        a.reject = reinterpret_cast<unsigned long long *>(words);
-        a.status = reinterpret_cast<uint32_t *>(words + 1);
+        place();
         if (clear() != cudaSuccess) return cuda_fail(e);
-        a.mats = scratch;
+        a.mats = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(space.sp.base) + 256);
         a.prods = a.mats + tile * 32;
         a.vin = a.prods + segs * 32;
         a.plas = a.vin + segs;
