@@ -76,7 +76,7 @@ typedef struct {
     uint32_t n_classes;      /* byte classes C (bytes read by exactly the same positions) */
     uint32_t n_dfa_states;   /* |Q| of the minimal DFA (0 if not built) */
     uint32_t q0_slot;        /* slot of {q0} */
-    uint64_t table_bytes;    /* device bytes of the RID tables */
+    uint64_t table_bytes;    /* device bytes of the RID tables, those of all kernels they may take */
     uint64_t dfa_table_bytes;/* device bytes of the DFA tables (0 if not built) */
 } ridfa_info;
 
@@ -456,10 +456,13 @@ typedef struct {
     uint32_t reserved;
     uint64_t device_budget;     /* admission by device memory: the resident programs' tables plus,
                                    for every admitted and unfinished request, its arena text and
-                                   its kernel scratch (chunk maps and summaries, 2k + 4 bytes per
-                                   chunk of at least chunk_len -- 1 KiB when adaptive -- plus 64)
-                                   may not exceed this many bytes; 0 = no budget (the arena and
-                                   max_requests alone admit) */
+                                   its kernel scratch may not exceed this many bytes; 0 = no
+                                   budget (the arena and max_requests alone admit).  Scratch: 64
+                                   bytes, and for automata whose runs merge 4 per 96 bytes of
+                                   text; otherwise 2k + 4 per chunk of chunk_len -- 1 KiB when
+                                   adaptive --, or for the set kernels' automata 44 per 512 bytes
+                                   of text if that is more.  Not counted: the batches' launch
+                                   descriptors, some KB each */
 } ridfa_server_opts;
 
 typedef struct {

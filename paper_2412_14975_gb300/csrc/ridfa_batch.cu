@@ -611,6 +611,14 @@ PlanStats plan_stats(const BatchPlan *pl) {
     return s;
 }
 
+uint64_t request_scratch(const HostAutomaton &H, uint64_t len, uint32_t L) {
+    constexpr uint64_t kDescriptors = 64;
+    if (H.stream.kind != kStreamNone) return 4 * std::max<uint64_t>(1, len / kStreamBatchPiece) + kDescriptors;
+    const uint64_t general = (len + L - 1) / L * (2ull * H.k + 4) + kDescriptors;
+    if (!H.set.ok) return general;               // (texts of set programs may take either kernels)
+    return std::max(general, (len + kSetBatchPiece - 1) / kSetBatchPiece * kSetBatchResult + kDescriptors);
+}
+
 int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, const ridfa_batch_item *items,
                uint32_t ni, uint32_t L, int device, const BatchShape &shape) {
     if (!pl || !progs || !np || (ni && !items) || L == 0) return RIDFA_E_ARG;

@@ -17,6 +17,8 @@
 
 namespace ridfa {
 
+struct HostAutomaton;
+
 struct BatchPlan;
 
 BatchPlan *plan_new();
@@ -43,6 +45,10 @@ size_t plan_status_offset(const BatchPlan *pl);  // byte offset of the status wo
 // Host image of the block for a block at device address `base` (pointers inside the
 // descriptors depend on it); `img` holds plan_image_bytes bytes.
 void plan_image(const BatchPlan *pl, uint8_t *base, uint8_t *img);
+
+// Device scratch that a plan takes for a text of `len` bytes, at most: what the kernels that its program takes
+// write per chunk (of L bytes) or piece, and its descriptors.
+uint64_t request_scratch(const HostAutomaton &H, uint64_t len, uint32_t L);
 
 // Streams and events that let the reach launches of one batch (one per table layout or form) run
 // concurrently: the first launch on the caller's stream, the further ones on the streams of aux,

@@ -837,12 +837,8 @@ extern "C" int ridfa_program_info(const ridfa_program *prog, ridfa_info *out) {
     out->n_classes = prog->rid.n_classes;
     out->n_dfa_states = prog->has_dfa ? prog->dfa.n_states : 0;
     out->q0_slot = prog->rid.q0_slot;
-    auto bytes = [](const ridfa::HostAutomaton &A) {
-        return static_cast<uint64_t>(A.trans.size() * 2 + 256 + A.final_bits.size() * 4 +
-                                     A.ifmask.size() * 4 + A.slot_state.size() * 2);
-    };
-    out->table_bytes = bytes(prog->rid);
-    out->dfa_table_bytes = prog->has_dfa ? bytes(prog->dfa) : 0;
+    out->table_bytes = ridfa::device_table_bytes(prog->rid);
+    out->dfa_table_bytes = prog->has_dfa ? ridfa::device_table_bytes(prog->dfa) : 0;
     return RIDFA_OK;
 }
 

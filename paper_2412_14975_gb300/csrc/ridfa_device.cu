@@ -52,43 +52,13 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
     std::vector<uint16_t> iota(H.n_states);
     for (uint32_t i = 0; i < H.n_states; ++i) iota[i] = static_cast<uint16_t>(i);
     // all tables in one host image, one allocation and one copy
-    std::vector<uint8_t> img;
-    auto put = [&](const void *src, size_t n) {
-        const size_t off = img.size();
-        img.resize(off + ((n + 255) & ~static_cast<size_t>(255)));
-        if (n) std::memcpy(img.data() + off, src, n);
-        return off;
-    };
-    auto put_v = [&](const auto &v) { return put(v.data(), v.size() * sizeof(v[0])); };
-    const HostMerge &G = H.merge;
-    const HostStream &T = H.stream;
-    const size_t o_trans = put_v(H.trans), o_cls = put_v(H.classmap), o_fin = put_v(H.final_bits), o_ifm = put_v(H.ifmask),
-                 o_slot = put_v(H.slot_state), o_all = put_v(iota);
-    const bool stream = T.kind != kStreamNone;
-    size_t o_walk = 0, o_edge = 0, o_np = 0, o_ni = 0, o_img = 0, o_part = 0, o_alive = 0, o_code = 0, o_words = 0;
-    if (stream) {
-        o_walk = put_v(G.walk);
-        o_edge = put_v(G.edge_pid);
-        o_np = put_v(G.node_part);
-        o_ni = put_v(G.node_img);
-        o_img = put_v(G.images);
-        o_part = put_v(G.part);
-        o_alive = put_v(G.slot_alive);
-        o_code = put_v(T.byte_code);
-        o_words = put_v(T.words);
-    }
-    const HostSet &Z = H.set;
-    size_t z_next = 0, z_leaf = 0, z_img = 0, z_part = 0, z_mask = 0, z_words = 0, z_bn = 0, z_bi = 0;
-    if (Z.ok) {
-        z_next = put_v(Z.next);
-        z_leaf = put_v(Z.leaf);
-        z_img = put_v(Z.images);
-        z_part = put_v(Z.part);
-        z_mask = put_v(Z.block_mask);
-        z_words = put_v(Z.table.words);
-        z_bn = put_v(Z.back_next);
-        z_bi = put_v(Z.back_images);
-    }
+    std::vector<uint8_t> img(device_table_bytes(H));
+    size_t at[kTables] = {}, end = 0;
+    each_table(H, [&](DeviceTable t, const void *src, size_t n) {
+        at[t] = end;
+        if (n) std::memcpy(img.data() + end, src ? src : iota.data(), n);
+        end += table_room(n);
+    });
     uint8_t *base = nullptr;
     cudaError_t e = cudaMalloc(&base, img.size());
     if (e != cudaSuccess) return cuda_fail(e);
@@ -98,34 +68,34 @@ int upload(const HostAutomaton &H, DeviceAutomaton &D, int dev) try {
         D = DeviceAutomaton{};
         return cuda_fail(e);
     }
-    auto u16 = [&](size_t off) { return reinterpret_cast<uint16_t *>(base + off); };
-    auto u32 = [&](size_t off) { return reinterpret_cast<uint32_t *>(base + off); };
-    D.trans = u16(o_trans);
-    D.classmap = base + o_cls;
-    D.final_bits = u32(o_fin);
-    D.ifmask = u32(o_ifm);
-    D.slot_state = u16(o_slot);
-    D.all_states = u16(o_all);
-    if (stream) {
-        D.mg_walk = u16(o_walk);
-        D.mg_edge_pid = u16(o_edge);
-        D.mg_node_part = u16(o_np);
-        D.mg_node_img = u32(o_ni);
-        D.mg_images = u16(o_img);
-        D.mg_part = u16(o_part);
-        D.mg_slot_alive = u32(o_alive);
-        D.st_code = u32(o_code);
-        D.st_words = u32(o_words);
+    auto u16 = [&](DeviceTable t) { return reinterpret_cast<uint16_t *>(base + at[t]); };
+    auto u32 = [&](DeviceTable t) { return reinterpret_cast<uint32_t *>(base + at[t]); };
+    D.trans = u16(kTabTrans);
+    D.classmap = base + at[kTabClass];
+    D.final_bits = u32(kTabFinal);
+    D.ifmask = u32(kTabIfmask);
+    D.slot_state = u16(kTabSlots);
+    D.all_states = u16(kTabAll);
+    if (H.stream.kind != kStreamNone) {
+        D.mg_walk = u16(kTabWalk);
+        D.mg_edge_pid = u16(kTabEdge);
+        D.mg_node_part = u16(kTabNodePart);
+        D.mg_node_img = u32(kTabNodeImg);
+        D.mg_images = u16(kTabImages);
+        D.mg_part = u16(kTabPart);
+        D.mg_slot_alive = u32(kTabAlive);
+        D.st_code = u32(kTabCode);
+        D.st_words = u32(kTabWords);
     }
-    if (Z.ok) {
-        D.set_next = u16(z_next);
-        D.set_leaf = u32(z_leaf);
-        D.set_images = u16(z_img);
-        D.set_part = base + z_part;
-        D.set_block_mask = u32(z_mask);
-        D.set_words = u32(z_words);
-        D.set_back_next = u16(z_bn);
-        D.set_back_images = u16(z_bi);
+    if (H.set.ok) {
+        D.set_next = u16(kTabSetNext);
+        D.set_leaf = u32(kTabSetLeaf);
+        D.set_images = u16(kTabSetImages);
+        D.set_part = base + at[kTabSetPart];
+        D.set_block_mask = u32(kTabSetMask);
+        D.set_words = u32(kTabSetWords);
+        D.set_back_next = u16(kTabBackNext);
+        D.set_back_images = u16(kTabBackImages);
     }
     D.bytes = img.size();
     return RIDFA_OK;

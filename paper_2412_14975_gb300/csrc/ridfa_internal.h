@@ -122,6 +122,53 @@ constexpr size_t kStreamWalkSmem = 24 * 1024;     // a walk table up to this siz
                                                   // a larger one is read through L1
 constexpr size_t kStreamStaging = 4096;           // per-warp staging (kStreamPair, kStreamSingle)
 
+// The tables of an automaton that go to the device, in the order they have there: f(table, data, bytes).
+// kTabAll (state s for every state s) has no data of its own.
+enum DeviceTable : uint32_t {
+    kTabTrans, kTabClass, kTabFinal, kTabIfmask, kTabSlots, kTabAll,
+    kTabWalk, kTabEdge, kTabNodePart, kTabNodeImg, kTabImages, kTabPart, kTabAlive, kTabCode, kTabWords,
+    kTabSetNext, kTabSetLeaf, kTabSetImages, kTabSetPart, kTabSetMask, kTabSetWords, kTabBackNext, kTabBackImages,
+    kTables
+};
+template <class F>
+void each_table(const HostAutomaton &H, F f) {
+    auto vec = [&](DeviceTable t, const auto &v) { f(t, static_cast<const void *>(v.data()), v.size() * sizeof(v[0])); };
+    vec(kTabTrans, H.trans);
+    vec(kTabClass, H.classmap);
+    vec(kTabFinal, H.final_bits);
+    vec(kTabIfmask, H.ifmask);
+    vec(kTabSlots, H.slot_state);
+    f(kTabAll, static_cast<const void *>(nullptr), static_cast<size_t>(H.n_states) * 2);
+    if (H.stream.kind != kStreamNone) {
+        vec(kTabWalk, H.merge.walk);
+        vec(kTabEdge, H.merge.edge_pid);
+        vec(kTabNodePart, H.merge.node_part);
+        vec(kTabNodeImg, H.merge.node_img);
+        vec(kTabImages, H.merge.images);
+        vec(kTabPart, H.merge.part);
+        vec(kTabAlive, H.merge.slot_alive);
+        vec(kTabCode, H.stream.byte_code);
+        vec(kTabWords, H.stream.words);
+    }
+    if (H.set.ok) {
+        vec(kTabSetNext, H.set.next);
+        vec(kTabSetLeaf, H.set.leaf);
+        vec(kTabSetImages, H.set.images);
+        vec(kTabSetPart, H.set.part);
+        vec(kTabSetMask, H.set.block_mask);
+        vec(kTabSetWords, H.set.table.words);
+        vec(kTabBackNext, H.set.back_next);
+        vec(kTabBackImages, H.set.back_images);
+    }
+}
+// Every table begins on a 256-byte boundary of one block of this many bytes.
+inline size_t table_room(size_t bytes) { return (bytes + 255) & ~static_cast<size_t>(255); }
+inline size_t device_table_bytes(const HostAutomaton &H) {
+    size_t total = 0;
+    each_table(H, [&](DeviceTable, const void *, size_t n) { total += table_room(n); });
+    return total;
+}
+
 // Device copy of one automaton (one per device it was uploaded to).
 struct DeviceAutomaton {
     int device = -1;

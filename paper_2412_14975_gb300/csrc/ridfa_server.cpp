@@ -52,13 +52,6 @@ struct Request {
     Clock::time_point t0;
 };
 
-// Device bytes of a program's tables as uploaded (the same count as ridfa_info.table_bytes).
-uint64_t table_bytes_of(const ridfa_program *prog) {
-    const HostAutomaton &A = prog->rid;
-    return static_cast<uint64_t>(A.trans.size() * 2 + 256 + A.final_bits.size() * 4 + A.ifmask.size() * 4 +
-                                 A.slot_state.size() * 2);
-}
-
 // Ring allocator over [0, cap): ranges are handed out in order and released in any order; space
 // is reclaimed from the oldest live range forward.
 class Ring {
@@ -473,7 +466,7 @@ extern "C" int ridfa_server_add_program(ridfa_server *S, const ridfa_program *pr
         if (!ridfa::device_copy(prog, false, S->device, &err)) return err;
     }
     std::lock_guard<std::mutex> lock(S->mu);
-    const uint64_t tb = ridfa::table_bytes_of(prog);
+    const uint64_t tb = ridfa::device_table_bytes(prog->rid);
     if (S->o.device_budget && S->tables + S->charged + tb > S->o.device_budget) {
         ++S->stats.rejected;
         return RIDFA_E_BUSY;
@@ -503,12 +496,9 @@ extern "C" int ridfa_server_submit(ridfa_server *S, uint32_t prog_slot, const ui
             return RIDFA_E_BUSY;
         }
         if (S->o.device_budget) {
-            // the arena text (a device text is the caller's) and the kernels' per-chunk scratch:
-            // chunk maps (k entries of 2 bytes) and summaries (4 bytes), chunks of at least
-            // chunk_len bytes (1 KiB when adaptive), plus descriptors
-            const uint64_t L = S->o.chunk_len ? S->o.chunk_len : 1024;
-            const uint64_t chunks = len ? (len + L - 1) / L : 0;
-            r.charge = (on_device ? 0 : ridfa::round16(len)) + chunks * (2ull * S->progs[prog_slot]->rid.k + 4) + 64;
+            // the arena text (a device text is the caller's) and the kernels' scratch for it
+            r.charge = (on_device ? 0 : ridfa::round16(len)) +
+                       ridfa::request_scratch(S->progs[prog_slot]->rid, len, S->o.chunk_len ? S->o.chunk_len : 1024);
             if (S->tables + r.charge > S->o.device_budget) return RIDFA_E_TOO_LARGE;
             if (S->tables + S->charged + r.charge > S->o.device_budget) {
                 ++S->stats.rejected;

@@ -750,7 +750,7 @@ void plan_set_batch(SetBatchPlan &P, const StreamBatchSource &src, uint32_t sms)
     uint64_t bytes = 0;
     for (const auto &it : src.items) bytes += it.len;
     // one round of pieces for the SMs' lanes, none longer than the others
-    const uint64_t piece = std::max<uint64_t>(512, bytes / (static_cast<uint64_t>(sms) * kSetBlock) + 1);
+    const uint64_t piece = std::max<uint64_t>(kSetBatchPiece, bytes / (static_cast<uint64_t>(sms) * kSetBlock) + 1);
     for (const auto &it : src.items) {
         StreamBatchText t{it.text, it.len, 0, P.pieces, 0, 0, it.item};
         // (one block joins a text's pieces, 23 ns each: longer ones for a text of very many, 64 MB in two
@@ -764,7 +764,7 @@ void plan_set_batch(SetBatchPlan &P, const StreamBatchSource &src, uint32_t sms)
     P.grid = std::min<uint32_t>(sms, (P.pieces + 31) / 32);
     P.o_bases = (P.texts.size() * sizeof(StreamBatchText) + 255) & ~static_cast<size_t>(255);
     P.image_bytes = P.o_bases + P.bases.size() * 4;
-    P.result_bytes = static_cast<size_t>(P.pieces) * (kSetRuns * 2 + 8 + 4);
+    P.result_bytes = static_cast<size_t>(P.pieces) * kSetBatchResult;
 }
 
 void set_batch_image(const SetBatchPlan &P, uint8_t *img) {

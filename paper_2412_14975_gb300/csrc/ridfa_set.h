@@ -34,6 +34,8 @@ cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st);
 // The texts of one program of a batch, each of kSetBatchText bytes or more, on `grid` SMs: only accept
 // bits are asked for, so a piece is entered through the interface slots, as a chunk is.
 constexpr uint64_t kSetBatchText = 32;         // (as deep as the graph may be)
+constexpr uint64_t kSetBatchPiece = 512;       // bytes a piece has at least, but a text's last
+constexpr size_t kSetBatchResult = kSetRuns * 2 + 8 + 4;     // bytes of scratch a piece
 // Text a batch's launch has to have.  (50 texts of 16 KB against 3 REs, one of them the codon RE: 242 us
 // with its texts in the general kernel, 58 us in this one; 30 texts of 2 KB: 181 and 56.)
 constexpr uint64_t kSetBatchBytes = 4096;

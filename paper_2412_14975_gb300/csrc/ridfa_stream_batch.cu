@@ -285,7 +285,7 @@ void plan_stream_batch(StreamBatchPlan &P, std::vector<StreamBatchSource> &src, 
     // program, about 150 KB through them); pieces of about 96 bytes then.  Otherwise two rounds of
     // pieces a lane, so that the shares even out.
     P.walk_only = P.bytes / blocks < 96 * 1024;
-    uint64_t piece = 96;
+    uint64_t piece = kStreamBatchPiece;
     if (!P.walk_only) {
         for (uint32_t p = 0; p < np; ++p)
             if (cost > 0) lanes += batch_warps(H[p]->stream) * 32.0 * (static_cast<double>(bytes[p]) * time_of(H[p]->stream) / cost);

@@ -11,6 +11,7 @@
 namespace ridfa {
 
 constexpr uint32_t kStreamBatchProgs = 64;       // programs of one plan at most
+constexpr uint64_t kStreamBatchPiece = 96;       // bytes a piece has at least, but a text of one piece
 // Shared memory that launches which run side by side take at least: over half of an SM's, so that each
 // of their blocks has an SM to itself (blocks of small tables otherwise met on one SM while others
 // stood idle).
