@@ -355,11 +355,12 @@ int ridfa_last_status(const ridfa_program *prog, void *stream);
  * events.  Errors: E_ARG (no profiled call yet), E_CUDA. */
 int ridfa_last_timings(const ridfa_program *prog, float *reach_ms, float *join_ms);
 
-/* The reach plan of the last ridfa_recognize / ridfa_recognize_dfa / ridfa_recognize_host call of
- * `prog` on the current device (diagnostics; the automatic choices the tuning fields override).
- * A call with the automatic tuning on an automaton whose runs merge runs in the stream kernels,
- * which have tables and a launch shape of their own; the report then describes the general reach
- * kernel's plan for the same call, the one that explicit tuning fields start from. */
+/* The general reach kernel's plan for the last ridfa_recognize / ridfa_recognize_dfa /
+ * ridfa_recognize_host call of `prog` on the current device (diagnostics; the automatic choices the
+ * tuning fields override, which explicit fields start from).  The call ran by that plan only where
+ * ridfa_last_kernel says general: with the automatic tuning, automata whose runs merge take the
+ * stream kernels, and most automata over at most four bytes whose runs stay apart the set kernels;
+ * both have tables and launch shapes of their own. */
 typedef struct {
     uint32_t table_mode;    /* table layout, numbered as ridfa_tuning::table_mode (1..11) */
     uint32_t text_path;     /* 1 global loads, 3 staged, 4 staged two chunks a lane, 5 set path */
@@ -370,6 +371,23 @@ typedef struct {
 } ridfa_plan_report;
 /* Errors: E_ARG (prog or out NULL, or no call on this device yet), E_CUDA. */
 int ridfa_last_plan(const ridfa_program *prog, ridfa_plan_report *out);
+
+/* The kernels that the same call ran in (diagnostics). */
+#define RIDFA_KERNEL_GENERAL 1u     /* ridfa_last_plan has the plan */
+#define RIDFA_KERNEL_STREAM 2u      /* runs that merge: one lane per chunk or piece */
+#define RIDFA_KERNEL_STREAM_WALK 3u /* the same in one-byte steps throughout (short texts) */
+#define RIDFA_KERNEL_SET 4u         /* runs that stay apart, over at most four bytes */
+typedef struct {
+    uint32_t kernel;           /* RIDFA_KERNEL_* */
+    uint32_t lookup_bytes;     /* text bytes per table lookup (0: general) */
+    uint32_t entry_bytes;      /* bytes of a table entry (0: general) */
+    uint32_t lane_copies;      /* copies of the table in shared memory (0: general) */
+    uint32_t pieces_per_chunk; /* pieces each chunk was cut into (0: general) */
+    uint32_t block_threads;    /* of the reach launch */
+    uint32_t grid_blocks;
+} ridfa_kernel_report;
+/* Errors: E_ARG (prog or out NULL, or no call on this device yet), E_CUDA. */
+int ridfa_last_kernel(const ridfa_program *prog, ridfa_kernel_report *out);
 
 /* ---- Batched recognition (the paper recognises one text at a time; a batch runs the same
  * reach and join, exactly, for many (text, program) items at once).

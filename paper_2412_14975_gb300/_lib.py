@@ -76,7 +76,15 @@ class PlanReport(_c.Structure):
                 ("block_threads", _u32), ("grid_blocks", _u32), ("pieces", _u32)]
 
 
+class KernelReport(_c.Structure):
+    _fields_ = [("kernel", _u32), ("lookup_bytes", _u32), ("entry_bytes", _u32), ("lane_copies", _u32),
+                ("pieces_per_chunk", _u32), ("block_threads", _u32), ("grid_blocks", _u32)]
+
+
+KERNELS = {1: "general", 2: "stream", 3: "stream_walk", 4: "set"}
+
 _decl("ridfa_last_plan", _c.c_int, [_vp, _c.POINTER(PlanReport)])
+_decl("ridfa_last_kernel", _c.c_int, [_vp, _c.POINTER(KernelReport)])
 
 
 class RidfaError(RuntimeError):
@@ -291,11 +299,23 @@ def ridfa_last_status(prog, stream=None):
 
 
 def ridfa_last_plan(prog):
-    """The reach plan of the program's last recognition on the current device: dict with
-    table_mode, text_path, lane_copies, block_threads, grid_blocks, pieces."""
+    """The general reach kernel's plan for the program's last recognition on the current device: dict
+    with table_mode, text_path, lane_copies, block_threads, grid_blocks, pieces.  The call ran by it
+    only where ridfa_last_kernel says "general"."""
     out = PlanReport()
     _check(_lib.ridfa_last_plan(prog, _c.byref(out)), "ridfa_last_plan")
     return {f: getattr(out, f) for f, _ in out._fields_}
+
+
+def ridfa_last_kernel(prog):
+    """What the program's last recognition on the current device ran in: dict with kernel ("general",
+    "stream", "stream_walk" or "set"), lookup_bytes, entry_bytes, lane_copies, pieces_per_chunk,
+    block_threads, grid_blocks."""
+    out = KernelReport()
+    _check(_lib.ridfa_last_kernel(prog, _c.byref(out)), "ridfa_last_kernel")
+    rep = {f: getattr(out, f) for f, _ in out._fields_}
+    rep["kernel"] = KERNELS[rep["kernel"]]
+    return rep
 
 
 def ridfa_last_timings(prog):

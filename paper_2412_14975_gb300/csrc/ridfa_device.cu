@@ -1023,6 +1023,7 @@ int recognize_stream(const ridfa_program *P, const HostAutomaton &H, const Devic
     NvtxRange range("ridfa reach");
     e = stream_launch(C, sh, st);
     if (e != cudaSuccess) return cuda_fail(e);
+    S->last_kernel = stream_report(H, sh);
     if (prof) {
         cudaEventRecord(static_cast<cudaEvent_t>(S->ev[2]), st);
         S->profiled = true;
@@ -1069,6 +1070,7 @@ int recognize_set(const ridfa_program *P, const HostAutomaton &H, const DeviceAu
     NvtxRange range("ridfa reach");
     e = set_launch(C, sms, st);
     if (e != cudaSuccess) return cuda_fail(e);
+    S->last_kernel = set_report(H, n_chunks, spc, sms);
     if (prof) {
         cudaEventRecord(static_cast<cudaEvent_t>(S->ev[2]), st);
         S->profiled = true;
@@ -1156,6 +1158,7 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
     DeviceScratch *S = scratch_for(P, dev, L.total, &err);
     if (!S) return err;
     S->last_plan = G.report();
+    S->last_kernel = {RIDFA_KERNEL_GENERAL, 0, 0, 0, 0, S->last_plan.block_threads, S->last_plan.grid_blocks};
     S->planned = true;
     S->stream_call = false;
     uint8_t *base = static_cast<uint8_t *>(S->base);
@@ -1490,6 +1493,19 @@ extern "C" int ridfa_last_plan(const ridfa_program *prog, ridfa_plan_report *out
                 s.stream_call = false;
             }
             *out = s.last_plan;
+            return RIDFA_OK;
+        }
+    return RIDFA_E_ARG;
+}
+
+extern "C" int ridfa_last_kernel(const ridfa_program *prog, ridfa_kernel_report *out) {
+    if (!prog || !out) return RIDFA_E_ARG;
+    std::lock_guard<std::mutex> lock(prog->mu);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return ridfa::cuda_fail(cudaGetLastError());
+    for (const auto &s : prog->scratch)
+        if (s.device == dev && s.planned) {
+            *out = s.last_kernel;
             return RIDFA_OK;
         }
     return RIDFA_E_ARG;

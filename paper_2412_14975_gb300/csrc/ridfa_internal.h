@@ -230,6 +230,7 @@ struct DeviceScratch {
     void *ev[3] = {nullptr, nullptr, nullptr};   // cudaEvent_t: before reach, before join, after
     bool profiled = false;
     ridfa_plan_report last_plan{};               // the reach plan of the last call on this device
+    ridfa_kernel_report last_kernel{};           // what it ran in
     bool planned = false;
     bool stream_call = false;                    // the last call took the stream kernels: its plan on the
     bool stream_dfa = false;                     // general path is worked out when asked for

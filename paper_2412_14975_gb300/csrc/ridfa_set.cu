@@ -656,6 +656,15 @@ size_t set_scratch(uint32_t c, uint32_t spc) {
     return (n + c) * (2 * kSetRuns * 2 + 8) + static_cast<size_t>(c) * 4 + static_cast<size_t>(set_join_blocks(c)) * kSetRuns * 4 + 64 * 256;
 }
 
+namespace {
+uint32_t set_grid(uint64_t pieces, int sms) { return static_cast<uint32_t>(std::min<uint64_t>(sms, (pieces + 31) / 32)); }
+}  // namespace
+
+ridfa_kernel_report set_report(const HostAutomaton &H, uint32_t c, uint32_t spc, int sms) {
+    const HostStream &T = H.set.table;
+    return {RIDFA_KERNEL_SET, T.group, T.entry, T.copies, spc, kSetBlock, set_grid(static_cast<uint64_t>(c) * spc, sms)};
+}
+
 cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     const HostAutomaton &H = *C.H;
     const DeviceAutomaton &D = *C.D;
@@ -685,7 +694,7 @@ cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {
     a.pids = pids;
     SetJoinArgs j{};
     const size_t smem = set_args(H, D, a, j);
-    cudaError_t e = set_reach(H, a, static_cast<uint32_t>(std::min<uint64_t>(sms, (pieces + 31) / 32)), smem, st);
+    cudaError_t e = set_reach(H, a, set_grid(pieces, sms), smem, st);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;

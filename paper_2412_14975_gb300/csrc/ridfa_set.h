@@ -29,6 +29,7 @@ struct SetCall {
 // Pieces the set kernels cut each chunk into; 0: the call is not theirs.
 uint32_t set_pieces(const HostAutomaton &H, uint64_t len, uint32_t c, int sms);
 size_t set_scratch(uint32_t c, uint32_t spc);
+ridfa_kernel_report set_report(const HostAutomaton &H, uint32_t c, uint32_t spc, int sms);
 cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st);
 
 // The texts of one program of a batch, each of kSetBatchText bytes or more, on `grid` SMs: only accept

@@ -724,6 +724,12 @@ StreamShape stream_shape(const HostAutomaton &H, uint64_t len, uint32_t c, int s
     return S;
 }
 
+ridfa_kernel_report stream_report(const HostAutomaton &H, const StreamShape &S) {
+    const HostStream &T = H.stream;
+    if (S.walk_only) return {RIDFA_KERNEL_STREAM_WALK, 1, 2, 1, S.per_chunk, S.block, S.grid};
+    return {RIDFA_KERNEL_STREAM, T.group, T.entry, T.copies, S.per_chunk, S.block, S.grid};
+}
+
 cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_t st) {
     const HostAutomaton &H = *C.H;
     const DeviceAutomaton &D = *C.D;

@@ -43,6 +43,7 @@ struct StreamCall {
 
 bool stream_takes(const HostAutomaton &H, uint64_t len, uint32_t c);
 StreamShape stream_shape(const HostAutomaton &H, uint64_t len, uint32_t c, int sms);
+ridfa_kernel_report stream_report(const HostAutomaton &H, const StreamShape &S);
 cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_t st);
 
 }  // namespace ridfa
