@@ -380,6 +380,7 @@ int ridfa_last_plan(const ridfa_program *prog, ridfa_plan_report *out);
 typedef struct {
     uint32_t kernel;           /* RIDFA_KERNEL_* */
     uint32_t lookup_bytes;     /* text bytes per table lookup (0: general) */
+    uint32_t class_lookups;    /* class lookups per text byte (0: general, or classes by arithmetic) */
     uint32_t entry_bytes;      /* bytes of a table entry (0: general) */
     uint32_t lane_copies;      /* copies of the table in shared memory (0: general) */
     uint32_t pieces_per_chunk; /* pieces each chunk was cut into (0: general) */
@@ -391,10 +392,16 @@ int ridfa_last_kernel(const ridfa_program *prog, ridfa_kernel_report *out);
 
 /* ---- Batched recognition (the paper recognises one text at a time; a batch runs the same
  * reach and join, exactly, for many (text, program) items at once).
- * All items' chunks run in one persistent reach launch per shared-memory table layout (CTAs take
- * tasks of up to 32 chunks per warp of one program from an atomic ticket and reload their tables
- * only when the program changes) followed by one join launch over all texts; create() captures
- * these launches into a CUDA graph that run() replays. */
+ * Texts of programs whose runs merge take the stream kernels, one reach and one join launch per
+ * table form; texts of at least 32 bytes of up to 16 programs whose runs stay apart, over at most
+ * four bytes and with at least 4 KB of such texts, take the set kernels, two launches a program.
+ * All other items' chunks run in one persistent reach launch per shared-memory table layout (CTAs
+ * take tasks of up to 32 chunks per warp of one program from an atomic ticket and reload their
+ * tables only when the program changes) followed by one join launch over their texts.  The launches
+ * run side by side; create() captures them into a CUDA graph that run() replays.
+ * The stream and set kernels cut texts by a rule of their own: n_chunks, chunk_len, block_warps and
+ * set_mode below concern the texts of the general kernels (accept bits do not depend on how a text
+ * is cut), and chunk_len == 0 times no batch whose programs' runs all merge. */
 typedef struct {
     const uint8_t *d_text;   /* device pointer (16-byte alignment of every text enables the
                                 cooperative staged text path; otherwise global loads are used) */
@@ -420,9 +427,9 @@ typedef struct {
 
 typedef struct {
     uint64_t total_bytes;
-    uint64_t total_chunks;
+    uint64_t total_chunks;   /* by n_chunks and chunk_len, whichever kernels a text takes */
     uint32_t n_programs, n_launches, n_tasks, n_segments;
-    uint32_t chunk_len;      /* the chunk length in use */
+    uint32_t chunk_len;      /* the chunk length in use (for the general kernels' texts) */
     uint32_t block_warps;    /* warps per block cap in use (0: as many as fit) */
     uint32_t set_mode;       /* run interleave in use (0/1 set path, 2 one run per lane) */
     uint32_t graph;          /* 1 if run() launches a CUDA graph */
