@@ -828,8 +828,9 @@ def main():
     lut_rate = lib.ridfa_bench_smem_gather(1 << 16) / 1e9
     text_rate = n / (reach_ms / 1e3) / 1e9
     # (the library's own choice; any override takes the general kernel)
-    override = args.table_mode or args.text_path or args.piece_len or args.probe
-    reach_kernel = "rid_reach_kernel" if override else "rid_set_kernel" if name == "c2" else "rid_stream_kernel"
+    ran = lib.ridfa_last_kernel(prog)
+    reach_kernel = {"general": "rid_reach_kernel", "stream": "rid_stream_kernel", "stream_walk": "rid_stream_walk_kernel",
+                    "set": "rid_set_kernel"}[ran["kernel"]]
     traffic = None
     if name == REACH_TRAFFIC["workload"] and args.table_mode == 0 and args.text_path == 0 and c == 155648:
         traffic = int(REACH_TRAFFIC["dram_bytes_per_text_byte"] * n)
@@ -906,11 +907,16 @@ def main():
             work.update({"nfa_w_paper_per_byte": round(nc["w_paper"] / n, 5),
                          "transition_ratio_nfa_over_rid": round(nc["w_paper"] / max(rc["w_paper"], 1), 4)})
         work["count_s"] = round(time.perf_counter() - t0, 2)
-        lpb = 1 + rc["w_conv"] / n
+        # lookups per byte of the kernel that ran: a class each (but for field codes) and a table step of one
+        # or more bytes, for the one run of a merged piece or for every live run
+        if ran["kernel"] == "general":
+            lpb = 1 + rc["w_conv"] / n / (2 if lib.ridfa_last_plan(prog)["table_mode"] >= 8 else 1)
+        else:
+            runs = rc["w_conv"] / n if ran["kernel"] == "set" else 1
+            lpb = ran["class_lookups"] + runs / ran["lookup_bytes"]
         roofline["smem_gather"]["lookups_per_byte"] = round(lpb, 5)
-        # the binding roof: the slower of the text at HBM bandwidth and the lookups of one-byte steps
-        # at the measured gather rate (the microbenchmark does 2 lookups per byte); kernels that step
-        # two or four bytes a lookup may pass the latter
+        # the binding roof: the slower of the text at HBM bandwidth and those lookups at the measured
+        # gather rate (the microbenchmark does 2 lookups per byte, free of bank conflicts)
         lut_text_rate = lut_rate * 2.0 / lpb
         roofline["smem_gather"]["roof_text_GBps"] = round(lut_text_rate, 1)
         roofline["smem_gather"]["roof_frac"] = round(text_rate / lut_text_rate, 4)

@@ -77,7 +77,7 @@ class PlanReport(_c.Structure):
 
 
 class KernelReport(_c.Structure):
-    _fields_ = [("kernel", _u32), ("lookup_bytes", _u32), ("entry_bytes", _u32), ("lane_copies", _u32),
+    _fields_ = [("kernel", _u32), ("lookup_bytes", _u32), ("class_lookups", _u32), ("entry_bytes", _u32), ("lane_copies", _u32),
                 ("pieces_per_chunk", _u32), ("block_threads", _u32), ("grid_blocks", _u32)]
 
 
@@ -309,8 +309,8 @@ def ridfa_last_plan(prog):
 
 def ridfa_last_kernel(prog):
     """What the program's last recognition on the current device ran in: dict with kernel ("general",
-    "stream", "stream_walk" or "set"), lookup_bytes, entry_bytes, lane_copies, pieces_per_chunk,
-    block_threads, grid_blocks."""
+    "stream", "stream_walk" or "set"), lookup_bytes, class_lookups, entry_bytes, lane_copies,
+    pieces_per_chunk, block_threads, grid_blocks."""
     out = KernelReport()
     _check(_lib.ridfa_last_kernel(prog, _c.byref(out)), "ridfa_last_kernel")
     rep = {f: getattr(out, f) for f, _ in out._fields_}

@@ -1158,7 +1158,7 @@ int recognize_impl(const ridfa_program *P, bool use_dfa, const uint8_t *d_text, 
     DeviceScratch *S = scratch_for(P, dev, L.total, &err);
     if (!S) return err;
     S->last_plan = G.report();
-    S->last_kernel = {RIDFA_KERNEL_GENERAL, 0, 0, 0, 0, S->last_plan.block_threads, S->last_plan.grid_blocks};
+    S->last_kernel = {RIDFA_KERNEL_GENERAL, 0, 0, 0, 0, 0, S->last_plan.block_threads, S->last_plan.grid_blocks};
     S->planned = true;
     S->stream_call = false;
     uint8_t *base = static_cast<uint8_t *>(S->base);

@@ -662,7 +662,7 @@ uint32_t set_grid(uint64_t pieces, int sms) { return static_cast<uint32_t>(std::
 
 ridfa_kernel_report set_report(const HostAutomaton &H, uint32_t c, uint32_t spc, int sms) {
     const HostStream &T = H.set.table;
-    return {RIDFA_KERNEL_SET, T.group, T.entry, T.copies, spc, kSetBlock, set_grid(static_cast<uint64_t>(c) * spc, sms)};
+    return {RIDFA_KERNEL_SET, T.group, 0, T.entry, T.copies, spc, kSetBlock, set_grid(static_cast<uint64_t>(c) * spc, sms)};
 }
 
 cudaError_t set_launch(const SetCall &C, int sms, cudaStream_t st) {

@@ -94,7 +94,7 @@ struct StreamJoinArgs {
     const uint16_t *tables;  // of the groups that did not merge (kTableResult)
     uint32_t per_chunk;      // pieces (or groups of them) per chunk
     uint32_t chunks;         // chunks per block
-    uint32_t k_magic;        // ceil(2^32 / k): e / k = umulhi(e, k_magic) for e < 2^16
+    uint32_t k_magic;        // ceil(2^32 / k): e / k = umulhi(e, k_magic) while e * k < 2^32 (e <= 257 k here)
     uint32_t *status;        // the call's status, written once by publish(); while it runs its bits are in j.status
     uint8_t *h_accept;
     uint32_t *h_status;
@@ -726,8 +726,8 @@ StreamShape stream_shape(const HostAutomaton &H, uint64_t len, uint32_t c, int s
 
 ridfa_kernel_report stream_report(const HostAutomaton &H, const StreamShape &S) {
     const HostStream &T = H.stream;
-    if (S.walk_only) return {RIDFA_KERNEL_STREAM_WALK, 1, 2, 1, S.per_chunk, S.block, S.grid};
-    return {RIDFA_KERNEL_STREAM, T.group, T.entry, T.copies, S.per_chunk, S.block, S.grid};
+    if (S.walk_only) return {RIDFA_KERNEL_STREAM_WALK, 1, 1, 2, 1, S.per_chunk, S.block, S.grid};
+    return {RIDFA_KERNEL_STREAM, T.group, T.kind == kStreamField ? 0u : 1u, T.entry, T.copies, S.per_chunk, S.block, S.grid};
 }
 
 cudaError_t stream_launch(const StreamCall &C, const StreamShape &S, cudaStream_t st) {
