@@ -754,8 +754,8 @@ int plan_build(BatchPlan *pl, const ridfa_program *const *progs, uint32_t np, co
         P.groups.push_back(g);
     }
     // The stream and set launches and the general groups run side by side, a block of any filling an SM:
-    // each gets SMs by its share of the work (the general kernels take some four times the time per
-    // byte), the general groups no more than they have tasks.
+    // each gets SMs by its share of the work (the general kernels take kGeneralWeight times a two-byte stream
+    // table's time per byte), the general groups no more than they have tasks.
     const uint64_t other_bytes = P.total_bytes - stream_bytes - all_set_bytes;
     double work = static_cast<double>(stream_bytes) + kGeneralWeight * static_cast<double>(other_bytes);
     for (size_t i = 0; i < set_sources.size(); ++i) work += set_batch_weight(*set_sources[i].H) * static_cast<double>(set_bytes[i]);

@@ -72,7 +72,7 @@ struct HostStream {
 };
 
 // Automata whose runs stay apart, over an alphabet of at most four bytes (set kernels, ridfa_set.cu): the
-// functions that the first `depth` bytes perform on the interface slots, all of which have at most
+// functions that the first `depth` bytes perform on the interface slots, all of which have fewer than
 // kSetRuns distinct values, so that a lane takes up a chunk's runs after walking `depth` edges.
 struct HostSet {
     bool ok = false;

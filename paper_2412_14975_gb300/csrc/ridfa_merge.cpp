@@ -17,8 +17,8 @@ namespace ridfa {
 namespace {
 
 // Limits of the graph: inner nodes (codon-like automata, whose runs stay apart, run into it),
-// entries of the partition table, and the images stepped while building (compile time: a step is
-// about 10 ns, so 1.5 M keep the construction under some 15 ms).
+// entries of the partition table, and the images stepped while building (compile time: 500,000 steps with
+// their partitions take up to some 20 ms on one core, which a graph over the limits costs for nothing).
 constexpr uint32_t kMaxInner = 6144;
 constexpr uint32_t kMaxInnerApart = 1536;      // without the merge hint
 constexpr uint64_t kMaxPartEntries = 1u << 20;

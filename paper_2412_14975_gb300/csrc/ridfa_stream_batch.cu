@@ -23,8 +23,7 @@ namespace {
 
 struct StreamBatchProg {
     uint32_t n;                  // states
-    uint32_t form;               // which instantiation of Steps
-    uint32_t k, kw, q0_slot, n_texts, np;
+    uint32_t kw, q0_slot, n_texts, np;
     uint32_t inner, n_images;    // nodes of the graph and their images
     const StreamBatchText *texts;
     const uint32_t *bases;
@@ -392,8 +391,6 @@ void stream_batch_image(const StreamBatchPlan &P, uint8_t *dev, uint32_t *res, u
         const DeviceAutomaton &D = *P.D[p];
         StreamBatchProg b{};
         b.n = H.n_states;
-        b.form = form_of(H.stream);
-        b.k = H.k;
         b.kw = H.kw;
         b.q0_slot = H.q0_slot;
         b.n_texts = (p + 1 < P.H.size() ? P.text0[p + 1] : static_cast<uint32_t>(P.texts.size())) - P.text0[p];

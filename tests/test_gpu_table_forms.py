@@ -1,7 +1,7 @@
 """GPU stream kernels on the table forms, each asserted to be the one that runs: fields of one and two bits by two
 and four bytes a lookup, pairs and single bytes, entries of one and two bytes, few and many lane copies.  Chunk
-maps against the general kernels' and accept bits against the serial host recognizer, single texts and batches;
-and what ridfa_last_kernel says of stream, set and general calls.  Tolerance 0."""
+maps against the general kernels' and accept bits against the serial host recognizer, single texts and batches.
+Tolerance 0."""
 import numpy as np
 import pytest
 
